@@ -1,0 +1,194 @@
+"""The work that users of the actor library have it do, as timed cases.
+
+A case names a scenario shape (agents, observation width, actions - the four of ``workloads.config``), a batch of
+environments, a hidden size, a precision and one of the public entry points:
+
+  rollout   ``Actor.rollout_staged``: T steps on environment output that is already on the device; with ``publish`` the
+            learner's new model is published first and takes effect halfway through the rollout
+  typed     the same with one network per unit type (``set_weights_typed``)
+  step      ``Actor.step``: one decision step, device buffers
+  host      ``Actor.step_host``: one decision step, host buffers (simulators on the host), copies and wait included
+  subset    ``Actor.step_subset``: one decision step for the environments of a list that changes from call to call
+  lagged    ``Actor.step_lagged``: the same, each action's outcome arriving with the next observation
+  sample    ``Actor.ring_sample``: the learner draws B episodes from the filled replay ring
+
+A pass returns everything it brings up to date: the ring (records and slot headers), the recurrent state and cursors,
+and the actions; the sampler returns its batch.
+"""
+import math
+
+import numpy as np
+import torch
+
+from paper_2205_05248_b200 import workloads
+from paper_2205_05248_b200.binding import Actor
+
+# scenario -> index of the workload that carries its shape, probabilities and exploration schedule
+SCENARIO = {"3m": 1, "8m": 2, "2s3z": 3, "5m_vs_6m": 4, "8m_sweep": 5}
+STEP_INPUTS = 8      # different inputs that the one-step cases take in turn, as a running worker would
+SAMPLE_DONE = 0.05   # end-of-game probability behind the sampler's ring: episodes of about 20 steps
+
+
+def listed():
+    return [
+        # one decision of a small worker (eight games of three agents): launch and latency
+        dict(name="step_3m_fp32", kind="step", scenario="3m", E=8, H=64, precision="fp32", S=8, L=32),
+        # simulators on the host: observations in, actions out, every step over the link
+        dict(name="host_8m", kind="host", scenario="8m", E=1024, H=64, precision="bf16", S=2, L=128),
+        # asynchronous actors: half of the environments have an observation ready
+        dict(name="subset_8m", kind="subset", scenario="8m_sweep", E=65536, M=32768, H=64, precision="bf16", S=1, L=32),
+        # the same with late outcomes, on rows that are not 16-byte multiples and a list of odd length
+        dict(name="lagged_5m_vs_6m", kind="lagged", scenario="5m_vs_6m", E=16384, M=9001, H=64, precision="bf16", S=1, L=64),
+        # an actor-learner iteration of ordinary size: a new model every rollout
+        dict(name="rollout_8m_publish", kind="rollout", scenario="8m", E=1024, H=64, precision="bf16", T=128, S=2, L=128, publish=True),
+        # two unit types, annealed exploration, availability rows that are not word-aligned
+        dict(name="rollout_2s3z", kind="rollout", scenario="2s3z", E=4096, H=64, precision="bf16", T=256, S=2, L=256, publish=False),
+        # observation rows that are not 16-byte multiples
+        dict(name="rollout_5m_vs_6m", kind="rollout", scenario="5m_vs_6m", E=16384, H=64, precision="bf16", T=128, S=1, L=128, publish=False),
+        # the largest batch of the throughput sweep
+        dict(name="rollout_8m_large", kind="rollout", scenario="8m_sweep", E=65536, H=64, precision="bf16", T=64, S=1, L=64, publish=False),
+        # the sweep's larger network
+        dict(name="rollout_8m_h128", kind="rollout", scenario="8m_sweep", E=16384, H=128, precision="bf16", T=64, S=1, L=96, publish=False),
+        # the sweep in full precision
+        dict(name="rollout_8m_fp32", kind="rollout", scenario="8m_sweep", E=4096, H=64, precision="fp32", T=64, S=2, L=96, publish=False),
+        # a heterogeneous team with a network per unit type
+        dict(name="typed_2s3z_fp32", kind="typed", scenario="2s3z", E=1024, H=64, precision="fp32", T=64, S=2, L=256),
+        # the learner's batch
+        dict(name="sample_8m", kind="sample", scenario="8m_sweep", E=4096, B=1024, H=64, precision="bf16", S=4, L=96),
+    ]
+
+
+def _log_int(rng, lo, hi):
+    return int(round(math.exp(rng.uniform(math.log(lo), math.log(hi)))))
+
+
+def draw(rng):
+    """One more case: every entry point, shape, precision and hidden size; sizes over their logarithm, mostly odd."""
+    kind = rng.choice(["rollout", "rollout", "rollout", "typed", "step", "host", "subset", "lagged", "sample"])
+    scenario = rng.choice(["3m", "8m", "2s3z", "5m_vs_6m"])
+    precision = rng.choice(["bf16", "bf16", "fp32"])
+    H = rng.choice([64, 64, 128])
+    c = dict(kind=kind, scenario=scenario, H=H, precision=precision, S=rng.choice([1, 2]), L=rng.choice([32, 64, 96]))
+    n = workloads.config(SCENARIO[scenario])["n"]
+    # relative cost of an agent step, so that no drawn case costs more than the largest listed one
+    weight = (12.0 if precision == "fp32" else 1.0) * (4.0 if H == 128 else 1.0)
+    most = 65536 * 8 * 64 / weight
+    if kind in ("rollout", "typed"):
+        c["T"] = _log_int(rng, 8, 128)
+        if kind == "typed":
+            c["scenario"], n, most = "2s3z", 5, most / (12.0 if precision == "bf16" else 1.0) / 2
+        else:
+            c["publish"] = rng.random() < 0.25
+        c["E"] = _log_int(rng, 8, max(16, min(65536, most / (n * c["T"]))))
+    elif kind == "sample":
+        c["E"], c["S"], c["B"] = _log_int(rng, 64, 4096), 4, _log_int(rng, 16, 1024)
+    elif kind == "host":
+        c["E"] = _log_int(rng, 8, 8192)
+    else:
+        c["E"] = _log_int(rng, 8, 65536 if precision == "bf16" else 16384)
+        if kind != "step":
+            c["M"] = max(1, int(c["E"] * rng.uniform(0.1, 1.0)))
+    return c
+
+
+def _config(case, seed):
+    """The workload's configuration at the case's size; every random stream follows from the seed."""
+    cfg = dict(workloads.config(SCENARIO[case["scenario"]]))
+    cfg.update(E=case["E"], C=case["E"] * case["S"], L=case["L"], H=case["H"], precision=case["precision"],
+               T=case.get("T", 1), seed=cfg["seed"] + 7919 * (seed + 1))
+    cfg["env"] = dict(cfg["env"], seed=cfg["seed"])
+    if case["kind"] == "typed":
+        cfg = workloads.typed(cfg)
+    return cfg
+
+
+def prepare(case, seed):
+    cfg = _config(case, seed)
+    kind, E, T = case["kind"], case["E"], case.get("T", 1)
+    n, env = cfg["n"], cfg["env"]
+    weights = workloads.make_weights_typed(cfg) if kind == "typed" else workloads.make_weights(cfg)
+    actor = Actor(cfg, work_steps=16 if kind == "sample" else 1)
+    if kind == "typed":
+        actor.set_weights_typed(weights)
+    else:
+        actor.set_weights(weights)
+    st = dict(kind=kind, cfg=cfg, actor=actor, T=T, turn=0, eps=cfg["eps_end"])
+    if kind == "sample":
+        env = dict(env, done_thresh24=workloads.thresh24(SAMPLE_DONE))
+        actor.rollout(env, 2 * case["S"] * 20, cfg["eps_start"])
+        st.update(B=case["B"])
+        return st
+    ring, state = actor.ring_view(), actor.get_state()
+    st["out"] = dict({k: ring[k] for k in ("obs", "avail", "action", "q", "reward", "done", "slot_epid", "slot_len", "slot_complete")},
+                     **{k: state[k] for k in ("h", "last_action", "slot", "pos", "ep_count")})
+    if kind in ("rollout", "typed"):
+        st["inputs"] = actor.env_generate(env, 0, T)
+        if case.get("publish"):
+            st["models"] = [workloads.make_weights(cfg, seed=cfg["seed"] + 1 + k) for k in range(2)]
+        return st
+    obs, avail, reward, done = actor.env_generate(env, 0, STEP_INPUTS)
+    if kind == "host":
+        obs, avail, reward, done = (t.cpu().pin_memory() for t in (obs, avail, reward, done))
+        st["actions"] = torch.empty((E, n), dtype=torch.int32).pin_memory()
+    elif kind == "step":
+        st["actions"] = torch.empty((E, n), dtype=torch.int32, device=actor.device)
+    else:
+        M = case["M"]
+        rng = np.random.Generator(np.random.Philox(key=cfg["seed"]))
+        st["lists"] = [rng.permutation(E)[:M].astype(np.int32) for _ in range(STEP_INPUTS)]
+        st["actions"] = torch.empty((M, n), dtype=torch.int32, device=actor.device)
+        obs, avail, reward, done = (t[:, :M].contiguous() for t in (obs, avail, reward, done))
+    st["inputs"] = [(obs[k], avail[k], reward[k], done[k]) for k in range(STEP_INPUTS)]
+    st["out"]["actions"] = st["actions"]
+    return st
+
+
+def run(st):
+    kind, actor, cfg = st["kind"], st["actor"], st["cfg"]
+    turn = st["turn"]
+    st["turn"] = turn + 1
+    if kind in ("rollout", "typed"):
+        if "models" in st:
+            actor.publish_weights(st["models"][turn % 2], version=turn + 2, effective_step=turn * st["T"] + st["T"] // 2)
+        actor.rollout_staged(*st["inputs"], st["T"], cfg["eps_start"], cfg["eps_end"], cfg["anneal_steps"])
+    elif kind == "sample":
+        return actor.ring_sample(turn, st["B"])
+    elif kind == "step":
+        actor.step(*st["inputs"][turn % STEP_INPUTS], st["eps"], st["actions"])
+    elif kind == "host":
+        actor.step_host(*st["inputs"][turn % STEP_INPUTS], st["eps"], st["actions"])
+    elif kind == "subset":
+        actor.step_subset(st["lists"][turn % STEP_INPUTS], *st["inputs"][turn % STEP_INPUTS], st["eps"], st["actions"])
+    else:
+        actor.step_lagged(st["lists"][turn % STEP_INPUTS], *st["inputs"][turn % STEP_INPUTS], st["eps"], st["actions"])
+    return st["out"]
+
+
+def work(case):
+    """Input once, record payload once, recurrent state in and out once a call, the network once; the products of the
+    network (one-hot columns as adds) and some 25 operations per hidden unit for the gates."""
+    cfg = _config(case, 0)
+    n, D, A, H, L = cfg["n"], cfg["D"], cfg["A"], case["H"], case["L"]
+    payload = n * (4 * D + A + 4 + 4 * A) + 5  # of one recorded environment step
+    if case["kind"] == "sample":
+        q = 1.0 - SAMPLE_DONE
+        mean = (1.0 - q ** L) / SAMPLE_DONE
+        return {"bytes": case["B"] * (mean + L) * payload, "flops": 0}
+    envs, T = case.get("M", case["E"]), case.get("T", 1)
+    wbytes = 2 if case["precision"] == "bf16" else 4
+    net = (H * (D + n + A) + 6 * H * H + A * H) * wbytes * (2 if case["kind"] == "typed" else 1)
+    state = 2 * (n * (4 * H + 4) + 16)
+    return {"bytes": envs * (T * (n * (4 * D + A) + 5 + payload) + state) + net,
+            "flops": envs * n * T * (2.0 * H * (D + 6 * H + A) + 25.0 * H)}
+
+
+def tolerance(case):
+    """Measured by running the cases with the hidden units of the network in another order (the same function, its sums
+    in another order) and, for bf16, on the CUDA-core kernel (another implementation at the same precision).  Without a
+    decision that differs the results agree to 3e-7 (fp32) and 8e-4 (bf16, whose operands are rounded).  But a greedy
+    choice whose runner-up lies at the edge of the tie band may go the other way, and the row's last action, hidden
+    state and Q differ from there to the end of its episode.  Over 16.8 million fp32 decisions that gave rel 1.7e-4, 7e-7
+    of the whole values and single values off by 0.6 of the root mean square; for bf16 rel 4e-3 and 4e-4."""
+    if case["precision"] == "fp32":
+        return {"rel": 7e-4, "max": 0.99, "differ": 1e-4}
+    return {"rel": 1.6e-2, "max": 0.99, "differ": 2e-3}
