@@ -26,6 +26,11 @@ from paper_2205_05248_b200.binding import Actor
 # scenario -> index of the workload that carries its shape, probabilities and exploration schedule
 SCENARIO = {"3m": 1, "8m": 2, "2s3z": 3, "5m_vs_6m": 4, "8m_sweep": 5}
 STEP_INPUTS = 8      # different inputs that the one-step cases take in turn, as a running worker would
+# Rollouts run with every action drawn, as workers do before a policy is learned.  The network, the greedy choice and the
+# draw are evaluated in every step whatever the rate; but a followed greedy choice whose runner-up lies at the edge of the
+# tie band goes either way in two correct implementations and sends the rest of its episode elsewhere, and over millions
+# of decisions that would hide real differences.  The one-step cases follow the greedy choice.
+EXPLORE = 1.0
 SAMPLE_DONE = 0.05   # end-of-game probability behind the sampler's ring: episodes of about 20 steps
 
 
@@ -41,7 +46,7 @@ def listed():
         dict(name="lagged_5m_vs_6m", kind="lagged", scenario="5m_vs_6m", E=16384, M=9001, H=64, precision="bf16", S=1, L=64),
         # an actor-learner iteration of ordinary size: a new model every rollout
         dict(name="rollout_8m_publish", kind="rollout", scenario="8m", E=1024, H=64, precision="bf16", T=128, S=2, L=128, publish=True),
-        # two unit types, annealed exploration, availability rows that are not word-aligned
+        # two unit types, availability rows that are not word-aligned
         dict(name="rollout_2s3z", kind="rollout", scenario="2s3z", E=4096, H=64, precision="bf16", T=256, S=2, L=256, publish=False),
         # observation rows that are not 16-byte multiples
         dict(name="rollout_5m_vs_6m", kind="rollout", scenario="5m_vs_6m", E=16384, H=64, precision="bf16", T=128, S=1, L=128, publish=False),
@@ -115,7 +120,7 @@ def prepare(case, seed):
     st = dict(kind=kind, cfg=cfg, actor=actor, T=T, turn=0, eps=cfg["eps_end"])
     if kind == "sample":
         env = dict(env, done_thresh24=workloads.thresh24(SAMPLE_DONE))
-        actor.rollout(env, 2 * case["S"] * 20, cfg["eps_start"])
+        actor.rollout(env, 2 * case["S"] * 20, EXPLORE)
         st.update(B=case["B"])
         return st
     ring, state = actor.ring_view(), actor.get_state()
@@ -150,7 +155,7 @@ def run(st):
     if kind in ("rollout", "typed"):
         if "models" in st:
             actor.publish_weights(st["models"][turn % 2], version=turn + 2, effective_step=turn * st["T"] + st["T"] // 2)
-        actor.rollout_staged(*st["inputs"], st["T"], cfg["eps_start"], cfg["eps_end"], cfg["anneal_steps"])
+        actor.rollout_staged(*st["inputs"], st["T"], EXPLORE, EXPLORE, cfg["anneal_steps"])
     elif kind == "sample":
         return actor.ring_sample(turn, st["B"])
     elif kind == "step":
@@ -183,12 +188,12 @@ def work(case):
 
 
 def tolerance(case):
-    """Measured by running the cases with the hidden units of the network in another order (the same function, its sums
-    in another order) and, for bf16, on the CUDA-core kernel (another implementation at the same precision).  Without a
-    decision that differs the results agree to 3e-7 (fp32) and 8e-4 (bf16, whose operands are rounded).  But a greedy
-    choice whose runner-up lies at the edge of the tie band may go the other way, and the row's last action, hidden
-    state and Q differ from there to the end of its episode.  Over 16.8 million fp32 decisions that gave rel 1.7e-4, 7e-7
-    of the whole values and single values off by 0.6 of the root mean square; for bf16 rel 4e-3 and 4e-4."""
-    if case["precision"] == "fp32":
-        return {"rel": 7e-4, "max": 0.99, "differ": 1e-4}
-    return {"rel": 1.6e-2, "max": 0.99, "differ": 2e-3}
+    """About four times what the cases and 34 drawn ones show when the hidden units of the network are put in another order
+    (the same function, its sums in another order) and, for bf16, on the CUDA-core kernel (another implementation at the
+    same precision): rollouts and samples rel 3.3e-7, max 2.6e-6 in fp32 and 5.1e-4, 1.7e-2 in bf16, no whole value differs.
+    The one-step cases follow the greedy choice, which goes the other way at the edge of the tie band in up to 2e-5 of the
+    bf16 rows (1e-6 in fp32) and then moves single values of the next step by more than their root mean square: rel 7.2e-4."""
+    fp32 = case["precision"] == "fp32"
+    if case["kind"] in ("rollout", "typed", "sample"):
+        return {"rel": 1.4e-6, "max": 1.1e-5, "differ": 0.0} if fp32 else {"rel": 2e-3, "max": 7e-2, "differ": 0.0}
+    return {"rel": 3e-4, "max": 0.99, "differ": 4e-6} if fp32 else {"rel": 3e-3, "max": 0.99, "differ": 8e-5}
