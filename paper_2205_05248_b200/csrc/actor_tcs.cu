@@ -1,0 +1,1262 @@
+// Split-operand tensor-core actor kernel for sm_100a: fp32 accuracy from bf16 tcgen05.mma, hidden size 64 or 128.
+//
+// An fp32 value is the exact sum of three bf16 values (8 + 8 + 8 significand bits, each rounded to nearest), and a
+// product of two bf16 values is exact in fp32.  So a matrix product of fp32 operands is the sum of the products of
+// their pieces: with x = x0 + x1 + x2 and w = w0 + w1 + w2 the six products of order 2^-16 and above are formed; what
+// is left out is below 2^-24 of |x||w|.  The accumulator of tcgen05.mma adds with truncation, so the order matters:
+// the five small products go first, while the accumulator is small, and x0 w0 last - few truncations at full
+// magnitude.  Measured on 128 x 80 x 64 products of uniform operands: rms error 4.7e-8, largest 3.0e-7; a chain of
+// fp32 fused multiply-adds: 9.4e-8 and 6.1e-7 (the six products interleaved K step by K step: 2.9e-7 and 2.1e-6).
+// With one piece (NS = 1) the same kernel is the bf16 precision with accurate gate functions.
+//
+// One thread block owns a tile of whole environments (up to 128 agent rows) and runs all T steps of the launch for it.
+// Weights stay in shared memory as far as they fit (hidden 64: all of them); the rest streams from L2 through a ring
+// of slices, every step again.  The left operands - observations, fc1 output, hidden state - are written to tensor
+// memory and read from there by tcgen05.mma (an A operand in shared memory costs at least 32 clocks a product, one in
+// tensor memory 3 at N = 16, 27 at N = 64); only the observations and the fc1 output of the three-piece hidden-128
+// variant live in shared memory.  Nothing assumes an alignment beyond that of the element type, and a tile's rows may
+// be those of a list (partial steps) or of one unit type (per-type networks: the block runs its tiles once per type,
+// on the rows of that type, with that type's network).
+//
+// Roles: warps 0-7 epilogue (two groups of 128 threads; a thread owns one row and 16 columns of every block of 32
+// hidden columns), warps 8-11 inputs and records (thread = row), warp 12 issues every tcgen05.mma (from the lane that
+// elect.sync picks: ptxas then knows that one lane runs and issues without a loop over lanes; 4 products take 325-400
+// clocks to completion against 577-700 behind "lane == 0"), warp 13 loads weights.
+// Per step:
+//   E1 (epilogue)  y = relu(fc1 + agent column + last-action column), pieces to the y operand
+//   E2 (epilogue)  per block of 32 hidden columns: gates, new hidden state (fp32 in registers); the next block's
+//                  products run meanwhile; then its pieces to the hidden operand
+//   E3 (group 0)   masked greedy choice
+//   inputs (beside E2) of the next step: ring cursor and headers, availability mask, epsilon draw, observation pieces
+//                  and record; then this step's Q record
+#include <cstring>
+
+#include "common.cuh"
+#include "launch_util.cuh"
+#include "tcgen05.cuh"
+
+namespace marl {
+
+constexpr int TS_EPI = 256, TS_PREP = 128, TS_THREADS = 512;
+constexpr int TS_ROWS = 128;
+constexpr int TS_BLK = 32;          // hidden columns of a gate block
+constexpr uint32_t TS_SMEM_MAX = 232448;
+constexpr int TS_MAX_SLOTS = 8;
+constexpr int TS_KCHUNK = 96;       // K of one W1 slice: no larger than a gate slice
+// Tensor-memory columns.  Two accumulator buffers of a gate block, laid out so that the columns fc1 uses at hidden 64
+// (the candidate-input parts of both) are contiguous: HN R Z IN | IN R Z HN.
+constexpr uint32_t TSM_HOP = 256, TSM_Q = 480;
+
+struct TsLayout {
+  int32_t Dk, NQ, nw1, nsl, nres, nslots;   // K of fc1; Q columns; W1 slices; slices; resident ones; ring slots
+  int32_t ept, ntypes;
+  uint32_t base_bytes, off_b2, off_bias, off_tabA, off_tabL;  // base part of the image: W2 pieces, biases, column tables
+  uint32_t img_bytes;
+  uint32_t off_sl, off_ring, off_xy, off_scr, off_recp, off_sel, off_pick, off_la, off_close, off_eid, off_row, off_bar, total;
+};
+
+struct TsBars {
+  uint64_t xrdy, fc1d, hset, yrdy, gd[2], accf[2], hr0, hr1, fc2d, qfree, res[2];
+  uint64_t full[TS_MAX_SLOTS], empty[TS_MAX_SLOTS];
+  uint32_t tmem_base, abort;
+};
+
+__host__ __device__ constexpr uint32_t ts_slice(int H) { return 96u * (uint32_t)H * 2u; }
+
+static uint32_t ts_up(uint32_t v, uint32_t a) { return (v + a - 1) / a * a; }
+
+// Bytes of slice i (order of use: W1, smallest pieces first; then per block the pieces of both gate matrices).
+__host__ __device__ inline uint32_t ts_slice_bytes(const TsLayout& L, int H, int ns, int i) {
+  if (i >= L.nw1) return ts_slice(H);
+  const int c = ns == 3 ? 0 : i;
+  const int k = L.Dk - c * TS_KCHUNK;
+  return (uint32_t)(k < TS_KCHUNK ? k : TS_KCHUNK) * (uint32_t)H * 2u;
+}
+__host__ __device__ inline uint32_t ts_slice_off(const TsLayout& L, int H, int ns, int i) {  // within the slices' part
+  const int w = i < L.nw1 ? i : L.nw1;
+  const uint32_t w1 = ns == 3 ? (uint32_t)w * (uint32_t)L.Dk * (uint32_t)H * 2u
+                              : (uint32_t)(w * TS_KCHUNK < L.Dk ? w * TS_KCHUNK : L.Dk) * (uint32_t)H * 2u;
+  return w1 + (uint32_t)(i - w) * ts_slice(H);
+}
+
+// The image of one network: [W2 pieces | biases and tables (fp32) | slices].
+static TsLayout ts_image(int n, int D, int A, int H, int ns) {
+  TsLayout L;
+  memset(&L, 0, sizeof(L));
+  L.Dk = (D + 15) & ~15;
+  L.NQ = A <= 16 ? 16 : 32;
+  L.nw1 = ns == 3 ? 3 : (L.Dk + TS_KCHUNK - 1) / TS_KCHUNK;
+  L.nsl = L.nw1 + (H / TS_BLK) * 2 * ns;
+  uint32_t o = (uint32_t)ns * (uint32_t)H * L.NQ * 2;
+  L.off_b2 = o; o += 32 * 4;
+  L.off_bias = o; o += 4u * H * 4;
+  L.off_tabA = o; o += (uint32_t)n * (H + 4) * 4;
+  L.off_tabL = o; o += (uint32_t)A * (H + 4) * 4;
+  L.base_bytes = ts_up(o, 128);
+  L.img_bytes = ts_up(L.base_bytes + ts_slice_off(L, H, ns, L.nsl), 256);
+  return L;
+}
+
+// nt_max: rows of an environment in one tile (the agents, or those of the largest unit type).  ept = 0: does not fit.
+static TsLayout ts_layout(int n, int D, int A, int H, int ns, int nt_max, int M, int sms) {
+  TsLayout L = ts_image(n, D, A, H, ns);
+  int ept = TS_ROWS / nt_max;
+  if (M > 0 && sms > 0) {  // even the tiles out over the waves they need anyway
+    const int tiles = (M + ept - 1) / ept, waves = (tiles + sms - 1) / sms;
+    const int e2 = (M + waves * sms - 1) / (waves * sms);
+    if (e2 < ept) ept = e2;
+  }
+  L.ept = ept;
+  uint32_t o = L.base_bytes;
+  L.off_xy = o;
+  if (ns == 3 && H == 128) o += 3u * (uint32_t)(L.Dk > H ? L.Dk : H) * TS_ROWS * 2;
+  L.off_scr = o; o += (TS_PREP / 32) * 2048;
+  L.off_bar = o; o += (uint32_t)sizeof(TsBars);
+  L.off_recp = o; o += 4u * (uint32_t)ept * 8;
+  L.off_sel = o; o += 4u * TS_ROWS * 4;
+  L.off_la = o; o += TS_ROWS * 4;
+  L.off_close = o; o += 4u * (uint32_t)ept * 4;
+  L.off_eid = o; o += (uint32_t)ept * 4;
+  L.off_pick = o; o += 4u * TS_ROWS;
+  L.off_row = o; o += TS_ROWS * 2;
+  o = ts_up(o, 128);
+  L.off_sl = o;
+  // resident slices: all of them, or what is left beside the ring (three slots where two slices are held at once)
+  const uint32_t all = ts_slice_off(L, H, ns, L.nsl);
+  if (o + all <= TS_SMEM_MAX) {
+    L.nres = L.nsl;
+    L.nslots = 0;
+    L.off_ring = L.total = o + all;
+    return L;
+  }
+  L.nslots = ns == 3 ? 3 : 2;
+  if (o + (uint32_t)L.nslots * ts_slice(H) > TS_SMEM_MAX) {
+    L.ept = 0;
+    return L;
+  }
+  const uint32_t room = TS_SMEM_MAX - o - (uint32_t)L.nslots * ts_slice(H);
+  while (ts_slice_off(L, H, ns, L.nres + 1) <= room) L.nres += 1;
+  L.off_ring = o + ts_slice_off(L, H, ns, L.nres);
+  while (L.nslots < TS_MAX_SLOTS && L.off_ring + (uint32_t)(L.nslots + 1) * ts_slice(H) <= TS_SMEM_MAX) L.nslots += 1;
+  L.total = L.off_ring + (uint32_t)L.nslots * ts_slice(H);
+  return L;
+}
+
+static int ts_pieces(int prec) { return prec == MARL_PRECISION_FP32 ? 3 : 1; }
+
+// Shapes this kernel takes: the operands fit their tensor-memory columns and what must be resident fits shared memory.
+// At hidden 64 everything is resident (the products are issued in an order that is not the stream's).
+bool tcs_supported(int n, int D, int A, int H, int prec) {
+  const int ns = ts_pieces(prec);
+  const TsLayout L = ts_layout(n, D, A, H, ns, 1, 0, 0);  // one-row environments: the largest per-tile arrays
+  if (L.ept == 0) return false;
+  if (H == 64 && L.nres < L.nsl) return false;
+  if (ns == 3 && L.Dk > TS_KCHUNK) return false;
+  const int xcols = ns * (L.Dk > H ? L.Dk : H) / 2;
+  return (ns == 3 && H == 128) || (int)TSM_HOP + ns * H / 2 + xcols <= (int)TSM_Q;
+}
+
+size_t tcs_image_bytes(int n, int D, int A, int H, int prec) {
+  return tcs_supported(n, D, A, H, prec) ? ts_image(n, D, A, H, ts_pieces(prec)).img_bytes : 0;
+}
+
+static uint16_t ts_bf16(float v) {  // round to nearest even
+  uint32_t u;
+  memcpy(&u, &v, 4);
+  if ((u & 0x7FFFFFFFu) > 0x7F800000u) return (uint16_t)(u >> 16);
+  u += 0x7FFFu + ((u >> 16) & 1u);
+  return (uint16_t)(u >> 16);
+}
+static float ts_float(uint16_t b) {
+  const uint32_t u = (uint32_t)b << 16;
+  float v;
+  memcpy(&v, &u, 4);
+  return v;
+}
+
+constexpr float TS_LOG2E = 1.44269504088896340736f;
+
+// One network into its image.  A matrix slice is [K / 8][rows][8] bf16.  Rows of a gate slice follow the accumulator
+// columns of the block's buffer: y side R Z IN (buffer 0) or IN R Z, hidden side HN R Z or R Z HN.
+void tcs_pack_weights(int n, int D, int A, int H, int prec, const float* W1, const float* b1, const float* Wih,
+                      const float* bih, const float* Whh, const float* bhh, const float* W2, const float* b2, uint8_t* dst) {
+  const int ns = ts_pieces(prec);
+  const TsLayout L = ts_image(n, D, A, H, ns);
+  const int I = D + n + A;
+  memset(dst, 0, L.img_bytes);
+  auto piece = [&](float v, int i) {  // piece i of v
+    for (int k = 0; k < i; ++k) v -= ts_float(ts_bf16(v));
+    return ts_bf16(v);
+  };
+  uint16_t* w2 = reinterpret_cast<uint16_t*>(dst);
+  for (int i = 0; i < ns; ++i)
+    for (int a = 0; a < A; ++a)
+      for (int k = 0; k < H; ++k) w2[(((size_t)i * (H / 8) + k / 8) * L.NQ + a) * 8 + k % 8] = piece(W2[(size_t)a * H + k], i);
+  uint8_t* sl = dst + L.base_bytes;
+  for (int s = 0; s < L.nw1; ++s) {
+    uint16_t* w = reinterpret_cast<uint16_t*>(sl + ts_slice_off(L, H, ns, s));
+    const int k0 = ns == 3 ? 0 : s * TS_KCHUNK, k1 = ns == 3 || k0 + TS_KCHUNK > D ? D : k0 + TS_KCHUNK;
+    for (int j = 0; j < H; ++j)
+      for (int k = k0; k < k1; ++k)
+        w[((size_t)((k - k0) / 8) * H + j) * 8 + k % 8] = piece(W1[(size_t)j * I + k], ns == 3 ? 2 - s : 0);
+  }
+  // gate slices of a block: three pieces h2 h1 y2 y1 h0 y0, one piece h0 y0
+  static const int order3[6][2] = {{1, 2}, {1, 1}, {0, 2}, {0, 1}, {1, 0}, {0, 0}}, order1[2][2] = {{1, 0}, {0, 0}};
+  for (int b = 0; b < H / TS_BLK; ++b) {
+    const int buf = H == 64 ? b : (b + 1) & 1;
+    for (int s = 0; s < 2 * ns; ++s) {
+      const int hid = ns == 3 ? order3[s][0] : order1[s][0], pc = ns == 3 ? order3[s][1] : order1[s][1];
+      const float* W = hid ? Whh : Wih;
+      uint16_t* w = reinterpret_cast<uint16_t*>(sl + ts_slice_off(L, H, ns, L.nw1 + b * 2 * ns + s));
+      // gate blocks of the source are r | z | n
+      static const int rows_y[2][3] = {{0, 1, 2}, {2, 0, 1}}, rows_h[2][3] = {{2, 0, 1}, {0, 1, 2}};
+      for (int g = 0; g < 3; ++g)
+        for (int j = 0; j < TS_BLK; ++j) {
+          const int src = (hid ? rows_h : rows_y)[buf][g] * H + b * TS_BLK + j;
+          for (int k = 0; k < H; ++k) w[((size_t)(k / 8) * 96 + g * TS_BLK + j) * 8 + k % 8] = piece(W[(size_t)src * H + k], pc);
+        }
+    }
+  }
+  memcpy(dst + L.off_b2, b2, sizeof(float) * A);
+  // biases: reset and update as the sigmoid's exponent wants them, candidate input, candidate hidden
+  float* bias = reinterpret_cast<float*>(dst + L.off_bias);
+  for (int j = 0; j < H; ++j) {
+    bias[j] = -TS_LOG2E * (bih[j] + bhh[j]);
+    bias[H + j] = -TS_LOG2E * (bih[H + j] + bhh[H + j]);
+    bias[2 * H + j] = bih[2 * H + j];
+    bias[3 * H + j] = bhh[2 * H + j];
+  }
+  auto col = [&](float v) { return ns == 1 ? ts_float(ts_bf16(v)) : v; };
+  float* tabA = reinterpret_cast<float*>(dst + L.off_tabA);
+  float* tabL = reinterpret_cast<float*>(dst + L.off_tabL);
+  for (int j = 0; j < H; ++j) {
+    for (int i = 0; i < n; ++i) tabA[i * (H + 4) + j] = b1[j] + col(W1[(size_t)j * I + D + i]);
+    for (int a = 0; a < A; ++a) tabL[a * (H + 4) + j] = col(W1[(size_t)j * I + D + n + a]);
+  }
+}
+
+// ------------------------------------------------------------------------------------------------
+namespace {
+
+__device__ __forceinline__ void ts_arrive(uint64_t* bar, int lane) {  // one arrival per warp
+  __syncwarp();
+  if (lane == 0) tc::mbar_arrive(bar);
+}
+
+__device__ __forceinline__ uint32_t ts_pack2(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+
+// The pieces of 16 consecutive values of this thread's row: piece i as 8 packed words to put(i, words).
+template <int NS, typename Put>
+__device__ __forceinline__ void ts_split16(float (&v)[16], Put put) {
+#pragma unroll
+  for (int i = 0; i < NS; ++i) {
+    uint32_t w[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      w[j] = ts_pack2(v[2 * j], v[2 * j + 1]);
+      if (i + 1 < NS) {
+        v[2 * j] -= __uint_as_float(w[j] << 16);
+        v[2 * j + 1] -= __uint_as_float(w[j] & 0xFFFF0000u);
+      }
+    }
+    put(i, w);
+  }
+}
+
+__device__ __forceinline__ float ts_ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float ts_rcp(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// sigmoid(v) with s = -log2(e) v: 1 / (1 + 2^s).  The approximate exponential's 2^-22.5 enters with weight
+// sigmoid (1 - sigmoid) <= 1/4.
+__device__ __forceinline__ float ts_sigmoid(float s) { return ts_rcp(1.0f + ts_ex2(s)); }
+// tanh: below 0.6 the odd polynomial u + u^3 P(u^2), P a degree-4 minimax fit (weighted least squares iterated to equal
+// ripple, 2.8e-9), else 1 - 2 / (1 + e^(2 |u|)), where the exponential's error has faded to an ulp.
+__device__ __forceinline__ float ts_tanh(float u) {
+  const float a = fabsf(u);
+  const float big = fmaf(-2.0f, ts_rcp(1.0f + ts_ex2(2.0f * TS_LOG2E * a)), 1.0f);
+  const float z = u * u;
+  float p = fmaf(-0.00589515688f, z, 0.0207959712f);
+  p = fmaf(p, z, -0.0537838303f);
+  p = fmaf(p, z, 0.133319244f);
+  p = fmaf(p, z, -0.333332986f);
+  const float small = fmaf(p * z, u, u);
+  return a < 0.6f ? small : copysignf(big, u);
+}
+
+// D (+)= A B^T, issued by one lane; A in shared memory (AS: descriptor) or in tensor memory (column address).
+template <bool AS>
+__device__ __forceinline__ void ts_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+  if (AS) tc::mma_bf16(d, a, b, idesc, acc);
+  else tc::mma_bf16_ts(d, (uint32_t)a, b, idesc, acc);
+}
+
+}  // namespace
+
+template <int NS, int NQ, int H>
+__global__ void __launch_bounds__(TS_THREADS, 1)
+    actor_tcs_kernel(const __grid_constant__ ActorParams p, const __grid_constant__ TsLayout L) {
+  using namespace tc;
+  constexpr int NBLK = H / TS_BLK, KH = H / 16;
+  constexpr bool XS = NS == 3 && H == 128;       // x and y pieces in shared memory
+  constexpr uint32_t TSM_XY = TSM_HOP + NS * H / 2;
+  constexpr uint32_t FC1 = H == 64 ? 96 : 0;     // fc1's accumulator: the candidate-input columns, or buffer 0
+  // Registers (setmaxnreg): launched with 128 a thread (512 * 128 = 65536); afterwards
+  // 256 * 144 + 128 * 128 + 128 * 96 or, hidden 128, 256 * 176 + 128 * 112 + 128 * 48 = 65536.
+  constexpr int REGS_EPI = H == 64 ? 144 : 176, REGS_PREP = H == 64 ? 128 : 112, REGS_SVC = H == 64 ? 96 : 48;
+  extern __shared__ __align__(1024) uint8_t smem[];
+  TsBars* B = reinterpret_cast<TsBars*>(smem + L.off_bar);
+  // per-step hand-offs, four buffers each: the input warps run up to two steps ahead of the choice
+  unsigned long long* recp_s = reinterpret_cast<unsigned long long*>(smem + L.off_recp);  // [4][ept] record of the step, 0: none
+  uint32_t* mask_s = reinterpret_cast<uint32_t*>(smem + L.off_sel);                       // [4][128] availability
+  int8_t* pick_s = reinterpret_cast<int8_t*>(smem + L.off_pick);                          // [4][128] random pick or -1
+  int32_t* close_s = reinterpret_cast<int32_t*>(smem + L.off_close);                      // [4][ept] the episode ends with the step
+  int32_t* la_s = reinterpret_cast<int32_t*>(smem + L.off_la);
+  int32_t* eid_s = reinterpret_cast<int32_t*>(smem + L.off_eid);                          // environment's index in the actor
+  uint8_t* rowel_s = smem + L.off_row;                                                    // [128] environment of the row, in the tile
+  uint8_t* rowag_s = rowel_s + TS_ROWS;                                                   // [128] agent of the row
+  const float* b2_s = reinterpret_cast<const float*>(smem + L.off_b2);
+  const float* bias_s = reinterpret_cast<const float*>(smem + L.off_bias);
+  volatile uint32_t* abortf = &B->abort;
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int n = p.n, D = p.D, A = p.A, T = p.T, ept = L.ept;
+  const bool lag = p.lagged != 0;
+  const int ntypes = L.ntypes;
+  const uint32_t rec_bytes = p.rl.rec_bytes;
+
+  if (tid == 0) {
+    mbar_init(&B->xrdy, TS_PREP / 32);
+    mbar_init(&B->fc1d, 1);
+    mbar_init(&B->hset, TS_EPI / 32);
+    mbar_init(&B->yrdy, TS_EPI / 32);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&B->gd[i], 1);
+      mbar_init(&B->accf[i], TS_EPI / 32);
+      mbar_init(&B->res[i], 1);
+    }
+    mbar_init(&B->hr0, TS_EPI / 32);
+    mbar_init(&B->hr1, TS_EPI / 32);
+    mbar_init(&B->fc2d, 1);
+    mbar_init(&B->qfree, TS_PREP / 32);
+    for (int i = 0; i < TS_MAX_SLOTS; ++i) {
+      mbar_init(&B->full[i], 1);
+      mbar_init(&B->empty[i], 1);
+    }
+    B->abort = 0;
+    mbar_init_fence();
+  }
+  if (warp == 12) tmem_alloc(&B->tmem_base, 512);
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+  const uint32_t tmem = B->tmem_base;
+  auto rows_per_env = [&](int typ) -> int {  // of a pass: the agents of its unit type
+    int nt = ntypes > 1 ? 0 : n;
+    if (ntypes > 1)
+      for (int i = 0; i < n; ++i) nt += (int)((p.agent_type_bits >> (2 * i)) & 3ull) == typ ? 1 : 0;
+    return nt;
+  };
+  const int my_tiles = blockIdx.x < p.num_tiles ? (p.num_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+
+  if (warp >= 12) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_SVC));
+    if (warp == 12) {
+      // =========================== MMA warp ===========================
+      const uint32_t sb = smem_u32(smem);
+      constexpr uint32_t id96 = idesc_bf16_f32(128, 96), id64 = idesc_bf16_f32(128, 64), id32 = idesc_bf16_f32(128, 32),
+                         idH = idesc_bf16_f32(128, H), idq = idesc_bf16_f32(128, NQ);
+      constexpr uint64_t ks_1 = (2 * H * 16) >> 4, ks_g = (2 * 96 * 16) >> 4, ks_q = (2 * NQ * 16) >> 4, st_q = (H / 16) * ks_q;
+      const int nk1 = L.Dk / 16;
+      // the left operands and the distance between their pieces and K steps
+      const uint64_t a_h = tmem + TSM_HOP;
+      constexpr uint64_t h_st = H / 2, h_ks = 8;
+      const uint64_t a_x = XS ? smem_desc(sb + L.off_xy, 2048, 128) : (uint64_t)(tmem + TSM_XY);
+      constexpr uint64_t x_ks = XS ? (2 * 2048) >> 4 : 8;
+      const uint64_t x_st = (uint64_t)nk1 * x_ks;
+      constexpr uint64_t y_st = KH * x_ks;
+      uint32_t g = 0, ri = 0, rpar = 0;  // steps so far; ring slot and its parity
+      uint32_t typ = 0;
+      bool first = true;
+
+      // slice i of the step: its address once it is in shared memory
+      auto get = [&](int i) -> uint32_t {
+        if (i < L.nres) {
+          if (first) mbar_wait(&B->res[i < L.nw1 ? 0 : 1], typ & 1, abortf);
+          return sb + L.off_sl + ts_slice_off(L, H, NS, i);
+        }
+        mbar_wait(&B->full[ri], rpar, abortf);
+        return sb + L.off_ring + ri * ts_slice(H);
+      };
+      auto next_slot = [&]() {
+        if (++ri == (uint32_t)L.nslots) { ri = 0; rpar ^= 1u; }
+      };
+      auto desc = [&](uint32_t addr, uint32_t lbo) { return smem_desc(addr, lbo, 128); };
+
+      // gate products of one piece pair over all K steps (the y side's first one starts the candidate-input columns)
+      auto prod_h = [&](int buf, uint32_t ai, uint64_t w, uint32_t acc) {
+        const uint32_t d = tmem + (buf ? 160u : 0u);
+#pragma unroll
+        for (int ks = 0; ks < KH; ++ks) ts_mma<false>(d, a_h + ai * h_st + ks * h_ks, w + ks * ks_g, id96, ks ? 1u : acc);
+      };
+      auto prod_y = [&](int buf, uint32_t ai, uint64_t w, bool start) {
+        const uint32_t d = tmem + (buf ? 128u : 32u);
+        const uint64_t a = a_x + ai * y_st;
+        if (start) {
+          // buffer 0: R Z at rows 0.., IN at rows 64..; buffer 1: IN at rows 0.., R Z at rows 32..
+          const uint64_t w_in = w + (buf ? 0 : (64 * 16) >> 4), w_rz = w + (buf ? (32 * 16) >> 4 : 0);
+          ts_mma<XS>(d + (buf ? 0u : 64u), a, w_in, id32, 0);
+          ts_mma<XS>(d + (buf ? 32u : 0u), a, w_rz, id64, 1);
+        } else {
+          ts_mma<XS>(d, a, w, id96, 1);
+        }
+#pragma unroll
+        for (int ks = 1; ks < KH; ++ks) ts_mma<XS>(d, a + ks * x_ks, w + ks * ks_g, id96, 1);
+      };
+
+      for (; typ < (uint32_t)ntypes; ++typ) {
+        if (typ > 0) __syncthreads();  // every role has left the previous type
+        first = true;
+        for (int tile = blockIdx.x; tile < p.num_tiles; tile += gridDim.x)
+          for (int s = 0; s < T; ++s, ++g, first = false) {
+            const uint32_t par = g & 1;
+            // ---- fc1 ----
+            mbar_wait(&B->xrdy, par, abortf);  // (E2 of the previous step has read the columns: hr1)
+            tc_fence_after_sync();
+            {
+              uint32_t acc = 0;
+              for (int i = 0; i < L.nw1; ++i) {
+                const uint64_t w = desc(get(i), H * 16);
+                if (elect_one()) {
+                  if (NS == 3) {  // piece 2 - i against the small products' left pieces, then the main product
+                    for (int ai = i == 2 ? 2 : i; ai >= (i == 2 ? 1 : 0); --ai)
+                      for (int ks = 0; ks < nk1; ++ks) {
+                        ts_mma<XS>(tmem + FC1, a_x + ai * x_st + ks * x_ks, w + ks * ks_1, idH, acc);
+                        acc = 1;
+                      }
+                    if (i == 2)
+                      for (int ks = 0; ks < nk1; ++ks) ts_mma<XS>(tmem + FC1, a_x + ks * x_ks, w + ks * ks_1, idH, 1);
+                  } else {
+                    const int k0 = i * (TS_KCHUNK / 16), k1 = min(nk1, k0 + TS_KCHUNK / 16);
+                    for (int ks = k0; ks < k1; ++ks) {
+                      ts_mma<XS>(tmem + FC1, a_x + ks * x_ks, w + (ks - k0) * ks_1, idH, acc);
+                      acc = 1;
+                    }
+                  }
+                  if (i >= L.nres) mma_commit(&B->empty[ri]);
+                  if (i == L.nw1 - 1) mma_commit(&B->fc1d);
+                }
+                __syncwarp();
+                acc = 1;
+                if (i >= L.nres) next_slot();
+              }
+            }
+            // ---- gates ----
+            if (H == 64) {
+              // everything resident: the hidden side's first products run before the fc1 output is there
+              mbar_wait(&B->hset, par, abortf);
+              tc_fence_after_sync();
+              const uint32_t sl0 = get(L.nw1);
+              constexpr uint32_t SL = ts_slice(H);
+#pragma unroll
+              for (int b = 0; b < NBLK; ++b) {
+                const uint32_t s0 = sl0 + (uint32_t)b * 2u * NS * SL;
+                if (elect_one()) {
+                  if (NS == 3) {
+                    const uint64_t h2 = desc(s0, 1536), h1 = desc(s0 + SL, 1536), h0 = desc(s0 + 4 * SL, 1536);
+                    prod_h(b, 0, h2, 0);
+                    prod_h(b, 1, h1, 1);
+                    prod_h(b, 2, h0, 1);
+                    prod_h(b, 0, h1, 1);
+                    prod_h(b, 1, h0, 1);
+                  } else {
+                    prod_h(b, 0, desc(s0, 1536), 0);
+                  }
+                }
+                __syncwarp();
+              }
+              mbar_wait(&B->yrdy, par, abortf);
+              tc_fence_after_sync();
+#pragma unroll
+              for (int b = 0; b < NBLK; ++b) {
+                const uint32_t s0 = sl0 + (uint32_t)b * 2u * NS * SL;
+                if (elect_one()) {
+                  if (NS == 3) {
+                    const uint64_t y2 = desc(s0 + 2 * SL, 1536), y1 = desc(s0 + 3 * SL, 1536), h0 = desc(s0 + 4 * SL, 1536), y0 = desc(s0 + 5 * SL, 1536);
+                    prod_y(b, 0, y2, true);
+                    prod_y(b, 1, y1, false);
+                    prod_y(b, 2, y0, false);
+                    prod_y(b, 0, y1, false);
+                    prod_y(b, 1, y0, false);
+                    prod_h(b, 0, h0, 1);
+                    prod_y(b, 0, y0, false);
+                  } else {
+                    prod_y(b, 0, desc(s0 + SL, 1536), true);
+                  }
+                  mma_commit(&B->gd[b]);
+                }
+                __syncwarp();
+              }
+            } else {
+              int i = L.nw1;
+#pragma unroll 1
+              for (int b = 0; b < NBLK; ++b) {
+                const int buf = (b + 1) & 1;
+                if (b == 0) {
+                  mbar_wait(&B->hset, par, abortf);
+                } else if (b >= 2) {
+                  mbar_wait(&B->accf[buf], par, abortf);
+                }
+                tc_fence_after_sync();
+                if (NS == 3) {
+                  // h2, h1, y2, y1, then h0 and y0 held together: their small products come before both main ones
+#pragma unroll 1
+                  for (int k = 0; k < 4; ++k, ++i) {
+                    if (b == 0 && k == 2) {
+                      mbar_wait(&B->yrdy, par, abortf);
+                      tc_fence_after_sync();
+                    }
+                    const uint64_t w = desc(get(i), 1536);
+                    if (elect_one()) {
+                      if (k == 0) {
+                        prod_h(buf, 0, w, 0);
+                      } else if (k == 1) {
+                        prod_h(buf, 1, w, 1);
+                        prod_h(buf, 0, w, 1);
+                      } else if (k == 2) {
+                        prod_y(buf, 0, w, true);
+                      } else {
+                        prod_y(buf, 1, w, false);
+                        prod_y(buf, 0, w, false);
+                      }
+                      if (i >= L.nres) mma_commit(&B->empty[ri]);
+                    }
+                    __syncwarp();
+                    if (i >= L.nres) next_slot();
+                  }
+                  const uint64_t wh = desc(get(i), 1536);
+                  const uint32_t rh = ri;
+                  if (elect_one()) {
+                    prod_h(buf, 2, wh, 1);
+                    prod_h(buf, 1, wh, 1);
+                  }
+                  __syncwarp();
+                  if (i >= L.nres) next_slot();
+                  const uint64_t wy = desc(get(i + 1), 1536);
+                  if (elect_one()) {
+                    prod_y(buf, 2, wy, false);
+                    prod_y(buf, 1, wy, false);
+                    prod_h(buf, 0, wh, 1);
+                    if (i >= L.nres) mma_commit(&B->empty[rh]);
+                    prod_y(buf, 0, wy, false);
+                    if (i + 1 >= L.nres) mma_commit(&B->empty[ri]);
+                    mma_commit(&B->gd[buf]);
+                  }
+                  __syncwarp();
+                  if (i + 1 >= L.nres) next_slot();
+                  i += 2;
+                } else {
+                  const uint64_t wh = desc(get(i), 1536);
+                  if (elect_one()) {
+                    prod_h(buf, 0, wh, 0);
+                    if (i >= L.nres) mma_commit(&B->empty[ri]);
+                  }
+                  __syncwarp();
+                  if (i >= L.nres) next_slot();
+                  ++i;
+                  const uint64_t wy = desc(get(i), 1536);
+                  if (b == 0) {
+                    mbar_wait(&B->yrdy, par, abortf);
+                    tc_fence_after_sync();
+                  }
+                  if (elect_one()) {
+                    prod_y(buf, 0, wy, true);
+                    if (i >= L.nres) mma_commit(&B->empty[ri]);
+                    mma_commit(&B->gd[buf]);
+                  }
+                  __syncwarp();
+                  if (i >= L.nres) next_slot();
+                  ++i;
+                }
+              }
+            }
+            // ---- fc2: the small products of all blocks but the last, then the rest ----
+            if (g > 0) mbar_wait(&B->qfree, par ^ 1u, abortf);  // the previous step's Q has been read
+            const uint64_t w2 = desc(sb, NQ * 16);
+            auto prod_q = [&](uint32_t ai, uint32_t wi, int k0, int k1, uint32_t acc) {
+#pragma unroll
+              for (int ks = k0; ks < k1; ++ks) ts_mma<false>(tmem + TSM_Q, a_h + ai * h_st + ks * h_ks, w2 + wi * st_q + ks * ks_q, idq, ks > k0 ? 1u : acc);
+            };
+            constexpr int K1 = KH - TS_BLK / 16;  // K steps of the earlier blocks
+            mbar_wait(&B->hr0, par, abortf);
+            tc_fence_after_sync();
+            if (elect_one()) {
+              if (NS == 3) {
+                prod_q(2, 0, 0, K1, 0);
+                prod_q(1, 1, 0, K1, 1);
+                prod_q(0, 2, 0, K1, 1);
+                prod_q(1, 0, 0, K1, 1);
+                prod_q(0, 1, 0, K1, 1);
+              } else {
+                prod_q(0, 0, 0, K1, 0);
+              }
+            }
+            __syncwarp();
+            mbar_wait(&B->hr1, par, abortf);
+            tc_fence_after_sync();
+            if (elect_one()) {
+              if (NS == 3) {
+                prod_q(2, 0, K1, KH, 1);
+                prod_q(1, 1, K1, KH, 1);
+                prod_q(0, 2, K1, KH, 1);
+                prod_q(1, 0, K1, KH, 1);
+                prod_q(0, 1, K1, KH, 1);
+                prod_q(0, 0, 0, KH, 1);
+              } else {
+                prod_q(0, 0, K1, KH, 1);
+              }
+              mma_commit(&B->fc2d);
+            }
+            __syncwarp();
+          }
+      }
+    } else if (warp == 13) {
+      // =========================== weight warp ===========================
+      uint32_t ri = 0, rpar = 1, used = 0;
+      for (int typ = 0; typ < ntypes; ++typ) {
+        if (typ > 0) __syncthreads();
+        if (my_tiles == 0) continue;
+        const uint8_t* img = reinterpret_cast<const uint8_t*>(p.wsplit) + (size_t)typ * p.wsplit_stride;
+        const uint8_t* sl = img + L.base_bytes;
+        if (lane == 0) {
+          // resident part: the base and W1 first, then the gate slices
+          const int r1 = min(L.nres, L.nw1);
+          const uint32_t b1 = ts_slice_off(L, H, NS, r1), b2 = ts_slice_off(L, H, NS, L.nres);
+          mbar_arrive_expect_tx(&B->res[0], L.base_bytes + b1);
+          bulk_load(smem, img, L.base_bytes, &B->res[0]);
+          if (b1) bulk_load(smem + L.off_sl, sl, b1, &B->res[0]);
+          mbar_arrive_expect_tx(&B->res[1], b2 - b1);
+          for (uint32_t o = b1; o < b2; o += 32768u) bulk_load(smem + L.off_sl + o, sl + o, min(32768u, b2 - o), &B->res[1]);
+        }
+        __syncwarp();
+        if (L.nres < L.nsl) {
+          const int steps = my_tiles * T;
+          for (int g = 0; g < steps; ++g)
+            for (int i = L.nres; i < L.nsl; ++i) {
+              if (used >= (uint32_t)L.nslots) mbar_wait(&B->empty[ri], rpar, abortf);
+              else ++used;
+              if (lane == 0) {
+                const uint32_t bytes = ts_slice_bytes(L, H, NS, i);
+                mbar_arrive_expect_tx(&B->full[ri], bytes);
+                bulk_load(smem + L.off_ring + ri * ts_slice(H), sl + ts_slice_off(L, H, NS, i), bytes, &B->full[ri]);
+              }
+              __syncwarp();
+              if (++ri == (uint32_t)L.nslots) {
+                ri = 0;
+                rpar ^= 1u;
+              }
+            }
+        }
+      }
+    } else {
+      for (int typ = 1; typ < ntypes; ++typ) __syncthreads();
+    }
+  } else if (warp >= 8) {
+    // =========================== inputs and records ===========================
+    if (REGS_PREP < 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_PREP));
+    const int row = tid - TS_EPI, pw = warp - 8;  // (the thread also keeps the cursor of the tile's environment `row`)
+    const uint32_t tm = tmem + ((uint32_t)(pw * 32) << 16);
+    unsigned long long c_episodes = 0, c_trunc = 0;
+    uint32_t st_bits = 0, g = 0;
+    for (int typ = 0; typ < ntypes; ++typ) {
+      if (typ > 0) __syncthreads();
+      const int nt = rows_per_env(typ);
+      bool fresh = true;
+      for (int tile = blockIdx.x; tile < p.num_tiles; tile += gridDim.x) {
+        const int e0 = tile * ept;
+        const int ne = min(ept, p.M - e0);
+        const int R = ne * nt;
+        const bool wlive = pw * 32 < R;   // warps without a live row only keep the barriers going
+        const bool live = row < R;
+        int32_t slot = 0, pos = 0, eok = 0;
+        long long epc = 0;
+        asm volatile("bar.sync 2, 384;" ::: "memory");  // the previous tile's shared arrays are done with
+        if (row < ne) {
+          const int e = p.env_ids ? __ldg(p.env_ids + e0 + row) : e0 + row;
+          slot = p.slot[e];
+          pos = p.pos[e];
+          epc = p.ep_count[e];
+          // (with late outcomes a full slot waits, at pos == L, for its last outcome before it is truncated)
+          eok = (slot >= 0 && slot < p.E * p.S && pos >= 0 && pos < p.L + (lag ? 1 : 0)) ? 1 : 0;
+          if (!eok) st_bits |= MARL_STATUS_BAD_INDEX;
+          int closed = 0;
+          if (lag && eok && pos > 0) {
+            // the outcome of the previous action completes the record at pos - 1 and may close the episode
+            const float r = p.reward[e0 + row];
+            const int d = p.done[e0 + row] ? 1 : 0;
+            if (typ == 0) {
+              uint8_t* rec = p.ring + (size_t)slot * p.slot_stride + (size_t)(pos - 1) * rec_bytes;
+              *reinterpret_cast<float*>(rec + p.rl.off_reward) = r;
+              rec[p.rl.off_done] = (uint8_t)d;
+            }
+            if (d || pos == p.L) {
+              if (typ == 0) {
+                p.slot_len[slot] = pos;
+                p.slot_complete[slot] = 1;
+                c_episodes += 1;
+                if (!d) c_trunc += 1;
+              }
+              epc += 1;
+              slot = e * p.S + (int)(epc % p.S);
+              pos = 0;
+              closed = 1;
+            }
+          }
+          eid_s[row] = e;
+          close_s[((g + 3) & 3) * ept + row] = closed;  // (as if by the step before the first)
+        }
+        asm volatile("bar.sync 2, 384;" ::: "memory");
+        const int el = rowel_s[row], ai = rowag_s[row];
+        const int e = eid_s[el];
+        const bool vec = (D & 3) == 0 && (reinterpret_cast<uintptr_t>(p.obs) & 15) == 0;
+        float4* scr = reinterpret_cast<float4*>(smem + L.off_scr + pw * 2048);  // this warp's 32 rows x 16 columns
+        // observation units: lane l takes columns 4 (l % 4) .. of rows 8 j + l / 4, so four lanes read 64 bytes of a row
+        const int c4 = lane & 3;
+        int srow[4];      // rows, and their offsets in the tile's observations (floats)
+        int soff[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          srow[j] = pw * 32 + 8 * j + (lane >> 2);
+          soff[j] = (rowel_s[srow[j]] * n + rowag_s[srow[j]]) * D + 4 * c4;
+        }
+        const int nk = L.Dk / 16;
+        float reward_next = 0.f;
+        uint32_t done_next = 0;
+        auto fetch_outcome = [&](int s) {
+          if (row < ne && !lag) {
+            reward_next = p.reward[(size_t)s * p.env_step_stride + e0 + row];
+            done_next = p.done[(size_t)s * p.env_step_stride + e0 + row];
+          }
+        };
+        fetch_outcome(0);
+        unsigned long long myrec = 0, prevrec = 0;  // records of this thread's row: the step prepared, the one before
+
+        auto prepare = [&](int s, uint32_t gk) {
+          const uint32_t b = gk & 3;
+          // availability row as aligned words (up to three bytes on either side are read and dropped)
+          constexpr int AW = NQ == 16 ? 5 : 9;
+          uint32_t aw[AW], ash = 0;
+          if (live) {
+            const uintptr_t a0 = reinterpret_cast<uintptr_t>(p.avail + (size_t)s * p.avail_step_stride + ((size_t)(e0 + el) * n + ai) * A);
+            const uint32_t* wp = reinterpret_cast<const uint32_t*>(a0 & ~(uintptr_t)3);
+            ash = (uint32_t)(a0 & 3u);
+            const uint32_t nw = (ash + (uint32_t)A + 3u) / 4u;
+#pragma unroll
+            for (int k = 0; k < AW; ++k) aw[k] = (uint32_t)k < nw ? __ldg(wp + k) : 0u;
+          }
+          const float* obs = p.obs + (size_t)s * p.obs_step_stride + (size_t)e0 * n * D;
+          auto load = [&](int ks, float4 (&v)[4]) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const int c = ks * 16 + 4 * c4;
+              v[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+              if (srow[j] < R) {
+                const float* src = obs + soff[j] + ks * 16;
+                if (vec) {
+                  if (c < D) v[j] = __ldg(reinterpret_cast<const float4*>(src));
+                } else {
+                  if (c < D) v[j].x = __ldg(src);
+                  if (c + 1 < D) v[j].y = __ldg(src + 1);
+                  if (c + 2 < D) v[j].z = __ldg(src + 2);
+                  if (c + 3 < D) v[j].w = __ldg(src + 3);
+                }
+              }
+            }
+          };
+          float4 cur[4], nxt[4];
+          if (wlive) load(0, cur);
+          if (row < ne) {
+            // ring cursor, headers, reward and done of this step; the cursor needs only the done flags
+            unsigned long long rec = 0;
+            int close = 0;
+            if (eok) {
+              uint8_t* rp = p.ring + (size_t)slot * p.slot_stride + (size_t)pos * rec_bytes;
+              rec = reinterpret_cast<unsigned long long>(rp);
+              const int done = done_next ? 1 : 0;
+              close = (!lag && (done || pos + 1 == p.L)) ? 1 : 0;
+              if (typ == 0) {
+                if (pos == 0) {  // an episode opens in this slot
+                  p.slot_epid[slot] = epc * (long long)p.E + eid_s[row];
+                  p.slot_len[slot] = 0;
+                  p.slot_complete[slot] = 0;
+                }
+                *reinterpret_cast<float*>(rp + p.rl.off_reward) = reward_next;
+                rp[p.rl.off_done] = (uint8_t)done;
+                if (close) {
+                  p.slot_len[slot] = pos + 1;
+                  p.slot_complete[slot] = 1;
+                  c_episodes += 1;
+                  if (!done) c_trunc += 1;
+                }
+              }
+              if (close) {
+                epc += 1;
+                slot = eid_s[row] * p.S + (int)(epc % p.S);
+                pos = 0;
+              } else {
+                pos += 1;
+              }
+            }
+            recp_s[b * ept + row] = rec;
+            close_s[b * ept + row] = close;
+          }
+          if (s + 1 < T) fetch_outcome(s + 1);
+          if (live) {
+            unsigned long long bits = 0;
+#pragma unroll
+            for (int k = 0; k < AW; ++k) {
+              const uint32_t v = aw[k];
+              const uint32_t nz = ((v | ((v & 0x7F7F7F7Fu) + 0x7F7F7F7Fu)) & 0x80808080u) >> 7;  // 0x01 per non-zero byte
+              bits |= (unsigned long long)((nz * 0x01020408u) >> 24 & 0xFu) << (4 * k);
+            }
+            const uint32_t mask = (uint32_t)(bits >> ash) & (A >= 32 ? 0xFFFFFFFFu : ((1u << A) - 1u));
+            const uint32_t t = p.t0 + (uint32_t)s;
+            const int pick = mask ? draw_explore(mask, eps_at(p, t), p.seed, t, (uint32_t)e, (uint32_t)ai) : -1;
+            mask_s[b * TS_ROWS + row] = mask;
+            pick_s[b * TS_ROWS + row] = (int8_t)pick;
+          }
+          asm volatile("bar.sync 3, 128;" ::: "memory");  // the step's records are known
+          prevrec = myrec;
+          myrec = live ? recp_s[b * ept + el] : 0ull;
+          unsigned long long orec[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            orec[j] = srow[j] < R ? recp_s[b * ept + rowel_s[srow[j]]] : 0ull;
+            if (orec[j]) orec[j] += p.rl.off_obs + (unsigned long long)(rowag_s[srow[j]] * D + 4 * c4) * 4u;
+          }
+          if (gk > 0) {  // the y operand (same place) has been read by the previous step's gate products
+            mbar_wait(H == 64 ? &B->gd[1] : &B->hr0, (gk - 1) & 1, abortf);  // (barriers with one phase a step)
+            tc_fence_after_sync();
+          }
+          if (wlive) {
+#pragma unroll 1
+            for (int ks = 0; ks < nk; ++ks) {
+              if (ks + 1 < nk) load(ks + 1, nxt);
+              __syncwarp();
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                const int r = 8 * j + (lane >> 2);
+                scr[r * 4 + (c4 ^ ((r >> 1) & 3))] = cur[j];
+              }
+              __syncwarp();
+              float v[16];
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                const float4 f = scr[lane * 4 + (k ^ ((lane >> 1) & 3))];
+                v[4 * k] = f.x; v[4 * k + 1] = f.y; v[4 * k + 2] = f.z; v[4 * k + 3] = f.w;
+              }
+              ts_split16<NS>(v, [&](int i, const uint32_t (&w)[8]) {
+                if (XS) {
+                  uint8_t* to = smem + L.off_xy + (uint32_t)(i * nk + ks) * 4096u + (uint32_t)row * 16u;
+                  *reinterpret_cast<uint4*>(to) = make_uint4(w[0], w[1], w[2], w[3]);
+                  *reinterpret_cast<uint4*>(to + 2048) = make_uint4(w[4], w[5], w[6], w[7]);
+                } else {
+                  tmem_st8(tm + TSM_XY + (uint32_t)(i * nk + ks) * 8u, w);
+                }
+              });
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                const int c = ks * 16 + 4 * c4;
+                if (orec[j]) {
+                  float* to = reinterpret_cast<float*>(orec[j]) + ks * 16;
+                  if ((D & 3) == 0) {
+                    if (c < D) *reinterpret_cast<float4*>(to) = cur[j];
+                  } else {
+                    if (c < D) to[0] = cur[j].x;
+                    if (c + 1 < D) to[1] = cur[j].y;
+                    if (c + 2 < D) to[2] = cur[j].z;
+                    if (c + 3 < D) to[3] = cur[j].w;
+                  }
+                }
+              }
+#pragma unroll
+              for (int j = 0; j < 4; ++j) cur[j] = nxt[j];
+            }
+            if (XS) fence_proxy_async_smem();
+            else tmem_st_wait();
+          }
+          tc_fence_before_sync();
+          ts_arrive(&B->xrdy, lane);
+          if (myrec) {
+            uint8_t* dst = reinterpret_cast<uint8_t*>(myrec + p.rl.off_avail) + ai * A;
+#pragma unroll
+            for (int j = 0; j < NQ / 4; ++j) {
+              const uint32_t v = __funnelshift_r(aw[j], aw[j + 1], 8u * ash);  // bytes 4 j .. 4 j + 3 of the row
+#pragma unroll
+              for (int c = 0; c < 4; ++c)
+                if (4 * j + c < A) dst[4 * j + c] = (uint8_t)(v >> (8 * c));
+            }
+          }
+          if (live && s + 1 < T) {  // first touch of the next step's lines
+            const float* o1 = p.obs + (size_t)(s + 1) * p.obs_step_stride + ((size_t)(e0 + el) * n + ai) * D;
+            for (int c = 0; c < D; c += 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(o1 + c));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(o1 + D - 1));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(p.avail + (size_t)(s + 1) * p.avail_step_stride + ((size_t)(e0 + el) * n + ai) * A));
+          }
+        };
+
+        prepare(0, g);
+        if (fresh) mbar_wait(&B->res[0], (uint32_t)typ & 1, abortf);  // the output biases are in place
+        for (int s = 0; s < T; ++s, ++g) {
+          if (s + 1 < T) prepare(s + 1, g + 1);
+          else prevrec = myrec;
+          mbar_wait(&B->fc2d, g & 1, abortf);
+          tc_fence_after_sync();
+          if (wlive) {
+            uint32_t qv[NQ];
+            tmem_ld16(tm + TSM_Q, *reinterpret_cast<uint32_t(*)[16]>(qv));
+            if (NQ == 32) tmem_ld16(tm + TSM_Q + 16, *reinterpret_cast<uint32_t(*)[16]>(qv + NQ - 16));
+            tmem_ld_wait();
+            tc_fence_before_sync();
+            ts_arrive(&B->qfree, lane);
+            if (prevrec) {
+              float* qrow = reinterpret_cast<float*>(prevrec + p.rl.off_q) + ai * A;
+              if ((A & 1) == 0) {  // rows of an even number of floats start on 8-byte boundaries
+#pragma unroll
+                for (int a = 0; a < NQ; a += 2)
+                  if (a < A) *reinterpret_cast<float2*>(qrow + a) = make_float2(__uint_as_float(qv[a]) + b2_s[a], __uint_as_float(qv[a + 1]) + b2_s[a + 1]);
+              } else {
+#pragma unroll
+                for (int a = 0; a < NQ; ++a)
+                  if (a < A) qrow[a] = __uint_as_float(qv[a]) + b2_s[a];
+              }
+            }
+            const int tk = p.trace_first + s;
+            if (live && tk < p.trace_cap && p.trace_q) {
+              float* tq = p.trace_q + (((size_t)tk * p.E + e) * n + ai) * A;
+#pragma unroll
+              for (int a = 0; a < NQ; ++a)
+                if (a < A) tq[a] = __uint_as_float(qv[a]) + b2_s[a];
+            }
+          } else {
+            ts_arrive(&B->qfree, lane);
+          }
+        }
+        if (row < ne && eok && typ == ntypes - 1) {
+          const int ee = eid_s[row];
+          p.slot[ee] = slot;
+          p.pos[ee] = pos;
+          p.ep_count[ee] = epc;
+          if (pos > 0) p.slot_len[slot] = pos;
+        }
+        fresh = false;
+      }
+    }
+    if (c_episodes) atomicAdd(p.counters + CNT_EPISODES, c_episodes);
+    if (c_trunc) atomicAdd(p.counters + CNT_TRUNCATED, c_trunc);
+    if (st_bits) atomicOr(p.status, st_bits);
+  } else {
+    // =========================== epilogue ===========================
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_EPI));
+    const int row = tid & 127, grp = warp >> 2;
+    const uint32_t tm = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    unsigned long long c_steps = 0, c_explore = 0, c_noavail = 0;
+    uint32_t st_bits = 0, g = 0;
+    for (int typ = 0; typ < ntypes; ++typ) {
+      if (typ > 0) __syncthreads();
+      const int nt = rows_per_env(typ);
+      bool fresh = true;
+      for (int tile = blockIdx.x; tile < p.num_tiles; tile += gridDim.x) {
+        const int e0 = tile * ept;
+        const int R = min(ept, p.M - e0) * nt;
+        const bool wlive = (warp & 3) * 32 < R;   // warps without a live row only keep the barriers going
+        const bool live = row < R;
+        asm volatile("bar.sync 2, 384;" ::: "memory");  // the previous tile's shared arrays are done with
+        if (grp == 0) {
+          // row -> (environment, agent): the agents of this pass' unit type, in rising order
+          uint8_t el = 0, ag = 0;
+          if (live) {
+            el = (uint8_t)(row / nt);
+            int k = row - el * nt, i = k;
+            if (ntypes > 1)
+              for (i = 0; i < n; ++i)
+                if ((int)((p.agent_type_bits >> (2 * i)) & 3ull) == typ && k-- == 0) break;
+            ag = (uint8_t)i;
+          }
+          rowel_s[row] = el;
+          rowag_s[row] = ag;
+        }
+        asm volatile("bar.sync 2, 384;" ::: "memory");
+        const int el = rowel_s[row], ai = rowag_s[row];
+        const int e = eid_s[el];
+        const size_t grow = (size_t)e * n + ai;
+        float h[NBLK][16];
+        auto store_h = [&](int b) {  // the pieces of one block's hidden state
+          float v[16];
+#pragma unroll
+          for (int j = 0; j < 16; ++j) v[j] = h[b][j];
+          ts_split16<NS>(v, [&](int i, const uint32_t (&w)[8]) {
+            tmem_st8(tm + TSM_HOP + (uint32_t)(i * (H / 2) + b * (TS_BLK / 2) + grp * 8), w);
+          });
+        };
+        {
+          const bool carry = live && !close_s[((g + 3) & 3) * ept + el];  // the row continues an episode
+#pragma unroll
+          for (int b = 0; b < NBLK; ++b) {
+            const float4* src = reinterpret_cast<const float4*>(p.h + grow * H + b * TS_BLK + grp * 16);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const float4 v = carry ? src[k] : make_float4(0.f, 0.f, 0.f, 0.f);
+              h[b][4 * k] = v.x; h[b][4 * k + 1] = v.y; h[b][4 * k + 2] = v.z; h[b][4 * k + 3] = v.w;
+            }
+          }
+          if (grp == 0) {
+            int la = carry ? p.last_action[grow] : -1;
+            if (la >= A) la = -1;
+            la_s[row] = la;
+          }
+          if (wlive) {
+#pragma unroll
+            for (int b = 0; b < NBLK; ++b) store_h(b);
+            tmem_st_wait();
+          }
+          tc_fence_before_sync();
+          ts_arrive(&B->hset, lane);
+          asm volatile("bar.sync 1, 256;" ::: "memory");
+          if (fresh) mbar_wait(&B->res[0], (uint32_t)typ & 1, abortf);  // tables and biases are in place
+        }
+        const float* ta = reinterpret_cast<const float*>(smem + L.off_tabA) + ai * (H + 4) + grp * 16;
+        const float* tl0 = reinterpret_cast<const float*>(smem + L.off_tabL) + grp * 16;
+
+        for (int s = 0; s < T; ++s, ++g) {
+          const uint32_t par = g & 1u, b4 = g & 3u;
+          // ---- E1 ----
+          // (the inputs' own barrier orders their records and draws; looked at here, before the input warps can be two
+          // phases ahead of a parity wait)
+          mbar_wait(&B->xrdy, par, abortf);
+          mbar_wait(&B->fc1d, par, abortf);
+          tc_fence_after_sync();
+          if (wlive) {
+            const int last = la_s[row];
+            const float* tl = tl0 + (last >= 0 ? last : 0) * (H + 4);
+#pragma unroll
+            for (int b = 0; b < NBLK; ++b) {
+              uint32_t a[16];
+              tmem_ld16(tm + FC1 + (uint32_t)(b * TS_BLK + grp * 16), a);
+              float y[16];
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                const float4 va = *reinterpret_cast<const float4*>(ta + b * TS_BLK + 4 * k);
+                float4 vl = *reinterpret_cast<const float4*>(tl + b * TS_BLK + 4 * k);
+                if (last < 0) vl = make_float4(0.f, 0.f, 0.f, 0.f);
+                y[4 * k] = va.x + vl.x; y[4 * k + 1] = va.y + vl.y; y[4 * k + 2] = va.z + vl.z; y[4 * k + 3] = va.w + vl.w;
+              }
+              tmem_ld_wait();
+#pragma unroll
+              for (int k = 0; k < 16; ++k) y[k] = fmaxf(__uint_as_float(a[k]) + y[k], 0.f);
+              ts_split16<NS>(y, [&](int i, const uint32_t (&w)[8]) {
+                const int k8 = b * (TS_BLK / 8) + grp * 2;  // first 8-column group
+                if (XS) {
+                  uint8_t* to = smem + L.off_xy + (uint32_t)(i * (H / 8) + k8) * 2048u + (uint32_t)row * 16u;
+                  *reinterpret_cast<uint4*>(to) = make_uint4(w[0], w[1], w[2], w[3]);
+                  *reinterpret_cast<uint4*>(to + 2048) = make_uint4(w[4], w[5], w[6], w[7]);
+                } else {
+                  tmem_st8(tm + TSM_XY + (uint32_t)(i * (H / 2) + k8 * 4), w);
+                }
+              });
+            }
+            if (XS) fence_proxy_async_smem();
+            else tmem_st_wait();
+          }
+          tc_fence_before_sync();
+          ts_arrive(&B->yrdy, lane);
+
+          // ---- E2 ----
+#pragma unroll
+          for (int b = 0; b < NBLK; ++b) {
+            const int buf = H == 64 ? b : (b + 1) & 1;
+            mbar_wait(&B->gd[buf], H == 64 ? par : (uint32_t)(b >> 1), abortf);
+            tc_fence_after_sync();
+            if (b == NBLK - 1) {  // no product reads the old hidden state any more
+              if (wlive) {
+#pragma unroll
+                for (int k = 0; k < NBLK - 1; ++k) store_h(k);
+                tmem_st_wait();
+              }
+              tc_fence_before_sync();
+              ts_arrive(&B->hr0, lane);
+            }
+            if (wlive) {
+              // columns of the buffer: HN R Z IN | IN R Z HN
+              const uint32_t base = tm + (buf ? 128u : 0u) + (uint32_t)grp * 16u;
+              const uint32_t c_in = buf ? 0u : 96u, c_hn = buf ? 96u : 0u;
+#pragma unroll
+              for (int c8 = 0; c8 < 2; ++c8) {
+                uint32_t v[4][8];
+                tmem_ld8(base + 32u + c8 * 8, v[0]);
+                tmem_ld8(base + 64u + c8 * 8, v[1]);
+                tmem_ld8(base + c_in + c8 * 8, v[2]);
+                tmem_ld8(base + c_hn + c8 * 8, v[3]);
+                tmem_ld_wait();
+                if (H == 128 && c8 == 1 && b < NBLK - 2) {
+                  tc_fence_before_sync();
+                  ts_arrive(&B->accf[buf], lane);
+                }
+                const float* bb = bias_s + b * TS_BLK + grp * 16 + c8 * 8;
+#pragma unroll
+                for (int j4 = 0; j4 < 2; ++j4) {
+                  const float4 br = *reinterpret_cast<const float4*>(bb + 4 * j4), bz = *reinterpret_cast<const float4*>(bb + H + 4 * j4),
+                               bi = *reinterpret_cast<const float4*>(bb + 2 * H + 4 * j4), bh = *reinterpret_cast<const float4*>(bb + 3 * H + 4 * j4);
+                  const float brv[4] = {br.x, br.y, br.z, br.w}, bzv[4] = {bz.x, bz.y, bz.z, bz.w}, biv[4] = {bi.x, bi.y, bi.z, bi.w},
+                              bhv[4] = {bh.x, bh.y, bh.z, bh.w};
+#pragma unroll
+                  for (int k = 0; k < 4; ++k) {
+                    const int j = 4 * j4 + k;
+                    const float rg = ts_sigmoid(fmaf(__uint_as_float(v[0][j]), -TS_LOG2E, brv[k]));
+                    const float zg = ts_sigmoid(fmaf(__uint_as_float(v[1][j]), -TS_LOG2E, bzv[k]));
+                    const float cand = ts_tanh(fmaf(rg, __uint_as_float(v[3][j]) + bhv[k], __uint_as_float(v[2][j]) + biv[k]));
+                    const float hp = h[b][c8 * 8 + j];
+                    h[b][c8 * 8 + j] = fmaf(zg, hp - cand, cand);  // (1 - z) * cand + z * h
+                  }
+                }
+              }
+            } else if (H == 128 && b < NBLK - 2) {
+              ts_arrive(&B->accf[buf], lane);
+            }
+          }
+          if (wlive) {
+            store_h(NBLK - 1);
+            tmem_st_wait();
+          }
+          tc_fence_before_sync();
+          ts_arrive(&B->hr1, lane);
+
+          // ---- E3 ----
+          const bool close = live && close_s[b4 * ept + el];
+          mbar_wait(&B->fc2d, par, abortf);
+          tc_fence_after_sync();
+          uint32_t qv[NQ];
+          if (grp == 0 && wlive) {
+            tmem_ld16(tm + TSM_Q, *reinterpret_cast<uint32_t(*)[16]>(qv));
+            if (NQ == 32) tmem_ld16(tm + TSM_Q + 16, *reinterpret_cast<uint32_t(*)[16]>(qv + NQ - 16));
+            tmem_ld_wait();
+          }
+          // a closed episode restarts from a zero hidden state and no last action
+          if (wlive && __any_sync(0xFFFFFFFFu, close)) {
+            if (close) {
+#pragma unroll
+              for (int b = 0; b < NBLK; ++b)
+#pragma unroll
+                for (int j = 0; j < 16; ++j) h[b][j] = 0.f;
+            }
+#pragma unroll
+            for (int b = 0; b < NBLK; ++b) store_h(b);
+            tmem_st_wait();
+          }
+          tc_fence_before_sync();
+          if (s + 1 < T) ts_arrive(&B->hset, lane);
+          int act = 0;
+          if (grp == 0 && live) {
+            const uint32_t mask = mask_s[b4 * TS_ROWS + row];
+            const int pick = pick_s[b4 * TS_ROWS + row];
+            // greedy rule: m = max over available, thr = m - 1e-4f, lowest available a with Q >= thr (a NaN never
+            // compares greater or equal and fmaxf ignores it)
+            float qf[NQ];
+            float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+            for (int a = 0; a < NQ; ++a) {
+              qf[a] = __uint_as_float(qv[a]) + b2_s[a];
+              m4[a & 3] = fmaxf(m4[a & 3], ((mask >> a) & 1u) ? qf[a] : -INFINITY);
+            }
+            const float thr = __fsub_rn(fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])), 1e-4f);
+            uint32_t ge = 0;
+#pragma unroll
+            for (int a = 0; a < NQ; ++a) ge |= (qf[a] >= thr ? 1u : 0u) << a;
+            ge &= mask;
+            const int greedy = ge ? __ffs(ge) - 1 : __ffs(mask) - 1;
+            act = mask == 0 ? 0 : (pick >= 0 ? pick : greedy);
+            la_s[row] = close ? -1 : act;
+            c_steps += 1;
+            c_explore += pick >= 0 ? 1u : 0u;
+            if (mask == 0) { c_noavail += 1; st_bits |= MARL_STATUS_NO_AVAIL; }
+          }
+          asm volatile("bar.sync 1, 256;" ::: "memory");  // last actions are in place
+          if (grp == 0 && live) {
+            const unsigned long long rec = recp_s[b4 * ept + el];
+            if (rec) reinterpret_cast<int32_t*>(rec + p.rl.off_action)[ai] = act;
+            const int tk = p.trace_first + s;
+            if (tk < p.trace_cap && p.trace_actions) p.trace_actions[((size_t)tk * p.E + e) * n + ai] = act;
+            if (p.actions_out && s == T - 1) p.actions_out[(size_t)(e0 + el) * n + ai] = act;
+          }
+        }
+        // ---- end of the tile: state back to global memory ----
+        if (live) {
+#pragma unroll
+          for (int b = 0; b < NBLK; ++b) {
+            float4* dst = reinterpret_cast<float4*>(p.h + grow * H + b * TS_BLK + grp * 16);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) dst[k] = make_float4(h[b][4 * k], h[b][4 * k + 1], h[b][4 * k + 2], h[b][4 * k + 3]);
+          }
+          if (grp == 0) p.last_action[grow] = la_s[row];
+        }
+        fresh = false;
+      }
+    }
+    if (c_steps) atomicAdd(p.counters + CNT_AGENT_STEPS, c_steps);
+    if (c_explore) atomicAdd(p.counters + CNT_EXPLORED, c_explore);
+    if (c_noavail) atomicAdd(p.counters + CNT_NO_AVAIL, c_noavail);
+    if (st_bits) atomicOr(p.status, st_bits);
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  if (tid == 0 && B->abort) {
+    atomicOr(p.status, MARL_STATUS_TIMEOUT);
+    atomicCAS(p.status + 1, 0u, ((((B->abort & 0xFFFFFu) - (smem_u32(B) & 0xFFFFFu)) >> 3) & 0xFFu) | (((B->abort >> 20) & 0xFFu) << 8));
+  }
+  if (warp == 12) tmem_dealloc(tmem, 512);
+}
+
+// Returns the number of kernels launched or a negative cudaError.
+int launch_actor_tcs(const ActorParams& p_in, int sms, cudaStream_t stream) {
+  ActorParams p = p_in;
+  int nt_max = p.n, ntypes = 1;
+  if (p.n_types > 1) {
+    ntypes = p.n_types;
+    nt_max = 1;
+    for (int k = 0; k < ntypes; ++k) {
+      int c = 0;
+      for (int i = 0; i < p.n; ++i) c += (int)((p.agent_type_bits >> (2 * i)) & 3ull) == k ? 1 : 0;
+      if (c > nt_max) nt_max = c;
+    }
+  }
+  const int ns = ts_pieces(p.prec);
+  TsLayout L = ts_layout(p.n, p.D, p.A, p.H, ns, nt_max, p.M, sms);
+  L.ntypes = ntypes;
+  p.ept = L.ept;
+  p.num_tiles = (p.M + L.ept - 1) / L.ept;
+  const int v = (ns == 3 ? 0 : 4) + (L.NQ == 16 ? 0 : 2) + (p.H == 64 ? 0 : 1);
+  decltype(&actor_tcs_kernel<3, 16, 64>) kernels[8] = {
+      actor_tcs_kernel<3, 16, 64>, actor_tcs_kernel<3, 16, 128>, actor_tcs_kernel<3, 32, 64>, actor_tcs_kernel<3, 32, 128>,
+      actor_tcs_kernel<1, 16, 64>, actor_tcs_kernel<1, 16, 128>, actor_tcs_kernel<1, 32, 64>, actor_tcs_kernel<1, 32, 128>};
+  static uint32_t configured[8][SMEM_OPTIN_DEVICES];
+  {
+    const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernels[v]), L.total, configured[v]);
+    if (e != cudaSuccess) return -(int)e;
+  }
+  int grid = p.num_tiles < sms ? p.num_tiles : sms;
+  if (grid < 1) grid = 1;
+  kernels[v]<<<grid, TS_THREADS, L.total, stream>>>(p, L);
+  const cudaError_t err = cudaGetLastError();
+  return err == cudaSuccess ? 1 : -(int)err;
+}
+
+}  // namespace marl

@@ -37,6 +37,9 @@ struct ActorParams {
   const float *W1T, *b1, *WihT, *bih, *WhhT, *bhh, *W2, *b2;
   // tensor-core kernel weights: one packed image (see actor_tc.cu)
   const void* wpack;
+  // split-operand kernel weights: one image per unit type, wsplit_stride bytes apart (see actor_tcs.cu)
+  const void* wsplit;
+  size_t wsplit_stride;
   // inputs; step k of the launch reads base + k * stride (elements)
   const float* obs;
   const uint8_t* avail;
@@ -64,12 +67,12 @@ struct ActorParams {
   int32_t trace_cap;
   unsigned long long* counters;
   uint32_t* status;
-  // partial step (FFMA kernel only): the call's rows are the M listed environments; null: all E in order
+  // partial step: the call's rows are the M listed environments; null: all E in order
   const int32_t* env_ids;
   int32_t M;
   // T == 1 over a list: reward/done are the outcome of each environment's PREVIOUS action (committed at pos - 1)
   int32_t lagged;
-  // One network per unit type (FFMA kernel only): n_types > 1, the FFMA image of type k starts type_stride floats
+  // One network per unit type (FFMA and split-operand kernels): n_types > 1, the FFMA image of type k starts type_stride floats
   // after the one of type k - 1, and agent i's type is bits 2i, 2i+1 of agent_type_bits.
   int32_t n_types;
   uint32_t type_stride;

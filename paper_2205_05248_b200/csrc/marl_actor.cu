@@ -32,6 +32,12 @@ bool tc2_supported(int n, int D, int A, int H, int prec);
 int launch_actor_tc2(const ActorParams& p, int sms, cudaStream_t stream);
 bool tcw_supported(int n, int D, int A, int H, int prec);
 int launch_actor_tcw(const ActorParams& p, int sms, cudaStream_t stream);
+// split-operand tensor-core kernel: the general path wherever its shape is supported
+bool tcs_supported(int n, int D, int A, int H, int prec);
+size_t tcs_image_bytes(int n, int D, int A, int H, int prec);
+void tcs_pack_weights(int n, int D, int A, int H, int prec, const float* W1, const float* b1, const float* Wih,
+                      const float* bih, const float* Whh, const float* bhh, const float* W2, const float* b2, uint8_t* dst);
+int launch_actor_tcs(const ActorParams& p, int sms, cudaStream_t stream);
 int launch_ring_sample(const SampleParams& p, cudaStream_t stream);
 }  // namespace marl
 
@@ -84,7 +90,8 @@ static FfmaWeightOffsets ffma_weight_offsets(int n, int D, int A, int H) {
   return w;
 }
 
-struct StateOffsets { size_t h, last_action, slot, pos, ep_count, counters, status, wff[2], wpack[2], ids, total; };  // two weight images
+// two weight images, each: per-type images of the general kernel (split-operand or FFMA), then the tensor-core image
+struct StateOffsets { size_t h, last_action, slot, pos, ep_count, counters, status, wgen[2], wpack[2], ids, total; };
 struct RingOffsets { size_t records, epid, len, complete, total; };
 struct WorkOffsets { size_t obs, avail, reward, done, actions, total; };
 
@@ -103,6 +110,17 @@ static RecordLayout record_layout(int n, int D, int A) {
   return r;
 }
 
+// The kernel behind the tensor-core ones - fp32, per-type networks, launches the others do not take - is the
+// split-operand kernel where it supports the shape, unless the caller asked for the CUDA-core kernel.
+static bool general_is_tcs(const marl_actor_config_t& c) {
+  return c.kernel != MARL_KERNEL_FFMA && tcs_supported(c.n_agents, c.obs_dim, c.n_actions, c.hidden, c.precision);
+}
+// Bytes of one network's image for the general kernel.
+static size_t general_image_bytes(const marl_actor_config_t& c) {
+  return general_is_tcs(c) ? tcs_image_bytes(c.n_agents, c.obs_dim, c.n_actions, c.hidden, c.precision)
+                           : ffma_weight_offsets(c.n_agents, c.obs_dim, c.n_actions, c.hidden).total;
+}
+
 static StateOffsets state_offsets(const marl_actor_config_t& c) {
   StateOffsets s;
   Carve cv;
@@ -114,9 +132,12 @@ static StateOffsets state_offsets(const marl_actor_config_t& c) {
   s.ep_count = cv.take(sizeof(int64_t) * c.n_envs);
   s.counters = cv.take(sizeof(uint64_t) * CNT_N);
   s.status = cv.take(sizeof(uint32_t) * 4);
-  const size_t types = c.n_agent_types > 1 ? (size_t)c.n_agent_types : 1;  // FFMA images of a typed actor, one per type
+  const size_t types = c.n_agent_types > 1 ? (size_t)c.n_agent_types : 1;
+  // (room for either image: the caller may size the buffers with another kernel choice than the one it creates with)
+  const size_t ff = ffma_weight_offsets(c.n_agents, c.obs_dim, c.n_actions, c.hidden).total;
+  const size_t sp = tcs_image_bytes(c.n_agents, c.obs_dim, c.n_actions, c.hidden, c.precision);
   for (int i = 0; i < 2; ++i) {
-    s.wff[i] = cv.take(types * ffma_weight_offsets(c.n_agents, c.obs_dim, c.n_actions, c.hidden).total);
+    s.wgen[i] = cv.take(types * (ff > sp ? ff : sp));
     s.wpack[i] = cv.take(tc_wpack_bytes(c.n_agents, c.obs_dim, c.n_actions, c.hidden));
   }
   s.ids = cv.take(sizeof(int32_t) * (size_t)c.n_envs);  // environment list of a partial step
@@ -173,6 +194,8 @@ struct marl_actor {
   marl_actor_config_t cfg;
   cudaStream_t stream;
   int device, sms;
+  bool use_tcs;  // the general kernel is the split-operand one (else the CUDA-core kernel)
+  size_t gen_bytes;  // one network's image for it
   bool use_tc;   // a tensor-core kernel steps this actor
   bool use_tcp;  // ... the pipelined one (falls back to the one-tile kernel for inputs it cannot bulk-copy)
   bool use_tc2;  // ... with two tiles resident per SM where a launch allows it (else the pipelined kernel, same results)
@@ -285,6 +308,8 @@ int marl_actor_create(const marl_actor_config_t* cfg, marl_actor_t** out) {
   a->ro = ring_offsets(*cfg);
   a->wo = ffma_weight_offsets(cfg->n_agents, cfg->obs_dim, cfg->n_actions, cfg->hidden);
   a->rl = record_layout(cfg->n_agents, cfg->obs_dim, cfg->n_actions);
+  a->use_tcs = general_is_tcs(*cfg);
+  a->gen_bytes = general_image_bytes(*cfg);
   a->ring = a->state = a->work = nullptr;
   a->own_ring = a->own_state = a->own_work = false;
   a->step = 0;
@@ -397,16 +422,13 @@ static float to_bf16_value(float v) {
   return v;
 }
 
-// Packs the network into `dst` as the kernels read it: the FFMA image (k-major fp32, bf16-representable values in
-// the bf16 precision) followed by the tensor-core image.
-static void pack_weights_host(marl_actor* a, const float* W1, const float* b1, const float* W_ih, const float* b_ih,
-                              const float* W_hh, const float* b_hh, const float* W2, const float* b2,
-                              uint8_t* hp) {
+// The network's image for the CUDA-core kernel: k-major fp32, bf16-representable values in the bf16 precision.
+static void pack_ffma_host(const marl_actor* a, const float* W1, const float* b1, const float* W_ih, const float* b_ih,
+                           const float* W_hh, const float* b_hh, const float* W2, const float* b2, uint8_t* hp) {
   const int n = a->cfg.n_agents, D = a->cfg.obs_dim, A = a->cfg.n_actions, H = a->cfg.hidden;
   const int I = D + n + A;
   const bool lowp = a->cfg.precision == MARL_PRECISION_BF16;
-  const size_t tcb = tc_wpack_bytes(n, D, A, H);
-  memset(hp, 0, a->wo.total + tcb);
+  memset(hp, 0, a->wo.total);
   auto q = [lowp](float v) { return lowp ? to_bf16_value(v) : v; };
   float* W1T = reinterpret_cast<float*>(hp + a->wo.W1T);
   for (int j = 0; j < H; ++j)
@@ -424,16 +446,30 @@ static void pack_weights_host(marl_actor* a, const float* W1, const float* b1, c
   memcpy(hp + a->wo.bih, b_ih, sizeof(float) * 3 * H);
   memcpy(hp + a->wo.bhh, b_hh, sizeof(float) * 3 * H);
   memcpy(hp + a->wo.b2, b2, sizeof(float) * A);
-  if (tcb && (tc_supported(n, D, A, H, a->cfg.precision) || tcp_supported(n, D, A, H, a->cfg.precision) ||
-              tcw_supported(n, D, A, H, a->cfg.precision)))
-    tc_pack_weights(n, D, A, H, W1, b1, W_ih, b_ih, W_hh, b_hh, W2, b2, hp + a->wo.total);
+}
+
+// Packs the network as the kernels read it: the general kernel's image to `gen`, the tensor-core image to `tc` (null:
+// not needed).
+static void pack_weights_host(const marl_actor* a, const float* W1, const float* b1, const float* W_ih, const float* b_ih,
+                              const float* W_hh, const float* b_hh, const float* W2, const float* b2, uint8_t* gen,
+                              uint8_t* tc) {
+  const int n = a->cfg.n_agents, D = a->cfg.obs_dim, A = a->cfg.n_actions, H = a->cfg.hidden;
+  if (a->use_tcs) tcs_pack_weights(n, D, A, H, a->cfg.precision, W1, b1, W_ih, b_ih, W_hh, b_hh, W2, b2, gen);
+  else pack_ffma_host(a, W1, b1, W_ih, b_ih, W_hh, b_hh, W2, b2, gen);
+  const size_t tcb = tc_wpack_bytes(n, D, A, H);
+  if (tc && tcb) {
+    memset(tc, 0, tcb);
+    if (tc_supported(n, D, A, H, a->cfg.precision) || tcp_supported(n, D, A, H, a->cfg.precision) ||
+        tcw_supported(n, D, A, H, a->cfg.precision))
+      tc_pack_weights(n, D, A, H, W1, b1, W_ih, b_ih, W_hh, b_hh, W2, b2, tc);
+  }
 }
 
 static int upload_weights(marl_actor* a, const uint8_t* src, int image, cudaStream_t stream) {
   const marl_actor_config_t& c = a->cfg;
   const size_t tcb = tc_wpack_bytes(c.n_agents, c.obs_dim, c.n_actions, c.hidden);
-  CU_TRY(cudaMemcpyAsync(a->state + a->so.wff[image], src, a->wo.total, cudaMemcpyHostToDevice, stream));
-  if (tcb) CU_TRY(cudaMemcpyAsync(a->state + a->so.wpack[image], src + a->wo.total, tcb, cudaMemcpyHostToDevice, stream));
+  CU_TRY(cudaMemcpyAsync(a->state + a->so.wgen[image], src, a->gen_bytes, cudaMemcpyHostToDevice, stream));
+  if (tcb) CU_TRY(cudaMemcpyAsync(a->state + a->so.wpack[image], src + a->gen_bytes, tcb, cudaMemcpyHostToDevice, stream));
   return MARL_OK;
 }
 
@@ -448,8 +484,8 @@ int marl_actor_set_weights(marl_actor_t* a, const float* W1, const float* b1, co
     CU_TRY(cudaStreamSynchronize(a->copy_stream));
     a->pending = false;
   }
-  a->host_pack.resize(a->wo.total + tc_wpack_bytes(a->cfg.n_agents, a->cfg.obs_dim, a->cfg.n_actions, a->cfg.hidden));
-  pack_weights_host(a, W1, b1, W_ih, b_ih, W_hh, b_hh, W2, b2, a->host_pack.data());
+  a->host_pack.resize(a->gen_bytes + tc_wpack_bytes(a->cfg.n_agents, a->cfg.obs_dim, a->cfg.n_actions, a->cfg.hidden));
+  pack_weights_host(a, W1, b1, W_ih, b_ih, W_hh, b_hh, W2, b2, a->host_pack.data(), a->host_pack.data() + a->gen_bytes);
   const int rc = upload_weights(a, a->host_pack.data(), a->wslot, a->stream);
   if (rc) return rc;
   CU_TRY(cudaStreamSynchronize(a->stream));
@@ -485,24 +521,22 @@ int marl_actor_set_weights_typed(marl_actor_t* a, int32_t n_types, const int32_t
   }
   const int n = c.n_agents, D = c.obs_dim, A = c.n_actions, H = c.hidden, I = D + n + A;
   const size_t tcb = tc_wpack_bytes(n, D, A, H);
-  a->host_pack.assign((size_t)n_types * a->wo.total + a->wo.total + tcb, 0);
-  std::vector<uint8_t> one(a->wo.total + tcb);
-  for (int k = 0; k < n_types; ++k) {  // the CUDA-core image of every type, one after the other
+  a->host_pack.resize((size_t)n_types * a->gen_bytes + tcb);
+  for (int k = 0; k < n_types; ++k)  // the general kernel's image of every type, one after the other
     pack_weights_host(a, W1 + (size_t)k * H * I, b1 + (size_t)k * H, W_ih + (size_t)k * 3 * H * H, b_ih + (size_t)k * 3 * H,
                       W_hh + (size_t)k * 3 * H * H, b_hh + (size_t)k * 3 * H, W2 + (size_t)k * A * H, b2 + (size_t)k * A,
-                      one.data());
-    memcpy(a->host_pack.data() + (size_t)k * a->wo.total, one.data(), a->wo.total);
-  }
-  CU_TRY(cudaMemcpyAsync(a->state + a->so.wff[a->wslot], a->host_pack.data(), (size_t)n_types * a->wo.total,
+                      a->host_pack.data() + (size_t)k * a->gen_bytes,
+                      n_types == 1 ? a->host_pack.data() + a->gen_bytes : nullptr);
+  CU_TRY(cudaMemcpyAsync(a->state + a->so.wgen[a->wslot], a->host_pack.data(), (size_t)n_types * a->gen_bytes,
                          cudaMemcpyHostToDevice, a->stream));
   CU_TRY(cudaStreamSynchronize(a->stream));
   a->weights_version = version;
   a->have_weights = true;
   a->n_types = n_types;
   a->agent_type_bits = bits;
-  a->use_tc = a->use_tcp = a->use_tc2 = false;  // per-type networks run on the CUDA-core kernel
+  a->use_tc = a->use_tcp = a->use_tc2 = false;  // per-type networks run on the general kernel
   if (n_types == 1) {              // a single type is the shared network: its tensor-core image as well
-    const int rc = upload_weights(a, one.data(), a->wslot, a->stream);
+    const int rc = upload_weights(a, a->host_pack.data(), a->wslot, a->stream);
     if (rc) return rc;
     CU_TRY(cudaStreamSynchronize(a->stream));
     a->use_tc = a->tc_allowed;
@@ -525,11 +559,11 @@ int marl_actor_publish_weights(marl_actor_t* a, const float* W1, const float* b1
     CU_TRY(cudaStreamCreateWithFlags(&a->copy_stream, cudaStreamNonBlocking));
     CU_TRY(cudaEventCreateWithFlags(&a->upload_done, cudaEventDisableTiming));
     CU_TRY(cudaEventCreateWithFlags(&a->image_free, cudaEventDisableTiming));
-    CU_TRY(cudaMallocHost(&a->host_pack2, a->wo.total + tc_wpack_bytes(a->cfg.n_agents, a->cfg.obs_dim, a->cfg.n_actions, a->cfg.hidden)));
+    CU_TRY(cudaMallocHost(&a->host_pack2, a->gen_bytes + tc_wpack_bytes(a->cfg.n_agents, a->cfg.obs_dim, a->cfg.n_actions, a->cfg.hidden)));
   }
   // an earlier publication's copy reads host_pack2 and writes the same image: let it finish (it is replaced)
   CU_TRY(cudaStreamSynchronize(a->copy_stream));
-  pack_weights_host(a, W1, b1, W_ih, b_ih, W_hh, b_hh, W2, b2, a->host_pack2);
+  pack_weights_host(a, W1, b1, W_ih, b_ih, W_hh, b_hh, W2, b2, a->host_pack2, a->host_pack2 + a->gen_bytes);
   // the idle image was last read by steps enqueued before the previous switch
   if (a->image_free_recorded) CU_TRY(cudaStreamWaitEvent(a->copy_stream, a->image_free, 0));
   const int rc = upload_weights(a, a->host_pack2, a->wslot ^ 1, a->copy_stream);
@@ -553,7 +587,9 @@ static void fill_params(marl_actor* a, ActorParams& p) {
   p.prec = c.precision;
   p.seed = c.seed;
   uint8_t* st = a->state;
-  const uint8_t* w = st + a->so.wff[a->wslot];
+  const uint8_t* w = st + a->so.wgen[a->wslot];
+  p.wsplit = w;
+  p.wsplit_stride = a->gen_bytes;
   p.W1T = reinterpret_cast<const float*>(w + a->wo.W1T);
   p.b1 = reinterpret_cast<const float*>(w + a->wo.b1);
   p.WihT = reinterpret_cast<const float*>(w + a->wo.WihT);
@@ -646,7 +682,9 @@ static int enqueue_steps(marl_actor* a, const float* obs, const uint8_t* avail, 
     // (the one-tile kernel bulk-copies the observations too; it copes with unaligned availability bytes itself)
     if (rc == 0 && a->use_tc && reinterpret_cast<uintptr_t>(obs) % 16 == 0) rc = launch_actor_tc(p, a->sms, a->stream);
   }
-  if (rc == 0) {
+  if (rc == 0 && a->use_tcs) {
+    rc = launch_actor_tcs(p, a->sms, a->stream);
+  } else if (rc == 0) {
     ffma_tiling(c.n_envs, c.n_agents, a->sms, &p.ept, &p.num_tiles);
     rc = launch_actor_ffma(p, a->sms, a->stream);
   }
@@ -728,7 +766,9 @@ static int step_list(marl_actor* a, const int32_t* env_ids, int32_t M, const flo
     tc_tiling(M, c.n_agents, a->sms, &p.ept, &p.num_tiles);
     rc = c.hidden == 128 ? 0 : launch_actor_tcp(p, a->sms, a->stream);  // (the hidden-128 kernel takes dense launches only)
   }
-  if (rc == 0) {
+  if (rc == 0 && a->use_tcs) {
+    rc = launch_actor_tcs(p, a->sms, a->stream);
+  } else if (rc == 0) {
     ffma_tiling(M, c.n_agents, a->sms, &p.ept, &p.num_tiles);
     rc = launch_actor_ffma(p, a->sms, a->stream);
   }

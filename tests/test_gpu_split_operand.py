@@ -1,0 +1,89 @@
+"""The split-operand tensor-core kernel (general path: fp32, per-type networks, launches and shapes the bf16 kernels do
+not take) at the edges of its tiles, slices and dispatch, against the oracle."""
+import pytest
+import torch
+
+from paper_2205_05248_b200 import binding, workloads
+from referee import referee, run_gpu_rollout
+
+pytestmark = pytest.mark.gpu
+
+
+# A tile has 128 rows = n * environments; fc1 goes in K steps of 16 observations and, in bf16, slices of 96; 16 and 17
+# actions lie on both sides of the width of the Q product; at hidden 128 the gate slices stream through the ring in fp32
+# and stay (nearly) resident in bf16 with few observations.
+@pytest.mark.parametrize("prec,H,shape", [
+    ("fp32", 64, dict(E=8, n=3, D=30, A=9)),            # one environment per block
+    ("fp32", 64, dict(E=300, n=1, D=1, A=1)),
+    # 128 environments per tile, a ragged last tile.  (Nine actions: the referee's error is relative to the row's largest
+    # |Q|, and with two of them it falls to about 1e-3 in one of 100,000 rows, where the rounding of 64 products of size
+    # 0.1 - up to 64 * 0.1 * 2^-24 = 4e-7 - is beyond 1e-5 of it in any order of summation.)
+    ("fp32", 64, dict(E=20000, n=1, D=17, A=9, L=4, T=5)),
+    ("fp32", 64, dict(E=600, n=32, D=16, A=17, T=6)),   # four environments per tile, the wide Q product
+    ("fp32", 64, dict(E=7, n=32, D=63, A=32)),
+    ("fp32", 64, dict(E=2500, n=8, D=80, A=16, T=6)),   # full tiles, the largest observation
+    ("fp32", 64, dict(E=331, n=5, D=64, A=11, C=662)),
+    ("bf16", 64, dict(E=331, n=3, D=30, A=9, C=662)),   # fewer agents than the pipelined kernel takes, unaligned rows
+    ("bf16", 64, dict(E=40, n=2, D=255, A=20)),         # three fc1 slices
+    ("bf16", 64, dict(E=3000, n=3, D=31, A=16, T=6)),
+    ("fp32", 128, dict(E=8, n=3, D=30, A=9)),
+    ("fp32", 128, dict(E=2500, n=8, D=80, A=14, T=6)),
+    ("fp32", 128, dict(E=40, n=5, D=96, A=16)),
+    ("bf16", 128, dict(E=331, n=3, D=30, A=9, C=662)),
+    ("bf16", 128, dict(E=1700, n=5, D=55, A=12, T=6)),
+    ("bf16", 128, dict(E=40, n=4, D=200, A=20)),        # three fc1 slices, the wide Q product
+])
+def test_shapes(prec, H, shape):
+    cfg = workloads.small_config(**{**dict(H=H, L=6, T=14, C=shape["E"], precision=prec), **shape})
+    w = workloads.make_weights(cfg)
+    T = cfg["T"]
+    actor, acts, q = run_gpu_rollout(cfg, w, splits=[1, T - 1], work_steps=T)
+    res = referee(cfg, w, actor, acts, q)
+    assert res["kernel"] == "ffma"          # the general path's name
+    actor.destroy()
+
+
+@pytest.mark.parametrize("H", [64, 128])
+def test_precision_is_that_of_the_fma_chain(H):
+    """fp32: the largest Q and hidden-state differences to the oracle are those of the CUDA-core kernel.  Both sum the same
+    products; bound of one summation order against the other: twice the CUDA-core kernel's own largest difference."""
+    cfg = dict(workloads.config(5, E=1024, H=H, precision="fp32"), T=16, C=1024)
+    w = workloads.make_weights(cfg)
+    err = {}
+    for kernel in ("auto", "ffma"):
+        actor, acts, q = run_gpu_rollout(cfg, w, kernel=kernel)
+        res = referee(cfg, w, actor, acts, q)
+        err[kernel] = (res["q_err"], res["h_err"])
+        actor.destroy()
+    print(f"largest row-wise relative differences to the oracle (Q, h): {err}")
+    assert err["auto"][0] <= 2 * err["ffma"][0] and err["auto"][1] <= 2 * err["ffma"][1]
+
+
+@pytest.mark.parametrize("D", [30, 32])
+def test_observations_at_any_float_address(D):
+    """Device inputs that start on a 4-byte boundary only give the same results as aligned ones."""
+    cfg = workloads.small_config(H=64, E=50, n=3, D=D, A=9, C=50, L=5, precision="fp32")
+    w = workloads.make_weights(cfg)
+    a, b = (binding.Actor(cfg) for _ in range(2))
+    for x in (a, b):
+        x.set_weights(w)
+    for t in range(7):
+        obs, avail, reward, done = (v[0] for v in a.env_generate(cfg["env"], t, 1))
+        shifted = torch.empty(obs.numel() + 1, device="cuda")[1:].view_as(obs).copy_(obs)
+        av1 = torch.empty(avail.numel() + 1, dtype=torch.uint8, device="cuda")[1:].view_as(avail).copy_(avail)
+        assert torch.equal(a.step(obs, avail, reward, done, 0.1), b.step(shifted, av1, reward, done, 0.1))
+    assert torch.equal(a.ring_mem, b.ring_mem) and torch.equal(a.get_state()["h"], b.get_state()["h"])
+    a.destroy()
+    b.destroy()
+
+
+@pytest.mark.parametrize("H", [64, 128])
+def test_types_without_agents_and_one_agent_per_type(H):
+    """A unit type that no agent has, and a team of one agent per type: every environment refereed."""
+    for n, types in ((3, [0, 0, 2]), (4, [3, 2, 1, 0])):
+        cfg = workloads.small_config(H=H, E=1500, n=n, D=13, A=6, C=3000, L=4, T=9, precision="fp32")
+        cfg["agent_type"] = types
+        ws = [workloads.make_weights(cfg, seed=100 + k) for k in range(max(types) + 1)]
+        actor, acts, q = run_gpu_rollout(cfg, ws, splits=[2, 7])
+        referee(cfg, ws, actor, acts, q)
+        actor.destroy()
