@@ -52,7 +52,9 @@ extern "C" {
 #define MARL_PRECISION_BF16 1 /* weight matrices and matmul operands rounded to bf16 (RNE), fp32 accumulate */
 
 #define MARL_KERNEL_AUTO 0   /* bf16: a tensor-core kernel (the pipelined one, else the one-tile one, as the shape allows)
-                              * wherever the shape is supported, at every batch size; otherwise, and for fp32, FFMA */
+                              * wherever the shape is supported, at every batch size; otherwise, for fp32, for per-type
+                              * networks and for launches those do not take, the general kernel: split-operand tensor-core
+                              * products (fp32 as three bf16 pieces) where the shape fits, else FFMA */
 #define MARL_KERNEL_FFMA 1   /* CUDA-core kernel: any shape, both precisions */
 #define MARL_KERNEL_TENSOR 2 /* one-tile tcgen05 kernel: bf16 only; create fails if the shape is unsupported */
 #define MARL_KERNEL_TENSOR_PIPELINED 3 /* pipelined tcgen05 kernel: bf16, at least 4 agents; hidden 64, or hidden 128
@@ -202,7 +204,7 @@ int marl_actor_set_weights(marl_actor_t* a, const float* W1, const float* b1, co
  * in [0, n_types); the eight weight arrays as for marl_actor_set_weights with a leading [n_types] axis
  * (W1 [K][H][D+n+A], b1 [K][H], ...).  n_types must not exceed the n_agent_types the actor was created with.
  * Blocking, like marl_actor_set_weights, and a pending publication is dropped.  With n_types > 1 the steps run on
- * the CUDA-core kernel (both precisions; the products are evaluated once per type), marl_actor_publish_weights is
+ * the general kernel (both precisions; a tile's rows of one type at a time), marl_actor_publish_weights is
  * refused, and marl_actor_kernel_name reports "ffma"; a later marl_actor_set_weights returns to the shared network
  * and the kernel chosen at creation. */
 int marl_actor_set_weights_typed(marl_actor_t* a, int32_t n_types, const int32_t* agent_type, const float* W1,
@@ -239,7 +241,7 @@ int marl_actor_step(marl_actor_t* a, const float* obs, const uint8_t* avail, con
  * done u8[M], actions_out i32[M][n] (may be NULL).  The call consumes one index of the global step counter, which
  * keys the exploration stream as (seed, step, environment, agent) with the environment's own index; a trace row
  * of this step is written at the environment's own index as well.  Runs on the pipelined tensor-core kernel where
- * the actor uses it and the arrays can be bulk-copied (16-byte aligned obs and avail), else on the CUDA-core kernel. */
+ * the actor uses it and the arrays can be bulk-copied (16-byte aligned obs and avail), else on the general kernel. */
 int marl_actor_step_subset(marl_actor_t* a, const int32_t* env_ids, int32_t M, const float* obs,
                            const uint8_t* avail, const float* reward, const uint8_t* done, float eps,
                            int32_t* actions_out);
@@ -363,7 +365,7 @@ int marl_selftest_bounded_wait(void* stream, uint32_t poll_limit, uint32_t* stat
  * at the clocks it actually sustains.  SYNCHRONISES the stream; takes a few tens of milliseconds. */
 int marl_measure_ffma_tflops(void* stream, double* tflops_out);
 
-/* Name of the step kernel in use: "ffma", "tcgen05" (one-tile tensor-core kernel), "tcgen05-pipelined",
+/* Name of the step kernel in use: "ffma" (the general path: split-operand tensor-core or CUDA-core kernel), "tcgen05" (one-tile tensor-core kernel), "tcgen05-pipelined",
  * "tcgen05-dual" (two resident tiles; its other launches run on the pipelined kernel), or
  * "tcgen05-streamed" (hidden size 128: the pipelined design with the weights streamed through shared memory). */
 const char* marl_actor_kernel_name(const marl_actor_t* a);

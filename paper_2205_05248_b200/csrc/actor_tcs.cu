@@ -19,9 +19,9 @@
 // on the rows of that type, with that type's network).
 //
 // Roles: warps 0-7 epilogue (two groups of 128 threads; a thread owns one row and 16 columns of every block of 32
-// hidden columns), warps 8-11 inputs and records (thread = row), warp 12 issues every tcgen05.mma (from the lane that
+// hidden columns), warps 8-15 inputs and records (two groups, thread = row), warp 16 issues every tcgen05.mma (from the lane that
 // elect.sync picks: ptxas then knows that one lane runs and issues without a loop over lanes; 4 products take 325-400
-// clocks to completion against 577-700 behind "lane == 0"), warp 13 loads weights.
+// clocks to completion against 577-700 behind "lane == 0"), warp 17 loads weights.
 // Per step:
 //   E1 (epilogue)  y = relu(fc1 + agent column + last-action column), pieces to the y operand
 //   E2 (epilogue)  per block of 32 hidden columns: gates, new hidden state (fp32 in registers); the next block's
@@ -30,6 +30,7 @@
 //   inputs (beside E2) of the next step: ring cursor and headers, availability mask, epsilon draw, observation pieces
 //                  and record; then this step's Q record
 #include <cstring>
+#include <type_traits>
 
 #include "common.cuh"
 #include "launch_util.cuh"
@@ -37,7 +38,8 @@
 
 namespace marl {
 
-constexpr int TS_EPI = 256, TS_PREP = 128, TS_THREADS = 512;
+constexpr int TS_EPI = 256, TS_PREP = 256, TS_THREADS = 640;
+constexpr int TS_UNIT = 2048;       // a staged unit of observations: 32 rows x 16 columns
 constexpr int TS_ROWS = 128;
 constexpr int TS_BLK = 32;          // hidden columns of a gate block
 constexpr uint32_t TS_SMEM_MAX = 232448;
@@ -49,6 +51,7 @@ constexpr uint32_t TSM_HOP = 256, TSM_Q = 480;
 
 struct TsLayout {
   int32_t Dk, NQ, nw1, nsl, nres, nslots;   // K of fc1; Q columns; W1 slices; slices; resident ones; ring slots
+  int32_t nu;                               // staged units per input warp
   int32_t ept, ntypes;
   uint32_t base_bytes, off_b2, off_bias, off_tabA, off_tabL;  // base part of the image: W2 pieces, biases, column tables
   uint32_t img_bytes;
@@ -110,7 +113,6 @@ static TsLayout ts_layout(int n, int D, int A, int H, int ns, int nt_max, int M,
   uint32_t o = L.base_bytes;
   L.off_xy = o;
   if (ns == 3 && H == 128) o += 3u * (uint32_t)(L.Dk > H ? L.Dk : H) * TS_ROWS * 2;
-  L.off_scr = o; o += (TS_PREP / 32) * 2048;
   L.off_bar = o; o += (uint32_t)sizeof(TsBars);
   L.off_recp = o; o += 4u * (uint32_t)ept * 8;
   L.off_sel = o; o += 4u * TS_ROWS * 4;
@@ -120,25 +122,36 @@ static TsLayout ts_layout(int n, int D, int A, int H, int ns, int nt_max, int M,
   L.off_pick = o; o += 4u * TS_ROWS;
   L.off_row = o; o += TS_ROWS * 2;
   o = ts_up(o, 128);
+  // observation units in flight: one per input warp at least, a whole step's (up to three) where there is room
+  constexpr uint32_t units = (uint32_t)(TS_PREP / 32) * TS_UNIT;
+  const int nu_max = (L.Dk / 16 + 1) / 2 < 3 ? (L.Dk / 16 + 1) / 2 : 3;
+  L.nu = 1;
+  auto more_units = [&]() {  // at the end of shared memory: shifts nothing but the end
+    L.off_scr = L.total - units;
+    while (L.nu < nu_max && L.total + units <= TS_SMEM_MAX) { L.nu += 1; L.total += units; }
+  };
   L.off_sl = o;
   // resident slices: all of them, or what is left beside the ring (three slots where two slices are held at once)
   const uint32_t all = ts_slice_off(L, H, ns, L.nsl);
-  if (o + all <= TS_SMEM_MAX) {
+  if (o + all + units <= TS_SMEM_MAX) {
     L.nres = L.nsl;
     L.nslots = 0;
-    L.off_ring = L.total = o + all;
+    L.off_ring = o + all;
+    L.total = o + all + units;
+    more_units();
     return L;
   }
   L.nslots = ns == 3 ? 3 : 2;
-  if (o + (uint32_t)L.nslots * ts_slice(H) > TS_SMEM_MAX) {
+  if (o + units + (uint32_t)L.nslots * ts_slice(H) > TS_SMEM_MAX) {
     L.ept = 0;
     return L;
   }
-  const uint32_t room = TS_SMEM_MAX - o - (uint32_t)L.nslots * ts_slice(H);
+  const uint32_t room = TS_SMEM_MAX - o - units - (uint32_t)L.nslots * ts_slice(H);
   while (ts_slice_off(L, H, ns, L.nres + 1) <= room) L.nres += 1;
   L.off_ring = o + ts_slice_off(L, H, ns, L.nres);
-  while (L.nslots < TS_MAX_SLOTS && L.off_ring + (uint32_t)(L.nslots + 1) * ts_slice(H) <= TS_SMEM_MAX) L.nslots += 1;
-  L.total = L.off_ring + (uint32_t)L.nslots * ts_slice(H);
+  while (L.nslots < TS_MAX_SLOTS && L.off_ring + (uint32_t)(L.nslots + 1) * ts_slice(H) + units <= TS_SMEM_MAX) L.nslots += 1;
+  L.total = L.off_ring + (uint32_t)L.nslots * ts_slice(H) + units;
+  more_units();
   return L;
 }
 
@@ -243,6 +256,14 @@ __device__ __forceinline__ void ts_arrive(uint64_t* bar, int lane) {  // one arr
   if (lane == 0) tc::mbar_arrive(bar);
 }
 
+// Copies 16 or 4 bytes, of which the first `bytes` are read and the others written as zeros.
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async4(uint32_t dst, const void* src, uint32_t bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+
 __device__ __forceinline__ uint32_t ts_pack2(float lo, float hi) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&v);
@@ -276,21 +297,71 @@ __device__ __forceinline__ float ts_rcp(float x) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// sigmoid(v) with s = -log2(e) v: 1 / (1 + 2^s).  The approximate exponential's 2^-22.5 enters with weight
-// sigmoid (1 - sigmoid) <= 1/4.
-__device__ __forceinline__ float ts_sigmoid(float s) { return ts_rcp(1.0f + ts_ex2(s)); }
-// tanh: below 0.6 the odd polynomial u + u^3 P(u^2), P a degree-4 minimax fit (weighted least squares iterated to equal
-// ripple, 2.8e-9), else 1 - 2 / (1 + e^(2 |u|)), where the exponential's error has faded to an ulp.
-__device__ __forceinline__ float ts_tanh(float u) {
-  const float a = fabsf(u);
-  const float big = fmaf(-2.0f, ts_rcp(1.0f + ts_ex2(2.0f * TS_LOG2E * a)), 1.0f);
-  const float z = u * u;
-  float p = fmaf(-0.00589515688f, z, 0.0207959712f);
-  p = fmaf(p, z, -0.0537838303f);
-  p = fmaf(p, z, 0.133319244f);
-  p = fmaf(p, z, -0.333332986f);
-  const float small = fmaf(p * z, u, u);
-  return a < 0.6f ? small : copysignf(big, u);
+__device__ __forceinline__ float ts_min(float x, float y) {  // (a NaN stays)
+  float d;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(x), "f"(y));
+  return d;
+}
+// Two fp32 values side by side (fma.rn.f32x2 and its like: each half rounds like the scalar operation).
+typedef unsigned long long ts_f2;
+__device__ __forceinline__ ts_f2 f2(float lo, float hi) {
+  ts_f2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+  return d;
+}
+__device__ __forceinline__ ts_f2 f2(float v) { return f2(v, v); }
+__device__ __forceinline__ void f2_get(ts_f2 v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ ts_f2 f2_fma(ts_f2 a, ts_f2 b, ts_f2 c) {
+  ts_f2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ ts_f2 f2_mul(ts_f2 a, ts_f2 b) {
+  ts_f2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ ts_f2 f2_add(ts_f2 a, ts_f2 b) {
+  ts_f2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
+// The GRU's gate math on two columns: accumulators r, z, candidate input, candidate hidden; biases (b[0], b[1] already
+// times -log2 e); h in and out.  Bound by the special-function unit (16 results per clock and SM), so reciprocals are
+// shared: 1 / (dr dz) serves reset and update gate, one more both candidates - 4.5 special functions per column
+// instead of 6 - and everything else runs two columns per instruction.
+//   sigmoid(v) = 1 / (1 + 2^s), s = -log2(e) v: the approximate exponential's 2^-22.5 enters with weight
+//   sigmoid (1 - sigmoid) <= 1/4.  Exponents are cut at 60: the products of two denominators stay finite.
+//   tanh(u): below 0.6 the odd polynomial u + u^3 P(u^2), P a degree-4 minimax fit (weighted least squares iterated to
+//   equal ripple, 2.8e-9), else 1 - 2 / (1 + e^(2 |u|)), where the exponential's error has faded to an ulp.
+__device__ __forceinline__ void ts_gates2(const float (&v)[4][2], const ts_f2 (&b)[4], float& h0, float& h1) {
+  const ts_f2 one = f2(1.0f);
+  float s0, s1, z0, z1;
+  f2_get(f2_fma(f2(v[0][0], v[0][1]), f2(-TS_LOG2E), b[0]), s0, s1);
+  f2_get(f2_fma(f2(v[1][0], v[1][1]), f2(-TS_LOG2E), b[1]), z0, z1);
+  const ts_f2 dr = f2_add(f2(ts_ex2(ts_min(s0, 60.f)), ts_ex2(ts_min(s1, 60.f))), one);
+  const ts_f2 dz = f2_add(f2(ts_ex2(ts_min(z0, 60.f)), ts_ex2(ts_min(z1, 60.f))), one);
+  float p0, p1;
+  f2_get(f2_mul(dr, dz), p0, p1);
+  const ts_f2 inv = f2(ts_rcp(p0), ts_rcp(p1));
+  const ts_f2 rg = f2_mul(inv, dz), zg = f2_mul(inv, dr);
+  const ts_f2 u = f2_fma(rg, f2_add(f2(v[3][0], v[3][1]), b[3]), f2_add(f2(v[2][0], v[2][1]), b[2]));
+  float u0, u1, d0, d1;
+  f2_get(u, u0, u1);
+  const float a0 = fabsf(u0), a1 = fabsf(u1);
+  f2_get(f2_add(f2(ts_ex2(ts_min(2.0f * TS_LOG2E * a0, 60.f)), ts_ex2(ts_min(2.0f * TS_LOG2E * a1, 60.f))), one), d0, d1);
+  const float q = ts_rcp(d0 * d1);
+  float g0, g1, l0, l1;
+  f2_get(f2_fma(f2(q * d1, q * d0), f2(-2.0f), one), g0, g1);
+  const ts_f2 w = f2_mul(u, u);
+  ts_f2 p = f2_fma(f2(-0.00589515688f), w, f2(0.0207959712f));
+  p = f2_fma(p, w, f2(-0.0537838303f));
+  p = f2_fma(p, w, f2(0.133319244f));
+  p = f2_fma(p, w, f2(-0.333332986f));
+  f2_get(f2_fma(f2_mul(p, w), u, u), l0, l1);
+  const ts_f2 c = f2(a0 < 0.6f ? l0 : copysignf(g0, u0), a1 < 0.6f ? l1 : copysignf(g1, u1));
+  f2_get(f2_fma(zg, f2_fma(c, f2(-1.0f), f2(h0, h1)), c), h0, h1);  // (1 - z) * cand + z * h
 }
 
 // D (+)= A B^T, issued by one lane; A in shared memory (AS: descriptor) or in tensor memory (column address).
@@ -310,9 +381,9 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
   constexpr bool XS = NS == 3 && H == 128;       // x and y pieces in shared memory
   constexpr uint32_t TSM_XY = TSM_HOP + NS * H / 2;
   constexpr uint32_t FC1 = H == 64 ? 96 : 0;     // fc1's accumulator: the candidate-input columns, or buffer 0
-  // Registers (setmaxnreg): launched with 128 a thread (512 * 128 = 65536); afterwards
-  // 256 * 144 + 128 * 128 + 128 * 96 or, hidden 128, 256 * 176 + 128 * 112 + 128 * 48 = 65536.
-  constexpr int REGS_EPI = H == 64 ? 144 : 176, REGS_PREP = H == 64 ? 128 : 112, REGS_SVC = H == 64 ? 96 : 48;
+  // Registers (setmaxnreg): launched with 96 a thread (640 * 96 = 61440); afterwards
+  // 256 * 120 + 256 * 88 + 128 * 64 or, hidden 128, 256 * 128 + 256 * 88 + 128 * 48.
+  constexpr int REGS_EPI = H == 64 ? 120 : 128, REGS_PREP = 88, REGS_SVC = H == 64 ? 64 : 48;
   extern __shared__ __align__(1024) uint8_t smem[];
   TsBars* B = reinterpret_cast<TsBars*>(smem + L.off_bar);
   // per-step hand-offs, four buffers each: the input warps run up to two steps ahead of the choice
@@ -347,7 +418,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
     mbar_init(&B->hr0, TS_EPI / 32);
     mbar_init(&B->hr1, TS_EPI / 32);
     mbar_init(&B->fc2d, 1);
-    mbar_init(&B->qfree, TS_PREP / 32);
+    mbar_init(&B->qfree, TS_PREP / 64);
     for (int i = 0; i < TS_MAX_SLOTS; ++i) {
       mbar_init(&B->full[i], 1);
       mbar_init(&B->empty[i], 1);
@@ -355,7 +426,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
     B->abort = 0;
     mbar_init_fence();
   }
-  if (warp == 12) tmem_alloc(&B->tmem_base, 512);
+  if (warp == 16) tmem_alloc(&B->tmem_base, 512);
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -368,9 +439,9 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
   };
   const int my_tiles = blockIdx.x < p.num_tiles ? (p.num_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
 
-  if (warp >= 12) {
+  if (warp >= 16) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_SVC));
-    if (warp == 12) {
+    if (warp == 16) {
       // =========================== MMA warp ===========================
       const uint32_t sb = smem_u32(smem);
       constexpr uint32_t id96 = idesc_bf16_f32(128, 96), id64 = idesc_bf16_f32(128, 64), id32 = idesc_bf16_f32(128, 32),
@@ -402,25 +473,32 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
       };
       auto desc = [&](uint32_t addr, uint32_t lbo) { return smem_desc(addr, lbo, 128); };
 
-      // gate products of one piece pair over all K steps (the y side's first one starts the candidate-input columns)
-      auto prod_h = [&](int buf, uint32_t ai, uint64_t w, uint32_t acc) {
-        const uint32_t d = tmem + (buf ? 160u : 0u);
+      // The gate products of one piece pair over all K steps.  (Measured per product
+      // of N = 64: 30 clocks in rolled loops around four unrolled ones, 56 in a loop over single ones.)
+      // side 1: hidden, side 0: y, whose first product of a step starts the candidate-input columns.
+      auto prod = [&](int buf, int hid, uint32_t ai, uint64_t w, uint32_t acc) {
+        const uint32_t d = tmem + (hid ? (buf ? 160u : 0u) : (buf ? 128u : 32u));
+        if (XS && !hid) {
+          const uint64_t a = a_x + ai * y_st;
+          if (acc) {
+            ts_mma<true>(d, a, w, id96, 1);
+          } else {  // buffer 0: R Z at rows 0.., IN at rows 64..; buffer 1: IN at rows 0.., R Z at rows 32..
+            ts_mma<true>(d + (buf ? 0u : 64u), a, w + (buf ? 0u : (64u * 16u) >> 4), id32, 0);
+            ts_mma<true>(d + (buf ? 32u : 0u), a, w + (buf ? (32u * 16u) >> 4 : 0u), id64, 1);
+          }
 #pragma unroll
-        for (int ks = 0; ks < KH; ++ks) ts_mma<false>(d, a_h + ai * h_st + ks * h_ks, w + ks * ks_g, id96, ks ? 1u : acc);
-      };
-      auto prod_y = [&](int buf, uint32_t ai, uint64_t w, bool start) {
-        const uint32_t d = tmem + (buf ? 128u : 32u);
-        const uint64_t a = a_x + ai * y_st;
-        if (start) {
-          // buffer 0: R Z at rows 0.., IN at rows 64..; buffer 1: IN at rows 0.., R Z at rows 32..
-          const uint64_t w_in = w + (buf ? 0 : (64 * 16) >> 4), w_rz = w + (buf ? (32 * 16) >> 4 : 0);
-          ts_mma<XS>(d + (buf ? 0u : 64u), a, w_in, id32, 0);
-          ts_mma<XS>(d + (buf ? 32u : 0u), a, w_rz, id64, 1);
+          for (int ks = 1; ks < KH; ++ks) ts_mma<true>(d, a + ks * x_ks, w + ks * ks_g, id96, 1);
         } else {
-          ts_mma<XS>(d, a, w, id96, 1);
-        }
+          const uint64_t a = hid ? a_h + ai * h_st : a_x + ai * y_st;
+          if (hid || acc) {
+            ts_mma<false>(d, a, w, id96, acc);
+          } else {
+            ts_mma<false>(d + (buf ? 0u : 64u), a, w + (buf ? 0u : (64u * 16u) >> 4), id32, 0);
+            ts_mma<false>(d + (buf ? 32u : 0u), a, w + (buf ? (32u * 16u) >> 4 : 0u), id64, 1);
+          }
 #pragma unroll
-        for (int ks = 1; ks < KH; ++ks) ts_mma<XS>(d, a + ks * x_ks, w + ks * ks_g, id96, 1);
+          for (int ks = 1; ks < KH; ++ks) ts_mma<false>(d, a + ks * 8, w + ks * ks_g, id96, 1);
+        }
       };
 
       for (; typ < (uint32_t)ntypes; ++typ) {
@@ -433,30 +511,27 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
             mbar_wait(&B->xrdy, par, abortf);  // (E2 of the previous step has read the columns: hr1)
             tc_fence_after_sync();
             {
-              uint32_t acc = 0;
               for (int i = 0; i < L.nw1; ++i) {
                 const uint64_t w = desc(get(i), H * 16);
                 if (elect_one()) {
-                  if (NS == 3) {  // piece 2 - i against the small products' left pieces, then the main product
-                    for (int ai = i == 2 ? 2 : i; ai >= (i == 2 ? 1 : 0); --ai)
-                      for (int ks = 0; ks < nk1; ++ks) {
-                        ts_mma<XS>(tmem + FC1, a_x + ai * x_st + ks * x_ks, w + ks * ks_1, idH, acc);
-                        acc = 1;
-                      }
-                    if (i == 2)
-                      for (int ks = 0; ks < nk1; ++ks) ts_mma<XS>(tmem + FC1, a_x + ks * x_ks, w + ks * ks_1, idH, 1);
-                  } else {
-                    const int k0 = i * (TS_KCHUNK / 16), k1 = min(nk1, k0 + TS_KCHUNK / 16);
-                    for (int ks = k0; ks < k1; ++ks) {
-                      ts_mma<XS>(tmem + FC1, a_x + ks * x_ks, w + (ks - k0) * ks_1, idH, acc);
-                      acc = 1;
+                  // piece 2 - i against the small products' left pieces, then the main product (one piece: the slice's)
+                  const int k0 = NS == 3 ? 0 : i * (TS_KCHUNK / 16), nk = min(nk1 - k0, TS_KCHUNK / 16);
+#pragma unroll 1
+                  for (int ai = NS == 3 ? i : 0; ai >= 0; --ai) {
+                    uint64_t a = a_x + ai * x_st + (uint32_t)k0 * x_ks, wk = w;
+                    uint32_t acc = i > 0 || (NS == 3 && ai < i);
+                    int ks = 0;
+#pragma unroll 1
+                    for (; ks + 2 <= nk; ks += 2, a += 2 * x_ks, wk += 2 * ks_1, acc = 1) {
+                      ts_mma<XS>(tmem + FC1, a, wk, idH, acc);
+                      ts_mma<XS>(tmem + FC1, a + x_ks, wk + ks_1, idH, 1);
                     }
+                    if (ks < nk) ts_mma<XS>(tmem + FC1, a, wk, idH, acc);
                   }
                   if (i >= L.nres) mma_commit(&B->empty[ri]);
                   if (i == L.nw1 - 1) mma_commit(&B->fc1d);
                 }
                 __syncwarp();
-                acc = 1;
                 if (i >= L.nres) next_slot();
               }
             }
@@ -465,47 +540,35 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
               // everything resident: the hidden side's first products run before the fc1 output is there
               mbar_wait(&B->hset, par, abortf);
               tc_fence_after_sync();
-              const uint32_t sl0 = get(L.nw1);
-              constexpr uint32_t SL = ts_slice(H);
-#pragma unroll
-              for (int b = 0; b < NBLK; ++b) {
-                const uint32_t s0 = sl0 + (uint32_t)b * 2u * NS * SL;
-                if (elect_one()) {
-                  if (NS == 3) {
-                    const uint64_t h2 = desc(s0, 1536), h1 = desc(s0 + SL, 1536), h0 = desc(s0 + 4 * SL, 1536);
-                    prod_h(b, 0, h2, 0);
-                    prod_h(b, 1, h1, 1);
-                    prod_h(b, 2, h0, 1);
-                    prod_h(b, 0, h1, 1);
-                    prod_h(b, 1, h0, 1);
-                  } else {
-                    prod_h(b, 0, desc(s0, 1536), 0);
-                  }
-                }
-                __syncwarp();
+              const uint64_t w0 = desc(get(L.nw1), 1536);
+              constexpr uint64_t SL = ts_slice(H) >> 4;
+              // pieces of the small products in order: left, and slice of the hidden and of the y side
+              constexpr uint32_t LEFT = 0x10210u, SH = 0x41410u, SY = 0x53532u;
+              if (elect_one()) {
+#pragma unroll 1
+                for (int b = 0; b < NBLK; ++b)
+#pragma unroll 1
+                  for (int j = 0; j < (NS == 3 ? 5 : 1); ++j)
+                    prod(b, 1, (LEFT >> (4 * j)) & 15u, w0 + (uint32_t)(b * 2 * NS) * SL + (NS == 3 ? (SH >> (4 * j)) & 15u : 0u) * SL, j > 0);
               }
+              __syncwarp();
               mbar_wait(&B->yrdy, par, abortf);
               tc_fence_after_sync();
-#pragma unroll
-              for (int b = 0; b < NBLK; ++b) {
-                const uint32_t s0 = sl0 + (uint32_t)b * 2u * NS * SL;
-                if (elect_one()) {
+              if (elect_one()) {
+#pragma unroll 1
+                for (int b = 0; b < NBLK; ++b) {
+                  const uint64_t wb = w0 + (uint32_t)(b * 2 * NS) * SL;
                   if (NS == 3) {
-                    const uint64_t y2 = desc(s0 + 2 * SL, 1536), y1 = desc(s0 + 3 * SL, 1536), h0 = desc(s0 + 4 * SL, 1536), y0 = desc(s0 + 5 * SL, 1536);
-                    prod_y(b, 0, y2, true);
-                    prod_y(b, 1, y1, false);
-                    prod_y(b, 2, y0, false);
-                    prod_y(b, 0, y1, false);
-                    prod_y(b, 1, y0, false);
-                    prod_h(b, 0, h0, 1);
-                    prod_y(b, 0, y0, false);
+#pragma unroll 1
+                    for (int j = 0; j < 7; ++j)  // five small ones, then the main products
+                      prod(b, j == 5, j < 5 ? (LEFT >> (4 * j)) & 15u : 0u, wb + (j < 5 ? (SY >> (4 * j)) & 15u : (uint32_t)j - 1u) * SL, j > 0);
                   } else {
-                    prod_y(b, 0, desc(s0 + SL, 1536), true);
+                    prod(b, 0, 0, wb + SL, 0);
                   }
                   mma_commit(&B->gd[b]);
                 }
-                __syncwarp();
               }
+              __syncwarp();
             } else {
               int i = L.nw1;
 #pragma unroll 1
@@ -519,55 +582,36 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
                 tc_fence_after_sync();
                 if (NS == 3) {
                   // h2, h1, y2, y1, then h0 and y0 held together: their small products come before both main ones
+                  uint64_t wh = 0;
+                  uint32_t rh = 0;
 #pragma unroll 1
-                  for (int k = 0; k < 4; ++k, ++i) {
+                  for (int k = 0; k < 6; ++k, ++i) {
                     if (b == 0 && k == 2) {
                       mbar_wait(&B->yrdy, par, abortf);
                       tc_fence_after_sync();
                     }
                     const uint64_t w = desc(get(i), 1536);
+                    const int hid = k < 2 || k == 4;
+                    if (k == 4) { wh = w; rh = ri; }
                     if (elect_one()) {
-                      if (k == 0) {
-                        prod_h(buf, 0, w, 0);
-                      } else if (k == 1) {
-                        prod_h(buf, 1, w, 1);
-                        prod_h(buf, 0, w, 1);
-                      } else if (k == 2) {
-                        prod_y(buf, 0, w, true);
-                      } else {
-                        prod_y(buf, 1, w, false);
-                        prod_y(buf, 0, w, false);
+                      // left pieces: k = 0, 2: 0; 1, 3: 1 0; 4, 5: 2 1; after the last the main products
+                      const int first_ai = k >= 4 ? 2 : k & 1, last_ai = k >= 4 ? 1 : 0;
+#pragma unroll 1
+                      for (int ai = first_ai; ai >= last_ai - (k == 5 ? 2 : 0); --ai) {
+                        const bool main = ai < last_ai, mh = main && ai == 0;  // (k == 5: 0 stands for the hidden main, -1 for the y main)
+                        prod(buf, main ? mh : hid, main ? 0u : (uint32_t)ai, mh ? wh : w, !((k == 0 || k == 2) && ai == first_ai));
+                        if (mh && i - 1 >= L.nres) mma_commit(&B->empty[rh]);
                       }
-                      if (i >= L.nres) mma_commit(&B->empty[ri]);
+                      if (i >= L.nres && k != 4) mma_commit(&B->empty[ri]);
+                      if (k == 5) mma_commit(&B->gd[buf]);
                     }
                     __syncwarp();
                     if (i >= L.nres) next_slot();
                   }
-                  const uint64_t wh = desc(get(i), 1536);
-                  const uint32_t rh = ri;
-                  if (elect_one()) {
-                    prod_h(buf, 2, wh, 1);
-                    prod_h(buf, 1, wh, 1);
-                  }
-                  __syncwarp();
-                  if (i >= L.nres) next_slot();
-                  const uint64_t wy = desc(get(i + 1), 1536);
-                  if (elect_one()) {
-                    prod_y(buf, 2, wy, false);
-                    prod_y(buf, 1, wy, false);
-                    prod_h(buf, 0, wh, 1);
-                    if (i >= L.nres) mma_commit(&B->empty[rh]);
-                    prod_y(buf, 0, wy, false);
-                    if (i + 1 >= L.nres) mma_commit(&B->empty[ri]);
-                    mma_commit(&B->gd[buf]);
-                  }
-                  __syncwarp();
-                  if (i + 1 >= L.nres) next_slot();
-                  i += 2;
                 } else {
                   const uint64_t wh = desc(get(i), 1536);
                   if (elect_one()) {
-                    prod_h(buf, 0, wh, 0);
+                    prod(buf, 1, 0, wh, 0);
                     if (i >= L.nres) mma_commit(&B->empty[ri]);
                   }
                   __syncwarp();
@@ -579,7 +623,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
                     tc_fence_after_sync();
                   }
                   if (elect_one()) {
-                    prod_y(buf, 0, wy, true);
+                    prod(buf, 0, 0, wy, 0);
                     if (i >= L.nres) mma_commit(&B->empty[ri]);
                     mma_commit(&B->gd[buf]);
                   }
@@ -592,44 +636,32 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
             // ---- fc2: the small products of all blocks but the last, then the rest ----
             if (g > 0) mbar_wait(&B->qfree, par ^ 1u, abortf);  // the previous step's Q has been read
             const uint64_t w2 = desc(sb, NQ * 16);
-            auto prod_q = [&](uint32_t ai, uint32_t wi, int k0, int k1, uint32_t acc) {
-#pragma unroll
-              for (int ks = k0; ks < k1; ++ks) ts_mma<false>(tmem + TSM_Q, a_h + ai * h_st + ks * h_ks, w2 + wi * st_q + ks * ks_q, idq, ks > k0 ? 1u : acc);
-            };
             constexpr int K1 = KH - TS_BLK / 16;  // K steps of the earlier blocks
-            mbar_wait(&B->hr0, par, abortf);
-            tc_fence_after_sync();
-            if (elect_one()) {
-              if (NS == 3) {
-                prod_q(2, 0, 0, K1, 0);
-                prod_q(1, 1, 0, K1, 1);
-                prod_q(0, 2, 0, K1, 1);
-                prod_q(1, 0, 0, K1, 1);
-                prod_q(0, 1, 0, K1, 1);
-              } else {
-                prod_q(0, 0, 0, K1, 0);
+            auto part_q = [&](auto half_c) {  // K steps [0, K1) or [K1, KH); the second part ends with the main product
+              constexpr int half = decltype(half_c)::value, k0 = half ? K1 : 0, k1 = half ? KH : K1;
+              mbar_wait(half ? &B->hr1 : &B->hr0, par, abortf);
+              tc_fence_after_sync();
+              if (elect_one()) {
+                if (NS == 3) {  // small products (left, right): (2,0) (1,1) (0,2) (1,0) (0,1)
+#pragma unroll 1
+                  for (int j = 0; j < 5; ++j) {
+                    const uint64_t a = a_h + ((0x01012u >> (4 * j)) & 15u) * h_st, w = w2 + ((0x10210u >> (4 * j)) & 15u) * st_q;
+#pragma unroll
+                    for (int ks = k0; ks < k1; ++ks) ts_mma<false>(tmem + TSM_Q, a + ks * h_ks, w + ks * ks_q, idq, ks > 0 || j > 0);
+                  }
+                }
+                if (NS == 1 || half)
+#pragma unroll
+                  for (int ks = NS == 3 ? 0 : k0; ks < k1; ++ks) ts_mma<false>(tmem + TSM_Q, a_h + ks * h_ks, w2 + ks * ks_q, idq, NS == 3 || ks > 0);
+                if (half) mma_commit(&B->fc2d);
               }
-            }
-            __syncwarp();
-            mbar_wait(&B->hr1, par, abortf);
-            tc_fence_after_sync();
-            if (elect_one()) {
-              if (NS == 3) {
-                prod_q(2, 0, K1, KH, 1);
-                prod_q(1, 1, K1, KH, 1);
-                prod_q(0, 2, K1, KH, 1);
-                prod_q(1, 0, K1, KH, 1);
-                prod_q(0, 1, K1, KH, 1);
-                prod_q(0, 0, 0, KH, 1);
-              } else {
-                prod_q(0, 0, K1, KH, 1);
-              }
-              mma_commit(&B->fc2d);
-            }
-            __syncwarp();
+              __syncwarp();
+            };
+            part_q(std::integral_constant<int, 0>());
+            part_q(std::integral_constant<int, 1>());
           }
       }
-    } else if (warp == 13) {
+    } else if (warp == 17) {
       // =========================== weight warp ===========================
       uint32_t ri = 0, rpar = 1, used = 0;
       for (int typ = 0; typ < ntypes; ++typ) {
@@ -672,11 +704,21 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
     }
   } else if (warp >= 8) {
     // =========================== inputs and records ===========================
-    if (REGS_PREP < 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_PREP));
-    const int row = tid - TS_EPI, pw = warp - 8;  // (the thread also keeps the cursor of the tile's environment `row`)
+    // Two groups of four warps share a tile's rows (row = lane of tensor memory): both convert observations, in turn
+    // unit by unit (16 columns); group 0 also makes the masks and draws and records the availability, group 1 keeps the
+    // ring cursors (of environment `row` of the tile), headers and outcomes and records Q.
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_PREP));
+    auto inputs = [&](auto grp_c) {  // (the group as a constant: each group's code keeps only its own registers)
+    constexpr int grp = decltype(grp_c)::value;
+    const int row = tid & 127, pw = warp & 3;
     const uint32_t tm = tmem + ((uint32_t)(pw * 32) << 16);
-    unsigned long long c_episodes = 0, c_trunc = 0;
-    uint32_t st_bits = 0, g = 0;
+    const int nk = L.Dk / 16, nloc = (nk + 1 - grp) / 2;  // units of a step; this group's (2 k + grp)
+    // Units are staged by cp.async: loads that return to registers need a line of L1 each while in flight, and beside
+    // 227 KB of shared memory there are too few (a step's requests took 5 k clocks to issue).
+    uint8_t* units = smem + L.off_scr + (warp - 8) * L.nu * TS_UNIT;
+    const int c4 = lane & 3;  // the unit's columns 4 c4 .. of rows 8 j + lane / 4 are this lane's to copy
+    const bool vec = (D & 3) == 0 && (reinterpret_cast<uintptr_t>(p.obs) & 15) == 0;
+    uint32_t c_episodes = 0, c_trunc = 0, st_bits = 0, g = 0;
     for (int typ = 0; typ < ntypes; ++typ) {
       if (typ > 0) __syncthreads();
       const int nt = rows_per_env(typ);
@@ -687,10 +729,11 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
         const int R = ne * nt;
         const bool wlive = pw * 32 < R;   // warps without a live row only keep the barriers going
         const bool live = row < R;
+        const bool cursor = grp == 1 && row < ne;
         int32_t slot = 0, pos = 0, eok = 0;
         long long epc = 0;
-        asm volatile("bar.sync 2, 384;" ::: "memory");  // the previous tile's shared arrays are done with
-        if (row < ne) {
+        asm volatile("bar.sync 2, 512;" ::: "memory");  // the previous tile's shared arrays are done with
+        if (cursor) {
           const int e = p.env_ids ? __ldg(p.env_ids + e0 + row) : e0 + row;
           slot = p.slot[e];
           pos = p.pos[e];
@@ -724,38 +767,55 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
           eid_s[row] = e;
           close_s[((g + 3) & 3) * ept + row] = closed;  // (as if by the step before the first)
         }
-        asm volatile("bar.sync 2, 384;" ::: "memory");
+        asm volatile("bar.sync 2, 512;" ::: "memory");
         const int el = rowel_s[row], ai = rowag_s[row];
         const int e = eid_s[el];
-        const bool vec = (D & 3) == 0 && (reinterpret_cast<uintptr_t>(p.obs) & 15) == 0;
-        float4* scr = reinterpret_cast<float4*>(smem + L.off_scr + pw * 2048);  // this warp's 32 rows x 16 columns
-        // observation units: lane l takes columns 4 (l % 4) .. of rows 8 j + l / 4, so four lanes read 64 bytes of a row
-        const int c4 = lane & 3;
-        int srow[4];      // rows, and their offsets in the tile's observations (floats)
-        int soff[4];
+        int soff[4], poff[4];  // offset of the lane's first column in the tile's observations and in its record (floats)
+        uint32_t uel = 0, ulive = 0;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          srow[j] = pw * 32 + 8 * j + (lane >> 2);
-          soff[j] = (rowel_s[srow[j]] * n + rowag_s[srow[j]]) * D + 4 * c4;
+          const int r = pw * 32 + 8 * j + (lane >> 2);
+          soff[j] = (rowel_s[r] * n + rowag_s[r]) * D + 4 * c4;
+          poff[j] = rowag_s[r] * D + 4 * c4;
+          uel |= (uint32_t)rowel_s[r] << (8 * j);
+          ulive |= (r < R ? 1u : 0u) << j;
         }
-        const int nk = L.Dk / 16;
+
+        // ---- staging: unit `rq` of the group's sequence over (step, unit) goes to slot rq % nu ----
+        int rq_s = 0, rq_k = 0, rq_slot = 0, cv_slot = 0;
+        auto request_unit = [&]() {  // one cp.async group per call, empty at the end
+          if (wlive && rq_s < T) {
+            const int c = (2 * rq_k + grp) * 16 + 4 * c4;  // first column
+            const float* obs = p.obs + (size_t)rq_s * p.obs_step_stride + (size_t)e0 * n * D + (c - 4 * c4);
+            uint8_t* to = units + rq_slot * TS_UNIT;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const int r = 8 * j + (lane >> 2);
+              const uint32_t dst = smem_u32(to) + (uint32_t)(r * 64 + ((c4 ^ ((r >> 1) & 3)) * 16));
+              const int left = (ulive >> j) & 1u ? D - c : 0;  // columns there are; the others become zeros
+              const float* src = left > 0 ? obs + soff[j] : p.obs;
+              if (vec) {
+                cp_async16(dst, src, left > 0 ? 16u : 0u);
+              } else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) cp_async4(dst + 4 * k, left > k ? src + k : p.obs, left > k ? 4u : 0u);
+              }
+            }
+            if (++rq_k == nloc) { rq_k = 0; rq_s += 1; }
+            if (++rq_slot == L.nu) rq_slot = 0;
+          }
+          asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        if (nloc > 0)
+          for (int k = 0; k < L.nu; ++k) request_unit();
+
         float reward_next = 0.f;
         uint32_t done_next = 0;
-        auto fetch_outcome = [&](int s) {
-          if (row < ne && !lag) {
-            reward_next = p.reward[(size_t)s * p.env_step_stride + e0 + row];
-            done_next = p.done[(size_t)s * p.env_step_stride + e0 + row];
-          }
-        };
-        fetch_outcome(0);
-        unsigned long long myrec = 0, prevrec = 0;  // records of this thread's row: the step prepared, the one before
-
-        auto prepare = [&](int s, uint32_t gk) {
-          const uint32_t b = gk & 3;
-          // availability row as aligned words (up to three bytes on either side are read and dropped)
-          constexpr int AW = NQ == 16 ? 5 : 9;
-          uint32_t aw[AW], ash = 0;
-          if (live) {
+        constexpr int AW = NQ == 16 ? 5 : 9;
+        uint32_t aw[AW], ash = 0;
+        // a step's small inputs, requested a step ahead
+        auto request_small = [&](int s) {
+          if (grp == 0 && live) {  // availability row as aligned words (up to three bytes on either side are read and dropped)
             const uintptr_t a0 = reinterpret_cast<uintptr_t>(p.avail + (size_t)s * p.avail_step_stride + ((size_t)(e0 + el) * n + ai) * A);
             const uint32_t* wp = reinterpret_cast<const uint32_t*>(a0 & ~(uintptr_t)3);
             ash = (uint32_t)(a0 & 3u);
@@ -763,64 +823,58 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
 #pragma unroll
             for (int k = 0; k < AW; ++k) aw[k] = (uint32_t)k < nw ? __ldg(wp + k) : 0u;
           }
-          const float* obs = p.obs + (size_t)s * p.obs_step_stride + (size_t)e0 * n * D;
-          auto load = [&](int ks, float4 (&v)[4]) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const int c = ks * 16 + 4 * c4;
-              v[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-              if (srow[j] < R) {
-                const float* src = obs + soff[j] + ks * 16;
-                if (vec) {
-                  if (c < D) v[j] = __ldg(reinterpret_cast<const float4*>(src));
-                } else {
-                  if (c < D) v[j].x = __ldg(src);
-                  if (c + 1 < D) v[j].y = __ldg(src + 1);
-                  if (c + 2 < D) v[j].z = __ldg(src + 2);
-                  if (c + 3 < D) v[j].w = __ldg(src + 3);
-                }
-              }
-            }
-          };
-          float4 cur[4], nxt[4];
-          if (wlive) load(0, cur);
-          if (row < ne) {
-            // ring cursor, headers, reward and done of this step; the cursor needs only the done flags
-            unsigned long long rec = 0;
-            int close = 0;
-            if (eok) {
-              uint8_t* rp = p.ring + (size_t)slot * p.slot_stride + (size_t)pos * rec_bytes;
-              rec = reinterpret_cast<unsigned long long>(rp);
-              const int done = done_next ? 1 : 0;
-              close = (!lag && (done || pos + 1 == p.L)) ? 1 : 0;
-              if (typ == 0) {
-                if (pos == 0) {  // an episode opens in this slot
-                  p.slot_epid[slot] = epc * (long long)p.E + eid_s[row];
-                  p.slot_len[slot] = 0;
-                  p.slot_complete[slot] = 0;
-                }
-                *reinterpret_cast<float*>(rp + p.rl.off_reward) = reward_next;
-                rp[p.rl.off_done] = (uint8_t)done;
-                if (close) {
-                  p.slot_len[slot] = pos + 1;
-                  p.slot_complete[slot] = 1;
-                  c_episodes += 1;
-                  if (!done) c_trunc += 1;
-                }
-              }
-              if (close) {
-                epc += 1;
-                slot = eid_s[row] * p.S + (int)(epc % p.S);
-                pos = 0;
-              } else {
-                pos += 1;
-              }
-            }
-            recp_s[b * ept + row] = rec;
-            close_s[b * ept + row] = close;
+          if (grp == 1 && live && 2 * L.nu * 16 < D) {  // first touch of the lines whose units wait for a slot
+            const float* o1 = p.obs + (size_t)s * p.obs_step_stride + ((size_t)(e0 + el) * n + ai) * D;
+            for (int c = 2 * L.nu * 16; c < D; c += 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(o1 + c));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(o1 + D - 1));
           }
-          if (s + 1 < T) fetch_outcome(s + 1);
-          if (live) {
+          if (cursor && !lag) {
+            reward_next = p.reward[(size_t)s * p.env_step_stride + e0 + row];
+            done_next = p.done[(size_t)s * p.env_step_stride + e0 + row];
+          }
+        };
+        request_small(0);
+        unsigned long long myrec = 0, prevrec = 0;  // records of this thread's row: the step prepared, the one before
+
+        auto prepare = [&](int s, uint32_t gk) {
+          const uint32_t b = gk & 3;
+          if constexpr (grp == 1) {
+            if (cursor) {
+              // ring cursor, headers, reward and done of this step; the cursor needs only the done flags
+              unsigned long long rec = 0;
+              int close = 0;
+              if (eok) {
+                uint8_t* rp = p.ring + (size_t)slot * p.slot_stride + (size_t)pos * rec_bytes;
+                rec = reinterpret_cast<unsigned long long>(rp);
+                const int done = done_next ? 1 : 0;
+                close = (!lag && (done || pos + 1 == p.L)) ? 1 : 0;
+                if (typ == 0) {
+                  if (pos == 0) {  // an episode opens in this slot
+                    p.slot_epid[slot] = epc * (long long)p.E + eid_s[row];
+                    p.slot_len[slot] = 0;
+                    p.slot_complete[slot] = 0;
+                  }
+                  *reinterpret_cast<float*>(rp + p.rl.off_reward) = reward_next;
+                  rp[p.rl.off_done] = (uint8_t)done;
+                  if (close) {
+                    p.slot_len[slot] = pos + 1;
+                    p.slot_complete[slot] = 1;
+                    c_episodes += 1;
+                    if (!done) c_trunc += 1;
+                  }
+                }
+                if (close) {
+                  epc += 1;
+                  slot = eid_s[row] * p.S + (int)(epc % p.S);
+                  pos = 0;
+                } else {
+                  pos += 1;
+                }
+              }
+              recp_s[b * ept + row] = rec;
+              close_s[b * ept + row] = close;
+            }
+          } else if (live) {
             unsigned long long bits = 0;
 #pragma unroll
             for (int k = 0; k < AW; ++k) {
@@ -834,34 +888,25 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
             mask_s[b * TS_ROWS + row] = mask;
             pick_s[b * TS_ROWS + row] = (int8_t)pick;
           }
-          asm volatile("bar.sync 3, 128;" ::: "memory");  // the step's records are known
+          asm volatile("bar.sync 3, 256;" ::: "memory");  // the step's records are known
           prevrec = myrec;
           myrec = live ? recp_s[b * ept + el] : 0ull;
-          unsigned long long orec[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            orec[j] = srow[j] < R ? recp_s[b * ept + rowel_s[srow[j]]] : 0ull;
-            if (orec[j]) orec[j] += p.rl.off_obs + (unsigned long long)(rowag_s[srow[j]] * D + 4 * c4) * 4u;
-          }
           if (gk > 0) {  // the y operand (same place) has been read by the previous step's gate products
             mbar_wait(H == 64 ? &B->gd[1] : &B->hr0, (gk - 1) & 1, abortf);  // (barriers with one phase a step)
             tc_fence_after_sync();
           }
           if (wlive) {
 #pragma unroll 1
-            for (int ks = 0; ks < nk; ++ks) {
-              if (ks + 1 < nk) load(ks + 1, nxt);
+            for (int ks = grp; ks < nk; ks += 2) {
+              if (L.nu == 1) asm volatile("cp.async.wait_group 0;" ::: "memory");
+              else if (L.nu == 2) asm volatile("cp.async.wait_group 1;" ::: "memory");
+              else asm volatile("cp.async.wait_group 2;" ::: "memory");
               __syncwarp();
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                const int r = 8 * j + (lane >> 2);
-                scr[r * 4 + (c4 ^ ((r >> 1) & 3))] = cur[j];
-              }
-              __syncwarp();
+              const float4* un = reinterpret_cast<const float4*>(units + cv_slot * TS_UNIT);
               float v[16];
 #pragma unroll
               for (int k = 0; k < 4; ++k) {
-                const float4 f = scr[lane * 4 + (k ^ ((lane >> 1) & 3))];
+                const float4 f = un[lane * 4 + (k ^ ((lane >> 1) & 3))];
                 v[4 * k] = f.x; v[4 * k + 1] = f.y; v[4 * k + 2] = f.z; v[4 * k + 3] = f.w;
               }
               ts_split16<NS>(v, [&](int i, const uint32_t (&w)[8]) {
@@ -873,30 +918,34 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
                   tmem_st8(tm + TSM_XY + (uint32_t)(i * nk + ks) * 8u, w);
                 }
               });
+              const int c = ks * 16 + 4 * c4;
 #pragma unroll
               for (int j = 0; j < 4; ++j) {
-                const int c = ks * 16 + 4 * c4;
-                if (orec[j]) {
-                  float* to = reinterpret_cast<float*>(orec[j]) + ks * 16;
+                const unsigned long long rec = (ulive >> j) & 1u ? recp_s[b * ept + ((uel >> (8 * j)) & 0xFFu)] : 0ull;
+                const int r = 8 * j + (lane >> 2);
+                const float4 f = un[r * 4 + (c4 ^ ((r >> 1) & 3))];
+                if (rec) {
+                  float* to = reinterpret_cast<float*>(rec + p.rl.off_obs) + poff[j] + ks * 16;
                   if ((D & 3) == 0) {
-                    if (c < D) *reinterpret_cast<float4*>(to) = cur[j];
+                    if (c < D) *reinterpret_cast<float4*>(to) = f;
                   } else {
-                    if (c < D) to[0] = cur[j].x;
-                    if (c + 1 < D) to[1] = cur[j].y;
-                    if (c + 2 < D) to[2] = cur[j].z;
-                    if (c + 3 < D) to[3] = cur[j].w;
+                    if (c < D) to[0] = f.x;
+                    if (c + 1 < D) to[1] = f.y;
+                    if (c + 2 < D) to[2] = f.z;
+                    if (c + 3 < D) to[3] = f.w;
                   }
                 }
               }
-#pragma unroll
-              for (int j = 0; j < 4; ++j) cur[j] = nxt[j];
+              __syncwarp();  // the slot has been read
+              if (++cv_slot == L.nu) cv_slot = 0;
+              request_unit();
             }
             if (XS) fence_proxy_async_smem();
             else tmem_st_wait();
           }
           tc_fence_before_sync();
           ts_arrive(&B->xrdy, lane);
-          if (myrec) {
+          if (grp == 0 && myrec) {
             uint8_t* dst = reinterpret_cast<uint8_t*>(myrec + p.rl.off_avail) + ai * A;
 #pragma unroll
             for (int j = 0; j < NQ / 4; ++j) {
@@ -906,20 +955,19 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
                 if (4 * j + c < A) dst[4 * j + c] = (uint8_t)(v >> (8 * c));
             }
           }
-          if (live && s + 1 < T) {  // first touch of the next step's lines
-            const float* o1 = p.obs + (size_t)(s + 1) * p.obs_step_stride + ((size_t)(e0 + el) * n + ai) * D;
-            for (int c = 0; c < D; c += 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(o1 + c));
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(o1 + D - 1));
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(p.avail + (size_t)(s + 1) * p.avail_step_stride + ((size_t)(e0 + el) * n + ai) * A));
-          }
+          if (s + 1 < T) request_small(s + 1);
         };
 
-        prepare(0, g);
-        if (fresh) mbar_wait(&B->res[0], (uint32_t)typ & 1, abortf);  // the output biases are in place
-        for (int s = 0; s < T; ++s, ++g) {
-          if (s + 1 < T) prepare(s + 1, g + 1);
+        for (int sp = 0; sp <= T; ++sp) {  // prepare step sp, then finish step sp - 1
+          if (sp < T) prepare(sp, g + (uint32_t)sp);
           else prevrec = myrec;
-          mbar_wait(&B->fc2d, g & 1, abortf);
+          if constexpr (grp == 0) continue;
+          if (sp == 0) {
+            if (fresh) mbar_wait(&B->res[0], (uint32_t)typ & 1, abortf);  // the output biases are in place
+            continue;
+          }
+          const int s = sp - 1;
+          mbar_wait(&B->fc2d, (g + (uint32_t)s) & 1, abortf);
           tc_fence_after_sync();
           if (wlive) {
             uint32_t qv[NQ];
@@ -951,19 +999,24 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
             ts_arrive(&B->qfree, lane);
           }
         }
-        if (row < ne && eok && typ == ntypes - 1) {
+        g += (uint32_t)T;
+        if (cursor && eok && typ == ntypes - 1) {
           const int ee = eid_s[row];
           p.slot[ee] = slot;
           p.pos[ee] = pos;
           p.ep_count[ee] = epc;
           if (pos > 0) p.slot_len[slot] = pos;
         }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
         fresh = false;
       }
     }
-    if (c_episodes) atomicAdd(p.counters + CNT_EPISODES, c_episodes);
-    if (c_trunc) atomicAdd(p.counters + CNT_TRUNCATED, c_trunc);
+    if (c_episodes) atomicAdd(p.counters + CNT_EPISODES, (unsigned long long)c_episodes);
+    if (c_trunc) atomicAdd(p.counters + CNT_TRUNCATED, (unsigned long long)c_trunc);
     if (st_bits) atomicOr(p.status, st_bits);
+    };
+    if (warp < 12) inputs(std::integral_constant<int, 0>());
+    else inputs(std::integral_constant<int, 1>());
   } else {
     // =========================== epilogue ===========================
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_EPI));
@@ -980,7 +1033,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
         const int R = min(ept, p.M - e0) * nt;
         const bool wlive = (warp & 3) * 32 < R;   // warps without a live row only keep the barriers going
         const bool live = row < R;
-        asm volatile("bar.sync 2, 384;" ::: "memory");  // the previous tile's shared arrays are done with
+        asm volatile("bar.sync 2, 512;" ::: "memory");  // the previous tile's shared arrays are done with
         if (grp == 0) {
           // row -> (environment, agent): the agents of this pass' unit type, in rising order
           uint8_t el = 0, ag = 0;
@@ -995,7 +1048,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
           rowel_s[row] = el;
           rowag_s[row] = ag;
         }
-        asm volatile("bar.sync 2, 384;" ::: "memory");
+        asm volatile("bar.sync 2, 512;" ::: "memory");
         const int el = rowel_s[row], ai = rowag_s[row];
         const int e = eid_s[el];
         const size_t grow = (size_t)e * n + ai;
@@ -1113,19 +1166,21 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
                 }
                 const float* bb = bias_s + b * TS_BLK + grp * 16 + c8 * 8;
 #pragma unroll
-                for (int j4 = 0; j4 < 2; ++j4) {
-                  const float4 br = *reinterpret_cast<const float4*>(bb + 4 * j4), bz = *reinterpret_cast<const float4*>(bb + H + 4 * j4),
-                               bi = *reinterpret_cast<const float4*>(bb + 2 * H + 4 * j4), bh = *reinterpret_cast<const float4*>(bb + 3 * H + 4 * j4);
-                  const float brv[4] = {br.x, br.y, br.z, br.w}, bzv[4] = {bz.x, bz.y, bz.z, bz.w}, biv[4] = {bi.x, bi.y, bi.z, bi.w},
-                              bhv[4] = {bh.x, bh.y, bh.z, bh.w};
+                for (int j = 0; j < 8; j += 4) {
+                  ulonglong2 bv[4];  // biases of four columns
 #pragma unroll
-                  for (int k = 0; k < 4; ++k) {
-                    const int j = 4 * j4 + k;
-                    const float rg = ts_sigmoid(fmaf(__uint_as_float(v[0][j]), -TS_LOG2E, brv[k]));
-                    const float zg = ts_sigmoid(fmaf(__uint_as_float(v[1][j]), -TS_LOG2E, bzv[k]));
-                    const float cand = ts_tanh(fmaf(rg, __uint_as_float(v[3][j]) + bhv[k], __uint_as_float(v[2][j]) + biv[k]));
-                    const float hp = h[b][c8 * 8 + j];
-                    h[b][c8 * 8 + j] = fmaf(zg, hp - cand, cand);  // (1 - z) * cand + z * h
+                  for (int k = 0; k < 4; ++k) bv[k] = *reinterpret_cast<const ulonglong2*>(bb + k * H + j);
+#pragma unroll
+                  for (int c = 0; c < 4; c += 2) {
+                    float a[4][2];
+                    ts_f2 b2[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                      a[k][0] = __uint_as_float(v[k][j + c]);
+                      a[k][1] = __uint_as_float(v[k][j + c + 1]);
+                      b2[k] = c == 0 ? bv[k].x : bv[k].y;
+                    }
+                    ts_gates2(a, b2, h[b][c8 * 8 + j + c], h[b][c8 * 8 + j + c + 1]);
                   }
                 }
               }
@@ -1222,7 +1277,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
     atomicOr(p.status, MARL_STATUS_TIMEOUT);
     atomicCAS(p.status + 1, 0u, ((((B->abort & 0xFFFFFu) - (smem_u32(B) & 0xFFFFFu)) >> 3) & 0xFFu) | (((B->abort >> 20) & 0xFFu) << 8));
   }
-  if (warp == 12) tmem_dealloc(tmem, 512);
+  if (warp == 16) tmem_dealloc(tmem, 512);
 }
 
 // Returns the number of kernels launched or a negative cudaError.

@@ -110,10 +110,11 @@ static RecordLayout record_layout(int n, int D, int A) {
   return r;
 }
 
-// The kernel behind the tensor-core ones - fp32, per-type networks, launches the others do not take - is the
-// split-operand kernel where it supports the shape, unless the caller asked for the CUDA-core kernel.
+// The kernel behind the bf16 tensor-core ones - fp32, per-type networks, launches the others do not take.  Chosen
+// automatically, it is the split-operand kernel where that supports the shape; a kernel asked for by name falls back to
+// the CUDA-core kernel.
 static bool general_is_tcs(const marl_actor_config_t& c) {
-  return c.kernel != MARL_KERNEL_FFMA && tcs_supported(c.n_agents, c.obs_dim, c.n_actions, c.hidden, c.precision);
+  return c.kernel == MARL_KERNEL_AUTO && tcs_supported(c.n_agents, c.obs_dim, c.n_actions, c.hidden, c.precision);
 }
 // Bytes of one network's image for the general kernel.
 static size_t general_image_bytes(const marl_actor_config_t& c) {
