@@ -169,14 +169,21 @@ constexpr uint64_t TP_K_A = (2 * TC_LBO_A) >> 4, TP_K_X = (2 * TC_LBO_X) >> 4, T
 __device__ __forceinline__ void tp_issue_fc1(const TpLayout& L, uint32_t sb, uint32_t tmem, int lane, uint64_t* fc1d) {
   using namespace tc;
   tc_fence_after_sync();
-  if (lane == 0) {
+  if (elect_one()) {
     const uint64_t d_x = smem_desc(sb + L.off_x, TC_LBO_X, 128), d_oh = smem_desc(sb + L.off_oh, TC_LBO_A, 128);
     const uint64_t d_W1 = smem_desc(sb + L.off_W1, TP_LBO_W1, 128);
     const uint64_t d_W1oh = smem_desc(sb + L.off_W1 + (uint32_t)L.nchunk * TP_LBO_W1, TP_LBO_W1, 128);
     const uint32_t id64 = idesc_bf16_f32(128, 64);
     const int ks_obs = L.Dk / 16, ks_oh = L.ohK / 16;
-    for (int ks = 0; ks < ks_obs; ++ks) mma_bf16(tmem + TM_FC1, d_x + ks * TP_K_X, d_W1 + ks * TP_K_W1, id64, ks > 0);
-    for (int ks = 0; ks < ks_oh; ++ks) mma_bf16(tmem + TM_FC1, d_oh + ks * TP_K_A, d_W1oh + ks * TP_K_W1, id64, 1);
+    int ks = 0;
+#pragma unroll 1
+    for (; ks + 2 <= ks_obs; ks += 2) {
+      mma_bf16(tmem + TM_FC1, d_x + ks * TP_K_X, d_W1 + ks * TP_K_W1, id64, ks > 0);
+      mma_bf16(tmem + TM_FC1, d_x + (ks + 1) * TP_K_X, d_W1 + (ks + 1) * TP_K_W1, id64, 1);
+    }
+    if (ks < ks_obs) mma_bf16(tmem + TM_FC1, d_x + ks * TP_K_X, d_W1 + ks * TP_K_W1, id64, ks > 0);
+#pragma unroll 1
+    for (ks = 0; ks < ks_oh; ++ks) mma_bf16(tmem + TM_FC1, d_oh + ks * TP_K_A, d_W1oh + ks * TP_K_W1, id64, 1);
     mma_commit(fc1d);
   }
   __syncwarp();
@@ -188,7 +195,7 @@ template <int NQ>
 __device__ __forceinline__ void tp_issue_hside(const TpLayout& L, uint32_t sb, uint32_t tmem, int lane, uint32_t qcol) {
   using namespace tc;
   tc_fence_after_sync();
-  if (lane == 0) {
+  if (elect_one()) {
     const uint64_t d_h = smem_desc(sb + L.off_hb, TC_LBO_A, 128), d_oh = smem_desc(sb + L.off_oh, TC_LBO_A, 128);
     const uint64_t d_Whh = smem_desc(sb + L.off_Whh, TP_LBO_G, 128);
     const uint64_t d_Whh_n = smem_desc(sb + L.off_Whh + 2 * TC_H * 16, TP_LBO_G, 128);  // the candidate rows of each k-chunk
@@ -299,7 +306,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
   if (warp >= 12) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(TP_REGS_SVC));
     if (warp == 12) {
-      // =========================== MMA warp: lane 0 issues every tcgen05.mma ===========================
+      // =========================== MMA warp: one elected lane issues every tcgen05.mma ===========================
       const uint32_t sb = smem_u32(smem);
       const int total = my_tiles * T;
       uint32_t tl = 0;
@@ -323,7 +330,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
         }
         mbar_wait(&B->yready, par, abortf);
         tc_fence_after_sync();
-        if (lane == 0) {
+        if (elect_one()) {
           const uint64_t d_y = smem_desc(sb + L.off_y, TC_LBO_A, 128), d_Wih = smem_desc(sb + L.off_Wih, TP_LBO_G, 128);
 #pragma unroll
           for (int ks = 0; ks < 4; ++ks) mma_bf16(tmem + TM_R, d_y + ks * TP_K_A, d_Wih + ks * TP_K_G, idesc_bf16_f32(128, 192), 1);
@@ -343,7 +350,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
         }
         mbar_wait(&B->hready, par, abortf);
         tc_fence_after_sync();
-        if (lane == 0) {
+        if (elect_one()) {
           const uint64_t d_h = smem_desc(sb + L.off_hb, TC_LBO_A, 128), d_W2 = smem_desc(sb + L.off_W2, NQ * 16, 128);
 #pragma unroll
           for (int ks = 0; ks < 4; ++ks)  // part 0 holds the bias already; parts 1..3 start from zero
