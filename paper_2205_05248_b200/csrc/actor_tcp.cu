@@ -55,7 +55,7 @@ struct TpLayout {
   int32_t Dk, NQ, nchunk, ept, ohK, ohc, NS, plain;
   uint32_t prefix_bytes, tail_bytes, chunk_bytes, obs_bytes, av_bytes, rs_env, rs_bytes, off_rstage;
   uint32_t off_W1, off_Wih, off_Whh, off_Bg, off_Bhn, off_W2, off_tab_la, wbytes;
-  uint32_t off_x, off_y, off_hb, off_oh, off_stage, off_tail, off_sel, off_la, off_close, off_closeany, off_rowenv, off_dstp, off_tdst, off_bar, total;
+  uint32_t off_x, off_scr, off_oh, off_stage, off_tail, off_sel, off_la, off_close, off_closeany, off_rowenv, off_dstp, off_tdst, off_bar, total;
 };
 
 struct TpBars {
@@ -70,7 +70,9 @@ struct TpBars {
 };
 
 // M, sms: the launch's batch and the number of blocks it may use (0: the largest tiles, for the shape check).
-static TpLayout tp_layout(int n, int D, int A, int rec_bytes, int M = 0, int sms = 0) {
+// fastx: the launch moves its hidden-state rows through a scratch (modes 1 to 3 of the kernel).
+static TpLayout tp_layout(int n, int D, int A, int rec_bytes, int M = 0, int sms = 0, bool fastx = true,
+                          uint32_t reserve = 0) {
   const TcLayout W = tc_layout(n, D, A, rec_bytes);
   TpLayout L;
   memset(&L, 0, sizeof(L));
@@ -105,8 +107,7 @@ static TpLayout tp_layout(int n, int D, int A, int rec_bytes, int M = 0, int sms
   L.chunk_bytes = L.plain ? TP_G * L.obs_bytes + up16(TP_G * L.av_bytes) + 16u : TP_G * L.prefix_bytes;
   uint32_t o = L.wbytes;
   L.off_x = o; o += up16((uint32_t)L.nchunk * TC_LBO_X);
-  L.off_y = o; o += 8 * TC_LBO_A;
-  L.off_hb = o; o += 8 * TC_LBO_A;
+  L.off_scr = o; o += fastx ? 8 * 2048u : 0;
   L.off_oh = o; o += (uint32_t)L.ohc * TC_LBO_A;
   L.off_tail = o; o += 2u * (uint32_t)L.ept * L.tail_bytes;
   L.off_sel = o; o += 4u * TC_ROWS * 8;
@@ -122,7 +123,7 @@ static TpLayout tp_layout(int n, int D, int A, int rec_bytes, int M = 0, int sms
   // block padded to 16 bytes), one image per staging slot, for the store warp's bulk stores
   L.rs_env = L.plain == 1 ? up16(L.obs_bytes) + up16(L.av_bytes) : 0;  // the record's prefix [obs | avail], padded as in the ring
   L.rs_bytes = TP_G * L.rs_env;
-  const uint32_t room = o + 64 < TC_SMEM_MAX ? TC_SMEM_MAX - o - 64 : 0;
+  const uint32_t room = o + reserve + 64 < TC_SMEM_MAX ? TC_SMEM_MAX - o - reserve - 64 : 0;
   int ns = (int)(room / (L.chunk_bytes + L.rs_bytes));
   if (ns > TP_MAX_STAGES) ns = TP_MAX_STAGES;
   if (ns < 0) ns = 0;
@@ -143,7 +144,8 @@ static TpLayout tp_layout(int n, int D, int A, int rec_bytes, int M = 0, int sms
 bool tcp_supported(int n, int D, int A, int H, int prec) {
   if (prec != MARL_PRECISION_BF16 || H != TC_H) return false;
   if (D < 1 || D > 256 || n < 4 || n > 32 || A < 1 || A > 32) return false;
-  const TpLayout L = tp_layout(n, D, A, rec_bytes_of(n, D, A));
+  // (16 KB are kept back: the domain stated in the header does not move with what a layout happens to leave over)
+  const TpLayout L = tp_layout(n, D, A, rec_bytes_of(n, D, A), 0, 0, true, 8 * TC_LBO_A);
   // enough staging for loads to run ahead of the network (tp_layout leaves 0 where the ring would be unsafe)
   return L.ept >= TP_G && L.NS >= 3 && L.total <= TC_SMEM_MAX;
 }
@@ -157,6 +159,11 @@ __device__ __forceinline__ void warp_arrive(uint64_t* bar, int lane) {
   __syncwarp();
   if (lane == 0) tc::mbar_arrive(bar);
 }
+
+// The gate layer's left operands - fc1 output and hidden state, bf16 pairs - live in tensor memory behind the Q buffers:
+// tcgen05.mma reads them there, so shared memory, whose port the converters, bulk copies and weight operands keep
+// busy, is spared about 100 of 390 KB a step, and the epilogues need no proxy fence.
+constexpr uint32_t TMP_Y = 448, TMP_H = 480;
 
 // ---- MMA issue helpers.  Descriptors are rebuilt from the layout (kernel parameter space) where they are used:
 //      nothing is kept in local memory, whose loads would go to L2 - the L1 left beside 227 KB of shared memory is
@@ -196,7 +203,7 @@ __device__ __forceinline__ void tp_issue_hside(const TpLayout& L, uint32_t sb, u
   using namespace tc;
   tc_fence_after_sync();
   if (elect_one()) {
-    const uint64_t d_h = smem_desc(sb + L.off_hb, TC_LBO_A, 128), d_oh = smem_desc(sb + L.off_oh, TC_LBO_A, 128);
+    const uint64_t d_oh = smem_desc(sb + L.off_oh, TC_LBO_A, 128);
     const uint64_t d_Whh = smem_desc(sb + L.off_Whh, TP_LBO_G, 128);
     const uint64_t d_Whh_n = smem_desc(sb + L.off_Whh + 2 * TC_H * 16, TP_LBO_G, 128);  // the candidate rows of each k-chunk
     const uint64_t d_Bg = smem_desc(sb + L.off_Bg, TP_LBO_G, 128), d_Bhn = smem_desc(sb + L.off_Bhn, TP_LBO_W1, 128);
@@ -205,8 +212,8 @@ __device__ __forceinline__ void tp_issue_hside(const TpLayout& L, uint32_t sb, u
     mma_bf16(tmem + TM_R, d_oh, d_Bg, id192, 0);
 #pragma unroll
     for (int ks = 0; ks < 4; ++ks) {
-      mma_bf16(tmem + TM_R, d_h + ks * TP_K_A, d_Whh + ks * TP_K_G, id128, 1);
-      mma_bf16(tmem + TM_HN, d_h + ks * TP_K_A, d_Whh_n + ks * TP_K_G, id64, ks > 0);
+      mma_bf16_ts(tmem + TM_R, tmem + TMP_H + ks * 8, d_Whh + ks * TP_K_G, id128, 1);
+      mma_bf16_ts(tmem + TM_HN, tmem + TMP_H + ks * 8, d_Whh_n + ks * TP_K_G, id64, ks > 0);
     }
     mma_bf16(tmem + TM_HN, d_oh, d_Bhn, id64, 1);
     mma_bf16(tmem + qcol, d_oh, d_W2b, idesc_bf16_f32(128, NQ), 0);
@@ -232,8 +239,6 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
   using namespace tc;
   TpBars* B = reinterpret_cast<TpBars*>(smem + L.off_bar);
   uint8_t* xb = smem + L.off_x;
-  uint8_t* yb = smem + L.off_y;
-  uint8_t* hb = smem + L.off_hb;
   uint8_t* oh = smem + L.off_oh;
   uint8_t* stage = smem + L.off_stage;
   uint8_t* tails = smem + L.off_tail;                                  // [2][ept][tail_bytes]
@@ -331,30 +336,32 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
         mbar_wait(&B->yready, par, abortf);
         tc_fence_after_sync();
         if (elect_one()) {
-          const uint64_t d_y = smem_desc(sb + L.off_y, TC_LBO_A, 128), d_Wih = smem_desc(sb + L.off_Wih, TP_LBO_G, 128);
+          const uint64_t d_Wih = smem_desc(sb + L.off_Wih, TP_LBO_G, 128);
 #pragma unroll
-          for (int ks = 0; ks < 4; ++ks) mma_bf16(tmem + TM_R, d_y + ks * TP_K_A, d_Wih + ks * TP_K_G, idesc_bf16_f32(128, 192), 1);
+          for (int ks = 0; ks < 4; ++ks) mma_bf16_ts(tmem + TM_R, tmem + TMP_Y + ks * 8, d_Wih + ks * TP_K_G, idesc_bf16_f32(128, 192), 1);
           mma_commit(&B->grud);
         }
         __syncwarp();
         // fc1 of the next step (possibly the next tile's first): its accumulator is free since epilogue 1 of
-        // this step has read it; issue it now if the operand is already converted, else after fc2
+        // this step has read it; issue it when its operand is converted, but not before fc2 if that is ready first
         bool pending = g + 1 < total;
-        if (pending) {
+        for (uint32_t i = 0; pending && i < (1u << 16); ++i) {  // (bounded; hready has the bounded wait behind it)
           // one lane looks (lanes looking separately could disagree and split the warp's control flow)
-          const uint32_t ready = __shfl_sync(0xFFFFFFFFu, lane == 0 ? (uint32_t)mbar_test_wait(&B->xready, par ^ 1u) : 0u, 0);
-          if (ready) {
+          const uint32_t ready = __shfl_sync(0xFFFFFFFFu, lane == 0 ? (uint32_t)mbar_test_wait(&B->xready, par ^ 1u) | (uint32_t)mbar_test_wait(&B->hready, par) << 1 : 0u, 0);
+          if (ready & 1u) {
             tp_issue_fc1(L, sb, tmem, lane, &B->fc1d);
             pending = false;
+          } else if (ready & 2u) {
+            break;
           }
         }
         mbar_wait(&B->hready, par, abortf);
         tc_fence_after_sync();
         if (elect_one()) {
-          const uint64_t d_h = smem_desc(sb + L.off_hb, TC_LBO_A, 128), d_W2 = smem_desc(sb + L.off_W2, NQ * 16, 128);
+          const uint64_t d_W2 = smem_desc(sb + L.off_W2, NQ * 16, 128);
 #pragma unroll
           for (int ks = 0; ks < 4; ++ks)  // part 0 holds the bias already; parts 1..3 start from zero
-            mma_bf16(tmem + qcol + (NQ == 16 ? ks * NQ : 0), d_h + ks * TP_K_A, d_W2 + ks * ((2 * NQ * 16) >> 4), idesc_bf16_f32(128, NQ),
+            mma_bf16_ts(tmem + qcol + (NQ == 16 ? ks * NQ : 0), tmem + TMP_H + ks * 8, d_W2 + ks * ((2 * NQ * 16) >> 4), idesc_bf16_f32(128, NQ),
                      (NQ == 16 && ks > 0) ? 0 : 1);
           mma_commit(&B->fc2d);
         }
@@ -765,6 +772,15 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
     unsigned long long c_steps = 0, c_explore = 0, c_noavail = 0;
     uint32_t st_bits = 0, it = 0;
     float h[32];
+    const uint32_t tm_y = tmem + lane_addr + TMP_Y + (uint32_t)cb / 2u, tm_h = tmem + lane_addr + TMP_H + (uint32_t)cb / 2u;
+    auto store_h = [&](int c0, int c1) {  // groups of eight columns [c0, c1) of the hidden operand
+#pragma unroll
+      for (int c8 = 0; c8 < 4; ++c8)
+        if (c8 >= c0 && c8 < c1) {
+          const float* hv = h + c8 * 8;
+          tmem_st4(tm_h + (uint32_t)c8 * 4u, pack_bf16x2(hv[0], hv[1]), pack_bf16x2(hv[2], hv[3]), pack_bf16x2(hv[4], hv[5]), pack_bf16x2(hv[6], hv[7]));
+        }
+    };
     // this thread's half (32 floats) of tile row r's hidden state in global memory
     auto h_row = [&](int e0, int r) -> float* {
       if (!LIST) return p.h + ((size_t)e0 * n + (size_t)r) * TC_H + cb;  // a tile's rows are contiguous
@@ -792,11 +808,10 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
         }
         const int la_mem = (carry && half == 0) ? p.last_action[grow] : -1;  // in flight beside the rows below
         // A thread owns 128 bytes of its row, so a warp reading "its own" pieces would touch 32 lines per
-        // instruction.  The rows go through a warp-private 2 KB scratch instead (the y operand buffer, idle
-        // between tiles): eight lanes fetch one row's 128 bytes, the scratch's piece index is xor-ed with the row so
+        // instruction.  The rows go through a warp-private 2 KB scratch instead: eight lanes fetch one row's 128 bytes, the scratch's piece index is xor-ed with the row so
         // that neither side has bank conflicts, and each thread then takes its row, 16 rows per pass.
         if constexpr (FASTX) {
-          uint4* sw = reinterpret_cast<uint4*>(yb) + warp * 128;  // this warp's scratch
+          uint4* sw = reinterpret_cast<uint4*>(smem + L.off_scr) + warp * 128;  // this warp's scratch
           const int wrow0 = (warp & 3) * 32;                      // first tile row of this warp
           uint4 f[2][4];
 #pragma unroll
@@ -838,18 +853,13 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
             h[4 * q] = v.x; h[4 * q + 1] = v.y; h[4 * q + 2] = v.z; h[4 * q + 3] = v.w;
           }
         }
-#pragma unroll
-        for (int cc = 0; cc < 4; ++cc) {
-          const uint4 o = make_uint4(pack_bf16x2(h[8 * cc], h[8 * cc + 1]), pack_bf16x2(h[8 * cc + 2], h[8 * cc + 3]),
-                                     pack_bf16x2(h[8 * cc + 4], h[8 * cc + 5]), pack_bf16x2(h[8 * cc + 6], h[8 * cc + 7]));
-          *reinterpret_cast<uint4*>(hb + (uint32_t)(half * 4 + cc) * TC_LBO_A + (uint32_t)row * 16u) = o;
-        }
+        store_h(0, 4);
+        tmem_st_wait();
         if (half == 0) {
           la = la_mem;
           if (la >= A) la = -1;
           la_s[row] = la;
         }
-        fence_proxy_async_smem();
         tc_fence_before_sync();
         asm volatile("bar.sync 1, 256;" ::: "memory");  // la_s is read by both threads of a row
         warp_arrive(&B->tiled, lane);
@@ -896,15 +906,13 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
               y[4 * q + 2] = fmaxf(__uint_as_float(v[4 * q + 2]) + l4.z, 0.f);
               y[4 * q + 3] = fmaxf(__uint_as_float(v[4 * q + 3]) + l4.w, 0.f);
             }
+            uint32_t w[8];
 #pragma unroll
-            for (int cc = 0; cc < 2; ++cc) {
-              const uint4 o = make_uint4(pack_bf16x2(y[8 * cc], y[8 * cc + 1]), pack_bf16x2(y[8 * cc + 2], y[8 * cc + 3]),
-                                         pack_bf16x2(y[8 * cc + 4], y[8 * cc + 5]), pack_bf16x2(y[8 * cc + 6], y[8 * cc + 7]));
-              *reinterpret_cast<uint4*>(yb + (uint32_t)(half * 4 + c16 * 2 + cc) * TC_LBO_A + (uint32_t)row * 16u) = o;
-            }
+            for (int k = 0; k < 8; ++k) w[k] = pack_bf16x2(y[2 * k], y[2 * k + 1]);
+            tmem_st8(tm_y + (uint32_t)c16 * 8u, w);
           }
         }
-        fence_proxy_async_smem();
+        tmem_st_wait();
         tc_fence_before_sync();
         warp_arrive(&B->yready, lane);
 
@@ -937,13 +945,10 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
               const float hp = h[c8 * 8 + j];
               h[c8 * 8 + j] = fmaf(zg, hp - cand, cand);  // (1 - z) * cand + z * h
             }
-            const float* hv = h + c8 * 8;
-            const uint4 o = make_uint4(pack_bf16x2(hv[0], hv[1]), pack_bf16x2(hv[2], hv[3]), pack_bf16x2(hv[4], hv[5]),
-                                       pack_bf16x2(hv[6], hv[7]));
-            *reinterpret_cast<uint4*>(hb + (uint32_t)(half * 4 + c8) * TC_LBO_A + (uint32_t)row * 16u) = o;
+            store_h(c8, c8 + 1);
           }
         }
-        fence_proxy_async_smem();
+        tmem_st_wait();
         tc_fence_before_sync();
         warp_arrive(&B->hready, lane);
 
@@ -1024,15 +1029,16 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
         }
         asm volatile("bar.sync 1, 256;" ::: "memory");
         // ---- a closed episode restarts from a zero hidden state and no last action ----
-        if (live && close_s[b * 32 + el]) {
+        const bool closed = live && close_s[b * 32 + el];
+        if (__any_sync(0xFFFFFFFFu, closed)) {
+          if (closed) {
 #pragma unroll
-          for (int j = 0; j < 32; ++j) h[j] = 0.f;
-#pragma unroll
-          for (int cc = 0; cc < 4; ++cc)
-            *reinterpret_cast<uint4*>(hb + (uint32_t)(half * 4 + cc) * TC_LBO_A + (uint32_t)row * 16u) = make_uint4(0, 0, 0, 0);
-          if (half == 0) la = -1;
+            for (int j = 0; j < 32; ++j) h[j] = 0.f;
+            if (half == 0) la = -1;
+          }
+          store_h(0, 4);  // (tensor-memory stores take the whole warp)
+          tmem_st_wait();
         }
-        fence_proxy_async_smem();
         tc_fence_before_sync();
         warp_arrive(&B->stepd, lane);
         ++it;
@@ -1041,7 +1047,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
       // ---- tile epilogue: state back to global memory ----
       if (is_row) p.last_action[grow] = la;
       if constexpr (FASTX) {
-        uint4* sw = reinterpret_cast<uint4*>(yb) + warp * 128;
+        uint4* sw = reinterpret_cast<uint4*>(smem + L.off_scr) + warp * 128;
         const int wrow0 = (warp & 3) * 32;
 #pragma unroll
       for (int ps = 0; ps < 2; ++ps) {  // the rows leave through the same scratch, coalesced
@@ -1085,7 +1091,8 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
 // Returns the number of kernels launched, 0 if this launch's pointers do not meet the kernel's alignment
 // needs (the caller then uses the one-tile kernel), or a negative cudaError.
 int launch_actor_tcp(const ActorParams& p_in, int sms, cudaStream_t stream) {
-  const TpLayout L = tp_layout(p_in.n, p_in.D, p_in.A, (int)p_in.rl.rec_bytes, p_in.M, sms);
+  const int mode = p_in.env_ids == nullptr ? (p_in.T < 8 ? 3 : 0) : (p_in.lagged ? 2 : 1);
+  const TpLayout L = tp_layout(p_in.n, p_in.D, p_in.A, (int)p_in.rl.rec_bytes, p_in.M, sms, mode != 0);
   ActorParams p = p_in;
   p.ept = L.ept;  // (tiles of whole chunks for the plain shapes)
   p.num_tiles = (p.M + L.ept - 1) / L.ept;
@@ -1095,7 +1102,6 @@ int launch_actor_tcp(const ActorParams& p_in, int sms, cudaStream_t stream) {
   // the last chunk's availability bytes must end inside the step's block
   if (L.plain == 1 && p.M % TP_G != 0) return 0;
   if (L.plain != 0 && ((size_t)p.M * p.n * p.A) % 16 != 0) return 0;
-  const int mode = p.env_ids == nullptr ? (p.T < 8 ? 3 : 0) : (p.lagged ? 2 : 1);
   if (p.lagged && (mode != 2 || p.T != 1)) return 0;  // late outcomes: one step per launch over a list
   auto pick = [&](auto nq) {
     constexpr int Q = decltype(nq)::value;
