@@ -367,7 +367,7 @@ int marl_measure_ffma_tflops(void* stream, double* tflops_out);
 
 /* Name of the step kernel in use: "ffma" (the general path: split-operand tensor-core or CUDA-core kernel), "tcgen05" (one-tile tensor-core kernel), "tcgen05-pipelined",
  * "tcgen05-dual" (two resident tiles; its other launches run on the pipelined kernel), or
- * "tcgen05-streamed" (hidden size 128: the pipelined design with the weights streamed through shared memory). */
+ * "tcgen05-streamed" (hidden size 128: weights kept in shared memory as far as they fit, the others streamed). */
 const char* marl_actor_kernel_name(const marl_actor_t* a);
 
 /* Launches of library kernels enqueued by this actor since creation (all kernels, all entry points). */

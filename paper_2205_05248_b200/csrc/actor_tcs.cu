@@ -47,19 +47,22 @@ constexpr int TS_MAX_SLOTS = 8;
 constexpr int TS_KCHUNK = 96;       // K of one W1 slice: no larger than a gate slice
 // Tensor-memory columns.  Two accumulator buffers of a gate block, laid out so that the columns fc1 uses at hidden 64
 // (the candidate-input parts of both) are contiguous: HN R Z IN | IN R Z HN.
-constexpr uint32_t TSM_HOP = 256, TSM_Q = 480;
+// Behind them the hidden operand, the y operand, the x operand - with room for all, else x and y share columns - and Q.
+constexpr uint32_t TSM_HOP = 256, TSM_COLS = 512;
 
 struct TsLayout {
   int32_t Dk, NQ, nw1, nsl, nres, nslots;   // K of fc1; Q columns; W1 slices; slices; resident ones; ring slots
   int32_t nu;                               // staged units per input warp
   int32_t ept, ntypes;
+  int32_t sep;                              // x and y operands have columns of their own
+  uint32_t tm_x, tm_q;                      // first columns of x (y follows the hidden operand) and Q
   uint32_t base_bytes, off_b2, off_bias, off_tabA, off_tabL;  // base part of the image: W2 pieces, biases, column tables
   uint32_t img_bytes;
   uint32_t off_sl, off_ring, off_xy, off_scr, off_recp, off_sel, off_pick, off_la, off_close, off_eid, off_row, off_bar, total;
 };
 
 struct TsBars {
-  uint64_t xrdy, fc1d, hset, yrdy, gd[2], accf[2], hr0, hr1, fc2d, qfree, res[2];
+  uint64_t xrdy, srdy[4], fc1d, hset, yrdy, gd[2], accf[2], hr0, hr1, fc2d, qfree, res[2];
   uint64_t full[TS_MAX_SLOTS], empty[TS_MAX_SLOTS];
   uint32_t tmem_base, abort;
 };
@@ -90,9 +93,13 @@ static TsLayout ts_image(int n, int D, int A, int H, int ns) {
   L.NQ = A <= 16 ? 16 : 32;
   L.nw1 = ns == 3 ? 3 : (L.Dk + TS_KCHUNK - 1) / TS_KCHUNK;
   L.nsl = L.nw1 + (H / TS_BLK) * 2 * ns;
+  const uint32_t tm_y = TSM_HOP + (uint32_t)(ns * H / 2);
+  L.sep = tm_y + (uint32_t)(ns * (H + L.Dk) / 2 + L.NQ) <= TSM_COLS;
+  L.tm_x = L.sep ? tm_y + (uint32_t)(ns * H / 2) : tm_y;
+  L.tm_q = TSM_COLS - (uint32_t)L.NQ;
   uint32_t o = (uint32_t)ns * (uint32_t)H * L.NQ * 2;
   L.off_b2 = o; o += 32 * 4;
-  L.off_bias = o; o += 4u * H * 4;
+  L.off_bias = o; o += (H == 128 ? 6u : 4u) * H * 4;  // (hidden 128: reset and update again, for the fast gates)
   L.off_tabA = o; o += (uint32_t)n * (H + 4) * 4;
   L.off_tabL = o; o += (uint32_t)A * (H + 4) * 4;
   L.base_bytes = ts_up(o, 128);
@@ -165,8 +172,15 @@ bool tcs_supported(int n, int D, int A, int H, int prec) {
   if (L.ept == 0) return false;
   if (H == 64 && L.nres < L.nsl) return false;
   if (ns == 3 && L.Dk > TS_KCHUNK) return false;
-  const int xcols = ns * (L.Dk > H ? L.Dk : H) / 2;
-  return (ns == 3 && H == 128) || (int)TSM_HOP + ns * H / 2 + xcols <= (int)TSM_Q;
+  const uint32_t xcols = (uint32_t)(ns * (L.Dk > H ? L.Dk : H) / 2);
+  return (ns == 3 && H == 128) || L.sep || TSM_HOP + (uint32_t)(ns * H / 2) + xcols <= L.tm_q;
+}
+
+// Dense launches with the hardware's gate functions: bf16 at hidden size 128 on the shapes of the scenarios' teams (the
+// domain that the header states for the pipelined kernel at this size).
+bool tcs_fast_supported(int n, int D, int A, int H, int prec) {
+  return prec == MARL_PRECISION_BF16 && H == 128 && n >= 4 && D <= 256 && D % 8 == 0 && A <= 16 && (n * A) % 16 == 0 &&
+         tcs_supported(n, D, A, H, prec);
 }
 
 size_t tcs_image_bytes(int n, int D, int A, int H, int prec) {
@@ -238,6 +252,10 @@ void tcs_pack_weights(int n, int D, int A, int H, int prec, const float* W1, con
     bias[H + j] = -TS_LOG2E * (bih[H + j] + bhh[H + j]);
     bias[2 * H + j] = bih[2 * H + j];
     bias[3 * H + j] = bhh[2 * H + j];
+    if (H == 128) {
+      bias[4 * H + j] = 0.5f * (bih[j] + bhh[j]);
+      bias[5 * H + j] = 0.5f * (bih[H + j] + bhh[H + j]);
+    }
   }
   auto col = [&](float v) { return ns == 1 ? ts_float(ts_bf16(v)) : v; };
   float* tabA = reinterpret_cast<float*>(dst + L.off_tabA);
@@ -364,6 +382,25 @@ __device__ __forceinline__ void ts_gates2(const float (&v)[4][2], const ts_f2 (&
   f2_get(f2_fma(zg, f2_fma(c, f2(-1.0f), f2(h0, h1)), c), h0, h1);  // (1 - z) * cand + z * h
 }
 
+// The same with the hardware's tanh (bf16 rollouts at hidden size 128, which have always used it): sigmoid(v) =
+// 0.5 tanh(v / 2) + 0.5, b[0] and b[1] halved.  Three special functions per column.
+__device__ __forceinline__ float ts_tanh_hw(float x) {
+  float y;
+  asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ void ts_gates2_fast(const float (&v)[4][2], const ts_f2 (&b)[4], float& h0, float& h1) {
+  const ts_f2 half = f2(0.5f);
+  float r0, r1, z0, z1, u0, u1;
+  f2_get(f2_fma(f2(v[0][0], v[0][1]), half, b[0]), r0, r1);
+  f2_get(f2_fma(f2(v[1][0], v[1][1]), half, b[1]), z0, z1);
+  const ts_f2 rg = f2_fma(f2(ts_tanh_hw(r0), ts_tanh_hw(r1)), half, half);
+  const ts_f2 zg = f2_fma(f2(ts_tanh_hw(z0), ts_tanh_hw(z1)), half, half);
+  f2_get(f2_fma(rg, f2_add(f2(v[3][0], v[3][1]), b[3]), f2_add(f2(v[2][0], v[2][1]), b[2])), u0, u1);
+  const ts_f2 c = f2(ts_tanh_hw(u0), ts_tanh_hw(u1));
+  f2_get(f2_fma(zg, f2_fma(c, f2(-1.0f), f2(h0, h1)), c), h0, h1);
+}
+
 // D (+)= A B^T, issued by one lane; A in shared memory (AS: descriptor) or in tensor memory (column address).
 template <bool AS>
 __device__ __forceinline__ void ts_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
@@ -373,17 +410,21 @@ __device__ __forceinline__ void ts_mma(uint32_t d, uint64_t a, uint64_t b, uint3
 
 }  // namespace
 
-template <int NS, int NQ, int H>
+template <int NS, int NQ, int H, bool FAST = false>
 __global__ void __launch_bounds__(TS_THREADS, 1)
     actor_tcs_kernel(const __grid_constant__ ActorParams p, const __grid_constant__ TsLayout L) {
   using namespace tc;
   constexpr int NBLK = H / TS_BLK, KH = H / 16;
+  // The epilogue's loops over blocks: rolled for one piece at hidden 64 (the shorter code misses the instruction cache
+  // less: 353 us against 400 for 4096 x 3 agents x 64 steps), unrolled where the hidden state's registers would have to
+  // rotate further (hidden 128: 3394 us against 3997) or the pieces' arithmetic hides the misses (fp32: 1047 against 1064).
+  constexpr int UB = NS == 1 && H == 64 ? 1 : NBLK;
   constexpr bool XS = NS == 3 && H == 128;       // x and y pieces in shared memory
-  constexpr uint32_t TSM_XY = TSM_HOP + NS * H / 2;
+  constexpr uint32_t TSM_Y = TSM_HOP + NS * H / 2;
   constexpr uint32_t FC1 = H == 64 ? 96 : 0;     // fc1's accumulator: the candidate-input columns, or buffer 0
   // Registers (setmaxnreg): launched with 96 a thread (640 * 96 = 61440); afterwards
-  // 256 * 120 + 256 * 88 + 128 * 64 or, hidden 128, 256 * 128 + 256 * 88 + 128 * 48.
-  constexpr int REGS_EPI = H == 64 ? 120 : 128, REGS_PREP = 88, REGS_SVC = H == 64 ? 64 : 48;
+  // 256 * 128 + 256 * 88 + 128 * 48 = 61440.
+  constexpr int REGS_EPI = 128, REGS_PREP = 88, REGS_SVC = 48;
   extern __shared__ __align__(1024) uint8_t smem[];
   TsBars* B = reinterpret_cast<TsBars*>(smem + L.off_bar);
   // per-step hand-offs, four buffers each: the input warps run up to two steps ahead of the choice
@@ -407,6 +448,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
 
   if (tid == 0) {
     mbar_init(&B->xrdy, TS_PREP / 32);
+    for (int i = 0; i < 4; ++i) mbar_init(&B->srdy[i], TS_PREP / 32);
     mbar_init(&B->fc1d, 1);
     mbar_init(&B->hset, TS_EPI / 32);
     mbar_init(&B->yrdy, TS_EPI / 32);
@@ -451,7 +493,8 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
       // the left operands and the distance between their pieces and K steps
       const uint64_t a_h = tmem + TSM_HOP;
       constexpr uint64_t h_st = H / 2, h_ks = 8;
-      const uint64_t a_x = XS ? smem_desc(sb + L.off_xy, 2048, 128) : (uint64_t)(tmem + TSM_XY);
+      const uint64_t a_x = XS ? smem_desc(sb + L.off_xy, 2048, 128) : (uint64_t)(tmem + L.tm_x);
+      const uint64_t a_y = XS ? a_x : (uint64_t)(tmem + TSM_Y);
       constexpr uint64_t x_ks = XS ? (2 * 2048) >> 4 : 8;
       const uint64_t x_st = (uint64_t)nk1 * x_ks;
       constexpr uint64_t y_st = KH * x_ks;
@@ -479,7 +522,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
       auto prod = [&](int buf, int hid, uint32_t ai, uint64_t w, uint32_t acc) {
         const uint32_t d = tmem + (hid ? (buf ? 160u : 0u) : (buf ? 128u : 32u));
         if (XS && !hid) {
-          const uint64_t a = a_x + ai * y_st;
+          const uint64_t a = a_y + ai * y_st;
           if (acc) {
             ts_mma<true>(d, a, w, id96, 1);
           } else {  // buffer 0: R Z at rows 0.., IN at rows 64..; buffer 1: IN at rows 0.., R Z at rows 32..
@@ -489,7 +532,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
 #pragma unroll
           for (int ks = 1; ks < KH; ++ks) ts_mma<true>(d, a + ks * x_ks, w + ks * ks_g, id96, 1);
         } else {
-          const uint64_t a = hid ? a_h + ai * h_st : a_x + ai * y_st;
+          const uint64_t a = hid ? a_h + ai * h_st : a_y + ai * y_st;
           if (hid || acc) {
             ts_mma<false>(d, a, w, id96, acc);
           } else {
@@ -647,12 +690,12 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
                   for (int j = 0; j < 5; ++j) {
                     const uint64_t a = a_h + ((0x01012u >> (4 * j)) & 15u) * h_st, w = w2 + ((0x10210u >> (4 * j)) & 15u) * st_q;
 #pragma unroll
-                    for (int ks = k0; ks < k1; ++ks) ts_mma<false>(tmem + TSM_Q, a + ks * h_ks, w + ks * ks_q, idq, ks > 0 || j > 0);
+                    for (int ks = k0; ks < k1; ++ks) ts_mma<false>(tmem + L.tm_q, a + ks * h_ks, w + ks * ks_q, idq, ks > 0 || j > 0);
                   }
                 }
                 if (NS == 1 || half)
 #pragma unroll
-                  for (int ks = NS == 3 ? 0 : k0; ks < k1; ++ks) ts_mma<false>(tmem + TSM_Q, a_h + ks * h_ks, w2 + ks * ks_q, idq, NS == 3 || ks > 0);
+                  for (int ks = NS == 3 ? 0 : k0; ks < k1; ++ks) ts_mma<false>(tmem + L.tm_q, a_h + ks * h_ks, w2 + ks * ks_q, idq, NS == 3 || ks > 0);
                 if (half) mma_commit(&B->fc2d);
               }
               __syncwarp();
@@ -889,10 +932,13 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
             pick_s[b * TS_ROWS + row] = (int8_t)pick;
           }
           asm volatile("bar.sync 3, 256;" ::: "memory");  // the step's records are known
+          ts_arrive(&B->srdy[b], lane);
           prevrec = myrec;
           myrec = live ? recp_s[b * ept + el] : 0ull;
-          if (gk > 0) {  // the y operand (same place) has been read by the previous step's gate products
-            mbar_wait(H == 64 ? &B->gd[1] : &B->hr0, (gk - 1) & 1, abortf);  // (barriers with one phase a step)
+          if (gk > 0) {
+            // the operand has been read by the previous step's fc1 or, where y takes its place, the y operand by the
+            // gate products (barriers with one phase a step)
+            mbar_wait(L.sep ? &B->fc1d : H == 64 ? &B->gd[1] : &B->hr0, (gk - 1) & 1, abortf);
             tc_fence_after_sync();
           }
           if (wlive) {
@@ -915,7 +961,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
                   *reinterpret_cast<uint4*>(to) = make_uint4(w[0], w[1], w[2], w[3]);
                   *reinterpret_cast<uint4*>(to + 2048) = make_uint4(w[4], w[5], w[6], w[7]);
                 } else {
-                  tmem_st8(tm + TSM_XY + (uint32_t)(i * nk + ks) * 8u, w);
+                  tmem_st8(tm + L.tm_x + (uint32_t)(i * nk + ks) * 8u, w);
                 }
               });
               const int c = ks * 16 + 4 * c4;
@@ -971,8 +1017,8 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
           tc_fence_after_sync();
           if (wlive) {
             uint32_t qv[NQ];
-            tmem_ld16(tm + TSM_Q, *reinterpret_cast<uint32_t(*)[16]>(qv));
-            if (NQ == 32) tmem_ld16(tm + TSM_Q + 16, *reinterpret_cast<uint32_t(*)[16]>(qv + NQ - 16));
+            tmem_ld16(tm + L.tm_q, *reinterpret_cast<uint32_t(*)[16]>(qv));
+            if (NQ == 32) tmem_ld16(tm + L.tm_q + 16, *reinterpret_cast<uint32_t(*)[16]>(qv + NQ - 16));
             tmem_ld_wait();
             tc_fence_before_sync();
             ts_arrive(&B->qfree, lane);
@@ -1053,10 +1099,10 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
         const int e = eid_s[el];
         const size_t grow = (size_t)e * n + ai;
         float h[NBLK][16];
-        auto store_h = [&](int b) {  // the pieces of one block's hidden state
+        auto store_h = [&](int b, const float (&hb)[16]) {  // the pieces of block b's hidden state
           float v[16];
 #pragma unroll
-          for (int j = 0; j < 16; ++j) v[j] = h[b][j];
+          for (int j = 0; j < 16; ++j) v[j] = hb[j];
           ts_split16<NS>(v, [&](int i, const uint32_t (&w)[8]) {
             tmem_st8(tm + TSM_HOP + (uint32_t)(i * (H / 2) + b * (TS_BLK / 2) + grp * 8), w);
           });
@@ -1079,7 +1125,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
           }
           if (wlive) {
 #pragma unroll
-            for (int b = 0; b < NBLK; ++b) store_h(b);
+            for (int b = 0; b < NBLK; ++b) store_h(b, h[b]);
             tmem_st_wait();
           }
           tc_fence_before_sync();
@@ -1093,15 +1139,12 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
         for (int s = 0; s < T; ++s, ++g) {
           const uint32_t par = g & 1u, b4 = g & 3u;
           // ---- E1 ----
-          // (the inputs' own barrier orders their records and draws; looked at here, before the input warps can be two
-          // phases ahead of a parity wait)
-          mbar_wait(&B->xrdy, par, abortf);
           mbar_wait(&B->fc1d, par, abortf);
           tc_fence_after_sync();
           if (wlive) {
             const int last = la_s[row];
             const float* tl = tl0 + (last >= 0 ? last : 0) * (H + 4);
-#pragma unroll
+#pragma unroll UB
             for (int b = 0; b < NBLK; ++b) {
               uint32_t a[16];
               tmem_ld16(tm + FC1 + (uint32_t)(b * TS_BLK + grp * 16), a);
@@ -1123,7 +1166,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
                   *reinterpret_cast<uint4*>(to) = make_uint4(w[0], w[1], w[2], w[3]);
                   *reinterpret_cast<uint4*>(to + 2048) = make_uint4(w[4], w[5], w[6], w[7]);
                 } else {
-                  tmem_st8(tm + TSM_XY + (uint32_t)(i * (H / 2) + k8 * 4), w);
+                  tmem_st8(tm + TSM_Y + (uint32_t)(i * (H / 2) + k8 * 4), w);
                 }
               });
             }
@@ -1134,7 +1177,8 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
           ts_arrive(&B->yrdy, lane);
 
           // ---- E2 ----
-#pragma unroll
+          // one block of 32 hidden columns per pass; the block at work is h[0], the others move up behind it
+#pragma unroll UB
           for (int b = 0; b < NBLK; ++b) {
             const int buf = H == 64 ? b : (b + 1) & 1;
             mbar_wait(&B->gd[buf], H == 64 ? par : (uint32_t)(b >> 1), abortf);
@@ -1142,7 +1186,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
             if (b == NBLK - 1) {  // no product reads the old hidden state any more
               if (wlive) {
 #pragma unroll
-                for (int k = 0; k < NBLK - 1; ++k) store_h(k);
+                for (int k = 0; k < NBLK - 1; ++k) store_h(k, h[k + 1]);
                 tmem_st_wait();
               }
               tc_fence_before_sync();
@@ -1169,7 +1213,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
                 for (int j = 0; j < 8; j += 4) {
                   ulonglong2 bv[4];  // biases of four columns
 #pragma unroll
-                  for (int k = 0; k < 4; ++k) bv[k] = *reinterpret_cast<const ulonglong2*>(bb + k * H + j);
+                  for (int k = 0; k < 4; ++k) bv[k] = *reinterpret_cast<const ulonglong2*>(bb + (FAST && k < 2 ? k + 4 : k) * H + j);
 #pragma unroll
                   for (int c = 0; c < 4; c += 2) {
                     float a[4][2];
@@ -1180,33 +1224,42 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
                       a[k][1] = __uint_as_float(v[k][j + c + 1]);
                       b2[k] = c == 0 ? bv[k].x : bv[k].y;
                     }
-                    ts_gates2(a, b2, h[b][c8 * 8 + j + c], h[b][c8 * 8 + j + c + 1]);
+                    if constexpr (FAST) ts_gates2_fast(a, b2, h[0][c8 * 8 + j + c], h[0][c8 * 8 + j + c + 1]);
+                    else ts_gates2(a, b2, h[0][c8 * 8 + j + c], h[0][c8 * 8 + j + c + 1]);
                   }
                 }
               }
             } else if (H == 128 && b < NBLK - 2) {
               ts_arrive(&B->accf[buf], lane);
             }
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              const float x = h[0][j];
+#pragma unroll
+              for (int k = 0; k + 1 < NBLK; ++k) h[k][j] = h[k + 1][j];
+              h[NBLK - 1][j] = x;
+            }
           }
           if (wlive) {
-            store_h(NBLK - 1);
+            store_h(NBLK - 1, h[NBLK - 1]);
             tmem_st_wait();
           }
           tc_fence_before_sync();
           ts_arrive(&B->hr1, lane);
 
           // ---- E3 ----
+          mbar_wait(&B->srdy[b4], (g >> 2) & 1u, abortf);  // the step's records and draws
           const bool close = live && close_s[b4 * ept + el];
           mbar_wait(&B->fc2d, par, abortf);
           tc_fence_after_sync();
           uint32_t qv[NQ];
           if (grp == 0 && wlive) {
-            tmem_ld16(tm + TSM_Q, *reinterpret_cast<uint32_t(*)[16]>(qv));
-            if (NQ == 32) tmem_ld16(tm + TSM_Q + 16, *reinterpret_cast<uint32_t(*)[16]>(qv + NQ - 16));
+            tmem_ld16(tm + L.tm_q, *reinterpret_cast<uint32_t(*)[16]>(qv));
+            if (NQ == 32) tmem_ld16(tm + L.tm_q + 16, *reinterpret_cast<uint32_t(*)[16]>(qv + NQ - 16));
             tmem_ld_wait();
           }
           // a closed episode restarts from a zero hidden state and no last action
-          if (wlive && __any_sync(0xFFFFFFFFu, close)) {
+          if (wlive && __builtin_expect(__any_sync(0xFFFFFFFFu, close), 0)) {
             if (close) {
 #pragma unroll
               for (int b = 0; b < NBLK; ++b)
@@ -1214,7 +1267,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
                 for (int j = 0; j < 16; ++j) h[b][j] = 0.f;
             }
 #pragma unroll
-            for (int b = 0; b < NBLK; ++b) store_h(b);
+            for (int b = 0; b < NBLK; ++b) store_h(b, h[b]);
             tmem_st_wait();
           }
           tc_fence_before_sync();
@@ -1280,8 +1333,8 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
   if (warp == 16) tmem_dealloc(tmem, 512);
 }
 
-// Returns the number of kernels launched or a negative cudaError.
-int launch_actor_tcs(const ActorParams& p_in, int sms, cudaStream_t stream) {
+// Returns the number of kernels launched or a negative cudaError.  fast_gates: the hardware tanh (bf16, hidden 128).
+int launch_actor_tcs(const ActorParams& p_in, int sms, bool fast_gates, cudaStream_t stream) {
   ActorParams p = p_in;
   int nt_max = p.n, ntypes = 1;
   if (p.n_types > 1) {
@@ -1296,13 +1349,20 @@ int launch_actor_tcs(const ActorParams& p_in, int sms, cudaStream_t stream) {
   const int ns = ts_pieces(p.prec);
   TsLayout L = ts_layout(p.n, p.D, p.A, p.H, ns, nt_max, p.M, sms);
   L.ntypes = ntypes;
+  if (p.H == 128 && !fast_gates) {
+    // the accurate gates keep the epilogue so busy that input warps running beside it all step long cost more than the
+    // wait for the shared columns (1216 against 1246 us for 4096 x 5 agents x 64 steps; fast gates: 3940 against 3410)
+    L.sep = 0;
+    L.tm_x = TSM_HOP + (uint32_t)(ns * p.H / 2);
+  }
   p.ept = L.ept;
   p.num_tiles = (p.M + L.ept - 1) / L.ept;
-  const int v = (ns == 3 ? 0 : 4) + (L.NQ == 16 ? 0 : 2) + (p.H == 64 ? 0 : 1);
-  decltype(&actor_tcs_kernel<3, 16, 64>) kernels[8] = {
+  const int v = fast_gates ? 8 : (ns == 3 ? 0 : 4) + (L.NQ == 16 ? 0 : 2) + (p.H == 64 ? 0 : 1);
+  decltype(&actor_tcs_kernel<3, 16, 64>) kernels[9] = {
       actor_tcs_kernel<3, 16, 64>, actor_tcs_kernel<3, 16, 128>, actor_tcs_kernel<3, 32, 64>, actor_tcs_kernel<3, 32, 128>,
-      actor_tcs_kernel<1, 16, 64>, actor_tcs_kernel<1, 16, 128>, actor_tcs_kernel<1, 32, 64>, actor_tcs_kernel<1, 32, 128>};
-  static uint32_t configured[8][SMEM_OPTIN_DEVICES];
+      actor_tcs_kernel<1, 16, 64>, actor_tcs_kernel<1, 16, 128>, actor_tcs_kernel<1, 32, 64>, actor_tcs_kernel<1, 32, 128>,
+      actor_tcs_kernel<1, 16, 128, true>};
+  static uint32_t configured[9][SMEM_OPTIN_DEVICES];
   {
     const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernels[v]), L.total, configured[v]);
     if (e != cudaSuccess) return -(int)e;

@@ -30,14 +30,13 @@ bool tcp_supported(int n, int D, int A, int H, int prec);
 int launch_actor_tcp(const ActorParams& p, int sms, cudaStream_t stream);
 bool tc2_supported(int n, int D, int A, int H, int prec);
 int launch_actor_tc2(const ActorParams& p, int sms, cudaStream_t stream);
-bool tcw_supported(int n, int D, int A, int H, int prec);
-int launch_actor_tcw(const ActorParams& p, int sms, cudaStream_t stream);
 // split-operand tensor-core kernel: the general path wherever its shape is supported
 bool tcs_supported(int n, int D, int A, int H, int prec);
 size_t tcs_image_bytes(int n, int D, int A, int H, int prec);
 void tcs_pack_weights(int n, int D, int A, int H, int prec, const float* W1, const float* b1, const float* Wih,
                       const float* bih, const float* Whh, const float* bhh, const float* W2, const float* b2, uint8_t* dst);
-int launch_actor_tcs(const ActorParams& p, int sms, cudaStream_t stream);
+bool tcs_fast_supported(int n, int D, int A, int H, int prec);
+int launch_actor_tcs(const ActorParams& p, int sms, bool fast_gates, cudaStream_t stream);
 int launch_ring_sample(const SampleParams& p, cudaStream_t stream);
 }  // namespace marl
 
@@ -114,7 +113,9 @@ static RecordLayout record_layout(int n, int D, int A) {
 // automatically, it is the split-operand kernel where that supports the shape; a kernel asked for by name falls back to
 // the CUDA-core kernel.
 static bool general_is_tcs(const marl_actor_config_t& c) {
-  return c.kernel == MARL_KERNEL_AUTO && tcs_supported(c.n_agents, c.obs_dim, c.n_actions, c.hidden, c.precision);
+  // (at hidden size 128 the pipelined choice is this kernel with the hardware's gate functions)
+  return (c.kernel == MARL_KERNEL_AUTO || (c.kernel == MARL_KERNEL_TENSOR_PIPELINED && c.hidden == 128)) &&
+         tcs_supported(c.n_agents, c.obs_dim, c.n_actions, c.hidden, c.precision);
 }
 // Bytes of one network's image for the general kernel.
 static size_t general_image_bytes(const marl_actor_config_t& c) {
@@ -333,7 +334,7 @@ int marl_actor_create(const marl_actor_config_t* cfg, marl_actor_t** out) {
 
   const bool tc_ok = tc_supported(cfg->n_agents, cfg->obs_dim, cfg->n_actions, cfg->hidden, cfg->precision);
   const bool tcp_ok = tcp_supported(cfg->n_agents, cfg->obs_dim, cfg->n_actions, cfg->hidden, cfg->precision) ||
-                      tcw_supported(cfg->n_agents, cfg->obs_dim, cfg->n_actions, cfg->hidden, cfg->precision);
+                      tcs_fast_supported(cfg->n_agents, cfg->obs_dim, cfg->n_actions, cfg->hidden, cfg->precision);
   const bool tc2_ok = tc2_supported(cfg->n_agents, cfg->obs_dim, cfg->n_actions, cfg->hidden, cfg->precision) && tcp_ok;
   if ((cfg->kernel == MARL_KERNEL_TENSOR && !tc_ok) || (cfg->kernel == MARL_KERNEL_TENSOR_PIPELINED && !tcp_ok) ||
       (cfg->kernel == MARL_KERNEL_TENSOR_DUAL && !tc2_ok)) {
@@ -460,8 +461,7 @@ static void pack_weights_host(const marl_actor* a, const float* W1, const float*
   const size_t tcb = tc_wpack_bytes(n, D, A, H);
   if (tc && tcb) {
     memset(tc, 0, tcb);
-    if (tc_supported(n, D, A, H, a->cfg.precision) || tcp_supported(n, D, A, H, a->cfg.precision) ||
-        tcw_supported(n, D, A, H, a->cfg.precision))
+    if (tc_supported(n, D, A, H, a->cfg.precision) || tcp_supported(n, D, A, H, a->cfg.precision))
       tc_pack_weights(n, D, A, H, W1, b1, W_ih, b_ih, W_hh, b_hh, W2, b2, tc);
   }
 }
@@ -679,12 +679,12 @@ static int enqueue_steps(marl_actor* a, const float* obs, const uint8_t* avail, 
     tc_tiling(c.n_envs, c.n_agents, a->sms, &p.ept, &p.num_tiles);
     if (a->use_tc2) rc = launch_actor_tc2(p, a->sms, a->stream);  // 0: not a launch for two resident tiles
     if (rc == 0 && a->use_tcp)  // 0: these pointers cannot be bulk-copied
-      rc = c.hidden == 128 ? launch_actor_tcw(p, a->sms, a->stream) : launch_actor_tcp(p, a->sms, a->stream);
+      rc = c.hidden == 128 ? launch_actor_tcs(p, a->sms, true, a->stream) : launch_actor_tcp(p, a->sms, a->stream);
     // (the one-tile kernel bulk-copies the observations too; it copes with unaligned availability bytes itself)
     if (rc == 0 && a->use_tc && reinterpret_cast<uintptr_t>(obs) % 16 == 0) rc = launch_actor_tc(p, a->sms, a->stream);
   }
   if (rc == 0 && a->use_tcs) {
-    rc = launch_actor_tcs(p, a->sms, a->stream);
+    rc = launch_actor_tcs(p, a->sms, false, a->stream);
   } else if (rc == 0) {
     ffma_tiling(c.n_envs, c.n_agents, a->sms, &p.ept, &p.num_tiles);
     rc = launch_actor_ffma(p, a->sms, a->stream);
@@ -768,7 +768,7 @@ static int step_list(marl_actor* a, const int32_t* env_ids, int32_t M, const flo
     rc = c.hidden == 128 ? 0 : launch_actor_tcp(p, a->sms, a->stream);  // (the hidden-128 kernel takes dense launches only)
   }
   if (rc == 0 && a->use_tcs) {
-    rc = launch_actor_tcs(p, a->sms, a->stream);
+    rc = launch_actor_tcs(p, a->sms, false, a->stream);
   } else if (rc == 0) {
     ffma_tiling(M, c.n_agents, a->sms, &p.ept, &p.num_tiles);
     rc = launch_actor_ffma(p, a->sms, a->stream);
