@@ -281,6 +281,9 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
     mbar_init(&B->flags, 1);
     B->abort = 0;
     mbar_init_fence();
+    fence_proxy_async_smem();
+    mbar_arrive_expect_tx(&B->wload, L.wbytes);  // (only the warps that read the weights wait for them)
+    bulk_load(smem, p.wpack, L.wbytes, &B->wload);
   }
   if (warp == 12) tmem_alloc(&B->tmem_base, TM_COLS);
   // operands, tails and hand-off arrays start as zeros (padding bytes of every stored record stay zero)
@@ -302,11 +305,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = B->tmem_base;
-  if (tid == 12 * 32) {
-    mbar_arrive_expect_tx(&B->wload, L.wbytes);
-    bulk_load(smem, p.wpack, L.wbytes, &B->wload);
-  }
-  mbar_wait(&B->wload, 0, abortf);
+  grid_wait();
 
   if (warp >= 12) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(TP_REGS_SVC));
@@ -316,6 +315,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
       const int total = my_tiles * T;
       uint32_t tl = 0;
       bool hside_issued = false;
+      mbar_wait(&B->wload, 0, abortf);
       if (total > 0) {
         mbar_wait(&B->xready, 0, abortf);
         tp_issue_fc1(L, sb, tmem, lane, &B->fc1d);
@@ -772,6 +772,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
     unsigned long long c_steps = 0, c_explore = 0, c_noavail = 0;
     uint32_t st_bits = 0, it = 0;
     float h[32];
+    bool fresh = true;  // the weights (here the last-action table) have not been waited for yet
     const uint32_t tm_y = tmem + lane_addr + TMP_Y + (uint32_t)cb / 2u, tm_h = tmem + lane_addr + TMP_H + (uint32_t)cb / 2u;
     auto store_h = [&](int c0, int c1) {  // groups of eight columns [c0, c1) of the hidden operand
 #pragma unroll
@@ -876,6 +877,8 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
         }
       }
 
+      if (fresh) mbar_wait(&B->wload, 0, abortf);
+      fresh = false;
       for (int s = 0; s < T; ++s) {
         const uint32_t b = it & 1, par = it & 1;
         uint8_t* tl = tails + b * tail_set + (uint32_t)el * L.tail_bytes;  // this row's environment tail
@@ -1121,8 +1124,7 @@ int launch_actor_tcp(const ActorParams& p_in, int sms, cudaStream_t stream) {
   }
   int grid = p.num_tiles < sms ? p.num_tiles : sms;
   if (grid < 1) grid = 1;
-  kernel<<<grid, TP_THREADS, L.total, stream>>>(p, L);
-  const cudaError_t err = cudaGetLastError();
+  const cudaError_t err = launch_overlapped(kernel, grid, TP_THREADS, L.total, stream, p.early != 0, p, L);
   return err == cudaSuccess ? 1 : -(int)err;
 }
 

@@ -751,6 +751,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
     // unit by unit (16 columns); group 0 also makes the masks and draws and records the availability, group 1 keeps the
     // ring cursors (of environment `row` of the tile), headers and outcomes and records Q.
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_PREP));
+    grid_wait();
     auto inputs = [&](auto grp_c) {  // (the group as a constant: each group's code keeps only its own registers)
     constexpr int grp = decltype(grp_c)::value;
     const int row = tid & 127, pw = warp & 3;
@@ -1066,6 +1067,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
   } else {
     // =========================== epilogue ===========================
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_EPI));
+    grid_wait();
     const int row = tid & 127, grp = warp >> 2;
     const uint32_t tm = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     unsigned long long c_steps = 0, c_explore = 0, c_noavail = 0;
@@ -1369,8 +1371,7 @@ int launch_actor_tcs(const ActorParams& p_in, int sms, bool fast_gates, cudaStre
   }
   int grid = p.num_tiles < sms ? p.num_tiles : sms;
   if (grid < 1) grid = 1;
-  kernels[v]<<<grid, TS_THREADS, L.total, stream>>>(p, L);
-  const cudaError_t err = cudaGetLastError();
+  const cudaError_t err = launch_overlapped(kernels[v], grid, TS_THREADS, L.total, stream, p.early != 0, p, L);
   return err == cudaSuccess ? 1 : -(int)err;
 }
 

@@ -21,4 +21,32 @@ inline cudaError_t ensure_dynamic_smem(const void* kernel, uint32_t bytes, uint3
   return e;
 }
 
+// Launches a kernel that may start while the kernel before it in the stream is still running (programmatic dependent
+// launch).  Such a kernel does what does not depend on earlier work - barriers, tensor memory, its weights - and then
+// executes grid_wait() in every thread that touches anything earlier work reads or writes.  early = false: an ordinary
+// launch (the step that first uses a newly uploaded weight image).
+template <typename... P>
+inline cudaError_t launch_overlapped(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t stream, bool early, const P&... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3((unsigned)grid);
+  c.blockDim = dim3((unsigned)block);
+  c.dynamicSmemBytes = smem;
+  c.stream = stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = at;
+  c.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&c, kernel, args...);
+}
+
+#ifdef __CUDACC__
+// Waits until all earlier work of the stream is done and visible, then lets the next kernel be scheduled: at most one
+// kernel is waiting behind a running one.
+__device__ __forceinline__ void grid_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
+
 }  // namespace marl

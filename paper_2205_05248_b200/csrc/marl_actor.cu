@@ -224,6 +224,7 @@ struct marl_actor {
   cudaStream_t copy_stream;
   cudaEvent_t upload_done, image_free;
   bool image_free_recorded, pending;
+  bool image_fresh;  // no launch has used the present weight image yet
   uint64_t pending_version, pending_step;
   std::vector<uint8_t> id_seen;  // scratch of marl_actor_step_subset
   // pinned staging of the environment list, two buffers in turn, each with the event of its last upload
@@ -329,7 +330,7 @@ int marl_actor_create(const marl_actor_config_t* cfg, marl_actor_t** out) {
   a->ids_next = 0;
   a->copy_stream = nullptr;
   a->upload_done = a->image_free = nullptr;
-  a->image_free_recorded = a->pending = false;
+  a->image_free_recorded = a->pending = a->image_fresh = false;
   a->pending_version = a->pending_step = 0;
 
   const bool tc_ok = tc_supported(cfg->n_agents, cfg->obs_dim, cfg->n_actions, cfg->hidden, cfg->precision);
@@ -623,6 +624,10 @@ static void fill_params(marl_actor* a, ActorParams& p) {
   p.trace_q = a->trace_q;
   p.trace_first = a->trace_next;
   p.trace_cap = (a->trace_actions || a->trace_q) ? a->trace_cap : 0;
+  // The first launch on a published image waits for everything before it; the later ones find the image in place and may
+  // load it while the kernel before them still runs.
+  p.early = a->image_fresh ? 0 : 1;
+  a->image_fresh = false;
 }
 
 // The published network becomes the one in use: the stream waits for its upload; the image used so far is idle once
@@ -632,6 +637,7 @@ static int switch_to_published(marl_actor* a) {
   CU_TRY(cudaEventRecord(a->image_free, a->stream));
   a->image_free_recorded = true;
   a->wslot ^= 1;
+  a->image_fresh = true;
   a->weights_version = a->pending_version;
   a->pending = false;
   return MARL_OK;
