@@ -260,7 +260,7 @@ int marl_actor_step_lagged(marl_actor_t* a, const int32_t* env_ids, int32_t M, c
 
 /* The same step with HOST buffers (the observation-action pipe of Algorithms 1 and 2 when the simulators
  * run on the host): copies the four inputs to the device, runs the step, copies the actions back and
- * SYNCHRONISES the stream before returning.  Pinned host memory makes the copies asynchronous. */
+ * SYNCHRONISES the stream before returning.  Pinned host arrays are read and written by the step kernel itself. */
 int marl_actor_step_host(marl_actor_t* a, const float* obs, const uint8_t* avail, const float* reward,
                          const uint8_t* done, float eps, int32_t* actions_out);
 

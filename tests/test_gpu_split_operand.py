@@ -87,3 +87,27 @@ def test_types_without_agents_and_one_agent_per_type(H):
         actor, acts, q = run_gpu_rollout(cfg, ws, splits=[2, 7])
         referee(cfg, ws, actor, acts, q)
         actor.destroy()
+
+
+@pytest.mark.parametrize("over", [dict(), dict(precision="fp32"), dict(n=3, A=9, D=30), dict(E=2300, D=240, precision="fp32")])
+def test_host_step_on_pinned_and_pageable_arrays(over):
+    """Pinned arrays are read by the step kernel, pageable ones copied, large observations (here 2300 x 8 x 240 floats, 17.7
+    MB) always copied: the same actions, records and state as the step on device arrays."""
+    cfg = workloads.small_config(**{**dict(H=64, E=70, n=8, D=80, A=14, L=5, precision="bf16"), **over})
+    cfg["C"] = cfg["E"]
+    w = workloads.make_weights(cfg)
+    dev, pin, page = (binding.Actor(cfg) for _ in range(3))
+    for a in (dev, pin, page):
+        a.set_weights(w)
+    for t in range(7):
+        x = [v[0] for v in dev.env_generate(cfg["env"], t, 1)]
+        want = dev.step(*x, 0.1).cpu()
+        h = [v.cpu() for v in x]
+        assert torch.equal(page.step_host(*h, 0.1, torch.empty_like(want)), want)
+        out = torch.empty_like(want).pin_memory() if t % 2 else torch.empty_like(want)
+        assert torch.equal(pin.step_host(*[v.pin_memory() for v in h], 0.1, out), want)
+    for a in (pin, page):
+        assert torch.equal(a.ring_mem, dev.ring_mem) and torch.equal(a.get_state()["h"], dev.get_state()["h"])
+        assert a.status()[0] == 0
+        a.destroy()
+    dev.destroy()
