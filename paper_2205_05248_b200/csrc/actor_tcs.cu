@@ -211,37 +211,57 @@ void tcs_pack_weights(int n, int D, int A, int H, int prec, const float* W1, con
   const TsLayout L = ts_image(n, D, A, H, ns);
   const int I = D + n + A;
   memset(dst, 0, L.img_bytes);
-  auto piece = [&](float v, int i) {  // piece i of v
-    for (int k = 0; k < i; ++k) v -= ts_float(ts_bf16(v));
-    return ts_bf16(v);
+  // Eight consecutive values of a row (n8 of them present) as their pieces, 16 bytes to each of to[piece].
+  auto put8 = [&](const float* v, int n8, uint16_t* const (&to)[3]) {
+    float r[8];
+    for (int k = 0; k < 8; ++k) r[k] = k < n8 ? v[k] : 0.f;
+    for (int i = 0; i < ns; ++i)
+      for (int k = 0; k < 8; ++k) {
+        const uint16_t h = ts_bf16(r[k]);
+        to[i][k] = h;
+        r[k] -= ts_float(h);
+      }
+  };
+  // rows of a K-major matrix: row r of the source's `cols` columns from k0 on to row (r0 + r) of `rows` in base[piece]
+  auto put_rows = [&](const float* src, size_t stride, int nrows, int k0, int k1, uint16_t* const (&base)[3], int rows, int r0) {
+    for (int r = 0; r < nrows; ++r)
+      for (int k = k0; k < k1; k += 8) {
+        uint16_t* to[3];
+        for (int i = 0; i < ns; ++i) to[i] = base[i] + ((size_t)((k - k0) / 8) * rows + r0 + r) * 8;
+        put8(src + r * stride + k, k1 - k < 8 ? k1 - k : 8, to);
+      }
   };
   uint16_t* w2 = reinterpret_cast<uint16_t*>(dst);
-  for (int i = 0; i < ns; ++i)
-    for (int a = 0; a < A; ++a)
-      for (int k = 0; k < H; ++k) w2[(((size_t)i * (H / 8) + k / 8) * L.NQ + a) * 8 + k % 8] = piece(W2[(size_t)a * H + k], i);
+  {
+    uint16_t* const base[3] = {w2, w2 + (size_t)H * L.NQ, w2 + (size_t)2 * H * L.NQ};
+    put_rows(W2, H, A, 0, H, base, L.NQ, 0);
+  }
   uint8_t* sl = dst + L.base_bytes;
-  for (int s = 0; s < L.nw1; ++s) {
-    uint16_t* w = reinterpret_cast<uint16_t*>(sl + ts_slice_off(L, H, ns, s));
-    const int k0 = ns == 3 ? 0 : s * TS_KCHUNK, k1 = ns == 3 || k0 + TS_KCHUNK > D ? D : k0 + TS_KCHUNK;
-    for (int j = 0; j < H; ++j)
-      for (int k = k0; k < k1; ++k)
-        w[((size_t)((k - k0) / 8) * H + j) * 8 + k % 8] = piece(W1[(size_t)j * I + k], ns == 3 ? 2 - s : 0);
+  auto slice = [&](int i) { return reinterpret_cast<uint16_t*>(sl + ts_slice_off(L, H, ns, i)); };
+  if (ns == 3) {  // smallest piece first
+    uint16_t* const base[3] = {slice(2), slice(1), slice(0)};
+    put_rows(W1, I, H, 0, D, base, H, 0);
+  } else {
+    for (int c = 0; c < L.nw1; ++c) {
+      const int k0 = c * TS_KCHUNK, k1 = k0 + TS_KCHUNK > D ? D : k0 + TS_KCHUNK;
+      uint16_t* const base[3] = {slice(c), nullptr, nullptr};
+      put_rows(W1, I, H, k0, k1, base, H, 0);
+    }
   }
   // gate slices of a block: three pieces h2 h1 y2 y1 h0 y0, one piece h0 y0
-  static const int order3[6][2] = {{1, 2}, {1, 1}, {0, 2}, {0, 1}, {1, 0}, {0, 0}}, order1[2][2] = {{1, 0}, {0, 0}};
   for (int b = 0; b < H / TS_BLK; ++b) {
-    const int buf = H == 64 ? b : (b + 1) & 1;
-    for (int s = 0; s < 2 * ns; ++s) {
-      const int hid = ns == 3 ? order3[s][0] : order1[s][0], pc = ns == 3 ? order3[s][1] : order1[s][1];
-      const float* W = hid ? Whh : Wih;
-      uint16_t* w = reinterpret_cast<uint16_t*>(sl + ts_slice_off(L, H, ns, L.nw1 + b * 2 * ns + s));
-      // gate blocks of the source are r | z | n
-      static const int rows_y[2][3] = {{0, 1, 2}, {2, 0, 1}}, rows_h[2][3] = {{2, 0, 1}, {0, 1, 2}};
+    const int buf = H == 64 ? b : (b + 1) & 1, i0 = L.nw1 + b * 2 * ns;
+    // gate blocks of the source are r | z | n
+    static const int rows_y[2][3] = {{0, 1, 2}, {2, 0, 1}}, rows_h[2][3] = {{2, 0, 1}, {0, 1, 2}};
+    for (int hid = 0; hid < 2; ++hid) {
+      uint16_t* base[3] = {slice(i0 + (ns == 3 ? (hid ? 4 : 5) : (hid ? 0 : 1))), nullptr, nullptr};
+      if (ns == 3) {
+        base[1] = slice(i0 + (hid ? 1 : 3));
+        base[2] = slice(i0 + (hid ? 0 : 2));
+      }
+      uint16_t* const to[3] = {base[0], base[1], base[2]};
       for (int g = 0; g < 3; ++g)
-        for (int j = 0; j < TS_BLK; ++j) {
-          const int src = (hid ? rows_h : rows_y)[buf][g] * H + b * TS_BLK + j;
-          for (int k = 0; k < H; ++k) w[((size_t)(k / 8) * 96 + g * TS_BLK + j) * 8 + k % 8] = piece(W[(size_t)src * H + k], pc);
-        }
+        put_rows((hid ? Whh : Wih) + (size_t)((hid ? rows_h : rows_y)[buf][g] * H + b * TS_BLK) * H, H, TS_BLK, 0, H, to, 96, g * TS_BLK);
     }
   }
   memcpy(dst + L.off_b2, b2, sizeof(float) * A);
