@@ -283,3 +283,33 @@ def test_list_steps_full_size_bench_configuration(lagged):
     assert status == 0 and counters["agent_steps"] == listed * n
     del staged, g_acts, g_q
     actor.destroy()
+
+
+@pytest.mark.parametrize("lagged", [False, True])
+def test_lists_in_flight_keep_their_own_buffers(lagged):
+    """More list steps enqueued at once than there are list buffers, the caller's array filled anew after each call: the
+    same state as when every step is waited for."""
+    cfg = workloads.small_config(H=64, D=40, E=1500, C=1500, L=8, n=4, A=9, precision="bf16")
+    w = workloads.make_weights(cfg)
+    rng = np.random.default_rng(5)
+    lists = [rng.permutation(1500)[:m].astype(np.int32) for m in (1500, 1, 700, 1499, 3, 1100, 64, 900, 1500, 2, 33, 800, 5)]
+    actors = [binding.Actor(cfg), binding.Actor(cfg)]
+    for a in actors:
+        a.set_weights(w)
+    steps = [[v[0][:len(ids)].contiguous() for v in actors[0].env_generate(cfg["env"], t, 1)] for t, ids in enumerate(lists)]
+    got = [[], []]
+    ids = np.empty(1500, np.int32)
+    for k, a in enumerate(actors):
+        for x, li in zip(steps, lists):
+            ids[:len(li)] = li
+            got[k].append(a.step_subset(ids[:len(li)], *x, 0.2, lagged=lagged))
+            ids[:] = -1
+            if k == 0:
+                torch.cuda.synchronize()
+    assert all(torch.equal(x, y) for x, y in zip(*got))
+    s0, s1 = actors[0].get_state(), actors[1].get_state()
+    assert torch.equal(s0["h"], s1["h"]) and torch.equal(s0["pos"], s1["pos"])
+    assert torch.equal(actors[0].ring_mem, actors[1].ring_mem)
+    for a in actors:
+        assert a.status()[0] == 0
+        a.destroy()
