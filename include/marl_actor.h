@@ -48,7 +48,7 @@ extern "C" {
 #define MARL_ECUDA (-3)  /* a CUDA call failed; marl_last_error() names it */
 #define MARL_ENOMEM (-4) /* a caller-provided buffer is too small, or an allocation failed */
 
-#define MARL_PRECISION_FP32 0 /* fp32 weights, fp32 FFMA arithmetic */
+#define MARL_PRECISION_FP32 0 /* fp32 weights, fp32 arithmetic (FFMA, or tensor-core products of three bf16 pieces a value) */
 #define MARL_PRECISION_BF16 1 /* weight matrices and matmul operands rounded to bf16 (RNE), fp32 accumulate */
 
 #define MARL_KERNEL_AUTO 0   /* bf16: a tensor-core kernel (the pipelined one, else the one-tile one, as the shape allows)
@@ -59,7 +59,7 @@ extern "C" {
 #define MARL_KERNEL_TENSOR 2 /* one-tile tcgen05 kernel: bf16 only; create fails if the shape is unsupported */
 #define MARL_KERNEL_TENSOR_PIPELINED 3 /* pipelined tcgen05 kernel: bf16, at least 4 agents; hidden 64, or hidden 128
                                         * with at most 16 actions, obs_dim a multiple of 8 and n_agents * n_actions a
-                                        * multiple of 16 (weights streamed from L2, dense launches only); create
+                                        * multiple of 16 (the split-operand kernel with one piece a value); create
                                         * fails otherwise.  Inputs that are not 16-byte aligned fall back, per call,
                                         * to the one-tile kernel where the shape allows it, else to the FFMA kernel;
                                         * so do calls whose availability block (batch * n_agents * n_actions bytes)
@@ -365,8 +365,8 @@ int marl_selftest_bounded_wait(void* stream, uint32_t poll_limit, uint32_t* stat
  * at the clocks it actually sustains.  SYNCHRONISES the stream; takes a few tens of milliseconds. */
 int marl_measure_ffma_tflops(void* stream, double* tflops_out);
 
-/* Name of the step kernel in use: "ffma" (the general path: split-operand tensor-core or CUDA-core kernel), "tcgen05" (one-tile tensor-core kernel), "tcgen05-pipelined",
- * "tcgen05-dual" (two resident tiles; its other launches run on the pipelined kernel), or
+/* Name of the step kernel in use: "ffma" (the general path: split-operand tensor-core or CUDA-core kernel), "tcgen05"
+ * (one-tile tensor-core kernel), "tcgen05-pipelined", "tcgen05-dual" (two resident tiles; its other launches run on the pipelined kernel), or
  * "tcgen05-streamed" (hidden size 128: weights kept in shared memory as far as they fit, the others streamed). */
 const char* marl_actor_kernel_name(const marl_actor_t* a);
 

@@ -372,8 +372,8 @@ int marl_actor_create(const marl_actor_config_t* cfg, marl_actor_t** out) {
     delete a;
     return fail(MARL_EINVAL, "the tensor-core kernel does not support this shape/precision");
   }
-  // Kernel choice.  fp32 precision: the CUDA-core kernel (tensor cores cannot meet its 1e-5 tolerance).  bf16: a
-  // tensor-core kernel wherever the shape is supported, at every batch size - timed on the same rollouts from 24
+  // Kernel choice.  fp32 precision: the general path, whose split-operand kernel multiplies three bf16 pieces a
+  // value (its error is that of an fp32 chain).  bf16: a tensor-core kernel wherever the shape is supported, at every batch size - timed on the same rollouts from 24
   // rows to 16384 (`bench.py --crossover`), one 128-row tcgen05 tile takes 3.3-5.2 us per
   // environment step against 18-21 us for the CUDA-core kernel's 64-row tiles, so there is no batch size at which
   // the CUDA cores win.
