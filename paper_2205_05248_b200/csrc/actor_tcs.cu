@@ -505,6 +505,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_SVC));
     if (warp == 16) {
       // =========================== MMA warp ===========================
+      grid_wait();  // (no bounded wait may include the run time of the kernel before: its inputs arrive only after that)
       const uint32_t sb = smem_u32(smem);
       constexpr uint32_t id96 = idesc_bf16_f32(128, 96), id64 = idesc_bf16_f32(128, 64), id32 = idesc_bf16_f32(128, 32),
                          idH = idesc_bf16_f32(128, H), idq = idesc_bf16_f32(128, NQ);
@@ -747,8 +748,11 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
           const int steps = my_tiles * T;
           for (int g = 0; g < steps; ++g)
             for (int i = L.nres; i < L.nsl; ++i) {
-              if (used >= (uint32_t)L.nslots) mbar_wait(&B->empty[ri], rpar, abortf);
-              else ++used;
+              if (used >= (uint32_t)L.nslots) {
+                mbar_wait(&B->empty[ri], rpar, abortf);
+              } else if (++used == (uint32_t)L.nslots) {
+                grid_wait();  // what is loaded so far was the weights' alone; the ring moves on with the steps
+              }
               if (lane == 0) {
                 const uint32_t bytes = ts_slice_bytes(L, H, NS, i);
                 mbar_arrive_expect_tx(&B->full[ri], bytes);

@@ -111,3 +111,32 @@ def test_host_step_on_pinned_and_pageable_arrays(over):
         assert a.status()[0] == 0
         a.destroy()
     dev.destroy()
+
+
+@pytest.mark.parametrize("prec,H,T", [("fp32", 64, 220_000), ("bf16", 128, 300_000)])
+def test_launch_behind_a_long_one(prec, H, T):
+    """A launch that starts beside its predecessor while that still runs for longer than a bounded wait lasts (about a
+    second): the wait for the predecessor counts against none of its own waits."""
+    cfg = workloads.small_config(H=H, E=1, n=4, D=8, A=4, C=2, L=50, precision=prec, seed=5)
+    w = workloads.make_weights(cfg)
+    states = []
+    for together in (True, False):
+        a = binding.Actor(cfg, work_steps=1)
+        a.set_weights(w)
+        staged = a.env_generate(cfg["env"], 0, T)
+        short = a.env_generate(cfg["env"], T, 40)
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        torch.cuda.synchronize()
+        ev[0].record()
+        a.rollout_staged(*staged, T, 0.2)
+        if not together:
+            torch.cuda.synchronize()
+        a.rollout_staged(*short, 40, 0.2)
+        ev[1].record()
+        torch.cuda.synchronize()
+        assert ev[0].elapsed_time(ev[1]) > 1200.0, "the first launch is too short for what is tested"
+        status, counters = a.status()
+        assert status == 0 and counters["agent_steps"] == 4 * (T + 40)
+        states.append((a.get_state()["h"].clone(), a.ring_mem.clone()))
+        a.destroy()
+    assert all(torch.equal(x, y) for x, y in zip(*states))
