@@ -46,6 +46,13 @@ constexpr int TP_MAX_STAGES = 8;
 // fc2 is four K = 16 steps.  Dependent tcgen05.mma on one accumulator run one after the other at a few hundred
 // cycles each whatever their width, so with 16 outputs the steps go to four accumulators (summed in epilogue 3).
 constexpr int TP_QPARTS = 4;
+// The next kernel is released when the inputs of the block's last three steps are about to be requested, some 10 us before
+// its end; a later release saves nothing to other streams that would show and loses part of the overlap (1024 environments x
+// 8 agents x 128 steps: 396 us a launch, 395 when released at its start, 398 when released once all inputs are requested).
+// The place matters more than the moment: with the test in the load warp's step loop the shapes of unaligned rows and
+// availability run up to 9 % faster than with the same test in the product, store or tail warp (5 agents x 55 observations,
+// 16384 environments x 128 steps: 2496 against 2756-2760 us; released at the start: 2757), the aligned ones as before.
+constexpr int TP_RELEASE = 3;
 constexpr int TP_DST_DEPTH = 16;      // steps of record addresses kept: the loads run at most TP_MAX_STAGES chunks (steps) ahead
 // Register split (setmaxnreg): launched with 128 registers per thread (512 * 128 = 65536); afterwards
 // 256 * 144 + 128 * 112 + 128 * 112 = 65536.
@@ -416,6 +423,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
           }
         }
         for (int s = 0; s < T; ++s, ++kstep) {
+          if ((int)kstep + TP_RELEASE >= my_tiles * T) grid_release();
           unsigned long long rec = 0;
           int closes = 0;
           if (mine && ok) {
@@ -463,6 +471,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
       }
     } else if (warp == 14) {
       // =========================== tail warp: cursors, slot headers, record tails (lane = environment) ===========
+      if (my_tiles * T <= TP_RELEASE) grid_release();  // (before the load warp has its first cursors)
       unsigned long long c_episodes = 0, c_trunc = 0;
       uint32_t st_bits = 0, sd = 0, it = 0;
       for (int tile = blockIdx.x; tile < p.num_tiles; tile += gridDim.x) {

@@ -1082,6 +1082,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
         fresh = false;
       }
     }
+    if constexpr (grp == 0) grid_release();  // the last step's inputs are in place
     if (c_episodes) atomicAdd(p.counters + CNT_EPISODES, (unsigned long long)c_episodes);
     if (c_trunc) atomicAdd(p.counters + CNT_TRUNCATED, (unsigned long long)c_trunc);
     if (st_bits) atomicOr(p.status, st_bits);

@@ -52,12 +52,13 @@ inline bool early_pays(int tiles, int grid, int T) {
 }
 
 #ifdef __CUDACC__
-// Waits until all earlier work of the stream is done and visible, then lets the next kernel be scheduled: at most one
-// kernel is waiting behind a running one.
-__device__ __forceinline__ void grid_wait() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
+// Waits until all earlier work of the stream is done and visible.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// The next kernel's blocks may be scheduled once some thread of every block has come here (or the block has ended): to be
+// called when a block's last step begins or a little before.  Waiting blocks hold an SM each; released at the start of a
+// long launch they took the SMs that it leaves free from the kernels of other streams.
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 #endif
 
 }  // namespace marl
