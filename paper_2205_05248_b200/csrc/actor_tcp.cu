@@ -1133,7 +1133,7 @@ int launch_actor_tcp(const ActorParams& p_in, int sms, cudaStream_t stream) {
   }
   int grid = p.num_tiles < sms ? p.num_tiles : sms;
   if (grid < 1) grid = 1;
-  const cudaError_t err = launch_overlapped(kernel, grid, TP_THREADS, L.total, stream, p.early != 0 && early_pays(p.num_tiles, grid, p.T), p, L);
+  const cudaError_t err = launch_overlapped(kernel, grid, TP_THREADS, L.total, stream, p.early != 0, p, L);
   return err == cudaSuccess ? 1 : -(int)err;
 }
 

@@ -25,6 +25,10 @@ inline cudaError_t ensure_dynamic_smem(const void* kernel, uint32_t bytes, uint3
 // launch).  Such a kernel does what does not depend on earlier work - barriers, tensor memory, its weights - and then
 // executes grid_wait() in every thread that touches anything earlier work reads or writes.  early = false: an ordinary
 // launch (the step that first uses a newly uploaded weight image).
+// Whatever share of the blocks has a tile more than the others: pipelined kernel, some thirty launches with 50 to 100 % such blocks, the
+// early start costs or saves less than 1 % (683 tiles of 128 steps on 148 blocks, 91 with a fifth: 2490 us, ordinary 2494);
+// split-operand kernel, 20 launches of fp32, hidden 128 and per-type networks, likewise (547 tiles of 64 steps in fp32 2101 us,
+// ordinary 2104; 556 tiles of hidden 128 1956 against 1954).  One-step launches gain 2.5 to 3.5 us of 11 to 41.
 template <typename... P>
 inline cudaError_t launch_overlapped(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t stream, bool early, const P&... args) {
   cudaLaunchConfig_t c = {};
@@ -38,17 +42,6 @@ inline cudaError_t launch_overlapped(void (*kernel)(P...), int grid, int block, 
   c.attrs = at;
   c.numAttrs = early ? 1 : 0;
   return cudaLaunchKernelEx(&c, kernel, args...);
-}
-
-// Whether a pipelined-kernel launch of T steps over blocks that take `tiles` in turn should start early.  Early blocks take
-// the SMs that the kernel before leaves idle first, so where more than half of the blocks, but not nearly all, have a tile
-// more than the others, those end up side by side instead of spread over the chip: 683 tiles of 128 steps on 148 blocks (91
-// with a fifth tile) 2885 us, against 2743 started after the kernel before.  Other shares gain: 293 tiles (145 with a second)
-// 1580 -> 1557 us, 342 tiles (46 with a third) 753 -> 740, 64 tiles 414 -> 409; and so do short launches, where start-up
-// weighs more.
-inline bool early_pays(int tiles, int grid, int T) {
-  const int rest = tiles % grid;  // blocks with a tile more than the others
-  return T < 8 || rest <= grid / 2 || rest > grid - grid / 8;
 }
 
 #ifdef __CUDACC__
