@@ -90,9 +90,9 @@ static FfmaWeightOffsets ffma_weight_offsets(int n, int D, int A, int H) {
 }
 
 // two weight images, each: per-type images of the general kernel (split-operand or FFMA), then the tensor-core image
-constexpr int ID_LISTS = 3;  // environment lists on their way to partial steps
+constexpr int ID_LISTS = 3;  // environment lists on their way to partial steps; one more device list for captured steps
 
-struct StateOffsets { size_t h, last_action, slot, pos, ep_count, counters, status, wgen[2], wpack[2], ids[ID_LISTS], total; };
+struct StateOffsets { size_t h, last_action, slot, pos, ep_count, counters, status, wgen[2], wpack[2], ids[ID_LISTS + 1], total; };
 struct RingOffsets { size_t records, epid, len, complete, total; };
 struct WorkOffsets { size_t obs, avail, reward, done, actions, total; };
 
@@ -230,8 +230,9 @@ struct marl_actor {
   uint64_t pending_version, pending_step;
   std::vector<uint8_t> id_seen;  // scratch of marl_actor_step_subset
   cudaStream_t ids_stream;       // carries the lists to the device
-  // pinned staging of the environment list, two buffers in turn, each with the event of its last upload
-  int32_t* ids_host[ID_LISTS];   // pinned, from a buffer's first use on
+  // pinned staging of the environment lists, in turn, each with the events of its last upload and of the step that read it
+  int32_t* ids_host;             // [ID_LISTS][n_envs], from the first list step on
+  std::vector<void*> ids_captured;  // pinned lists of captured steps: their graphs read them at every replay
   cudaEvent_t ids_copied[ID_LISTS], ids_read[ID_LISTS];
   bool ids_in_flight[ID_LISTS];
   int ids_next;
@@ -294,11 +295,22 @@ static void destroy_list_stream(marl_actor* a) {
     cudaStreamSynchronize(a->ids_stream);
     cudaStreamDestroy(a->ids_stream);
   }
+  if (a->ids_host) cudaFreeHost(a->ids_host);
+  for (void* list : a->ids_captured) cudaFreeHost(list);
   for (int i = 0; i < ID_LISTS; ++i) {
-    if (a->ids_host[i]) cudaFreeHost(a->ids_host[i]);
     if (a->ids_copied[i]) cudaEventDestroy(a->ids_copied[i]);
     if (a->ids_read[i]) cudaEventDestroy(a->ids_read[i]);
   }
+}
+
+// Pinned memory, also while the calling thread captures (the allocation is no part of what is captured).
+static cudaError_t malloc_pinned(void** out, size_t bytes) {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) return e;
+  e = cudaMallocHost(out, bytes);
+  const cudaError_t back = cudaThreadExchangeStreamCaptureMode(&mode);
+  return e != cudaSuccess ? e : back;
 }
 
 extern "C" {
@@ -352,8 +364,8 @@ int marl_actor_create(const marl_actor_config_t* cfg, marl_actor_t** out) {
   a->wslot = 0;
   a->host_pack2 = nullptr;
   a->ids_stream = nullptr;
+  a->ids_host = nullptr;
   for (int i = 0; i < ID_LISTS; ++i) {
-    a->ids_host[i] = nullptr;
     a->ids_copied[i] = a->ids_read[i] = nullptr;
     a->ids_in_flight[i] = false;
   }
@@ -780,19 +792,28 @@ static int step_list(marl_actor* a, const int32_t* env_ids, int32_t M, const flo
   // pinned staging owned by the actor and uploaded from there, on a stream of its own so that it travels while the
   // previous step computes (in the actor's stream the copy and the gaps around it came between two kernels: a list of
   // 9001 x 5 agents 60.8 -> 51.1 us, 32768 x 8 agents 129 -> 115 us).  ID_LISTS buffers take turns, on the host and
-  // on the device; each is filled again only when the kernel that read it is done.  A stream that is being captured gets
-  // the copy as a node of its own graph.
-  const int ib = a->ids_next;
-  int32_t* d_ids = reinterpret_cast<int32_t*>(a->state + a->so.ids[ib]);
-  if (!a->ids_host[ib]) CU_TRY(cudaMallocHost(reinterpret_cast<void**>(&a->ids_host[ib]), sizeof(int32_t) * (size_t)c.n_envs));
-  if (a->ids_in_flight[ib]) CU_TRY(cudaEventSynchronize(a->ids_read[ib]));
-  memcpy(a->ids_host[ib], env_ids, sizeof(int32_t) * (size_t)M);
+  // on the device; each is filled again only when the kernel that read it is done.
+  // A captured step's copy is a node of the graph, before the step's and in its stream, from pinned memory of its own (a
+  // replay reads it again) to a device list that no other step uses.
+  const size_t list_bytes = sizeof(int32_t) * (size_t)M;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   CU_TRY(cudaStreamIsCapturing(a->stream, &cap));
-  const cudaStream_t up = cap == cudaStreamCaptureStatusNone ? a->ids_stream : a->stream;
-  CU_TRY(cudaMemcpyAsync(d_ids, a->ids_host[ib], sizeof(int32_t) * (size_t)M, cudaMemcpyHostToDevice, up));
-  if (up != a->stream) {
-    CU_TRY(cudaEventRecord(a->ids_copied[ib], up));
+  const bool captured = cap != cudaStreamCaptureStatusNone;
+  const int ib = captured ? ID_LISTS : a->ids_next;
+  int32_t* d_ids = reinterpret_cast<int32_t*>(a->state + a->so.ids[ib]);
+  if (!a->ids_host) CU_TRY(malloc_pinned(reinterpret_cast<void**>(&a->ids_host), sizeof(int32_t) * (size_t)c.n_envs * ID_LISTS));
+  if (captured) {
+    void* list = nullptr;
+    CU_TRY(malloc_pinned(&list, list_bytes));
+    a->ids_captured.push_back(list);
+    memcpy(list, env_ids, list_bytes);
+    CU_TRY(cudaMemcpyAsync(d_ids, list, list_bytes, cudaMemcpyHostToDevice, a->stream));
+  } else {
+    int32_t* list = a->ids_host + (size_t)ib * c.n_envs;
+    if (a->ids_in_flight[ib]) CU_TRY(cudaEventSynchronize(a->ids_read[ib]));
+    memcpy(list, env_ids, list_bytes);
+    CU_TRY(cudaMemcpyAsync(d_ids, list, list_bytes, cudaMemcpyHostToDevice, a->ids_stream));
+    CU_TRY(cudaEventRecord(a->ids_copied[ib], a->ids_stream));
     CU_TRY(cudaStreamWaitEvent(a->stream, a->ids_copied[ib], 0));
   }
   ActorParams p;
@@ -821,12 +842,14 @@ static int step_list(marl_actor* a, const int32_t* env_ids, int32_t M, const flo
     rc = launch_actor_ffma(p, a->sms, a->stream);
   }
   if (rc < 0) {
-    cudaStreamSynchronize(a->ids_stream);  // the staging may be filled again
+    if (!captured) cudaStreamSynchronize(a->ids_stream);  // the staging may be filled again
     return fail(MARL_ECUDA, "actor kernel launch: %s", cudaGetErrorString((cudaError_t)(-rc)));
   }
-  CU_TRY(cudaEventRecord(a->ids_read[ib], a->stream));
-  a->ids_in_flight[ib] = true;
-  a->ids_next = (ib + 1) % ID_LISTS;
+  if (!captured) {
+    CU_TRY(cudaEventRecord(a->ids_read[ib], a->stream));
+    a->ids_in_flight[ib] = true;
+    a->ids_next = (ib + 1) % ID_LISTS;
+  }
   a->launches += (uint64_t)rc;
   a->step += 1;
   if (a->trace_actions || a->trace_q) a->trace_next = a->trace_next + 1 > a->trace_cap ? a->trace_cap : a->trace_next + 1;

@@ -313,3 +313,47 @@ def test_lists_in_flight_keep_their_own_buffers(lagged):
     for a in actors:
         assert a.status()[0] == 0
         a.destroy()
+
+
+@pytest.mark.parametrize("lagged", [False, True])
+@pytest.mark.parametrize("prec,warm", [("bf16", 1), ("fp32", 1), ("fp32", 0)])
+def test_captured_list_steps(prec, warm, lagged):
+    """List steps captured into a graph after at most one call, two in one graph, replayed after other list steps have used
+    every list buffer: the captured lists are stepped, and steps outside the graph go on working.  (Nothing explores and
+    the random stream is not read, so a replay is the step it would have been at its turn.)"""
+    cfg = workloads.small_config(H=64, D=40, E=600, C=1200, L=6, n=4, A=8, precision=prec)
+    w = workloads.make_weights(cfg)
+    rng = np.random.default_rng(9)
+    lists = [rng.permutation(600)[:m].astype(np.int32) for m in (600, 333, 4, 600, 1, 500, 7, 600, 64)]
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        actors = [binding.Actor(cfg), binding.Actor(cfg)]
+        for a in actors:
+            a.set_weights(w)
+        steps = [[v[0][:len(ids)].contiguous() for v in actors[0].env_generate(cfg["env"], t, 1)] for t, ids in enumerate(lists)]
+        out = [torch.empty((len(ids), 4), dtype=torch.int32, device="cuda") for ids in lists]
+        torch.cuda.synchronize()
+
+        def call(a, k, to=None):
+            return a.step_subset(lists[k], *steps[k], 0.0, lagged=lagged, actions_out=to)
+        for k in range(warm):
+            call(actors[0], k)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=side):
+            for k in (1, 2):
+                call(actors[0], k, out[k])
+        for k in (3, 4, 5, 6):
+            call(actors[0], k)
+        graph.replay()
+        for k in (7, 8):
+            out[k] = call(actors[0], k)
+        want = {k: call(actors[1], k) for k in (*range(warm), 3, 4, 5, 6, 1, 2, 7, 8)}
+        torch.cuda.synchronize()
+    assert all(torch.equal(out[k], want[k]) for k in (1, 2, 7, 8))
+    s0, s1 = actors[0].get_state(), actors[1].get_state()
+    assert all(torch.equal(s0[k], s1[k]) for k in ("h", "last_action", "slot", "pos", "ep_count"))
+    assert torch.equal(actors[0].ring_mem, actors[1].ring_mem)
+    graph.reset()
+    for a in actors:
+        assert a.status()[0] == 0
+        a.destroy()
