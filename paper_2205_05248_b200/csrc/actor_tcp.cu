@@ -1100,6 +1100,11 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
   if (warp == 12) tmem_dealloc(tmem, TM_COLS);
 }
 
+// Whether a dense step of M environments runs on this kernel when its input arrays start on 16-byte boundaries.
+bool tcp_takes_batch(int n, int D, int A, int M) {
+  return ((size_t)M * n * D * 4) % 16 == 0 && ((size_t)M * n * A) % 16 == 0 && (D % 8 == 0 || M % TP_G == 0);
+}
+
 // Returns the number of kernels launched, 0 if this launch's pointers do not meet the kernel's alignment
 // needs (the caller then uses the one-tile kernel), or a negative cudaError.
 int launch_actor_tcp(const ActorParams& p_in, int sms, cudaStream_t stream) {

@@ -2,6 +2,8 @@
 // launch planning and the entry points declared in include/marl_actor.h.  All arithmetic of the actor
 // step runs in the kernels (actor_ffma.cu, actor_tc.cu, env_kernel.cu); nothing here computes on the CPU
 // and there is no CPU fallback.
+#include <cuda.h>
+
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -11,6 +13,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "host_span.cuh"
 
 namespace marl {
 int launch_env_generate(const marl_synth_env_t& env, int E, int n, int D, int A, uint32_t t0, int n_steps,
@@ -27,6 +30,7 @@ void tc_pack_weights(int n, int D, int A, int H, const float* W1, const float* b
 void tc_tiling(int E, int n, int sms, int* ept, int* num_tiles);
 int launch_actor_tc(const ActorParams& p, int sms, cudaStream_t stream);
 bool tcp_supported(int n, int D, int A, int H, int prec);
+bool tcp_takes_batch(int n, int D, int A, int M);
 int launch_actor_tcp(const ActorParams& p, int sms, cudaStream_t stream);
 bool tc2_supported(int n, int D, int A, int H, int prec);
 int launch_actor_tc2(const ActorParams& p, int sms, cudaStream_t stream);
@@ -756,14 +760,26 @@ int marl_actor_step(marl_actor_t* a, const float* obs, const uint8_t* avail, con
 
 }  // extern "C"
 
-// The device's address of a pinned host array, or null if the array is not one that kernels can read.
-static const void* mapped_host(const void* host) {
-  cudaPointerAttributes at;
-  if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
-    cudaGetLastError();
-    return nullptr;
-  }
-  return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
+// The device's address of a pinned host array, or null if the array is not one that the step kernels can access as it is.
+static const void* mapped_host(const void* host, size_t bytes, size_t align) {
+  // (the extent of an allocation is an attribute of the driver interface only)
+  typedef CUresult (*get_attributes_t)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+  static const get_attributes_t get_attributes = [] {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &fn, cudaEnableDefault, &found) != cudaSuccess) cudaGetLastError();
+    return reinterpret_cast<get_attributes_t>(fn);
+  }();
+  if (!get_attributes) return nullptr;
+  unsigned int type = 0, managed = 0;
+  CUdeviceptr device = 0, start = 0;
+  size_t size = 0;
+  CUpointer_attribute what[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                 CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* to[5] = {&type, &managed, &device, &start, &size};
+  if (get_attributes(5, what, to, reinterpret_cast<CUdeviceptr>(host)) != CUDA_SUCCESS) return nullptr;
+  const HostRange r = {type == CU_MEMORYTYPE_HOST && !managed, reinterpret_cast<const void*>(device), static_cast<uintptr_t>(start), size};
+  return kernel_span(r, host, bytes, align);
 }
 
 // One step over a host list of environments; lagged: reward/done belong to each environment's previous action.
@@ -889,21 +905,24 @@ int marl_actor_step_host(marl_actor_t* a, const float* obs, const uint8_t* avail
   // 11 MB 743 -> 247 us.  From some 16 MB on the copy engine is the faster reader of the observations (22 MB: 479
   // against 540 us, 175 MB: 3260 against 3460 us), the small arrays stay with the kernel.  The CUDA-core kernel reads the
   // availability rows twice and keeps the copies.
+  // Arrays that do not start where the kernels want them (observations and availability on 16-byte boundaries: others would
+  // change the kernel) or that are not pinned as a whole are copied.
+  const size_t obs_bytes = sizeof(float) * rows * c.obs_dim, avail_bytes = rows * c.n_actions;
   const void* in[4] = {obs, avail, reward, done};
-  bool mapped = a->use_tcp || a->use_tc || a->use_tcs;
-  for (int i = 0; i < 4 && mapped; ++i) mapped = (in[i] = mapped_host(in[i])) != nullptr;
-  const size_t obs_bytes = sizeof(float) * rows * c.obs_dim;
+  const size_t in_bytes[4] = {obs_bytes, avail_bytes, sizeof(float) * c.n_envs, (size_t)c.n_envs}, in_align[4] = {16, 16, 4, 1};
+  bool mapped = a->use_tcs || a->use_tc || (a->use_tcp && tcp_takes_batch(c.n_agents, c.obs_dim, c.n_actions, c.n_envs));
+  for (int i = 0; i < 4 && mapped; ++i) mapped = (in[i] = mapped_host(in[i], in_bytes[i], in_align[i])) != nullptr;
   if (!mapped || obs_bytes >= ((size_t)16 << 20)) {
     CU_TRY(cudaMemcpyAsync(d_obs, obs, obs_bytes, cudaMemcpyHostToDevice, a->stream));
     in[0] = d_obs;
   }
   if (!mapped) {
-    CU_TRY(cudaMemcpyAsync(d_avail, avail, rows * c.n_actions, cudaMemcpyHostToDevice, a->stream));
+    CU_TRY(cudaMemcpyAsync(d_avail, avail, avail_bytes, cudaMemcpyHostToDevice, a->stream));
     CU_TRY(cudaMemcpyAsync(d_reward, reward, sizeof(float) * c.n_envs, cudaMemcpyHostToDevice, a->stream));
     CU_TRY(cudaMemcpyAsync(d_done, done, (size_t)c.n_envs, cudaMemcpyHostToDevice, a->stream));
     in[1] = d_avail; in[2] = d_reward; in[3] = d_done;
   }
-  int32_t* out = mapped && actions_out ? static_cast<int32_t*>(const_cast<void*>(mapped_host(actions_out))) : nullptr;
+  int32_t* out = mapped && actions_out ? static_cast<int32_t*>(const_cast<void*>(mapped_host(actions_out, sizeof(int32_t) * rows, 4))) : nullptr;
   const int rc = enqueue_steps(a, static_cast<const float*>(in[0]), static_cast<const uint8_t*>(in[1]), static_cast<const float*>(in[2]),
                                static_cast<const uint8_t*>(in[3]), 1, true, eps, 0, 0, 0, out ? out : d_act);
   if (rc) return rc;

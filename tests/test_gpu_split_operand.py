@@ -1,5 +1,7 @@
 """The split-operand tensor-core kernel (general path: fp32, per-type networks, launches and shapes the bf16 kernels do
 not take) at the edges of its tiles, slices and dispatch, against the oracle."""
+import ctypes as C
+
 import pytest
 import torch
 
@@ -140,3 +142,31 @@ def test_launch_behind_a_long_one(prec, H, T):
         states.append((a.get_state()["h"].clone(), a.ring_mem.clone()))
         a.destroy()
     assert all(torch.equal(x, y) for x, y in zip(*states))
+
+
+@pytest.mark.parametrize("over,kernel", [(dict(), "auto"), (dict(precision="fp32"), "auto"), (dict(H=128), "auto"),
+                                         (dict(n=5, D=55, A=12), "pipelined"), (dict(n=5, D=55, A=12, E=72), "pipelined")])
+def test_host_step_on_pinned_arrays_at_any_address(over, kernel):
+    """Pinned arrays that start where the kernels could not read them, or read them on another kernel, are copied: the same
+    actions, records and state as the step on device arrays, whatever the addresses."""
+    cfg = workloads.small_config(**{**dict(H=64, E=70, n=8, D=80, A=14, L=5, precision="bf16"), **over})
+    cfg["C"] = cfg["E"]
+    w = workloads.make_weights(cfg)
+    dev, pin = (binding.Actor(cfg, kernel=kernel) for _ in range(2))
+    for a in (dev, pin):
+        a.set_weights(w)
+    offsets = [(0, 0, 0, 0, 0), (16, 16, 4, 1, 4), (4, 0, 0, 0, 0), (0, 3, 0, 0, 0), (0, 0, 2, 0, 0), (0, 0, 0, 3, 2), (8, 8, 1, 1, 1)]
+    for t, off in enumerate(offsets):
+        x = [v[0] for v in dev.env_generate(cfg["env"], t, 1)]
+        want = dev.step(*x, 0.1).cpu()
+        host = [torch.empty(v.numel() * v.element_size() + 32, dtype=torch.uint8).pin_memory() for v in (*x, want)]
+        for b, o, v in zip(host, off, x):
+            b[o:o + v.numel() * v.element_size()] = v.cpu().contiguous().view(-1).view(torch.uint8)
+        at = [C.c_void_p(b.data_ptr() + o) for b, o in zip(host, off)]
+        binding._check(pin.lib.marl_actor_step_host(pin.handle, *at[:4], C.c_float(0.1), at[4]))
+        got = host[4][off[4]:off[4] + want.numel() * 4].clone().view(torch.int32).view_as(want)
+        assert torch.equal(got, want), off
+    assert torch.equal(pin.ring_mem, dev.ring_mem) and torch.equal(pin.get_state()["h"], dev.get_state()["h"])
+    for a in (pin, dev):
+        assert a.status()[0] == 0
+        a.destroy()
