@@ -729,8 +729,11 @@ static int enqueue_steps(marl_actor* a, const float* obs, const uint8_t* avail, 
   if (a->use_tcp || a->use_tc) {
     tc_tiling(c.n_envs, c.n_agents, a->sms, &p.ept, &p.num_tiles);
     if (a->use_tc2) rc = launch_actor_tc2(p, a->sms, a->stream);  // 0: not a launch for two resident tiles
+    // Hidden 128: only aligned inputs take the hardware's gate functions.  The kernel could read others too, but those calls
+    // have always had the accurate ones.
+    const bool aligned = (reinterpret_cast<uintptr_t>(obs) | reinterpret_cast<uintptr_t>(avail)) % 16 == 0;
     if (rc == 0 && a->use_tcp)  // 0: these pointers cannot be bulk-copied
-      rc = c.hidden == 128 ? launch_actor_tcs(p, a->sms, true, a->stream) : launch_actor_tcp(p, a->sms, a->stream);
+      rc = c.hidden != 128 ? launch_actor_tcp(p, a->sms, a->stream) : aligned ? launch_actor_tcs(p, a->sms, true, a->stream) : 0;
     // (the one-tile kernel bulk-copies the observations too; it copes with unaligned availability bytes itself)
     if (rc == 0 && a->use_tc && reinterpret_cast<uintptr_t>(obs) % 16 == 0) rc = launch_actor_tc(p, a->sms, a->stream);
   }

@@ -2,6 +2,7 @@
 not take) at the edges of its tiles, slices and dispatch, against the oracle."""
 import ctypes as C
 
+import numpy as np
 import pytest
 import torch
 
@@ -170,3 +171,29 @@ def test_host_step_on_pinned_arrays_at_any_address(over, kernel):
     for a in (pin, dev):
         assert a.status()[0] == 0
         a.destroy()
+
+
+@pytest.mark.parametrize("shift", ["obs", "avail"])
+def test_hidden_128_gates_of_unaligned_inputs_are_the_accurate_ones(shift):
+    """bf16 at hidden 128: a dense step on inputs off a 16-byte boundary has the gate functions of the general path.  So it is,
+    bit for bit, the step over the list of all environments, which always has them; the aligned dense step is not."""
+    cfg = workloads.small_config(H=128, E=200, n=8, D=80, A=14, C=200, L=5, precision="bf16")
+    w = workloads.make_weights(cfg)
+    h = {}
+    for how in ("aligned", "shifted", "list"):
+        a = binding.Actor(cfg)
+        a.set_weights(w)
+        obs, avail, reward, done = (v[0] for v in a.env_generate(cfg["env"], 0, 1))
+        if how == "shifted" and shift == "obs":
+            obs = torch.empty(obs.numel() + 1, device="cuda")[1:].view_as(obs).copy_(obs)
+        elif how == "shifted":
+            avail = torch.empty(avail.numel() + 1, dtype=torch.uint8, device="cuda")[1:].view_as(avail).copy_(avail)
+        if how == "list":
+            a.step_subset(np.arange(200), obs, avail, reward, done, 0.1)
+        else:
+            a.step(obs, avail, reward, done, 0.1)
+        torch.cuda.synchronize()
+        h[how] = a.get_state()["h"].clone()
+        assert a.status()[0] == 0
+        a.destroy()
+    assert torch.equal(h["shifted"], h["list"]) and not torch.equal(h["aligned"], h["list"])
