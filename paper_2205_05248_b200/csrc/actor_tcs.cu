@@ -217,7 +217,16 @@ void tcs_pack_weights(int n, int D, int A, int H, int prec, const float* W1, con
     for (int k = 0; k < 8; ++k) r[k] = k < n8 ? v[k] : 0.f;
     for (int i = 0; i < ns; ++i)
       for (int k = 0; k < 8; ++k) {
-        const uint16_t h = ts_bf16(r[k]);
+        uint16_t h = ts_bf16(r[k]);
+        if (i + 1 < ns && (h & 0x7FFFu) == 0x7F80u) {
+          // rounds to infinity: the largest finite piece; an infinity keeps its sign in the smallest one, so that the rest
+          // of an infinite operand meets no zero, and stands in the last piece
+          const bool inf = r[k] - r[k] != 0.f;
+          h = (uint16_t)((h & 0x8000u) | (!inf ? 0x7F7Fu : i == 0 ? 0x0080u : 0u));
+          to[i][k] = h;
+          if (!inf) r[k] -= ts_float(h);
+          continue;
+        }
         to[i][k] = h;
         r[k] -= ts_float(h);
       }
@@ -307,7 +316,17 @@ __device__ __forceinline__ uint32_t ts_pack2(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-// The pieces of 16 consecutive values of this thread's row: piece i as 8 packed words to put(i, words).
+// The same, cut at the largest finite bf16.
+__device__ __forceinline__ uint32_t ts_pack2_finite(float lo, float hi) {
+  uint32_t d;
+  asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
+  return d;
+}
+
+// The pieces of 16 consecutive values of this thread's row: piece i as 8 packed words to put(i, words).  All but the last are
+// cut at the largest finite value: what bf16 would round to infinity splits into finite pieces, and an infinity stands in
+// the last piece alone, which meets only the weights' first pieces - infinite pieces against weight pieces of either sign
+// would be NaN.  (Finite large pieces stay below an infinite sum for weights up to some 128 in magnitude.)
 template <int NS, typename Put>
 __device__ __forceinline__ void ts_split16(float (&v)[16], Put put) {
 #pragma unroll
@@ -315,7 +334,7 @@ __device__ __forceinline__ void ts_split16(float (&v)[16], Put put) {
     uint32_t w[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      w[j] = ts_pack2(v[2 * j], v[2 * j + 1]);
+      w[j] = i + 1 < NS ? ts_pack2_finite(v[2 * j], v[2 * j + 1]) : ts_pack2(v[2 * j], v[2 * j + 1]);
       if (i + 1 < NS) {
         v[2 * j] -= __uint_as_float(w[j] << 16);
         v[2 * j + 1] -= __uint_as_float(w[j] & 0xFFFF0000u);

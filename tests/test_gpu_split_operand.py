@@ -197,3 +197,53 @@ def test_hidden_128_gates_of_unaligned_inputs_are_the_accurate_ones(shift):
         assert a.status()[0] == 0
         a.destroy()
     assert torch.equal(h["shifted"], h["list"]) and not torch.equal(h["aligned"], h["list"])
+
+
+@pytest.mark.parametrize("H", [64, 128])
+@pytest.mark.parametrize("net", ["mixed", "one sign", "large weights"])
+def test_infinite_and_very_large_values_fp32(H, net):
+    """fp32: infinities, NaN and values beyond the largest finite bf16 (3.39e38) go through the network as on the CUDA-core
+    kernel: the same infinities and NaN, other values to 1e-5, the same actions."""
+    cfg = workloads.small_config(H=H, E=16, n=2, D=20, A=4, C=16, L=5, precision="fp32")
+    w = {k: v.copy() for k, v in workloads.make_weights(cfg).items()}
+    rng = np.random.default_rng(3)
+    big = 3.4e38
+    if net == "one sign":                      # every unit infinite, every gate's sum of one sign: h stays finite
+        w["W1"][:, 0] = 0.3
+        w["W_ih"][:H] = np.abs(w["W_ih"][:H]) + 0.01
+        w["W_ih"][H:2 * H] = -np.abs(w["W_ih"][H:2 * H]) - 0.01
+        w["W_ih"][2 * H:] = np.abs(w["W_ih"][2 * H:]) * rng.choice([-1.0, 1.0], size=(H, 1)).astype(np.float32)
+    w["W1"][:, 1] *= 1e-3                      # (large observations: no overflow of a sum, whatever its order)
+    if net == "large weights":
+        w["W1"][3, 5] = np.inf
+        w["W2"][1, 7] = big
+        w["W2"][2, 9] = -np.inf
+        w["W1"][4, 6] = -big
+    got = {}
+    for kernel in ("auto", "ffma"):
+        a = binding.Actor(cfg, kernel=kernel)
+        a.set_weights(w)
+        acts, q = a.set_trace(2)
+        for t in range(2):
+            obs, avail, reward, done = (v[0] for v in a.env_generate(dict(cfg["env"], done_thresh24=0), t, 1))
+            if net != "large weights":
+                for e, (col, v) in enumerate([(0, np.inf), (0, -np.inf), (1, big), (1, -big), (1, 3.3895e38), (0, np.nan), (0, 1e30)]):
+                    obs[e, 0, col] = v
+            else:
+                obs[:, :, 6] *= 1e-3
+                obs[3, 1, 5] = 0.0
+            a.step(obs, avail, reward, done, 0.0)
+        torch.cuda.synchronize()
+        got[kernel] = (acts.cpu(), q.double().cpu(), a.get_state()["h"].double().cpu())
+        a.destroy()
+    assert torch.equal(got["auto"][0], got["ffma"][0])
+    # a Q value is bounded by its row of W2 (|h| <= 1): differences are measured against that
+    scale = torch.as_tensor(np.maximum(np.abs(np.where(np.isfinite(w["W2"]), w["W2"], 0)).max(axis=1), 1.0)).double()
+    for x, y, sc in ((got["auto"][1], got["ffma"][1], scale), (got["auto"][2], got["ffma"][2], torch.ones(H).double())):
+        assert torch.equal(x.isnan(), y.isnan()) and torch.equal(x.isinf(), y.isinf())
+        assert torch.equal(x[x.isinf()], y[y.isinf()])
+        f = torch.isfinite(y)
+        assert f.any()
+        assert bool(((x - y).abs() <= 1e-5 * sc)[f].all())
+    if net != "mixed":
+        assert (~torch.isfinite(got["ffma"][1])).any() == (net == "large weights")
