@@ -525,6 +525,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
     if (warp == 16) {
       // =========================== MMA warp ===========================
       grid_wait();  // (no bounded wait may include the run time of the kernel before: its inputs arrive only after that)
+      if (my_tiles * T * ntypes <= 2) grid_release();  // (the input warps would come to it too late to gain from it)
       const uint32_t sb = smem_u32(smem);
       constexpr uint32_t id96 = idesc_bf16_f32(128, 96), id64 = idesc_bf16_f32(128, 64), id32 = idesc_bf16_f32(128, 32),
                          idH = idesc_bf16_f32(128, H), idq = idesc_bf16_f32(128, NQ);
