@@ -370,6 +370,11 @@ int marl_measure_ffma_tflops(void* stream, double* tflops_out);
  * "tcgen05-streamed" (hidden size 128: weights kept in shared memory as far as they fit, the others streamed). */
 const char* marl_actor_kernel_name(const marl_actor_t* a);
 
+/* Name of the CUDA kernel that the latest step ran on: "actor_tcp_kernel" (pipelined), "actor_tcs_kernel" (split-operand),
+ * "actor_tc_kernel" (one-tile), "actor_tc2_kernel" (two resident tiles) or "actor_ffma_kernel" (CUDA cores); "" before the
+ * first step.  Unlike marl_actor_kernel_name it tells the two kernels of the general path apart, call by call. */
+const char* marl_actor_step_kernel(const marl_actor_t* a);
+
 /* Launches of library kernels enqueued by this actor since creation (all kernels, all entry points). */
 uint64_t marl_actor_launch_count(const marl_actor_t* a);
 

@@ -34,6 +34,7 @@ EXPORTS = [
     "marl_actor_step", "marl_actor_step_subset", "marl_actor_step_lagged", "marl_actor_step_host", "marl_env_generate", "marl_rollout_staged", "marl_rollout",
     "marl_actor_set_trace", "marl_ring_view", "marl_ring_sample", "marl_actor_get_state", "marl_actor_set_state",
     "marl_actor_status", "marl_actor_reset", "marl_actor_destroy", "marl_actor_kernel_name",
+    "marl_actor_step_kernel",
     "marl_actor_launch_count", "marl_last_error", "marl_rollout_noalloc", "marl_selftest_bounded_wait",
     "marl_measure_ffma_tflops",
 ]
@@ -101,6 +102,8 @@ def load_library():
         lib.marl_last_error.restype = C.c_char_p
         lib.marl_actor_kernel_name.restype = C.c_char_p
         lib.marl_actor_kernel_name.argtypes = [P]
+        lib.marl_actor_step_kernel.restype = C.c_char_p
+        lib.marl_actor_step_kernel.argtypes = [P]
         lib.marl_actor_launch_count.restype = C.c_uint64
         lib.marl_actor_launch_count.argtypes = [P]
         lib.marl_actor_weights_version.restype = C.c_uint64
@@ -461,6 +464,11 @@ class Actor:
     @property
     def kernel_name(self) -> str:
         return self.lib.marl_actor_kernel_name(self.handle).decode()
+
+    @property
+    def step_kernel(self) -> str:
+        """The CUDA kernel of the latest step ("" before the first)."""
+        return self.lib.marl_actor_step_kernel(self.handle).decode()
 
     @property
     def launch_count(self) -> int:

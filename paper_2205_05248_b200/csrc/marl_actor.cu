@@ -224,6 +224,7 @@ struct marl_actor {
   float* trace_q;
   int32_t trace_cap, trace_next;
   uint64_t launches;
+  const char* step_kernel;       // kernel of the latest step
   std::vector<uint8_t> host_pack;
   // weight publication: the image in use, the copy stream, and the publication waiting for its step
   int wslot;
@@ -365,6 +366,7 @@ int marl_actor_create(const marl_actor_config_t* cfg, marl_actor_t** out) {
   a->trace_q = nullptr;
   a->trace_cap = a->trace_next = 0;
   a->launches = 0;
+  a->step_kernel = "";
   a->wslot = 0;
   a->host_pack2 = nullptr;
   a->ids_stream = nullptr;
@@ -726,25 +728,31 @@ static int enqueue_steps(marl_actor* a, const float* obs, const uint8_t* avail, 
   p.env_step_stride = c.n_envs;
   p.actions_out = actions_out;
   int rc = 0;
+  const char* kernel = "";
+  auto tried = [&](const char* name, int launched) {  // 0: not a launch for that kernel, the next one takes it
+    rc = launched;
+    if (rc > 0) kernel = name;
+  };
   if (a->use_tcp || a->use_tc) {
     tc_tiling(c.n_envs, c.n_agents, a->sms, &p.ept, &p.num_tiles);
-    if (a->use_tc2) rc = launch_actor_tc2(p, a->sms, a->stream);  // 0: not a launch for two resident tiles
     // Hidden 128: only aligned inputs take the hardware's gate functions.  The kernel could read others too, but those calls
     // have always had the accurate ones.
     const bool aligned = (reinterpret_cast<uintptr_t>(obs) | reinterpret_cast<uintptr_t>(avail)) % 16 == 0;
-    if (rc == 0 && a->use_tcp)  // 0: these pointers cannot be bulk-copied
-      rc = c.hidden != 128 ? launch_actor_tcp(p, a->sms, a->stream) : aligned ? launch_actor_tcs(p, a->sms, true, a->stream) : 0;
+    if (a->use_tc2) tried("actor_tc2_kernel", launch_actor_tc2(p, a->sms, a->stream));  // (a launch for two resident tiles?)
+    if (rc == 0 && a->use_tcp && c.hidden != 128) tried("actor_tcp_kernel", launch_actor_tcp(p, a->sms, a->stream));
+    if (rc == 0 && a->use_tcp && c.hidden == 128 && aligned) tried("actor_tcs_kernel", launch_actor_tcs(p, a->sms, true, a->stream));
     // (the one-tile kernel bulk-copies the observations too; it copes with unaligned availability bytes itself)
-    if (rc == 0 && a->use_tc && reinterpret_cast<uintptr_t>(obs) % 16 == 0) rc = launch_actor_tc(p, a->sms, a->stream);
+    if (rc == 0 && a->use_tc && reinterpret_cast<uintptr_t>(obs) % 16 == 0) tried("actor_tc_kernel", launch_actor_tc(p, a->sms, a->stream));
   }
   if (rc == 0 && a->use_tcs) {
-    rc = launch_actor_tcs(p, a->sms, false, a->stream);
+    tried("actor_tcs_kernel", launch_actor_tcs(p, a->sms, false, a->stream));
   } else if (rc == 0) {
     ffma_tiling(c.n_envs, c.n_agents, a->sms, &p.ept, &p.num_tiles);
-    rc = launch_actor_ffma(p, a->sms, a->stream);
+    tried("actor_ffma_kernel", launch_actor_ffma(p, a->sms, a->stream));
   }
   if (rc < 0) return fail(MARL_ECUDA, "actor kernel launch: %s", cudaGetErrorString((cudaError_t)(-rc)));
   a->launches += (uint64_t)rc;
+  a->step_kernel = kernel;
   a->step += (uint64_t)T;
   if (a->trace_actions || a->trace_q) {
     const long long nx = (long long)a->trace_next + T;
@@ -850,13 +858,16 @@ static int step_list(marl_actor* a, const int32_t* env_ids, int32_t M, const flo
   p.M = M;
   p.lagged = lagged ? 1 : 0;
   int rc = 0;
-  if (a->use_tcp) {  // 0: these pointers or this list length cannot be bulk-copied
+  const char* kernel = "actor_tcp_kernel";
+  if (a->use_tcp && c.hidden != 128) {  // 0: these pointers or this list length cannot be bulk-copied
     tc_tiling(M, c.n_agents, a->sms, &p.ept, &p.num_tiles);
-    rc = c.hidden == 128 ? 0 : launch_actor_tcp(p, a->sms, a->stream);  // (the hidden-128 kernel takes dense launches only)
+    rc = launch_actor_tcp(p, a->sms, a->stream);
   }
   if (rc == 0 && a->use_tcs) {
+    kernel = "actor_tcs_kernel";
     rc = launch_actor_tcs(p, a->sms, false, a->stream);
   } else if (rc == 0) {
+    kernel = "actor_ffma_kernel";
     ffma_tiling(M, c.n_agents, a->sms, &p.ept, &p.num_tiles);
     rc = launch_actor_ffma(p, a->sms, a->stream);
   }
@@ -870,6 +881,7 @@ static int step_list(marl_actor* a, const int32_t* env_ids, int32_t M, const flo
     a->ids_next = (ib + 1) % ID_LISTS;
   }
   a->launches += (uint64_t)rc;
+  a->step_kernel = kernel;
   a->step += 1;
   if (a->trace_actions || a->trace_q) a->trace_next = a->trace_next + 1 > a->trace_cap ? a->trace_cap : a->trace_next + 1;
   return MARL_OK;
@@ -1106,12 +1118,14 @@ int marl_actor_reset(marl_actor_t* a) {
   return enqueue_reset(a);
 }
 
-const char* marl_actor_kernel_name(const marl_actor_t* a) { 
+const char* marl_actor_kernel_name(const marl_actor_t* a) {
   if (!a) return "ffma";
   if (a->use_tc2) return "tcgen05-dual";
   if (a->use_tcp) return a->cfg.hidden == 128 ? "tcgen05-streamed" : "tcgen05-pipelined";
   return a->use_tc ? "tcgen05" : "ffma";
 }
+
+const char* marl_actor_step_kernel(const marl_actor_t* a) { return a ? a->step_kernel : ""; }
 
 uint64_t marl_actor_launch_count(const marl_actor_t* a) { return a ? a->launches : 0; }
 

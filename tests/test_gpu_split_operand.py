@@ -43,6 +43,7 @@ def test_shapes(prec, H, shape):
     actor, acts, q = run_gpu_rollout(cfg, w, splits=[1, T - 1], work_steps=T)
     res = referee(cfg, w, actor, acts, q)
     assert res["kernel"] == "ffma"          # the general path's name
+    assert actor.step_kernel == "actor_tcs_kernel"
     actor.destroy()
 
 
@@ -57,9 +58,30 @@ def test_precision_is_that_of_the_fma_chain(H):
         actor, acts, q = run_gpu_rollout(cfg, w, kernel=kernel)
         res = referee(cfg, w, actor, acts, q)
         err[kernel] = (res["q_err"], res["h_err"])
+        assert actor.step_kernel == {"auto": "actor_tcs_kernel", "ffma": "actor_ffma_kernel"}[kernel]
         actor.destroy()
     print(f"largest row-wise relative differences to the oracle (Q, h): {err}")
     assert err["auto"][0] <= 2 * err["ffma"][0] and err["auto"][1] <= 2 * err["ffma"][1]
+
+
+@pytest.mark.parametrize("prec,H,shape,kernel", [
+    ("fp32", 64, dict(n=3, D=97, A=9), "actor_ffma_kernel"), ("fp32", 64, dict(n=3, D=96, A=17), "actor_ffma_kernel"),
+    ("fp32", 64, dict(n=3, D=96, A=16), "actor_tcs_kernel"), ("fp32", 128, dict(n=3, D=16, A=17), "actor_ffma_kernel"),
+    ("fp32", 128, dict(n=3, D=97, A=9), "actor_ffma_kernel"), ("bf16", 128, dict(n=3, D=321, A=17), "actor_ffma_kernel"),
+    ("bf16", 64, dict(n=3, D=30, A=9), "actor_tcs_kernel"), ("bf16", 64, dict(n=4, D=30, A=8), "actor_tcp_kernel"),
+    ("bf16", 128, dict(n=8, D=80, A=14), "actor_tcs_kernel")])
+def test_kernel_of_a_step(prec, H, shape, kernel):
+    """Which kernel a dense step and a list step run on, at the edges of the shapes that the split-operand kernel takes."""
+    cfg = workloads.small_config(H=H, E=8, C=8, L=4, precision=prec, **shape)
+    a = binding.Actor(cfg)
+    a.set_weights(workloads.make_weights(cfg))
+    assert a.step_kernel == ""
+    x = [v[0] for v in a.env_generate(cfg["env"], 0, 1)]
+    a.step(*x, 0.1)
+    assert a.step_kernel == kernel
+    a.step_subset(np.arange(3), *[v[:3].contiguous() for v in x], 0.1)
+    assert a.step_kernel == ("actor_tcs_kernel" if kernel == "actor_tcp_kernel" else kernel)   # (three environments: no whole chunk)
+    a.destroy()
 
 
 @pytest.mark.parametrize("D", [30, 32])
