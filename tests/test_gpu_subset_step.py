@@ -11,6 +11,16 @@ from referee import RTOL, check_near_ties, near_tie_rows_allowed, row_rel_err, s
 pytestmark = pytest.mark.gpu
 
 
+def _networks(cfg):
+    """The network, or one for each unit type."""
+    types = cfg.get("agent_type")
+    return workloads.make_weights(cfg) if types is None else [workloads.make_weights(cfg, seed=70 + k) for k in range(max(types) + 1)]
+
+
+def _load(actor, w):
+    actor.set_weights(w) if isinstance(w, dict) else actor.set_weights_typed(w)
+
+
 def _env_block(cfg, T):
     E = cfg["E"]
     obs = np.zeros((T, E, cfg["n"], cfg["D"]), np.float32)
@@ -31,17 +41,26 @@ def _env_block(cfg, T):
     ("bf16", "pipelined", dict(E=96, n=4, A=8, D=24, C=192), 5),
     ("bf16", "pipelined", dict(E=700, n=8, A=14, D=80, C=700), 0),
     # rows that are not 16-byte multiples: lists whose length is not a multiple of four go to the CUDA-core kernel
-    ("bf16", "pipelined", dict(E=300, n=5, A=12, D=55, C=300), 6)])
+    ("bf16", "pipelined", dict(E=300, n=5, A=12, D=55, C=300), 6),
+    # the split-operand kernel; every seventh list has one environment
+    ("fp32", "auto", dict(E=96, n=4, A=7, D=24, C=192), 0),
+    ("fp32", "auto", dict(E=701, n=5, A=12, D=55, C=701), 6),
+    ("fp32", "auto", dict(H=128, E=300, n=3, A=9, D=30, C=300), 0),
+    ("bf16", "auto", dict(H=128, E=303, n=5, A=12, D=55, C=606), 5),
+    ("bf16", "auto", dict(H=128, E=90, n=8, A=14, D=80, C=90), 0),
+    ("bf16", "auto", dict(E=260, n=3, A=9, D=31, C=260), 0),
+    ("fp32", "auto", dict(E=150, n=5, A=11, D=40, C=300, agent_type=[0, 1, 1, 0, 2]), 4)])
 def test_subset_steps_match_the_oracle(prec, kernel, shape, full_every):
-    cfg = workloads.small_config(H=64, L=5, T=22, precision=prec, env=dict(done_thresh24=1 << 21), **shape)
+    cfg = workloads.small_config(**{**dict(H=64, L=5, T=22, precision=prec, env=dict(done_thresh24=1 << 21)), **shape})
     E, n, A, T = cfg["E"], cfg["n"], cfg["A"], cfg["T"]
-    w = workloads.make_weights(cfg)
+    w = _networks(cfg)
     obs, avail, rew, done = _env_block(cfg, T)
     dev = "cuda:0"
     d_obs, d_avail, d_rew, d_done = (torch.as_tensor(x, device=dev) for x in (obs, avail, rew, done))
     actor = binding.Actor(cfg, device=dev, kernel=kernel)
-    actor.set_weights(w)
-    assert actor.kernel_name == {"ffma": "ffma", "pipelined": "tcgen05-pipelined"}[kernel]
+    _load(actor, w)
+    if kernel != "auto":
+        assert actor.kernel_name == {"ffma": "ffma", "pipelined": "tcgen05-pipelined"}[kernel]
     g_acts, g_q = actor.set_trace(T, want_q=True)
     sess = oracle.Session(cfg, w, np.arange(E))
     rng = np.random.default_rng(7)
@@ -53,11 +72,14 @@ def test_subset_steps_match_the_oracle(prec, kernel, shape, full_every):
             act = actor.step(d_obs[t], d_avail[t], d_rew[t], d_done[t], eps)
         else:
             M = int(rng.integers(1, E + 1)) if t % 3 else E          # every third call lists everybody, shuffled
+            if kernel == "auto" and t % 7 == 1:
+                M = 1
             ids = rng.permutation(E)[:M].astype(np.int32)
             tid = torch.as_tensor(ids, device=dev, dtype=torch.long)
             act = actor.step_subset(ids, d_obs[t].index_select(0, tid).contiguous(),
                                     d_avail[t].index_select(0, tid).contiguous(), d_rew[t].index_select(0, tid).contiguous(),
                                     d_done[t].index_select(0, tid).contiguous(), eps)
+        assert kernel != "auto" or actor.step_kernel == "actor_tcs_kernel"
         act = act.cpu().numpy()
         tid = torch.as_tensor(ids, device=dev, dtype=torch.long)
         q_rows = g_q[t].index_select(0, tid).cpu().numpy()
@@ -129,17 +151,24 @@ def test_subset_list_is_validated_on_the_host():
                                                ("bf16", "ffma", dict(E=500, n=5, A=11, D=16, C=1000)),
                                                ("bf16", "pipelined", dict(E=64, n=4, A=8, D=24, C=128)),
                                                ("bf16", "pipelined", dict(E=700, n=8, A=14, D=80, C=1400)),
-                                               ("bf16", "pipelined", dict(E=300, n=5, A=12, D=55, C=600))])
+                                               ("bf16", "pipelined", dict(E=300, n=5, A=12, D=55, C=600)),
+                                               # the split-operand kernel; every seventh list has one environment
+                                               ("fp32", "auto", dict(E=80, n=3, A=6, D=20, C=240)),
+                                               ("fp32", "auto", dict(E=501, n=5, A=12, D=55, C=1002)),
+                                               ("fp32", "auto", dict(H=128, E=300, n=8, A=16, D=15, C=300)),
+                                               ("bf16", "auto", dict(H=128, E=303, n=5, A=12, D=55, C=606)),
+                                               ("bf16", "auto", dict(E=260, n=3, A=9, D=31, C=520)),
+                                               ("fp32", "auto", dict(E=150, n=5, A=11, D=40, C=300, agent_type=[0, 1, 1, 0, 2]))])
 def test_lagged_steps_match_the_oracle(prec, kernel, shape):
     """Environments that answer after the action (Algorithm 1): every environment runs on its own clock, a call lists
     those with a new observation and brings the outcome of their previous action."""
-    cfg = workloads.small_config(H=64, L=4, T=26, precision=prec, env=dict(done_thresh24=1 << 22), **shape)
+    cfg = workloads.small_config(**{**dict(H=64, L=4, T=26, precision=prec, env=dict(done_thresh24=1 << 22)), **shape})
     E, n, A, T = cfg["E"], cfg["n"], cfg["A"], cfg["T"]
-    w = workloads.make_weights(cfg)
+    w = _networks(cfg)
     obs, avail, rew, done = _env_block(cfg, T)            # [k][e]: the k-th exchange of environment e
     dev = "cuda:0"
     actor = binding.Actor(cfg, device=dev, kernel=kernel)
-    actor.set_weights(w)
+    _load(actor, w)
     g_acts, g_q = actor.set_trace(T, want_q=True)
     sess = oracle.Session(cfg, w, np.arange(E))
     rng = np.random.default_rng(11)
@@ -148,6 +177,8 @@ def test_lagged_steps_match_the_oracle(prec, kernel, shape):
     near = greedy = 0
     for t in range(T):
         M = E if t == 0 else int(rng.integers(1, E + 1))
+        if kernel == "auto" and t % 7 == 1:
+            M = 1
         ids = rng.permutation(E)[:M].astype(np.int32)
         k = k_of[ids]
         first = k == 0
@@ -155,6 +186,7 @@ def test_lagged_steps_match_the_oracle(prec, kernel, shape):
         p_done = np.where(first, 1, done[np.maximum(k - 1, 0), ids]).astype(np.uint8)   # ignored on a first call
         o, av = obs[k, ids], avail[k, ids]
         act = actor.step_lagged(ids, *(torch.as_tensor(x, device=dev) for x in (o, av, p_rew, p_done)), eps).cpu().numpy()
+        assert kernel != "auto" or actor.step_kernel == "actor_tcs_kernel"
         tid = torch.as_tensor(ids, device=dev, dtype=torch.long)
         q_rows = g_q[t].index_select(0, tid).cpu().numpy()
         _, tr = sess.step_lagged(ids, o, av, p_rew, p_done, eps, adopt=act, trace=("q", "action_free", "explore"))
