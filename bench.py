@@ -79,6 +79,37 @@ def flops_per_agent_step(cfg: dict) -> float:
     return 2.0 * H * (D + 6 * H + A) + 25.0 * H
 
 
+def step_roofline(cfg: dict, kernel: str, kernel_ms: float, T_launch: float, agent_steps: float, peaks: dict, peak_kind: str,
+                  ffma_peak: float | None = None) -> dict:
+    """The roofline record of a launch of `agent_steps` agent-steps (T_launch environment steps) that took kernel_ms.
+
+    The bound is the slower of the algorithmic bytes at the measured HBM bandwidth and the products at the measured tensor
+    throughput (the sustained figure: the timed region is a loop of seconds).  In fp32 the split-operand kernel forms six bf16
+    products for each fp32 one; the CUDA-core kernel in fp32 is bound by plain FFMA arithmetic instead."""
+    seconds = kernel_ms * 1e-3
+    nbytes = algorithmic_bytes_per_agent_step(cfg, T_launch) * agent_steps
+    flops = flops_per_agent_step(cfg)
+    achieved, flop_rate = nbytes / seconds / 1e9, flops * agent_steps / seconds / 1e12
+    if ffma_peak is not None:
+        return {"bound": "alu", "achieved": flop_rate, "peak": ffma_peak, "unit": "TFLOP/s", "frac": flop_rate / ffma_peak,
+                "traffic": None, "peak_source": "measured (FFMA loop, this run)", "kernel": kernel, "kernel_ms": kernel_ms,
+                "flops_per_agent_step": flops, "hbm_gbs_achieved": achieved}
+    tf_peak = peaks.get("bf16_tflops_sustained") or peaks["bf16_tflops"]
+    products = 6 if cfg["precision"] == "fp32" else 1
+    tensor_rate = flop_rate * products
+    common = {"peak_source": peak_kind, "kernel": kernel, "kernel_ms": kernel_ms,
+              "algorithmic_bytes_per_agent_step": algorithmic_bytes_per_agent_step(cfg, T_launch),
+              "flops_per_agent_step": flops, "hbm_gbs_achieved": achieved, "tflops_effective": flop_rate,
+              "hbm_frac": achieved / peaks["hbm_gbs"], "tensor_frac": tensor_rate / tf_peak}
+    if products > 1:
+        common["bf16_products_per_product"] = products
+    if tensor_rate / tf_peak > achieved / peaks["hbm_gbs"]:
+        return {"bound": "tensor", "achieved": tensor_rate, "peak": tf_peak, "unit": "TFLOP/s", "frac": tensor_rate / tf_peak,
+                "traffic": None, **common}
+    return {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": achieved / peaks["hbm_gbs"],
+            **traffic_record(kernel, agent_steps, nbytes), **common}
+
+
 def traffic_record(kernel_name: str, agent_steps_per_launch: float, algorithmic_bytes: float) -> dict:
     """DRAM bytes per launch from the committed ncu record of this kernel: {"traffic": bytes or None, ...}.  None if
     there is no record or the kernel sources have changed since the counters were taken.  The record comes from a
@@ -480,35 +511,9 @@ def main():
     peaks, peak_kind = load_peaks()
     kernel_ms = ms_local / max(launches, 1)            # one actor kernel per bench step (two when it is split)
     T_launch = T * args.steps / max(launches, 1)       # environment steps one launch covers
-    bytes_per_launch = algorithmic_bytes_per_agent_step(cfg, T_launch) * E * n * T_launch
-    achieved = bytes_per_launch / (kernel_ms * 1e-3) / 1e9
-    flop_rate = flops_per_agent_step(cfg) * E * n * T_launch / (kernel_ms * 1e-3) / 1e12
-    kname = {"tcgen05-pipelined": "actor_tcp_kernel", "tcgen05": "actor_tc_kernel", "tcgen05-dual": "actor_tc2_kernel",
-             "tcgen05-streamed": "actor_tcs_kernel"}.get(actor.kernel_name, "actor_ffma_kernel")
-    if cfg["precision"] == "fp32":
-        # the fp32 path is bound by plain FFMA arithmetic: peak measured on this device by the library's FMA loop
-        ffma_peak = binding.marl_measure_ffma_tflops()
-        roofline = {"bound": "alu", "achieved": flop_rate, "peak": ffma_peak, "unit": "TFLOP/s",
-                    "frac": flop_rate / ffma_peak, "traffic": None, "peak_source": "measured (FFMA loop, this run)",
-                    "kernel": kname, "kernel_ms": kernel_ms, "flops_per_agent_step": flops_per_agent_step(cfg),
-                    "hbm_gbs_achieved": achieved}
-    else:
-        # The step's roofline is the slower of its bytes at the measured HBM bandwidth and its FLOPs at the measured
-        # bf16 tensor throughput (the sustained figure: the timed region is a loop of seconds).
-        tf_peak = peaks.get("bf16_tflops_sustained") or peaks["bf16_tflops"]
-        t_hbm = bytes_per_launch / (peaks["hbm_gbs"] * 1e9)
-        t_tensor = flops_per_agent_step(cfg) * E * n * T_launch / (tf_peak * 1e12)
-        common = {"peak_source": peak_kind, "kernel": kname, "kernel_ms": kernel_ms,
-                  "algorithmic_bytes_per_agent_step": algorithmic_bytes_per_agent_step(cfg, T_launch),
-                  "flops_per_agent_step": flops_per_agent_step(cfg), "hbm_gbs_achieved": achieved,
-                  "tflops_effective": flop_rate, "hbm_frac": achieved / peaks["hbm_gbs"], "tensor_frac": flop_rate / tf_peak}
-        if t_tensor > t_hbm:
-            roofline = {"bound": "tensor", "achieved": flop_rate, "peak": tf_peak, "unit": "TFLOP/s",
-                        "frac": flop_rate / tf_peak, "traffic": None, **common}
-        else:
-            roofline = {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
-                        "frac": achieved / peaks["hbm_gbs"], **traffic_record(kname, E * n * T_launch, bytes_per_launch),
-                        **common}
+    kname = actor.step_kernel
+    ffma_peak = binding.marl_measure_ffma_tflops() if kname == "actor_ffma_kernel" and cfg["precision"] == "fp32" else None
+    roofline = step_roofline(cfg, kname, kernel_ms, T_launch, E * n * T_launch, peaks, peak_kind, ffma_peak)
 
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms_total / args.steps, "ms_per_step_median": ms_median,

@@ -50,3 +50,22 @@ def test_algorithmic_bytes_formula():
     cfg = workloads.config(5)
     assert abs(bench.algorithmic_bytes_per_agent_step(cfg, 64) - 737.25) < 1e-9
     assert abs(bench.flops_per_agent_step(cfg) - (2 * 64 * (80 + 384 + 14) + 25 * 64)) < 1e-9
+
+
+def test_roofline_of_each_kernel():
+    """The bound follows the kernel that ran: HBM or tensor cores, in fp32 six bf16 products a product on the split-operand
+    kernel, plain FFMA on the CUDA-core kernel."""
+    sys.path.insert(0, ROOT)
+    import bench
+    from paper_2205_05248_b200 import workloads
+    peaks = {"hbm_gbs": 6500.0, "bf16_tflops": 1600.0, "bf16_tflops_sustained": 1400.0}
+    cfg = workloads.config(5, E=4096, precision="fp32")
+    steps = 4096 * 8 * 64
+    flops = bench.flops_per_agent_step(cfg)
+    r = bench.step_roofline(cfg, "actor_tcs_kernel", 1.1, 64, steps, peaks, "measured")
+    assert r["bound"] == "tensor" and r["kernel"] == "actor_tcs_kernel" and r["peak"] == 1400.0
+    assert abs(r["achieved"] - 6 * flops * steps / 1.1e-3 / 1e12) < 1e-6 and r["frac"] < 1.0
+    r = bench.step_roofline(cfg, "actor_ffma_kernel", 4.9, 64, steps, peaks, "measured", ffma_peak=72.0)
+    assert r["bound"] == "alu" and r["peak"] == 72.0 and abs(r["achieved"] - flops * steps / 4.9e-3 / 1e12) < 1e-6
+    r = bench.step_roofline(workloads.config(5), "actor_tcp_kernel", 5.7, 64, 65536 * 8 * 64, peaks, "measured")
+    assert r["bound"] == "hbm" and abs(r["achieved"] - 737.25 * 65536 * 8 * 64 / 5.7e-3 / 1e9) < 1e-6
