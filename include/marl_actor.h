@@ -61,7 +61,8 @@ extern "C" {
                                         * with at most 16 actions, obs_dim a multiple of 8 and n_agents * n_actions a
                                         * multiple of 16 (the split-operand kernel with one piece a value); create
                                         * fails otherwise.  Inputs that are not 16-byte aligned fall back, per call,
-                                        * to the one-tile kernel where the shape allows it, else to the FFMA kernel;
+                                        * to the one-tile kernel where the shape allows it, else to the general one (an
+                                        * actor made with this choice at hidden 64: the CUDA-core kernel);
                                         * so do calls whose availability block (batch * n_agents * n_actions bytes)
                                         * is not a 16-byte multiple when an environment's is not, and calls with an
                                         * environment count that is not a multiple of 4 when obs_dim is not a
@@ -241,7 +242,9 @@ int marl_actor_step(marl_actor_t* a, const float* obs, const uint8_t* avail, con
  * done u8[M], actions_out i32[M][n] (may be NULL).  The call consumes one index of the global step counter, which
  * keys the exploration stream as (seed, step, environment, agent) with the environment's own index; a trace row
  * of this step is written at the environment's own index as well.  Runs on the pipelined tensor-core kernel where
- * the actor uses it and the arrays can be bulk-copied (16-byte aligned obs and avail), else on the general kernel. */
+ * the actor uses it and the arrays can be bulk-copied (16-byte aligned obs and avail), else on the general kernel.
+ * May be captured into a graph, from the actor's first list step on or before: a captured call keeps its list in pinned memory of
+ * its own until the actor is destroyed (a replay reads it again). */
 int marl_actor_step_subset(marl_actor_t* a, const int32_t* env_ids, int32_t M, const float* obs,
                            const uint8_t* avail, const float* reward, const uint8_t* done, float eps,
                            int32_t* actions_out);
@@ -260,7 +263,8 @@ int marl_actor_step_lagged(marl_actor_t* a, const int32_t* env_ids, int32_t M, c
 
 /* The same step with HOST buffers (the observation-action pipe of Algorithms 1 and 2 when the simulators
  * run on the host): copies the four inputs to the device, runs the step, copies the actions back and
- * SYNCHRONISES the stream before returning.  Pinned host arrays are read and written by the step kernel itself. */
+ * SYNCHRONISES the stream before returning.  Pinned host arrays are read and written by the step kernel itself where they are
+ * pinned as a whole and start on boundaries of 16 bytes (obs, avail) and 4 bytes (reward, actions); others are copied. */
 int marl_actor_step_host(marl_actor_t* a, const float* obs, const uint8_t* avail, const float* reward,
                          const uint8_t* done, float eps, int32_t* actions_out);
 

@@ -180,7 +180,7 @@ constexpr uint64_t TP_K_A = (2 * TC_LBO_A) >> 4, TP_K_X = (2 * TC_LBO_X) >> 4, T
                    TP_K_G = (2 * TP_LBO_G) >> 4;                       // descriptor increments of one K = 16 step
 
 // fc1 of one step: observations x W1, then the one-hot tile x (bias pieces, agent-id columns); commits to fc1d.
-__device__ __forceinline__ void tp_issue_fc1(const TpLayout& L, uint32_t sb, uint32_t tmem, int lane, uint64_t* fc1d) {
+__device__ __forceinline__ void tp_issue_fc1(const TpLayout& L, uint32_t sb, uint32_t tmem, uint64_t* fc1d) {
   using namespace tc;
   tc_fence_after_sync();
   if (elect_one()) {
@@ -206,7 +206,7 @@ __device__ __forceinline__ void tp_issue_fc1(const TpLayout& L, uint32_t sb, uin
 // h-side gate products of one step: the first MMA seeds r | z | candidate-input with their biases (contiguous in
 // tensor memory: one N = 192 accumulator), the last one seeds the step's Q accumulator with the output bias.
 template <int NQ>
-__device__ __forceinline__ void tp_issue_hside(const TpLayout& L, uint32_t sb, uint32_t tmem, int lane, uint32_t qcol) {
+__device__ __forceinline__ void tp_issue_hside(const TpLayout& L, uint32_t sb, uint32_t tmem, uint32_t qcol) {
   using namespace tc;
   tc_fence_after_sync();
   if (elect_one()) {
@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
       mbar_wait(&B->wload, 0, abortf);
       if (total > 0) {
         mbar_wait(&B->xready, 0, abortf);
-        tp_issue_fc1(L, sb, tmem, lane, &B->fc1d);
+        tp_issue_fc1(L, sb, tmem, &B->fc1d);
       }
       for (int g = 0, s = 0; g < total; ++g) {
         const uint32_t par = (uint32_t)g & 1u;
@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
           } else {
             mbar_wait(&B->stepd, par ^ 1u, abortf);
           }
-          tp_issue_hside<NQ>(L, sb, tmem, lane, qcol);
+          tp_issue_hside<NQ>(L, sb, tmem, qcol);
         }
         mbar_wait(&B->yready, par, abortf);
         tc_fence_after_sync();
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
           // one lane looks (lanes looking separately could disagree and split the warp's control flow)
           const uint32_t ready = __shfl_sync(0xFFFFFFFFu, lane == 0 ? (uint32_t)mbar_test_wait(&B->xready, par ^ 1u) | (uint32_t)mbar_test_wait(&B->hready, par) << 1 : 0u, 0);
           if (ready & 1u) {
-            tp_issue_fc1(L, sb, tmem, lane, &B->fc1d);
+            tp_issue_fc1(L, sb, tmem, &B->fc1d);
             pending = false;
           } else if (ready & 2u) {
             break;
@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
         __syncwarp();
         if (pending) {
           mbar_wait(&B->xready, par ^ 1u, abortf);
-          tp_issue_fc1(L, sb, tmem, lane, &B->fc1d);
+          tp_issue_fc1(L, sb, tmem, &B->fc1d);
         }
         // The next step's h-side products need only the new hidden state, which is in place unless an episode
         // of this tile ends with this step (its rows are cleared after fc2): issue them now, off the critical
@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
         } else {
           // (published by the load warp before this step's inputs were requested: ordered before the fc1 operand)
           if (closeany_s[g & (TP_DST_DEPTH - 1)] == 0) {
-            tp_issue_hside<NQ>(L, sb, tmem, lane, TM_Q + (par ^ 1u) * tp_qstride(NQ));
+            tp_issue_hside<NQ>(L, sb, tmem, TM_Q + (par ^ 1u) * tp_qstride(NQ));
             hside_issued = true;
           }
         }

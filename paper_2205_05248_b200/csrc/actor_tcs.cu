@@ -20,8 +20,7 @@
 //
 // Roles: warps 0-7 epilogue (two groups of 128 threads; a thread owns one row and 16 columns of every block of 32
 // hidden columns), warps 8-15 inputs and records (two groups, thread = row), warp 16 issues every tcgen05.mma (from the lane that
-// elect.sync picks: ptxas then knows that one lane runs and issues without a loop over lanes; 4 products take 325-400
-// clocks to completion against 577-700 behind "lane == 0"), warp 17 loads weights.
+// elect.sync picks: 4 products take 325-400 clocks to completion against 577-700 behind "lane == 0"), warp 17 loads weights.
 // Per step:
 //   E1 (epilogue)  y = relu(fc1 + agent column + last-action column), pieces to the y operand
 //   E2 (epilogue)  per block of 32 hidden columns: gates, new hidden state (fp32 in registers); the next block's
@@ -456,7 +455,8 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
   constexpr int NBLK = H / TS_BLK, KH = H / 16;
   // The epilogue's loops over blocks: rolled for one piece at hidden 64 (the shorter code misses the instruction cache
   // less: 353 us against 400 for 4096 x 3 agents x 64 steps), unrolled where the hidden state's registers would have to
-  // rotate further (hidden 128: 3394 us against 3997) or the pieces' arithmetic hides the misses (fp32: 1047 against 1064).
+  // rotate further (hidden 128: 3394 us against 3997, one launch repeated on the same inputs) or the pieces' arithmetic hides the misses (fp32: 1047
+  // against 1064).
   constexpr int UB = NS == 1 && H == 64 ? 1 : NBLK;
   constexpr bool XS = NS == 3 && H == 128;       // x and y pieces in shared memory
   constexpr uint32_t TSM_Y = TSM_HOP + NS * H / 2;
@@ -1398,7 +1398,8 @@ int launch_actor_tcs(const ActorParams& p_in, int sms, bool fast_gates, cudaStre
   L.ntypes = ntypes;
   if (p.H == 128 && !fast_gates) {
     // the accurate gates keep the epilogue so busy that input warps running beside it all step long cost more than the
-    // wait for the shared columns (1216 against 1246 us for 4096 x 5 agents x 64 steps; fast gates: 3940 against 3410)
+    // wait for the shared columns (1216 against 1246 us for 4096 x 5 agents x 64 steps; fast gates, 16384 x 8 agents: 3940 against 3410;
+    // each one launch repeated on the same inputs)
     L.sep = 0;
     L.tm_x = TSM_HOP + (uint32_t)(ns * p.H / 2);
   }

@@ -1,6 +1,6 @@
 // Host runtime and C ABI of the actor library: configuration checks, buffer carving, weight repacking,
 // launch planning and the entry points declared in include/marl_actor.h.  All arithmetic of the actor
-// step runs in the kernels (actor_ffma.cu, actor_tc.cu, env_kernel.cu); nothing here computes on the CPU
+// step runs in the kernels (actor_*.cu, env_kernel.cu); nothing here computes on the CPU
 // and there is no CPU fallback.
 #include <cuda.h>
 
@@ -916,8 +916,8 @@ int marl_actor_step_host(marl_actor_t* a, const float* obs, const uint8_t* avail
   int32_t* d_act = reinterpret_cast<int32_t*>(a->work + wo.actions);
   // Pinned arrays are read by the step kernel itself, over the link and as its tiles need them: four copies, each with
   // its set-up, the kernel behind them and the copy back behind that become one launch.  Every input byte is read once.
-  // Measured with the copies' and the kernel's route in turn on one machine: 2.7 MB (1024 environments) 220 -> 85 us,
-  // 11 MB 743 -> 247 us.  From some 16 MB on the copy engine is the faster reader of the observations (22 MB: 479
+  // Measured with the copies' and the kernel's route in turn: 2.7 MB (1024 environments) 101 -> 81 us; with other traffic on the
+  // link 220 -> 85 us, and 11 MB 743 -> 247 us.  From some 16 MB on the copy engine is the faster reader of the observations (22 MB: 479
   // against 540 us, 175 MB: 3260 against 3460 us), the small arrays stay with the kernel.  The CUDA-core kernel reads the
   // availability rows twice and keeps the copies.
   // Arrays that do not start where the kernels want them (observations and availability on 16-byte boundaries: others would

@@ -116,7 +116,9 @@ __global__ void __launch_bounds__(GATHER_THREADS) ring_gather_kernel(const __gri
 int launch_ring_sample(const SampleParams& p, cudaStream_t stream) {
   // Equal ranges of steps per block.  Each block first makes its element's draw - some 1.5 us of dependent loads - so it
   // should move some 32 KB; twelve blocks for each that the device holds at once keep the last wave short.  Measured for
-  // 1024 episodes of 96 x 3 KB: one block of 83 and one of 13 steps per episode 87 us, nine of 11: 75 us.
+  // 1024 episodes of 96 x 3 KB: one block of 83 and one of 13 steps per episode 87 us, nine of 11: 75 us;
+  // 1024 x 96 of 2.2 KB (5 agents x 80 observations) 79 -> 53 us, 700 x 64 of 3 KB 47 -> 43, of 1.6 KB 39 -> 33.  Batches of a few
+  // hundred short episodes take the 30 us of a call whatever the split.
   const long long rows = (long long)p.L * p.B, resident = 148 * 8;
   const long long payload = 4ll * p.n * p.D + 5ll * p.n * p.A + 4ll * p.n + 5;
   long long spb = rows / (12 * resident), unit = (32768 + payload - 1) / payload, fill = rows / resident;
