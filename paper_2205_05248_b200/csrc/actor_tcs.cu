@@ -107,15 +107,17 @@ static TsLayout ts_image(int n, int D, int A, int H, int ns) {
 }
 
 // nt_max: rows of an environment in one tile (the agents, or those of the largest unit type).  ept = 0: does not fit.
-static TsLayout ts_layout(int n, int D, int A, int H, int ns, int nt_max, int M, int sms) {
+static TsLayout ts_layout(int n, int D, int A, int H, int ns, int nt_max, int M, int sms, int ntypes = 1) {
   TsLayout L = ts_image(n, D, A, H, ns);
   int ept = TS_ROWS / nt_max;
-  if (M > 0 && sms > 0) {  // even the tiles out over the waves they need anyway
-    const int tiles = (M + ept - 1) / ept, waves = (tiles + sms - 1) / sms;
-    const int e2 = (M + waves * sms - 1) / (waves * sms);
+  if (M > 0 && sms > 0) {  // even the tiles (of every type) out over the waves they need anyway
+    const int tiles = (M + ept - 1) / ept * ntypes, waves = (tiles + sms - 1) / sms;
+    const int per_type = waves * sms / ntypes;
+    const int e2 = per_type > 0 ? (M + per_type - 1) / per_type : ept;
     if (e2 < ept) ept = e2;
   }
   L.ept = ept;
+  L.ntypes = ntypes;
   uint32_t o = L.base_bytes;
   L.off_xy = o;
   if (ns == 3 && H == 128) o += 3u * (uint32_t)(L.Dk > H ? L.Dk : H) * TS_ROWS * 2;
@@ -518,14 +520,22 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
       for (int i = 0; i < n; ++i) nt += (int)((p.agent_type_bits >> (2 * i)) & 3ull) == typ ? 1 : 0;
     return nt;
   };
-  const int my_tiles = blockIdx.x < p.num_tiles ? (p.num_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+  // Work units: the tiles of type 0, then those of type 1, ...; a block takes every gridDim.x-th.
+  const int my_tiles = (p.num_tiles * ntypes - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;
+  auto unit_at = [&](int& tile, int& typ) -> bool {  // moves a tile number beyond its type's tiles on to the next type
+    while (tile >= p.num_tiles) {
+      tile -= p.num_tiles;
+      if (++typ == ntypes) return false;
+    }
+    return true;
+  };
 
   if (warp >= 16) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_SVC));
     if (warp == 16) {
       // =========================== MMA warp ===========================
       grid_wait();  // (no bounded wait may include the run time of the kernel before: its inputs arrive only after that)
-      if (my_tiles * T * ntypes <= 2) grid_release();  // (the input warps would come to it too late to gain from it)
+      if (my_tiles * T <= 2) grid_release();  // (the input warps would come to it too late to gain from it)
       const uint32_t sb = smem_u32(smem);
       constexpr uint32_t id96 = idesc_bf16_f32(128, 96), id64 = idesc_bf16_f32(128, 64), id32 = idesc_bf16_f32(128, 32),
                          idH = idesc_bf16_f32(128, H), idq = idesc_bf16_f32(128, NQ);
@@ -540,13 +550,13 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
       const uint64_t x_st = (uint64_t)nk1 * x_ks;
       constexpr uint64_t y_st = KH * x_ks;
       uint32_t g = 0, ri = 0, rpar = 0;  // steps so far; ring slot and its parity
-      uint32_t typ = 0;
+      uint32_t loads = 0;  // networks loaded so far
       bool first = true;
 
       // slice i of the step: its address once it is in shared memory
       auto get = [&](int i) -> uint32_t {
         if (i < L.nres) {
-          if (first) mbar_wait(&B->res[i < L.nw1 ? 0 : 1], typ & 1, abortf);
+          if (first) mbar_wait(&B->res[i < L.nw1 ? 0 : 1], (loads - 1) & 1, abortf);
           return sb + L.off_sl + ts_slice_off(L, H, NS, i);
         }
         mbar_wait(&B->full[ri], rpar, abortf);
@@ -585,172 +595,175 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
         }
       };
 
-      for (; typ < (uint32_t)ntypes; ++typ) {
-        if (typ > 0) __syncthreads();  // every role has left the previous type
-        first = true;
-        for (int tile = blockIdx.x; tile < p.num_tiles; tile += gridDim.x)
-          for (int s = 0; s < T; ++s, ++g, first = false) {
-            const uint32_t par = g & 1;
-            // ---- fc1 ----
-            mbar_wait(&B->xrdy, par, abortf);  // (E2 of the previous step has read the columns: hr1)
-            tc_fence_after_sync();
-            {
-              for (int i = 0; i < L.nw1; ++i) {
-                const uint64_t w = desc(get(i), H * 16);
-                if (elect_one()) {
-                  // piece 2 - i against the small products' left pieces, then the main product (one piece: the slice's)
-                  const int k0 = NS == 3 ? 0 : i * (TS_KCHUNK / 16), nk = min(nk1 - k0, TS_KCHUNK / 16);
+      for (int tile = blockIdx.x, typ = 0, cur = -1; unit_at(tile, typ); tile += gridDim.x) {
+        if (typ != cur) {
+          cur = typ;
+          first = true;
+          if (loads++ > 0) __syncthreads();  // every role has left the previous type
+        }
+        for (int s = 0; s < T; ++s, ++g, first = false) {
+          const uint32_t par = g & 1;
+          // ---- fc1 ----
+          mbar_wait(&B->xrdy, par, abortf);  // (E2 of the previous step has read the columns: hr1)
+          tc_fence_after_sync();
+          {
+            for (int i = 0; i < L.nw1; ++i) {
+              const uint64_t w = desc(get(i), H * 16);
+              if (elect_one()) {
+                // piece 2 - i against the small products' left pieces, then the main product (one piece: the slice's)
+                const int k0 = NS == 3 ? 0 : i * (TS_KCHUNK / 16), nk = min(nk1 - k0, TS_KCHUNK / 16);
 #pragma unroll 1
-                  for (int ai = NS == 3 ? i : 0; ai >= 0; --ai) {
-                    uint64_t a = a_x + ai * x_st + (uint32_t)k0 * x_ks, wk = w;
-                    uint32_t acc = i > 0 || (NS == 3 && ai < i);
-                    int ks = 0;
+                for (int ai = NS == 3 ? i : 0; ai >= 0; --ai) {
+                  uint64_t a = a_x + ai * x_st + (uint32_t)k0 * x_ks, wk = w;
+                  uint32_t acc = i > 0 || (NS == 3 && ai < i);
+                  int ks = 0;
 #pragma unroll 1
-                    for (; ks + 2 <= nk; ks += 2, a += 2 * x_ks, wk += 2 * ks_1, acc = 1) {
-                      ts_mma<XS>(tmem + FC1, a, wk, idH, acc);
-                      ts_mma<XS>(tmem + FC1, a + x_ks, wk + ks_1, idH, 1);
-                    }
-                    if (ks < nk) ts_mma<XS>(tmem + FC1, a, wk, idH, acc);
+                  for (; ks + 2 <= nk; ks += 2, a += 2 * x_ks, wk += 2 * ks_1, acc = 1) {
+                    ts_mma<XS>(tmem + FC1, a, wk, idH, acc);
+                    ts_mma<XS>(tmem + FC1, a + x_ks, wk + ks_1, idH, 1);
                   }
-                  if (i >= L.nres) mma_commit(&B->empty[ri]);
-                  if (i == L.nw1 - 1) mma_commit(&B->fc1d);
+                  if (ks < nk) ts_mma<XS>(tmem + FC1, a, wk, idH, acc);
                 }
-                __syncwarp();
-                if (i >= L.nres) next_slot();
+                if (i >= L.nres) mma_commit(&B->empty[ri]);
+                if (i == L.nw1 - 1) mma_commit(&B->fc1d);
               }
+              __syncwarp();
+              if (i >= L.nres) next_slot();
             }
-            // ---- gates ----
-            if (H == 64) {
-              // everything resident: the hidden side's first products run before the fc1 output is there
-              mbar_wait(&B->hset, par, abortf);
-              tc_fence_after_sync();
-              const uint64_t w0 = desc(get(L.nw1), 1536);
-              constexpr uint64_t SL = ts_slice(H) >> 4;
-              // pieces of the small products in order: left, and slice of the hidden and of the y side
-              constexpr uint32_t LEFT = 0x10210u, SH = 0x41410u, SY = 0x53532u;
-              if (elect_one()) {
+          }
+          // ---- gates ----
+          if (H == 64) {
+            // everything resident: the hidden side's first products run before the fc1 output is there
+            mbar_wait(&B->hset, par, abortf);
+            tc_fence_after_sync();
+            const uint64_t w0 = desc(get(L.nw1), 1536);
+            constexpr uint64_t SL = ts_slice(H) >> 4;
+            // pieces of the small products in order: left, and slice of the hidden and of the y side
+            constexpr uint32_t LEFT = 0x10210u, SH = 0x41410u, SY = 0x53532u;
+            if (elect_one()) {
 #pragma unroll 1
-                for (int b = 0; b < NBLK; ++b)
+              for (int b = 0; b < NBLK; ++b)
 #pragma unroll 1
-                  for (int j = 0; j < (NS == 3 ? 5 : 1); ++j)
-                    prod(b, 1, (LEFT >> (4 * j)) & 15u, w0 + (uint32_t)(b * 2 * NS) * SL + (NS == 3 ? (SH >> (4 * j)) & 15u : 0u) * SL, j > 0);
-              }
-              __syncwarp();
-              mbar_wait(&B->yrdy, par, abortf);
-              tc_fence_after_sync();
-              if (elect_one()) {
-#pragma unroll 1
-                for (int b = 0; b < NBLK; ++b) {
-                  const uint64_t wb = w0 + (uint32_t)(b * 2 * NS) * SL;
-                  if (NS == 3) {
-#pragma unroll 1
-                    for (int j = 0; j < 7; ++j)  // five small ones, then the main products
-                      prod(b, j == 5, j < 5 ? (LEFT >> (4 * j)) & 15u : 0u, wb + (j < 5 ? (SY >> (4 * j)) & 15u : (uint32_t)j - 1u) * SL, j > 0);
-                  } else {
-                    prod(b, 0, 0, wb + SL, 0);
-                  }
-                  mma_commit(&B->gd[b]);
-                }
-              }
-              __syncwarp();
-            } else {
-              int i = L.nw1;
+                for (int j = 0; j < (NS == 3 ? 5 : 1); ++j)
+                  prod(b, 1, (LEFT >> (4 * j)) & 15u, w0 + (uint32_t)(b * 2 * NS) * SL + (NS == 3 ? (SH >> (4 * j)) & 15u : 0u) * SL, j > 0);
+            }
+            __syncwarp();
+            mbar_wait(&B->yrdy, par, abortf);
+            tc_fence_after_sync();
+            if (elect_one()) {
 #pragma unroll 1
               for (int b = 0; b < NBLK; ++b) {
-                const int buf = (b + 1) & 1;
-                if (b == 0) {
-                  mbar_wait(&B->hset, par, abortf);
-                } else if (b >= 2) {
-                  mbar_wait(&B->accf[buf], par, abortf);
-                }
-                tc_fence_after_sync();
+                const uint64_t wb = w0 + (uint32_t)(b * 2 * NS) * SL;
                 if (NS == 3) {
-                  // h2, h1, y2, y1, then h0 and y0 held together: their small products come before both main ones
-                  uint64_t wh = 0;
-                  uint32_t rh = 0;
 #pragma unroll 1
-                  for (int k = 0; k < 6; ++k, ++i) {
-                    if (b == 0 && k == 2) {
-                      mbar_wait(&B->yrdy, par, abortf);
-                      tc_fence_after_sync();
-                    }
-                    const uint64_t w = desc(get(i), 1536);
-                    const int hid = k < 2 || k == 4;
-                    if (k == 4) { wh = w; rh = ri; }
-                    if (elect_one()) {
-                      // left pieces: k = 0, 2: 0; 1, 3: 1 0; 4, 5: 2 1; after the last the main products
-                      const int first_ai = k >= 4 ? 2 : k & 1, last_ai = k >= 4 ? 1 : 0;
-#pragma unroll 1
-                      for (int ai = first_ai; ai >= last_ai - (k == 5 ? 2 : 0); --ai) {
-                        const bool main = ai < last_ai, mh = main && ai == 0;  // (k == 5: 0 stands for the hidden main, -1 for the y main)
-                        prod(buf, main ? mh : hid, main ? 0u : (uint32_t)ai, mh ? wh : w, !((k == 0 || k == 2) && ai == first_ai));
-                        if (mh && i - 1 >= L.nres) mma_commit(&B->empty[rh]);
-                      }
-                      if (i >= L.nres && k != 4) mma_commit(&B->empty[ri]);
-                      if (k == 5) mma_commit(&B->gd[buf]);
-                    }
-                    __syncwarp();
-                    if (i >= L.nres) next_slot();
-                  }
+                  for (int j = 0; j < 7; ++j)  // five small ones, then the main products
+                    prod(b, j == 5, j < 5 ? (LEFT >> (4 * j)) & 15u : 0u, wb + (j < 5 ? (SY >> (4 * j)) & 15u : (uint32_t)j - 1u) * SL, j > 0);
                 } else {
-                  const uint64_t wh = desc(get(i), 1536);
-                  if (elect_one()) {
-                    prod(buf, 1, 0, wh, 0);
-                    if (i >= L.nres) mma_commit(&B->empty[ri]);
-                  }
-                  __syncwarp();
-                  if (i >= L.nres) next_slot();
-                  ++i;
-                  const uint64_t wy = desc(get(i), 1536);
-                  if (b == 0) {
+                  prod(b, 0, 0, wb + SL, 0);
+                }
+                mma_commit(&B->gd[b]);
+              }
+            }
+            __syncwarp();
+          } else {
+            int i = L.nw1;
+#pragma unroll 1
+            for (int b = 0; b < NBLK; ++b) {
+              const int buf = (b + 1) & 1;
+              if (b == 0) {
+                mbar_wait(&B->hset, par, abortf);
+              } else if (b >= 2) {
+                mbar_wait(&B->accf[buf], par, abortf);
+              }
+              tc_fence_after_sync();
+              if (NS == 3) {
+                // h2, h1, y2, y1, then h0 and y0 held together: their small products come before both main ones
+                uint64_t wh = 0;
+                uint32_t rh = 0;
+#pragma unroll 1
+                for (int k = 0; k < 6; ++k, ++i) {
+                  if (b == 0 && k == 2) {
                     mbar_wait(&B->yrdy, par, abortf);
                     tc_fence_after_sync();
                   }
+                  const uint64_t w = desc(get(i), 1536);
+                  const int hid = k < 2 || k == 4;
+                  if (k == 4) { wh = w; rh = ri; }
                   if (elect_one()) {
-                    prod(buf, 0, 0, wy, 0);
-                    if (i >= L.nres) mma_commit(&B->empty[ri]);
-                    mma_commit(&B->gd[buf]);
+                    // left pieces: k = 0, 2: 0; 1, 3: 1 0; 4, 5: 2 1; after the last the main products
+                    const int first_ai = k >= 4 ? 2 : k & 1, last_ai = k >= 4 ? 1 : 0;
+#pragma unroll 1
+                    for (int ai = first_ai; ai >= last_ai - (k == 5 ? 2 : 0); --ai) {
+                      const bool main = ai < last_ai, mh = main && ai == 0;  // (k == 5: 0 stands for the hidden main, -1 for the y main)
+                      prod(buf, main ? mh : hid, main ? 0u : (uint32_t)ai, mh ? wh : w, !((k == 0 || k == 2) && ai == first_ai));
+                      if (mh && i - 1 >= L.nres) mma_commit(&B->empty[rh]);
+                    }
+                    if (i >= L.nres && k != 4) mma_commit(&B->empty[ri]);
+                    if (k == 5) mma_commit(&B->gd[buf]);
                   }
                   __syncwarp();
                   if (i >= L.nres) next_slot();
-                  ++i;
                 }
+              } else {
+                const uint64_t wh = desc(get(i), 1536);
+                if (elect_one()) {
+                  prod(buf, 1, 0, wh, 0);
+                  if (i >= L.nres) mma_commit(&B->empty[ri]);
+                }
+                __syncwarp();
+                if (i >= L.nres) next_slot();
+                ++i;
+                const uint64_t wy = desc(get(i), 1536);
+                if (b == 0) {
+                  mbar_wait(&B->yrdy, par, abortf);
+                  tc_fence_after_sync();
+                }
+                if (elect_one()) {
+                  prod(buf, 0, 0, wy, 0);
+                  if (i >= L.nres) mma_commit(&B->empty[ri]);
+                  mma_commit(&B->gd[buf]);
+                }
+                __syncwarp();
+                if (i >= L.nres) next_slot();
+                ++i;
               }
             }
-            // ---- fc2: the small products of all blocks but the last, then the rest ----
-            if (g > 0) mbar_wait(&B->qfree, par ^ 1u, abortf);  // the previous step's Q has been read
-            const uint64_t w2 = desc(sb, NQ * 16);
-            constexpr int K1 = KH - TS_BLK / 16;  // K steps of the earlier blocks
-            auto part_q = [&](auto half_c) {  // K steps [0, K1) or [K1, KH); the second part ends with the main product
-              constexpr int half = decltype(half_c)::value, k0 = half ? K1 : 0, k1 = half ? KH : K1;
-              mbar_wait(half ? &B->hr1 : &B->hr0, par, abortf);
-              tc_fence_after_sync();
-              if (elect_one()) {
-                if (NS == 3) {  // small products (left, right): (2,0) (1,1) (0,2) (1,0) (0,1)
-#pragma unroll 1
-                  for (int j = 0; j < 5; ++j) {
-                    const uint64_t a = a_h + ((0x01012u >> (4 * j)) & 15u) * h_st, w = w2 + ((0x10210u >> (4 * j)) & 15u) * st_q;
-#pragma unroll
-                    for (int ks = k0; ks < k1; ++ks) ts_mma<false>(tmem + L.tm_q, a + ks * h_ks, w + ks * ks_q, idq, ks > 0 || j > 0);
-                  }
-                }
-                if (NS == 1 || half)
-#pragma unroll
-                  for (int ks = NS == 3 ? 0 : k0; ks < k1; ++ks) ts_mma<false>(tmem + L.tm_q, a_h + ks * h_ks, w2 + ks * ks_q, idq, NS == 3 || ks > 0);
-                if (half) mma_commit(&B->fc2d);
-              }
-              __syncwarp();
-            };
-            part_q(std::integral_constant<int, 0>());
-            part_q(std::integral_constant<int, 1>());
           }
+          // ---- fc2: the small products of all blocks but the last, then the rest ----
+          if (g > 0) mbar_wait(&B->qfree, par ^ 1u, abortf);  // the previous step's Q has been read
+          const uint64_t w2 = desc(sb, NQ * 16);
+          constexpr int K1 = KH - TS_BLK / 16;  // K steps of the earlier blocks
+          auto part_q = [&](auto half_c) {  // K steps [0, K1) or [K1, KH); the second part ends with the main product
+            constexpr int half = decltype(half_c)::value, k0 = half ? K1 : 0, k1 = half ? KH : K1;
+            mbar_wait(half ? &B->hr1 : &B->hr0, par, abortf);
+            tc_fence_after_sync();
+            if (elect_one()) {
+              if (NS == 3) {  // small products (left, right): (2,0) (1,1) (0,2) (1,0) (0,1)
+#pragma unroll 1
+                for (int j = 0; j < 5; ++j) {
+                  const uint64_t a = a_h + ((0x01012u >> (4 * j)) & 15u) * h_st, w = w2 + ((0x10210u >> (4 * j)) & 15u) * st_q;
+#pragma unroll
+                  for (int ks = k0; ks < k1; ++ks) ts_mma<false>(tmem + L.tm_q, a + ks * h_ks, w + ks * ks_q, idq, ks > 0 || j > 0);
+                }
+              }
+              if (NS == 1 || half)
+#pragma unroll
+                for (int ks = NS == 3 ? 0 : k0; ks < k1; ++ks) ts_mma<false>(tmem + L.tm_q, a_h + ks * h_ks, w2 + ks * ks_q, idq, NS == 3 || ks > 0);
+              if (half) mma_commit(&B->fc2d);
+            }
+            __syncwarp();
+          };
+          part_q(std::integral_constant<int, 0>());
+          part_q(std::integral_constant<int, 1>());
+        }
       }
     } else if (warp == 17) {
       // =========================== weight warp ===========================
       uint32_t ri = 0, rpar = 1, used = 0;
-      for (int typ = 0; typ < ntypes; ++typ) {
-        if (typ > 0) __syncthreads();
-        if (my_tiles == 0) continue;
+      for (int tile = blockIdx.x, typ = 0, cur = -1; unit_at(tile, typ); tile += gridDim.x) {
+        if (typ == cur) continue;
+        if (cur >= 0) __syncthreads();
+        cur = typ;
         const uint8_t* img = reinterpret_cast<const uint8_t*>(p.wsplit) + (size_t)typ * p.wsplit_stride;
         const uint8_t* sl = img + L.base_bytes;
         if (lane == 0) {
@@ -765,7 +778,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
         }
         __syncwarp();
         if (L.nres < L.nsl) {
-          const int steps = my_tiles * T;
+          const int steps = ((p.num_tiles - 1 - tile) / (int)gridDim.x + 1) * T;
           for (int g = 0; g < steps; ++g)
             for (int i = L.nres; i < L.nsl; ++i) {
               if (used >= (uint32_t)L.nslots) {
@@ -787,7 +800,10 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
         }
       }
     } else {
-      for (int typ = 1; typ < ntypes; ++typ) __syncthreads();
+      for (int tile = blockIdx.x, typ = 0, cur = -1; unit_at(tile, typ); tile += gridDim.x) {
+        if (typ != cur && cur >= 0) __syncthreads();
+        cur = typ;
+      }
     }
   } else if (warp >= 8) {
     // =========================== inputs and records ===========================
@@ -806,301 +822,314 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
     uint8_t* units = smem + L.off_scr + (warp - 8) * L.nu * TS_UNIT;
     const int c4 = lane & 3;  // the unit's columns 4 c4 .. of rows 8 j + lane / 4 are this lane's to copy
     const bool vec = (D & 3) == 0 && (reinterpret_cast<uintptr_t>(p.obs) & 15) == 0;
-    uint32_t c_episodes = 0, c_trunc = 0, st_bits = 0, g = 0;
-    for (int typ = 0; typ < ntypes; ++typ) {
-      if (typ > 0) __syncthreads();
-      const int nt = rows_per_env(typ);
-      bool fresh = true;
-      for (int tile = blockIdx.x; tile < p.num_tiles; tile += gridDim.x) {
-        const int e0 = tile * ept;
-        const int ne = min(ept, p.M - e0);
-        const int R = ne * nt;
-        const bool wlive = pw * 32 < R;   // warps without a live row only keep the barriers going
-        const bool live = row < R;
-        const bool cursor = grp == 1 && row < ne;
-        int32_t slot = 0, pos = 0, eok = 0;
-        long long epc = 0;
-        asm volatile("bar.sync 2, 512;" ::: "memory");  // the previous tile's shared arrays are done with
-        if (cursor) {
-          const int e = p.env_ids ? __ldg(p.env_ids + e0 + row) : e0 + row;
-          slot = p.slot[e];
-          pos = p.pos[e];
-          epc = p.ep_count[e];
-          // (with late outcomes a full slot waits, at pos == L, for its last outcome before it is truncated)
-          eok = (slot >= 0 && slot < p.E * p.S && pos >= 0 && pos < p.L + (lag ? 1 : 0)) ? 1 : 0;
-          if (!eok) st_bits |= MARL_STATUS_BAD_INDEX;
-          int closed = 0;
-          if (lag && eok && pos > 0) {
-            // the outcome of the previous action completes the record at pos - 1 and may close the episode
-            const float r = p.reward[e0 + row];
-            const int d = p.done[e0 + row] ? 1 : 0;
+    uint32_t c_episodes = 0, c_trunc = 0, st_bits = 0, g = 0, loads = 0;
+    int nt = 0;
+    bool fresh = true;
+    for (int tile = blockIdx.x, typ = 0, cur = -1; unit_at(tile, typ); tile += gridDim.x) {
+      if (typ != cur) {
+        cur = typ;
+        nt = rows_per_env(typ);
+        fresh = true;
+        if (loads++ > 0) __syncthreads();
+      }
+      const int e0 = tile * ept;
+      const int ne = min(ept, p.M - e0);
+      const int R = ne * nt;
+      const bool wlive = pw * 32 < R;   // warps without a live row only keep the barriers going
+      const bool live = row < R;
+      const bool cursor = grp == 1 && row < ne;
+      int32_t slot = 0, pos = 0, eok = 0;
+      long long epc = 0;
+      asm volatile("bar.sync 2, 512;" ::: "memory");  // the previous tile's shared arrays are done with
+      if (cursor) {
+        const int e = p.env_ids ? __ldg(p.env_ids + e0 + row) : e0 + row;
+        slot = p.slot[e];
+        pos = p.pos[e];
+        epc = p.ep_count[e];
+        // (with late outcomes a full slot waits, at pos == L, for its last outcome before it is truncated)
+        eok = (slot >= 0 && slot < p.E * p.S && pos >= 0 && pos < p.L + (lag ? 1 : 0)) ? 1 : 0;
+        if (!eok) st_bits |= MARL_STATUS_BAD_INDEX;
+        int closed = 0;
+        if (lag && eok && pos > 0) {
+          // the outcome of the previous action completes the record at pos - 1 and may close the episode
+          const float r = p.reward[e0 + row];
+          const int d = p.done[e0 + row] ? 1 : 0;
+          if (typ == 0) {
+            uint8_t* rec = p.ring + (size_t)slot * p.slot_stride + (size_t)(pos - 1) * rec_bytes;
+            *reinterpret_cast<float*>(rec + p.rl.off_reward) = r;
+            rec[p.rl.off_done] = (uint8_t)d;
+          }
+          if (d || pos == p.L) {
             if (typ == 0) {
-              uint8_t* rec = p.ring + (size_t)slot * p.slot_stride + (size_t)(pos - 1) * rec_bytes;
-              *reinterpret_cast<float*>(rec + p.rl.off_reward) = r;
-              rec[p.rl.off_done] = (uint8_t)d;
+              p.slot_len[slot] = pos;
+              p.slot_complete[slot] = 1;
+              c_episodes += 1;
+              if (!d) c_trunc += 1;
             }
-            if (d || pos == p.L) {
-              if (typ == 0) {
-                p.slot_len[slot] = pos;
-                p.slot_complete[slot] = 1;
-                c_episodes += 1;
-                if (!d) c_trunc += 1;
-              }
-              epc += 1;
-              slot = e * p.S + (int)(epc % p.S);
-              pos = 0;
-              closed = 1;
+            epc += 1;
+            slot = e * p.S + (int)(epc % p.S);
+            pos = 0;
+            closed = 1;
+          }
+        }
+        eid_s[row] = e;
+        close_s[((g + 3) & 3) * ept + row] = closed;  // (as if by the step before the first)
+      }
+      asm volatile("bar.sync 2, 512;" ::: "memory");
+      const int el = rowel_s[row], ai = rowag_s[row];
+      const int e = eid_s[el];
+      int soff[4], poff[4];  // offset of the lane's first column in the tile's observations and in its record (floats)
+      uint32_t uel = 0, ulive = 0;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int r = pw * 32 + 8 * j + (lane >> 2);
+        soff[j] = (rowel_s[r] * n + rowag_s[r]) * D + 4 * c4;
+        poff[j] = rowag_s[r] * D + 4 * c4;
+        uel |= (uint32_t)rowel_s[r] << (8 * j);
+        ulive |= (r < R ? 1u : 0u) << j;
+      }
+
+      // ---- staging: unit `rq` of the group's sequence over (step, unit) goes to slot rq % nu ----
+      int rq_s = 0, rq_k = 0, rq_slot = 0, cv_slot = 0;
+      auto request_unit = [&]() {  // one cp.async group per call, empty at the end
+        if (wlive && rq_s < T) {
+          const int c = (2 * rq_k + grp) * 16 + 4 * c4;  // first column
+          const float* obs = p.obs + (size_t)rq_s * p.obs_step_stride + (size_t)e0 * n * D + (c - 4 * c4);
+          uint8_t* to = units + rq_slot * TS_UNIT;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int r = 8 * j + (lane >> 2);
+            const uint32_t dst = smem_u32(to) + (uint32_t)(r * 64 + ((c4 ^ ((r >> 1) & 3)) * 16));
+            const int left = (ulive >> j) & 1u ? D - c : 0;  // columns there are; the others become zeros
+            const float* src = left > 0 ? obs + soff[j] : p.obs;
+            if (vec) {
+              cp_async16(dst, src, left > 0 ? 16u : 0u);
+            } else {
+#pragma unroll
+              for (int k = 0; k < 4; ++k) cp_async4(dst + 4 * k, left > k ? src + k : p.obs, left > k ? 4u : 0u);
             }
           }
-          eid_s[row] = e;
-          close_s[((g + 3) & 3) * ept + row] = closed;  // (as if by the step before the first)
+          if (++rq_k == nloc) { rq_k = 0; rq_s += 1; }
+          if (++rq_slot == L.nu) rq_slot = 0;
         }
-        asm volatile("bar.sync 2, 512;" ::: "memory");
-        const int el = rowel_s[row], ai = rowag_s[row];
-        const int e = eid_s[el];
-        int soff[4], poff[4];  // offset of the lane's first column in the tile's observations and in its record (floats)
-        uint32_t uel = 0, ulive = 0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int r = pw * 32 + 8 * j + (lane >> 2);
-          soff[j] = (rowel_s[r] * n + rowag_s[r]) * D + 4 * c4;
-          poff[j] = rowag_s[r] * D + 4 * c4;
-          uel |= (uint32_t)rowel_s[r] << (8 * j);
-          ulive |= (r < R ? 1u : 0u) << j;
-        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+      };
+      if (nloc > 0)
+        for (int k = 0; k < L.nu; ++k) request_unit();
 
-        // ---- staging: unit `rq` of the group's sequence over (step, unit) goes to slot rq % nu ----
-        int rq_s = 0, rq_k = 0, rq_slot = 0, cv_slot = 0;
-        auto request_unit = [&]() {  // one cp.async group per call, empty at the end
-          if (wlive && rq_s < T) {
-            const int c = (2 * rq_k + grp) * 16 + 4 * c4;  // first column
-            const float* obs = p.obs + (size_t)rq_s * p.obs_step_stride + (size_t)e0 * n * D + (c - 4 * c4);
-            uint8_t* to = units + rq_slot * TS_UNIT;
+      float reward_next = 0.f;
+      uint32_t done_next = 0;
+      constexpr int AW = NQ == 16 ? 5 : 9;
+      uint32_t aw[AW], ash = 0;
+      // a step's small inputs, requested a step ahead
+      auto request_small = [&](int s) {
+        if (grp == 0 && live) {  // availability row as aligned words (up to three bytes on either side are read and dropped)
+          const uintptr_t a0 = reinterpret_cast<uintptr_t>(p.avail + (size_t)s * p.avail_step_stride + ((size_t)(e0 + el) * n + ai) * A);
+          const uint32_t* wp = reinterpret_cast<const uint32_t*>(a0 & ~(uintptr_t)3);
+          ash = (uint32_t)(a0 & 3u);
+          const uint32_t nw = (ash + (uint32_t)A + 3u) / 4u;
+#pragma unroll
+          for (int k = 0; k < AW; ++k) aw[k] = (uint32_t)k < nw ? __ldg(wp + k) : 0u;
+        }
+        if (grp == 1 && live && 2 * L.nu * 16 < D) {  // first touch of the lines whose units wait for a slot
+          const float* o1 = p.obs + (size_t)s * p.obs_step_stride + ((size_t)(e0 + el) * n + ai) * D;
+          for (int c = 2 * L.nu * 16; c < D; c += 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(o1 + c));
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(o1 + D - 1));
+        }
+        if (cursor && !lag) {
+          reward_next = p.reward[(size_t)s * p.env_step_stride + e0 + row];
+          done_next = p.done[(size_t)s * p.env_step_stride + e0 + row];
+        }
+      };
+      request_small(0);
+      unsigned long long myrec = 0, prevrec = 0;  // records of this thread's row: the step prepared, the one before
+
+      auto prepare = [&](int s, uint32_t gk) {
+        const uint32_t b = gk & 3;
+        if constexpr (grp == 1) {
+          if (cursor) {
+            // ring cursor, headers, reward and done of this step; the cursor needs only the done flags
+            unsigned long long rec = 0;
+            int close = 0;
+            if (eok) {
+              uint8_t* rp = p.ring + (size_t)slot * p.slot_stride + (size_t)pos * rec_bytes;
+              rec = reinterpret_cast<unsigned long long>(rp);
+              const int done = done_next ? 1 : 0;
+              close = (!lag && (done || pos + 1 == p.L)) ? 1 : 0;
+              if (typ == 0) {
+                if (pos == 0) {  // an episode opens in this slot
+                  p.slot_epid[slot] = epc * (long long)p.E + eid_s[row];
+                  p.slot_len[slot] = 0;
+                  p.slot_complete[slot] = 0;
+                }
+                *reinterpret_cast<float*>(rp + p.rl.off_reward) = reward_next;
+                rp[p.rl.off_done] = (uint8_t)done;
+                if (close) {
+                  p.slot_len[slot] = pos + 1;
+                  p.slot_complete[slot] = 1;
+                  c_episodes += 1;
+                  if (!done) c_trunc += 1;
+                }
+              }
+              if (close) {
+                epc += 1;
+                slot = eid_s[row] * p.S + (int)(epc % p.S);
+                pos = 0;
+              } else {
+                pos += 1;
+              }
+            }
+            recp_s[b * ept + row] = rec;
+            close_s[b * ept + row] = close;
+          }
+        } else if (live) {
+          unsigned long long bits = 0;
+#pragma unroll
+          for (int k = 0; k < AW; ++k) {
+            const uint32_t v = aw[k];
+            const uint32_t nz = ((v | ((v & 0x7F7F7F7Fu) + 0x7F7F7F7Fu)) & 0x80808080u) >> 7;  // 0x01 per non-zero byte
+            bits |= (unsigned long long)((nz * 0x01020408u) >> 24 & 0xFu) << (4 * k);
+          }
+          const uint32_t mask = (uint32_t)(bits >> ash) & (A >= 32 ? 0xFFFFFFFFu : ((1u << A) - 1u));
+          const uint32_t t = p.t0 + (uint32_t)s;
+          const int pick = mask ? draw_explore(mask, eps_at(p, t), p.seed, t, (uint32_t)e, (uint32_t)ai) : -1;
+          mask_s[b * TS_ROWS + row] = mask;
+          pick_s[b * TS_ROWS + row] = (int8_t)pick;
+        }
+        asm volatile("bar.sync 3, 256;" ::: "memory");  // the step's records are known
+        ts_arrive(&B->srdy[b], lane);
+        prevrec = myrec;
+        myrec = live ? recp_s[b * ept + el] : 0ull;
+        if (gk > 0) {
+          // the operand has been read by the previous step's fc1 or, where y takes its place, the y operand by the
+          // gate products (barriers with one phase a step)
+          mbar_wait(L.sep ? &B->fc1d : H == 64 ? &B->gd[1] : &B->hr0, (gk - 1) & 1, abortf);
+          tc_fence_after_sync();
+        }
+        if (wlive) {
+#pragma unroll 1
+          for (int ks = grp; ks < nk; ks += 2) {
+            if (L.nu == 1) asm volatile("cp.async.wait_group 0;" ::: "memory");
+            else if (L.nu == 2) asm volatile("cp.async.wait_group 1;" ::: "memory");
+            else asm volatile("cp.async.wait_group 2;" ::: "memory");
+            __syncwarp();
+            const float4* un = reinterpret_cast<const float4*>(units + cv_slot * TS_UNIT);
+            float v[16];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const float4 f = un[lane * 4 + (k ^ ((lane >> 1) & 3))];
+              v[4 * k] = f.x; v[4 * k + 1] = f.y; v[4 * k + 2] = f.z; v[4 * k + 3] = f.w;
+            }
+            ts_split16<NS>(v, [&](int i, const uint32_t (&w)[8]) {
+              if (XS) {
+                uint8_t* to = smem + L.off_xy + (uint32_t)(i * nk + ks) * 4096u + (uint32_t)row * 16u;
+                *reinterpret_cast<uint4*>(to) = make_uint4(w[0], w[1], w[2], w[3]);
+                *reinterpret_cast<uint4*>(to + 2048) = make_uint4(w[4], w[5], w[6], w[7]);
+              } else {
+                tmem_st8(tm + L.tm_x + (uint32_t)(i * nk + ks) * 8u, w);
+              }
+            });
+            const int c = ks * 16 + 4 * c4;
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
+              const unsigned long long rec = (ulive >> j) & 1u ? recp_s[b * ept + ((uel >> (8 * j)) & 0xFFu)] : 0ull;
               const int r = 8 * j + (lane >> 2);
-              const uint32_t dst = smem_u32(to) + (uint32_t)(r * 64 + ((c4 ^ ((r >> 1) & 3)) * 16));
-              const int left = (ulive >> j) & 1u ? D - c : 0;  // columns there are; the others become zeros
-              const float* src = left > 0 ? obs + soff[j] : p.obs;
-              if (vec) {
-                cp_async16(dst, src, left > 0 ? 16u : 0u);
-              } else {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) cp_async4(dst + 4 * k, left > k ? src + k : p.obs, left > k ? 4u : 0u);
-              }
-            }
-            if (++rq_k == nloc) { rq_k = 0; rq_s += 1; }
-            if (++rq_slot == L.nu) rq_slot = 0;
-          }
-          asm volatile("cp.async.commit_group;" ::: "memory");
-        };
-        if (nloc > 0)
-          for (int k = 0; k < L.nu; ++k) request_unit();
-
-        float reward_next = 0.f;
-        uint32_t done_next = 0;
-        constexpr int AW = NQ == 16 ? 5 : 9;
-        uint32_t aw[AW], ash = 0;
-        // a step's small inputs, requested a step ahead
-        auto request_small = [&](int s) {
-          if (grp == 0 && live) {  // availability row as aligned words (up to three bytes on either side are read and dropped)
-            const uintptr_t a0 = reinterpret_cast<uintptr_t>(p.avail + (size_t)s * p.avail_step_stride + ((size_t)(e0 + el) * n + ai) * A);
-            const uint32_t* wp = reinterpret_cast<const uint32_t*>(a0 & ~(uintptr_t)3);
-            ash = (uint32_t)(a0 & 3u);
-            const uint32_t nw = (ash + (uint32_t)A + 3u) / 4u;
-#pragma unroll
-            for (int k = 0; k < AW; ++k) aw[k] = (uint32_t)k < nw ? __ldg(wp + k) : 0u;
-          }
-          if (grp == 1 && live && 2 * L.nu * 16 < D) {  // first touch of the lines whose units wait for a slot
-            const float* o1 = p.obs + (size_t)s * p.obs_step_stride + ((size_t)(e0 + el) * n + ai) * D;
-            for (int c = 2 * L.nu * 16; c < D; c += 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(o1 + c));
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(o1 + D - 1));
-          }
-          if (cursor && !lag) {
-            reward_next = p.reward[(size_t)s * p.env_step_stride + e0 + row];
-            done_next = p.done[(size_t)s * p.env_step_stride + e0 + row];
-          }
-        };
-        request_small(0);
-        unsigned long long myrec = 0, prevrec = 0;  // records of this thread's row: the step prepared, the one before
-
-        auto prepare = [&](int s, uint32_t gk) {
-          const uint32_t b = gk & 3;
-          if constexpr (grp == 1) {
-            if (cursor) {
-              // ring cursor, headers, reward and done of this step; the cursor needs only the done flags
-              unsigned long long rec = 0;
-              int close = 0;
-              if (eok) {
-                uint8_t* rp = p.ring + (size_t)slot * p.slot_stride + (size_t)pos * rec_bytes;
-                rec = reinterpret_cast<unsigned long long>(rp);
-                const int done = done_next ? 1 : 0;
-                close = (!lag && (done || pos + 1 == p.L)) ? 1 : 0;
-                if (typ == 0) {
-                  if (pos == 0) {  // an episode opens in this slot
-                    p.slot_epid[slot] = epc * (long long)p.E + eid_s[row];
-                    p.slot_len[slot] = 0;
-                    p.slot_complete[slot] = 0;
-                  }
-                  *reinterpret_cast<float*>(rp + p.rl.off_reward) = reward_next;
-                  rp[p.rl.off_done] = (uint8_t)done;
-                  if (close) {
-                    p.slot_len[slot] = pos + 1;
-                    p.slot_complete[slot] = 1;
-                    c_episodes += 1;
-                    if (!done) c_trunc += 1;
-                  }
-                }
-                if (close) {
-                  epc += 1;
-                  slot = eid_s[row] * p.S + (int)(epc % p.S);
-                  pos = 0;
+              const float4 f = un[r * 4 + (c4 ^ ((r >> 1) & 3))];
+              if (rec) {
+                float* to = reinterpret_cast<float*>(rec + p.rl.off_obs) + poff[j] + ks * 16;
+                if ((D & 3) == 0) {
+                  if (c < D) *reinterpret_cast<float4*>(to) = f;
                 } else {
-                  pos += 1;
+                  if (c < D) to[0] = f.x;
+                  if (c + 1 < D) to[1] = f.y;
+                  if (c + 2 < D) to[2] = f.z;
+                  if (c + 3 < D) to[3] = f.w;
                 }
               }
-              recp_s[b * ept + row] = rec;
-              close_s[b * ept + row] = close;
             }
-          } else if (live) {
-            unsigned long long bits = 0;
-#pragma unroll
-            for (int k = 0; k < AW; ++k) {
-              const uint32_t v = aw[k];
-              const uint32_t nz = ((v | ((v & 0x7F7F7F7Fu) + 0x7F7F7F7Fu)) & 0x80808080u) >> 7;  // 0x01 per non-zero byte
-              bits |= (unsigned long long)((nz * 0x01020408u) >> 24 & 0xFu) << (4 * k);
-            }
-            const uint32_t mask = (uint32_t)(bits >> ash) & (A >= 32 ? 0xFFFFFFFFu : ((1u << A) - 1u));
-            const uint32_t t = p.t0 + (uint32_t)s;
-            const int pick = mask ? draw_explore(mask, eps_at(p, t), p.seed, t, (uint32_t)e, (uint32_t)ai) : -1;
-            mask_s[b * TS_ROWS + row] = mask;
-            pick_s[b * TS_ROWS + row] = (int8_t)pick;
+            __syncwarp();  // the slot has been read
+            if (++cv_slot == L.nu) cv_slot = 0;
+            request_unit();
           }
-          asm volatile("bar.sync 3, 256;" ::: "memory");  // the step's records are known
-          ts_arrive(&B->srdy[b], lane);
-          prevrec = myrec;
-          myrec = live ? recp_s[b * ept + el] : 0ull;
-          if (gk > 0) {
-            // the operand has been read by the previous step's fc1 or, where y takes its place, the y operand by the
-            // gate products (barriers with one phase a step)
-            mbar_wait(L.sep ? &B->fc1d : H == 64 ? &B->gd[1] : &B->hr0, (gk - 1) & 1, abortf);
-            tc_fence_after_sync();
-          }
-          if (wlive) {
-#pragma unroll 1
-            for (int ks = grp; ks < nk; ks += 2) {
-              if (L.nu == 1) asm volatile("cp.async.wait_group 0;" ::: "memory");
-              else if (L.nu == 2) asm volatile("cp.async.wait_group 1;" ::: "memory");
-              else asm volatile("cp.async.wait_group 2;" ::: "memory");
-              __syncwarp();
-              const float4* un = reinterpret_cast<const float4*>(units + cv_slot * TS_UNIT);
-              float v[16];
+          if (XS) fence_proxy_async_smem();
+          else tmem_st_wait();
+        }
+        tc_fence_before_sync();
+        ts_arrive(&B->xrdy, lane);
+        if (grp == 0 && myrec) {
+          uint8_t* dst = reinterpret_cast<uint8_t*>(myrec + p.rl.off_avail) + ai * A;
 #pragma unroll
-              for (int k = 0; k < 4; ++k) {
-                const float4 f = un[lane * 4 + (k ^ ((lane >> 1) & 3))];
-                v[4 * k] = f.x; v[4 * k + 1] = f.y; v[4 * k + 2] = f.z; v[4 * k + 3] = f.w;
-              }
-              ts_split16<NS>(v, [&](int i, const uint32_t (&w)[8]) {
-                if (XS) {
-                  uint8_t* to = smem + L.off_xy + (uint32_t)(i * nk + ks) * 4096u + (uint32_t)row * 16u;
-                  *reinterpret_cast<uint4*>(to) = make_uint4(w[0], w[1], w[2], w[3]);
-                  *reinterpret_cast<uint4*>(to + 2048) = make_uint4(w[4], w[5], w[6], w[7]);
-                } else {
-                  tmem_st8(tm + L.tm_x + (uint32_t)(i * nk + ks) * 8u, w);
-                }
-              });
-              const int c = ks * 16 + 4 * c4;
+          for (int j = 0; j < NQ / 4; ++j) {
+            const uint32_t v = __funnelshift_r(aw[j], aw[j + 1], 8u * ash);  // bytes 4 j .. 4 j + 3 of the row
 #pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                const unsigned long long rec = (ulive >> j) & 1u ? recp_s[b * ept + ((uel >> (8 * j)) & 0xFFu)] : 0ull;
-                const int r = 8 * j + (lane >> 2);
-                const float4 f = un[r * 4 + (c4 ^ ((r >> 1) & 3))];
-                if (rec) {
-                  float* to = reinterpret_cast<float*>(rec + p.rl.off_obs) + poff[j] + ks * 16;
-                  if ((D & 3) == 0) {
-                    if (c < D) *reinterpret_cast<float4*>(to) = f;
-                  } else {
-                    if (c < D) to[0] = f.x;
-                    if (c + 1 < D) to[1] = f.y;
-                    if (c + 2 < D) to[2] = f.z;
-                    if (c + 3 < D) to[3] = f.w;
-                  }
-                }
-              }
-              __syncwarp();  // the slot has been read
-              if (++cv_slot == L.nu) cv_slot = 0;
-              request_unit();
-            }
-            if (XS) fence_proxy_async_smem();
-            else tmem_st_wait();
-          }
-          tc_fence_before_sync();
-          ts_arrive(&B->xrdy, lane);
-          if (grp == 0 && myrec) {
-            uint8_t* dst = reinterpret_cast<uint8_t*>(myrec + p.rl.off_avail) + ai * A;
-#pragma unroll
-            for (int j = 0; j < NQ / 4; ++j) {
-              const uint32_t v = __funnelshift_r(aw[j], aw[j + 1], 8u * ash);  // bytes 4 j .. 4 j + 3 of the row
-#pragma unroll
-              for (int c = 0; c < 4; ++c)
-                if (4 * j + c < A) dst[4 * j + c] = (uint8_t)(v >> (8 * c));
-            }
-          }
-          if (s + 1 < T) request_small(s + 1);
-        };
-
-        for (int sp = 0; sp <= T; ++sp) {  // prepare step sp, then finish step sp - 1
-          if (sp < T) prepare(sp, g + (uint32_t)sp);
-          else prevrec = myrec;
-          if constexpr (grp == 0) continue;
-          if (sp == 0) {
-            if (fresh) mbar_wait(&B->res[0], (uint32_t)typ & 1, abortf);  // the output biases are in place
-            continue;
-          }
-          const int s = sp - 1;
-          mbar_wait(&B->fc2d, (g + (uint32_t)s) & 1, abortf);
-          tc_fence_after_sync();
-          if (wlive) {
-            uint32_t qv[NQ];
-            tmem_ld16(tm + L.tm_q, *reinterpret_cast<uint32_t(*)[16]>(qv));
-            if (NQ == 32) tmem_ld16(tm + L.tm_q + 16, *reinterpret_cast<uint32_t(*)[16]>(qv + NQ - 16));
-            tmem_ld_wait();
-            tc_fence_before_sync();
-            ts_arrive(&B->qfree, lane);
-            if (prevrec) {
-              float* qrow = reinterpret_cast<float*>(prevrec + p.rl.off_q) + ai * A;
-              if ((A & 1) == 0) {  // rows of an even number of floats start on 8-byte boundaries
-#pragma unroll
-                for (int a = 0; a < NQ; a += 2)
-                  if (a < A) *reinterpret_cast<float2*>(qrow + a) = make_float2(__uint_as_float(qv[a]) + b2_s[a], __uint_as_float(qv[a + 1]) + b2_s[a + 1]);
-              } else {
-#pragma unroll
-                for (int a = 0; a < NQ; ++a)
-                  if (a < A) qrow[a] = __uint_as_float(qv[a]) + b2_s[a];
-              }
-            }
-            const int tk = p.trace_first + s;
-            if (live && tk < p.trace_cap && p.trace_q) {
-              float* tq = p.trace_q + (((size_t)tk * p.E + e) * n + ai) * A;
-#pragma unroll
-              for (int a = 0; a < NQ; ++a)
-                if (a < A) tq[a] = __uint_as_float(qv[a]) + b2_s[a];
-            }
-          } else {
-            ts_arrive(&B->qfree, lane);
+            for (int c = 0; c < 4; ++c)
+              if (4 * j + c < A) dst[4 * j + c] = (uint8_t)(v >> (8 * c));
           }
         }
-        g += (uint32_t)T;
-        if (cursor && eok && typ == ntypes - 1) {
-          const int ee = eid_s[row];
+        if (s + 1 < T) request_small(s + 1);
+      };
+
+      for (int sp = 0; sp <= T; ++sp) {  // prepare step sp, then finish step sp - 1
+        if (sp < T) prepare(sp, g + (uint32_t)sp);
+        else prevrec = myrec;
+        if constexpr (grp == 0) continue;
+        if (sp == 0) {
+          if (fresh) mbar_wait(&B->res[0], (loads - 1) & 1, abortf);  // the output biases are in place
+          continue;
+        }
+        const int s = sp - 1;
+        mbar_wait(&B->fc2d, (g + (uint32_t)s) & 1, abortf);
+        tc_fence_after_sync();
+        if (wlive) {
+          uint32_t qv[NQ];
+          tmem_ld16(tm + L.tm_q, *reinterpret_cast<uint32_t(*)[16]>(qv));
+          if (NQ == 32) tmem_ld16(tm + L.tm_q + 16, *reinterpret_cast<uint32_t(*)[16]>(qv + NQ - 16));
+          tmem_ld_wait();
+          tc_fence_before_sync();
+          ts_arrive(&B->qfree, lane);
+          if (prevrec) {
+            float* qrow = reinterpret_cast<float*>(prevrec + p.rl.off_q) + ai * A;
+            if ((A & 1) == 0) {  // rows of an even number of floats start on 8-byte boundaries
+#pragma unroll
+              for (int a = 0; a < NQ; a += 2)
+                if (a < A) *reinterpret_cast<float2*>(qrow + a) = make_float2(__uint_as_float(qv[a]) + b2_s[a], __uint_as_float(qv[a + 1]) + b2_s[a + 1]);
+            } else {
+#pragma unroll
+              for (int a = 0; a < NQ; ++a)
+                if (a < A) qrow[a] = __uint_as_float(qv[a]) + b2_s[a];
+            }
+          }
+          const int tk = p.trace_first + s;
+          if (live && tk < p.trace_cap && p.trace_q) {
+            float* tq = p.trace_q + (((size_t)tk * p.E + e) * n + ai) * A;
+#pragma unroll
+            for (int a = 0; a < NQ; ++a)
+              if (a < A) tq[a] = __uint_as_float(qv[a]) + b2_s[a];
+          }
+        } else {
+          ts_arrive(&B->qfree, lane);
+        }
+      }
+      g += (uint32_t)T;
+      if (cursor && eok) {
+        const int ee = eid_s[row];
+        if (typ == 0 && pos > 0) p.slot_len[slot] = pos;
+        // The types' tiles of an environment run in any order, on any block: the last one to finish writes the
+        // cursor (all have read it by then, and all have come to the same one).
+        bool last = true;
+        if (ntypes > 1) {
+          __threadfence();
+          last = atomicAdd(p.type_count + ee, 1) == ntypes - 1;
+          if (last) p.type_count[ee] = 0;
+        }
+        if (last) {
           p.slot[ee] = slot;
           p.pos[ee] = pos;
           p.ep_count[ee] = epc;
-          if (pos > 0) p.slot_len[slot] = pos;
         }
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        fresh = false;
       }
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      fresh = false;
     }
     if constexpr (grp == 0) grid_release();  // the last step's inputs are in place
     if (c_episodes) atomicAdd(p.counters + CNT_EPISODES, (unsigned long long)c_episodes);
@@ -1116,255 +1145,258 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
     const int row = tid & 127, grp = warp >> 2;
     const uint32_t tm = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     unsigned long long c_steps = 0, c_explore = 0, c_noavail = 0;
-    uint32_t st_bits = 0, g = 0;
-    for (int typ = 0; typ < ntypes; ++typ) {
-      if (typ > 0) __syncthreads();
-      const int nt = rows_per_env(typ);
-      bool fresh = true;
-      for (int tile = blockIdx.x; tile < p.num_tiles; tile += gridDim.x) {
-        const int e0 = tile * ept;
-        const int R = min(ept, p.M - e0) * nt;
-        const bool wlive = (warp & 3) * 32 < R;   // warps without a live row only keep the barriers going
-        const bool live = row < R;
-        asm volatile("bar.sync 2, 512;" ::: "memory");  // the previous tile's shared arrays are done with
-        if (grp == 0) {
-          // row -> (environment, agent): the agents of this pass' unit type, in rising order
-          uint8_t el = 0, ag = 0;
-          if (live) {
-            el = (uint8_t)(row / nt);
-            int k = row - el * nt, i = k;
-            if (ntypes > 1)
-              for (i = 0; i < n; ++i)
-                if ((int)((p.agent_type_bits >> (2 * i)) & 3ull) == typ && k-- == 0) break;
-            ag = (uint8_t)i;
-          }
-          rowel_s[row] = el;
-          rowag_s[row] = ag;
+    uint32_t st_bits = 0, g = 0, loads = 0;
+    int nt = 0;
+    bool fresh = true;
+    for (int tile = blockIdx.x, typ = 0, cur = -1; unit_at(tile, typ); tile += gridDim.x) {
+      if (typ != cur) {
+        cur = typ;
+        nt = rows_per_env(typ);
+        fresh = true;
+        if (loads++ > 0) __syncthreads();
+      }
+      const int e0 = tile * ept;
+      const int R = min(ept, p.M - e0) * nt;
+      const bool wlive = (warp & 3) * 32 < R;   // warps without a live row only keep the barriers going
+      const bool live = row < R;
+      asm volatile("bar.sync 2, 512;" ::: "memory");  // the previous tile's shared arrays are done with
+      if (grp == 0) {
+        // row -> (environment, agent): the agents of this pass' unit type, in rising order
+        uint8_t el = 0, ag = 0;
+        if (live) {
+          el = (uint8_t)(row / nt);
+          int k = row - el * nt, i = k;
+          if (ntypes > 1)
+            for (i = 0; i < n; ++i)
+              if ((int)((p.agent_type_bits >> (2 * i)) & 3ull) == typ && k-- == 0) break;
+          ag = (uint8_t)i;
         }
-        asm volatile("bar.sync 2, 512;" ::: "memory");
-        const int el = rowel_s[row], ai = rowag_s[row];
-        const int e = eid_s[el];
-        const size_t grow = (size_t)e * n + ai;
-        float h[NBLK][16];
-        auto store_h = [&](int b, const float (&hb)[16]) {  // the pieces of block b's hidden state
-          float v[16];
+        rowel_s[row] = el;
+        rowag_s[row] = ag;
+      }
+      asm volatile("bar.sync 2, 512;" ::: "memory");
+      const int el = rowel_s[row], ai = rowag_s[row];
+      const int e = eid_s[el];
+      const size_t grow = (size_t)e * n + ai;
+      float h[NBLK][16];
+      auto store_h = [&](int b, const float (&hb)[16]) {  // the pieces of block b's hidden state
+        float v[16];
 #pragma unroll
-          for (int j = 0; j < 16; ++j) v[j] = hb[j];
-          ts_split16<NS>(v, [&](int i, const uint32_t (&w)[8]) {
-            tmem_st8(tm + TSM_HOP + (uint32_t)(i * (H / 2) + b * (TS_BLK / 2) + grp * 8), w);
-          });
-        };
-        {
-          const bool carry = live && !close_s[((g + 3) & 3) * ept + el];  // the row continues an episode
+        for (int j = 0; j < 16; ++j) v[j] = hb[j];
+        ts_split16<NS>(v, [&](int i, const uint32_t (&w)[8]) {
+          tmem_st8(tm + TSM_HOP + (uint32_t)(i * (H / 2) + b * (TS_BLK / 2) + grp * 8), w);
+        });
+      };
+      {
+        const bool carry = live && !close_s[((g + 3) & 3) * ept + el];  // the row continues an episode
 #pragma unroll
+        for (int b = 0; b < NBLK; ++b) {
+          const float4* src = reinterpret_cast<const float4*>(p.h + grow * H + b * TS_BLK + grp * 16);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float4 v = carry ? src[k] : make_float4(0.f, 0.f, 0.f, 0.f);
+            h[b][4 * k] = v.x; h[b][4 * k + 1] = v.y; h[b][4 * k + 2] = v.z; h[b][4 * k + 3] = v.w;
+          }
+        }
+        if (grp == 0) {
+          int la = carry ? p.last_action[grow] : -1;
+          if (la >= A) la = -1;
+          la_s[row] = la;
+        }
+        if (wlive) {
+#pragma unroll
+          for (int b = 0; b < NBLK; ++b) store_h(b, h[b]);
+          tmem_st_wait();
+        }
+        tc_fence_before_sync();
+        ts_arrive(&B->hset, lane);
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        if (fresh) mbar_wait(&B->res[0], (loads - 1) & 1, abortf);  // tables and biases are in place
+      }
+      const float* ta = reinterpret_cast<const float*>(smem + L.off_tabA) + ai * (H + 4) + grp * 16;
+      const float* tl0 = reinterpret_cast<const float*>(smem + L.off_tabL) + grp * 16;
+
+      for (int s = 0; s < T; ++s, ++g) {
+        const uint32_t par = g & 1u, b4 = g & 3u;
+        // ---- E1 ----
+        mbar_wait(&B->fc1d, par, abortf);
+        tc_fence_after_sync();
+        if (wlive) {
+          const int last = la_s[row];
+          const float* tl = tl0 + (last >= 0 ? last : 0) * (H + 4);
+#pragma unroll UB
           for (int b = 0; b < NBLK; ++b) {
-            const float4* src = reinterpret_cast<const float4*>(p.h + grow * H + b * TS_BLK + grp * 16);
+            uint32_t a[16];
+            tmem_ld16(tm + FC1 + (uint32_t)(b * TS_BLK + grp * 16), a);
+            float y[16];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              const float4 v = carry ? src[k] : make_float4(0.f, 0.f, 0.f, 0.f);
-              h[b][4 * k] = v.x; h[b][4 * k + 1] = v.y; h[b][4 * k + 2] = v.z; h[b][4 * k + 3] = v.w;
+              const float4 va = *reinterpret_cast<const float4*>(ta + b * TS_BLK + 4 * k);
+              float4 vl = *reinterpret_cast<const float4*>(tl + b * TS_BLK + 4 * k);
+              if (last < 0) vl = make_float4(0.f, 0.f, 0.f, 0.f);
+              y[4 * k] = va.x + vl.x; y[4 * k + 1] = va.y + vl.y; y[4 * k + 2] = va.z + vl.z; y[4 * k + 3] = va.w + vl.w;
             }
-          }
-          if (grp == 0) {
-            int la = carry ? p.last_action[grow] : -1;
-            if (la >= A) la = -1;
-            la_s[row] = la;
-          }
-          if (wlive) {
-#pragma unroll
-            for (int b = 0; b < NBLK; ++b) store_h(b, h[b]);
-            tmem_st_wait();
-          }
-          tc_fence_before_sync();
-          ts_arrive(&B->hset, lane);
-          asm volatile("bar.sync 1, 256;" ::: "memory");
-          if (fresh) mbar_wait(&B->res[0], (uint32_t)typ & 1, abortf);  // tables and biases are in place
-        }
-        const float* ta = reinterpret_cast<const float*>(smem + L.off_tabA) + ai * (H + 4) + grp * 16;
-        const float* tl0 = reinterpret_cast<const float*>(smem + L.off_tabL) + grp * 16;
-
-        for (int s = 0; s < T; ++s, ++g) {
-          const uint32_t par = g & 1u, b4 = g & 3u;
-          // ---- E1 ----
-          mbar_wait(&B->fc1d, par, abortf);
-          tc_fence_after_sync();
-          if (wlive) {
-            const int last = la_s[row];
-            const float* tl = tl0 + (last >= 0 ? last : 0) * (H + 4);
-#pragma unroll UB
-            for (int b = 0; b < NBLK; ++b) {
-              uint32_t a[16];
-              tmem_ld16(tm + FC1 + (uint32_t)(b * TS_BLK + grp * 16), a);
-              float y[16];
-#pragma unroll
-              for (int k = 0; k < 4; ++k) {
-                const float4 va = *reinterpret_cast<const float4*>(ta + b * TS_BLK + 4 * k);
-                float4 vl = *reinterpret_cast<const float4*>(tl + b * TS_BLK + 4 * k);
-                if (last < 0) vl = make_float4(0.f, 0.f, 0.f, 0.f);
-                y[4 * k] = va.x + vl.x; y[4 * k + 1] = va.y + vl.y; y[4 * k + 2] = va.z + vl.z; y[4 * k + 3] = va.w + vl.w;
-              }
-              tmem_ld_wait();
-#pragma unroll
-              for (int k = 0; k < 16; ++k) y[k] = fmaxf(__uint_as_float(a[k]) + y[k], 0.f);
-              ts_split16<NS>(y, [&](int i, const uint32_t (&w)[8]) {
-                const int k8 = b * (TS_BLK / 8) + grp * 2;  // first 8-column group
-                if (XS) {
-                  uint8_t* to = smem + L.off_xy + (uint32_t)(i * (H / 8) + k8) * 2048u + (uint32_t)row * 16u;
-                  *reinterpret_cast<uint4*>(to) = make_uint4(w[0], w[1], w[2], w[3]);
-                  *reinterpret_cast<uint4*>(to + 2048) = make_uint4(w[4], w[5], w[6], w[7]);
-                } else {
-                  tmem_st8(tm + TSM_Y + (uint32_t)(i * (H / 2) + k8 * 4), w);
-                }
-              });
-            }
-            if (XS) fence_proxy_async_smem();
-            else tmem_st_wait();
-          }
-          tc_fence_before_sync();
-          ts_arrive(&B->yrdy, lane);
-
-          // ---- E2 ----
-          // one block of 32 hidden columns per pass; the block at work is h[0], the others move up behind it
-#pragma unroll UB
-          for (int b = 0; b < NBLK; ++b) {
-            const int buf = H == 64 ? b : (b + 1) & 1;
-            mbar_wait(&B->gd[buf], H == 64 ? par : (uint32_t)(b >> 1), abortf);
-            tc_fence_after_sync();
-            if (b == NBLK - 1) {  // no product reads the old hidden state any more
-              if (wlive) {
-#pragma unroll
-                for (int k = 0; k < NBLK - 1; ++k) store_h(k, h[k + 1]);
-                tmem_st_wait();
-              }
-              tc_fence_before_sync();
-              ts_arrive(&B->hr0, lane);
-            }
-            if (wlive) {
-              // columns of the buffer: HN R Z IN | IN R Z HN
-              const uint32_t base = tm + (buf ? 128u : 0u) + (uint32_t)grp * 16u;
-              const uint32_t c_in = buf ? 0u : 96u, c_hn = buf ? 96u : 0u;
-#pragma unroll
-              for (int c8 = 0; c8 < 2; ++c8) {
-                uint32_t v[4][8];
-                tmem_ld8(base + 32u + c8 * 8, v[0]);
-                tmem_ld8(base + 64u + c8 * 8, v[1]);
-                tmem_ld8(base + c_in + c8 * 8, v[2]);
-                tmem_ld8(base + c_hn + c8 * 8, v[3]);
-                tmem_ld_wait();
-                if (H == 128 && c8 == 1 && b < NBLK - 2) {
-                  tc_fence_before_sync();
-                  ts_arrive(&B->accf[buf], lane);
-                }
-                const float* bb = bias_s + b * TS_BLK + grp * 16 + c8 * 8;
-#pragma unroll
-                for (int j = 0; j < 8; j += 4) {
-                  ulonglong2 bv[4];  // biases of four columns
-#pragma unroll
-                  for (int k = 0; k < 4; ++k) bv[k] = *reinterpret_cast<const ulonglong2*>(bb + (FAST && k < 2 ? k + 4 : k) * H + j);
-#pragma unroll
-                  for (int c = 0; c < 4; c += 2) {
-                    float a[4][2];
-                    ts_f2 b2[4];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                      a[k][0] = __uint_as_float(v[k][j + c]);
-                      a[k][1] = __uint_as_float(v[k][j + c + 1]);
-                      b2[k] = c == 0 ? bv[k].x : bv[k].y;
-                    }
-                    if constexpr (FAST) ts_gates2_fast(a, b2, h[0][c8 * 8 + j + c], h[0][c8 * 8 + j + c + 1]);
-                    else ts_gates2(a, b2, h[0][c8 * 8 + j + c], h[0][c8 * 8 + j + c + 1]);
-                  }
-                }
-              }
-            } else if (H == 128 && b < NBLK - 2) {
-              ts_arrive(&B->accf[buf], lane);
-            }
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const float x = h[0][j];
-#pragma unroll
-              for (int k = 0; k + 1 < NBLK; ++k) h[k][j] = h[k + 1][j];
-              h[NBLK - 1][j] = x;
-            }
-          }
-          if (wlive) {
-            store_h(NBLK - 1, h[NBLK - 1]);
-            tmem_st_wait();
-          }
-          tc_fence_before_sync();
-          ts_arrive(&B->hr1, lane);
-
-          // ---- E3 ----
-          mbar_wait(&B->srdy[b4], (g >> 2) & 1u, abortf);  // the step's records and draws
-          const bool close = live && close_s[b4 * ept + el];
-          mbar_wait(&B->fc2d, par, abortf);
-          tc_fence_after_sync();
-          uint32_t qv[NQ];
-          if (grp == 0 && wlive) {
-            tmem_ld16(tm + L.tm_q, *reinterpret_cast<uint32_t(*)[16]>(qv));
-            if (NQ == 32) tmem_ld16(tm + L.tm_q + 16, *reinterpret_cast<uint32_t(*)[16]>(qv + NQ - 16));
             tmem_ld_wait();
+#pragma unroll
+            for (int k = 0; k < 16; ++k) y[k] = fmaxf(__uint_as_float(a[k]) + y[k], 0.f);
+            ts_split16<NS>(y, [&](int i, const uint32_t (&w)[8]) {
+              const int k8 = b * (TS_BLK / 8) + grp * 2;  // first 8-column group
+              if (XS) {
+                uint8_t* to = smem + L.off_xy + (uint32_t)(i * (H / 8) + k8) * 2048u + (uint32_t)row * 16u;
+                *reinterpret_cast<uint4*>(to) = make_uint4(w[0], w[1], w[2], w[3]);
+                *reinterpret_cast<uint4*>(to + 2048) = make_uint4(w[4], w[5], w[6], w[7]);
+              } else {
+                tmem_st8(tm + TSM_Y + (uint32_t)(i * (H / 2) + k8 * 4), w);
+              }
+            });
           }
-          // a closed episode restarts from a zero hidden state and no last action
-          if (wlive && __builtin_expect(__any_sync(0xFFFFFFFFu, close), 0)) {
-            if (close) {
+          if (XS) fence_proxy_async_smem();
+          else tmem_st_wait();
+        }
+        tc_fence_before_sync();
+        ts_arrive(&B->yrdy, lane);
+
+        // ---- E2 ----
+        // one block of 32 hidden columns per pass; the block at work is h[0], the others move up behind it
+#pragma unroll UB
+        for (int b = 0; b < NBLK; ++b) {
+          const int buf = H == 64 ? b : (b + 1) & 1;
+          mbar_wait(&B->gd[buf], H == 64 ? par : (uint32_t)(b >> 1), abortf);
+          tc_fence_after_sync();
+          if (b == NBLK - 1) {  // no product reads the old hidden state any more
+            if (wlive) {
 #pragma unroll
-              for (int b = 0; b < NBLK; ++b)
-#pragma unroll
-                for (int j = 0; j < 16; ++j) h[b][j] = 0.f;
+              for (int k = 0; k < NBLK - 1; ++k) store_h(k, h[k + 1]);
+              tmem_st_wait();
             }
-#pragma unroll
-            for (int b = 0; b < NBLK; ++b) store_h(b, h[b]);
-            tmem_st_wait();
+            tc_fence_before_sync();
+            ts_arrive(&B->hr0, lane);
           }
-          tc_fence_before_sync();
-          if (s + 1 < T) ts_arrive(&B->hset, lane);
-          int act = 0;
-          if (grp == 0 && live) {
-            const uint32_t mask = mask_s[b4 * TS_ROWS + row];
-            const int pick = pick_s[b4 * TS_ROWS + row];
-            // greedy rule: m = max over available, thr = m - 1e-4f, lowest available a with Q >= thr (a NaN never
-            // compares greater or equal and fmaxf ignores it)
-            float qf[NQ];
-            float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+          if (wlive) {
+            // columns of the buffer: HN R Z IN | IN R Z HN
+            const uint32_t base = tm + (buf ? 128u : 0u) + (uint32_t)grp * 16u;
+            const uint32_t c_in = buf ? 0u : 96u, c_hn = buf ? 96u : 0u;
 #pragma unroll
-            for (int a = 0; a < NQ; ++a) {
-              qf[a] = __uint_as_float(qv[a]) + b2_s[a];
-              m4[a & 3] = fmaxf(m4[a & 3], ((mask >> a) & 1u) ? qf[a] : -INFINITY);
+            for (int c8 = 0; c8 < 2; ++c8) {
+              uint32_t v[4][8];
+              tmem_ld8(base + 32u + c8 * 8, v[0]);
+              tmem_ld8(base + 64u + c8 * 8, v[1]);
+              tmem_ld8(base + c_in + c8 * 8, v[2]);
+              tmem_ld8(base + c_hn + c8 * 8, v[3]);
+              tmem_ld_wait();
+              if (H == 128 && c8 == 1 && b < NBLK - 2) {
+                tc_fence_before_sync();
+                ts_arrive(&B->accf[buf], lane);
+              }
+              const float* bb = bias_s + b * TS_BLK + grp * 16 + c8 * 8;
+#pragma unroll
+              for (int j = 0; j < 8; j += 4) {
+                ulonglong2 bv[4];  // biases of four columns
+#pragma unroll
+                for (int k = 0; k < 4; ++k) bv[k] = *reinterpret_cast<const ulonglong2*>(bb + (FAST && k < 2 ? k + 4 : k) * H + j);
+#pragma unroll
+                for (int c = 0; c < 4; c += 2) {
+                  float a[4][2];
+                  ts_f2 b2[4];
+#pragma unroll
+                  for (int k = 0; k < 4; ++k) {
+                    a[k][0] = __uint_as_float(v[k][j + c]);
+                    a[k][1] = __uint_as_float(v[k][j + c + 1]);
+                    b2[k] = c == 0 ? bv[k].x : bv[k].y;
+                  }
+                  if constexpr (FAST) ts_gates2_fast(a, b2, h[0][c8 * 8 + j + c], h[0][c8 * 8 + j + c + 1]);
+                  else ts_gates2(a, b2, h[0][c8 * 8 + j + c], h[0][c8 * 8 + j + c + 1]);
+                }
+              }
             }
-            const float thr = __fsub_rn(fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])), 1e-4f);
-            uint32_t ge = 0;
-#pragma unroll
-            for (int a = 0; a < NQ; ++a) ge |= (qf[a] >= thr ? 1u : 0u) << a;
-            ge &= mask;
-            const int greedy = ge ? __ffs(ge) - 1 : __ffs(mask) - 1;
-            act = mask == 0 ? 0 : (pick >= 0 ? pick : greedy);
-            la_s[row] = close ? -1 : act;
-            c_steps += 1;
-            c_explore += pick >= 0 ? 1u : 0u;
-            if (mask == 0) { c_noavail += 1; st_bits |= MARL_STATUS_NO_AVAIL; }
+          } else if (H == 128 && b < NBLK - 2) {
+            ts_arrive(&B->accf[buf], lane);
           }
-          asm volatile("bar.sync 1, 256;" ::: "memory");  // last actions are in place
-          if (grp == 0 && live) {
-            const unsigned long long rec = recp_s[b4 * ept + el];
-            if (rec) reinterpret_cast<int32_t*>(rec + p.rl.off_action)[ai] = act;
-            const int tk = p.trace_first + s;
-            if (tk < p.trace_cap && p.trace_actions) p.trace_actions[((size_t)tk * p.E + e) * n + ai] = act;
-            if (p.actions_out && s == T - 1) p.actions_out[(size_t)(e0 + el) * n + ai] = act;
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const float x = h[0][j];
+#pragma unroll
+            for (int k = 0; k + 1 < NBLK; ++k) h[k][j] = h[k + 1][j];
+            h[NBLK - 1][j] = x;
           }
         }
-        // ---- end of the tile: state back to global memory ----
-        if (live) {
-#pragma unroll
-          for (int b = 0; b < NBLK; ++b) {
-            float4* dst = reinterpret_cast<float4*>(p.h + grow * H + b * TS_BLK + grp * 16);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) dst[k] = make_float4(h[b][4 * k], h[b][4 * k + 1], h[b][4 * k + 2], h[b][4 * k + 3]);
-          }
-          if (grp == 0) p.last_action[grow] = la_s[row];
+        if (wlive) {
+          store_h(NBLK - 1, h[NBLK - 1]);
+          tmem_st_wait();
         }
-        fresh = false;
+        tc_fence_before_sync();
+        ts_arrive(&B->hr1, lane);
+
+        // ---- E3 ----
+        mbar_wait(&B->srdy[b4], (g >> 2) & 1u, abortf);  // the step's records and draws
+        const bool close = live && close_s[b4 * ept + el];
+        mbar_wait(&B->fc2d, par, abortf);
+        tc_fence_after_sync();
+        uint32_t qv[NQ];
+        if (grp == 0 && wlive) {
+          tmem_ld16(tm + L.tm_q, *reinterpret_cast<uint32_t(*)[16]>(qv));
+          if (NQ == 32) tmem_ld16(tm + L.tm_q + 16, *reinterpret_cast<uint32_t(*)[16]>(qv + NQ - 16));
+          tmem_ld_wait();
+        }
+        // a closed episode restarts from a zero hidden state and no last action
+        if (wlive && __builtin_expect(__any_sync(0xFFFFFFFFu, close), 0)) {
+          if (close) {
+#pragma unroll
+            for (int b = 0; b < NBLK; ++b)
+#pragma unroll
+              for (int j = 0; j < 16; ++j) h[b][j] = 0.f;
+          }
+#pragma unroll
+          for (int b = 0; b < NBLK; ++b) store_h(b, h[b]);
+          tmem_st_wait();
+        }
+        tc_fence_before_sync();
+        if (s + 1 < T) ts_arrive(&B->hset, lane);
+        int act = 0;
+        if (grp == 0 && live) {
+          const uint32_t mask = mask_s[b4 * TS_ROWS + row];
+          const int pick = pick_s[b4 * TS_ROWS + row];
+          // greedy rule: m = max over available, thr = m - 1e-4f, lowest available a with Q >= thr (a NaN never
+          // compares greater or equal and fmaxf ignores it)
+          float qf[NQ];
+          float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+          for (int a = 0; a < NQ; ++a) {
+            qf[a] = __uint_as_float(qv[a]) + b2_s[a];
+            m4[a & 3] = fmaxf(m4[a & 3], ((mask >> a) & 1u) ? qf[a] : -INFINITY);
+          }
+          const float thr = __fsub_rn(fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])), 1e-4f);
+          uint32_t ge = 0;
+#pragma unroll
+          for (int a = 0; a < NQ; ++a) ge |= (qf[a] >= thr ? 1u : 0u) << a;
+          ge &= mask;
+          const int greedy = ge ? __ffs(ge) - 1 : __ffs(mask) - 1;
+          act = mask == 0 ? 0 : (pick >= 0 ? pick : greedy);
+          la_s[row] = close ? -1 : act;
+          c_steps += 1;
+          c_explore += pick >= 0 ? 1u : 0u;
+          if (mask == 0) { c_noavail += 1; st_bits |= MARL_STATUS_NO_AVAIL; }
+        }
+        asm volatile("bar.sync 1, 256;" ::: "memory");  // last actions are in place
+        if (grp == 0 && live) {
+          const unsigned long long rec = recp_s[b4 * ept + el];
+          if (rec) reinterpret_cast<int32_t*>(rec + p.rl.off_action)[ai] = act;
+          const int tk = p.trace_first + s;
+          if (tk < p.trace_cap && p.trace_actions) p.trace_actions[((size_t)tk * p.E + e) * n + ai] = act;
+          if (p.actions_out && s == T - 1) p.actions_out[(size_t)(e0 + el) * n + ai] = act;
+        }
       }
+      // ---- end of the tile: state back to global memory ----
+      if (live) {
+#pragma unroll
+        for (int b = 0; b < NBLK; ++b) {
+          float4* dst = reinterpret_cast<float4*>(p.h + grow * H + b * TS_BLK + grp * 16);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) dst[k] = make_float4(h[b][4 * k], h[b][4 * k + 1], h[b][4 * k + 2], h[b][4 * k + 3]);
+        }
+        if (grp == 0) p.last_action[grow] = la_s[row];
+      }
+      fresh = false;
     }
     if (c_steps) atomicAdd(p.counters + CNT_AGENT_STEPS, c_steps);
     if (c_explore) atomicAdd(p.counters + CNT_EXPLORED, c_explore);
@@ -1394,8 +1426,7 @@ int launch_actor_tcs(const ActorParams& p_in, int sms, bool fast_gates, cudaStre
     }
   }
   const int ns = ts_pieces(p.prec);
-  TsLayout L = ts_layout(p.n, p.D, p.A, p.H, ns, nt_max, p.M, sms);
-  L.ntypes = ntypes;
+  TsLayout L = ts_layout(p.n, p.D, p.A, p.H, ns, nt_max, p.M, sms, ntypes);
   if (p.H == 128 && !fast_gates) {
     // the accurate gates keep the epilogue so busy that input warps running beside it all step long cost more than the
     // wait for the shared columns (1216 against 1246 us for 4096 x 5 agents x 64 steps; fast gates, 16384 x 8 agents: 3940 against 3410;
@@ -1415,7 +1446,7 @@ int launch_actor_tcs(const ActorParams& p_in, int sms, bool fast_gates, cudaStre
     const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernels[v]), L.total, configured[v]);
     if (e != cudaSuccess) return -(int)e;
   }
-  int grid = p.num_tiles < sms ? p.num_tiles : sms;
+  int grid = p.num_tiles * ntypes < sms ? p.num_tiles * ntypes : sms;
   if (grid < 1) grid = 1;
   const cudaError_t err = launch_overlapped(kernels[v], grid, TS_THREADS, L.total, stream, p.early != 0, p, L);
   return err == cudaSuccess ? 1 : -(int)err;

@@ -77,6 +77,7 @@ struct ActorParams {
   int32_t n_types;
   uint32_t type_stride;
   uint64_t agent_type_bits;
+  int32_t* type_count;      // [E] types of an environment that are done with the launch (split-operand kernel, zero between launches)
   int32_t early;            // host only: the launch may start beside the kernel before it (see launch_overlapped)
 };
 

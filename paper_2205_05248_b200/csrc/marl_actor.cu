@@ -96,7 +96,7 @@ static FfmaWeightOffsets ffma_weight_offsets(int n, int D, int A, int H) {
 // two weight images, each: per-type images of the general kernel (split-operand or FFMA), then the tensor-core image
 constexpr int ID_LISTS = 3;  // environment lists on their way to partial steps; one more device list for captured steps
 
-struct StateOffsets { size_t h, last_action, slot, pos, ep_count, counters, status, wgen[2], wpack[2], ids[ID_LISTS + 1], total; };
+struct StateOffsets { size_t h, last_action, slot, pos, ep_count, counters, status, wgen[2], wpack[2], ids[ID_LISTS + 1], type_count, total; };
 struct RingOffsets { size_t records, epid, len, complete, total; };
 struct WorkOffsets { size_t obs, avail, reward, done, actions, total; };
 
@@ -149,6 +149,7 @@ static StateOffsets state_offsets(const marl_actor_config_t& c) {
     s.wpack[i] = cv.take(tc_wpack_bytes(c.n_agents, c.obs_dim, c.n_actions, c.hidden));
   }
   for (size_t& ids : s.ids) ids = cv.take(sizeof(int32_t) * (size_t)c.n_envs);  // environment lists of partial steps
+  s.type_count = cv.take(types > 1 ? sizeof(int32_t) * (size_t)c.n_envs : 0);
   s.total = cv.off;
   return s;
 }
@@ -246,7 +247,8 @@ struct marl_actor {
 
 __global__ void init_state_kernel(int E, int n, int H, int S, int C, float* h, int32_t* la, int32_t* slot,
                                   int32_t* pos, long long* epc, long long* epid, int32_t* len,
-                                  uint8_t* complete, unsigned long long* counters, uint32_t* status) {
+                                  uint8_t* complete, unsigned long long* counters, uint32_t* status,
+                                  int32_t* type_count) {
   const long long rows = (long long)E * n;
   const long long stride = (long long)gridDim.x * blockDim.x;
   const long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -256,6 +258,7 @@ __global__ void init_state_kernel(int E, int n, int H, int S, int C, float* h, i
     slot[i] = (int32_t)(i * S);
     pos[i] = 0;
     epc[i] = 0;
+    if (type_count) type_count[i] = 0;
   }
   for (long long i = i0; i < C; i += stride) {
     epid[i] = -1;
@@ -275,7 +278,8 @@ static int enqueue_reset(marl_actor* a) {
       reinterpret_cast<int32_t*>(st + a->so.slot), reinterpret_cast<int32_t*>(st + a->so.pos),
       reinterpret_cast<long long*>(st + a->so.ep_count), reinterpret_cast<long long*>(a->ring + a->ro.epid),
       reinterpret_cast<int32_t*>(a->ring + a->ro.len), a->ring + a->ro.complete,
-      reinterpret_cast<unsigned long long*>(st + a->so.counters), reinterpret_cast<uint32_t*>(st + a->so.status));
+      reinterpret_cast<unsigned long long*>(st + a->so.counters), reinterpret_cast<uint32_t*>(st + a->so.status),
+      c.n_agent_types > 1 ? reinterpret_cast<int32_t*>(st + a->so.type_count) : nullptr);
   CU_TRY(cudaGetLastError());
   a->launches += 1;
   a->step = 0;
@@ -667,6 +671,7 @@ static void fill_params(marl_actor* a, ActorParams& p) {
   p.n_types = a->n_types;
   p.type_stride = (uint32_t)(a->wo.total / sizeof(float));
   p.agent_type_bits = a->agent_type_bits;
+  p.type_count = reinterpret_cast<int32_t*>(st + a->so.type_count);
   p.trace_actions = a->trace_actions;
   p.trace_q = a->trace_q;
   p.trace_first = a->trace_next;
