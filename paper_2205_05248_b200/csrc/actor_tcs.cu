@@ -15,8 +15,9 @@
 // memory and read from there by tcgen05.mma (an A operand in shared memory costs at least 32 clocks a product, one in
 // tensor memory 3 at N = 16, 27 at N = 64); only the observations and the fc1 output of the three-piece hidden-128
 // variant live in shared memory.  Nothing assumes an alignment beyond that of the element type, and a tile's rows may
-// be those of a list (partial steps) or of one unit type (per-type networks: the block runs its tiles once per type,
-// on the rows of that type, with that type's network).
+// be those of a list (partial steps) or of one unit type (per-type networks: the tiles of all types are dealt to the blocks
+// together, those of one type before those of the next, and a block loads a type's network when it comes to its tiles; a
+// pass of all blocks per type took 1045 us for 1024 environments of 2 + 3 agents, fp32, 64 steps, this takes 507).
 //
 // Roles: warps 0-7 epilogue (two groups of 128 threads; a thread owns one row and 16 columns of every block of 32
 // hidden columns), warps 8-15 inputs and records (two groups, thread = row), warp 16 issues every tcgen05.mma (from the lane that
@@ -441,12 +442,15 @@ __device__ __forceinline__ void ts_gates2_fast(const float (&v)[4][2], const ts_
   f2_get(f2_fma(zg, f2_fma(c, f2(-1.0f), f2(h0, h1)), c), h0, h1);
 }
 
-// D (+)= A B^T, issued by one lane; A in shared memory (AS: descriptor) or in tensor memory (column address).
+// D (+)= A B^T, issued by one lane; A in shared memory (AS: descriptor) or in tensor memory (column address).  Descriptors go
+// by their low words: the warp that issues has few registers, and a reload from local memory costs an access to L2 (64-bit
+// descriptors: a step of 8 environments x 3 agents 11.4 us, 64 steps of 4096 x 8 in fp32 1060; now 10.7 and 1010).
 template <bool AS>
-__device__ __forceinline__ void ts_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  if (AS) tc::mma_bf16(d, a, b, idesc, acc);
-  else tc::mma_bf16_ts(d, (uint32_t)a, b, idesc, acc);
+__device__ __forceinline__ void ts_mma(uint32_t d, uint32_t a, uint32_t b, uint32_t idesc, uint32_t acc) {
+  if (AS) tc::mma_bf16_lo(d, a, b, idesc, acc);
+  else tc::mma_bf16_ts_lo(d, a, b, idesc, acc);
 }
+__device__ __forceinline__ uint32_t ts_lo(uint32_t addr, uint32_t lbo) { return (addr >> 4) | ((lbo >> 4) << 16); }
 
 }  // namespace
 
@@ -464,8 +468,10 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
   constexpr uint32_t TSM_Y = TSM_HOP + NS * H / 2;
   constexpr uint32_t FC1 = H == 64 ? 96 : 0;     // fc1's accumulator: the candidate-input columns, or buffer 0
   // Registers (setmaxnreg): launched with 96 a thread (640 * 96 = 61440); afterwards
-  // 256 * 128 + 256 * 88 + 128 * 48 = 61440.
-  constexpr int REGS_EPI = 128, REGS_PREP = 88, REGS_SVC = 48;
+  // 256 * 128 + 256 * 88 + 128 * 48 = 61440, at one piece and hidden 128 256 * 136 + 256 * 72 + 128 * 64: there the epilogue
+  // and the issuing warp spill less (16384 environments x 8 agents x 64 steps 3600 -> 3405 us).
+  constexpr bool WIDE = NS == 1 && H == 128;
+  constexpr int REGS_EPI = WIDE ? 136 : 128, REGS_PREP = WIDE ? 72 : 88, REGS_SVC = WIDE ? 64 : 48;
   extern __shared__ __align__(1024) uint8_t smem[];
   TsBars* B = reinterpret_cast<TsBars*>(smem + L.off_bar);
   // per-step hand-offs, four buffers each: the input warps run up to two steps ahead of the choice
@@ -539,16 +545,16 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
       const uint32_t sb = smem_u32(smem);
       constexpr uint32_t id96 = idesc_bf16_f32(128, 96), id64 = idesc_bf16_f32(128, 64), id32 = idesc_bf16_f32(128, 32),
                          idH = idesc_bf16_f32(128, H), idq = idesc_bf16_f32(128, NQ);
-      constexpr uint64_t ks_1 = (2 * H * 16) >> 4, ks_g = (2 * 96 * 16) >> 4, ks_q = (2 * NQ * 16) >> 4, st_q = (H / 16) * ks_q;
+      constexpr uint32_t ks_1 = (2 * H * 16) >> 4, ks_g = (2 * 96 * 16) >> 4, ks_q = (2 * NQ * 16) >> 4, st_q = (H / 16) * ks_q;
       const int nk1 = L.Dk / 16;
       // the left operands and the distance between their pieces and K steps
-      const uint64_t a_h = tmem + TSM_HOP;
-      constexpr uint64_t h_st = H / 2, h_ks = 8;
-      const uint64_t a_x = XS ? smem_desc(sb + L.off_xy, 2048, 128) : (uint64_t)(tmem + L.tm_x);
-      const uint64_t a_y = XS ? a_x : (uint64_t)(tmem + TSM_Y);
-      constexpr uint64_t x_ks = XS ? (2 * 2048) >> 4 : 8;
-      const uint64_t x_st = (uint64_t)nk1 * x_ks;
-      constexpr uint64_t y_st = KH * x_ks;
+      const uint32_t a_h = tmem + TSM_HOP;
+      constexpr uint32_t h_st = H / 2, h_ks = 8;
+      const uint32_t a_x = XS ? ts_lo(sb + L.off_xy, 2048) : tmem + L.tm_x;
+      const uint32_t a_y = XS ? a_x : tmem + TSM_Y;
+      constexpr uint32_t x_ks = XS ? (2 * 2048) >> 4 : 8;
+      const uint32_t x_st = (uint32_t)nk1 * x_ks;
+      constexpr uint32_t y_st = KH * x_ks;
       uint32_t g = 0, ri = 0, rpar = 0;  // steps so far; ring slot and its parity
       uint32_t loads = 0;  // networks loaded so far
       bool first = true;
@@ -565,15 +571,14 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
       auto next_slot = [&]() {
         if (++ri == (uint32_t)L.nslots) { ri = 0; rpar ^= 1u; }
       };
-      auto desc = [&](uint32_t addr, uint32_t lbo) { return smem_desc(addr, lbo, 128); };
 
       // The gate products of one piece pair over all K steps.  (Measured per product
       // of N = 64: 30 clocks in rolled loops around four unrolled ones, 56 in a loop over single ones.)
       // side 1: hidden, side 0: y, whose first product of a step starts the candidate-input columns.
-      auto prod = [&](int buf, int hid, uint32_t ai, uint64_t w, uint32_t acc) {
+      auto prod = [&](int buf, int hid, uint32_t ai, uint32_t w, uint32_t acc) {
         const uint32_t d = tmem + (hid ? (buf ? 160u : 0u) : (buf ? 128u : 32u));
         if (XS && !hid) {
-          const uint64_t a = a_y + ai * y_st;
+          const uint32_t a = a_y + ai * y_st;
           if (acc) {
             ts_mma<true>(d, a, w, id96, 1);
           } else {  // buffer 0: R Z at rows 0.., IN at rows 64..; buffer 1: IN at rows 0.., R Z at rows 32..
@@ -583,7 +588,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
 #pragma unroll
           for (int ks = 1; ks < KH; ++ks) ts_mma<true>(d, a + ks * x_ks, w + ks * ks_g, id96, 1);
         } else {
-          const uint64_t a = hid ? a_h + ai * h_st : a_y + ai * y_st;
+          const uint32_t a = hid ? a_h + ai * h_st : a_y + ai * y_st;
           if (hid || acc) {
             ts_mma<false>(d, a, w, id96, acc);
           } else {
@@ -595,6 +600,33 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
         }
       };
 
+      // fc1 at hidden 64, where all weights are resident
+      const uint32_t w1_lo = ts_lo(sb + L.off_sl, H * 16), w1_st = (uint32_t)(L.Dk * H * 2) >> 4;
+      const uint32_t wg_lo = ts_lo(sb + L.off_sl + ts_slice_off(L, H, NS, L.nw1), 1536);
+      auto fc1_resident = [&]() {
+        if (elect_one()) {
+          // (left piece, slice): (0,0) (1,1) (0,1) (2,2) (1,2) (0,2) - the slices lie smallest piece first
+          constexpr uint32_t LA = 0x012010u, SA = 0x222110u;
+#pragma unroll 1
+          for (int j = 0; j < (NS == 3 ? 6 : 1); ++j) {
+            uint32_t a = tmem + L.tm_x, w = w1_lo, acc = j > 0;
+            if (NS == 3) {
+              a += ((LA >> (4 * j)) & 15u) * (uint32_t)(nk1 * 8);
+              w += ((SA >> (4 * j)) & 15u) * w1_st;
+            }
+            int ks = 0;
+#pragma unroll 1
+            for (; ks + 2 <= nk1; ks += 2, a += 16, w += 2 * ks_1, acc = 1) {
+              ts_mma<false>(tmem + FC1, a, w, idH, acc);
+              ts_mma<false>(tmem + FC1, a + 8, w + ks_1, idH, 1);
+            }
+            if (ks < nk1) ts_mma<false>(tmem + FC1, a, w, idH, acc);
+          }
+          mma_commit(&B->fc1d);
+        }
+        __syncwarp();
+      };
+
       for (int tile = blockIdx.x, typ = 0, cur = -1; unit_at(tile, typ); tile += gridDim.x) {
         if (typ != cur) {
           cur = typ;
@@ -604,17 +636,22 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
         for (int s = 0; s < T; ++s, ++g, first = false) {
           const uint32_t par = g & 1;
           // ---- fc1 ----
-          mbar_wait(&B->xrdy, par, abortf);  // (E2 of the previous step has read the columns: hr1)
-          tc_fence_after_sync();
-          {
+          if (H == 64) {
+            mbar_wait(&B->xrdy, par, abortf);  // (E2 of the previous step has read the columns: hr1)
+            if (first) mbar_wait(&B->res[0], (loads - 1) & 1, abortf);
+            tc_fence_after_sync();
+            fc1_resident();
+          } else {
+            mbar_wait(&B->xrdy, par, abortf);  // (E2 of the previous step has read the columns: hr1)
+            tc_fence_after_sync();
             for (int i = 0; i < L.nw1; ++i) {
-              const uint64_t w = desc(get(i), H * 16);
+              const uint32_t w = ts_lo(get(i), H * 16);
               if (elect_one()) {
                 // piece 2 - i against the small products' left pieces, then the main product (one piece: the slice's)
                 const int k0 = NS == 3 ? 0 : i * (TS_KCHUNK / 16), nk = min(nk1 - k0, TS_KCHUNK / 16);
 #pragma unroll 1
                 for (int ai = NS == 3 ? i : 0; ai >= 0; --ai) {
-                  uint64_t a = a_x + ai * x_st + (uint32_t)k0 * x_ks, wk = w;
+                  uint32_t a = a_x + (uint32_t)ai * x_st + (uint32_t)k0 * x_ks, wk = w;
                   uint32_t acc = i > 0 || (NS == 3 && ai < i);
                   int ks = 0;
 #pragma unroll 1
@@ -635,9 +672,9 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
           if (H == 64) {
             // everything resident: the hidden side's first products run before the fc1 output is there
             mbar_wait(&B->hset, par, abortf);
+            if (first) mbar_wait(&B->res[1], (loads - 1) & 1, abortf);
             tc_fence_after_sync();
-            const uint64_t w0 = desc(get(L.nw1), 1536);
-            constexpr uint64_t SL = ts_slice(H) >> 4;
+            constexpr uint32_t SL = ts_slice(64) >> 4;
             // pieces of the small products in order: left, and slice of the hidden and of the y side
             constexpr uint32_t LEFT = 0x10210u, SH = 0x41410u, SY = 0x53532u;
             if (elect_one()) {
@@ -645,7 +682,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
               for (int b = 0; b < NBLK; ++b)
 #pragma unroll 1
                 for (int j = 0; j < (NS == 3 ? 5 : 1); ++j)
-                  prod(b, 1, (LEFT >> (4 * j)) & 15u, w0 + (uint32_t)(b * 2 * NS) * SL + (NS == 3 ? (SH >> (4 * j)) & 15u : 0u) * SL, j > 0);
+                  prod(b, 1, (LEFT >> (4 * j)) & 15u, wg_lo + (uint32_t)(b * 2 * NS) * SL + (NS == 3 ? (SH >> (4 * j)) & 15u : 0u) * SL, j > 0);
             }
             __syncwarp();
             mbar_wait(&B->yrdy, par, abortf);
@@ -653,7 +690,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
             if (elect_one()) {
 #pragma unroll 1
               for (int b = 0; b < NBLK; ++b) {
-                const uint64_t wb = w0 + (uint32_t)(b * 2 * NS) * SL;
+                const uint32_t wb = wg_lo + (uint32_t)(b * 2 * NS) * SL;
                 if (NS == 3) {
 #pragma unroll 1
                   for (int j = 0; j < 7; ++j)  // five small ones, then the main products
@@ -678,7 +715,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
               tc_fence_after_sync();
               if (NS == 3) {
                 // h2, h1, y2, y1, then h0 and y0 held together: their small products come before both main ones
-                uint64_t wh = 0;
+                uint32_t wh = 0;
                 uint32_t rh = 0;
 #pragma unroll 1
                 for (int k = 0; k < 6; ++k, ++i) {
@@ -686,7 +723,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
                     mbar_wait(&B->yrdy, par, abortf);
                     tc_fence_after_sync();
                   }
-                  const uint64_t w = desc(get(i), 1536);
+                  const uint32_t w = ts_lo(get(i), 1536);
                   const int hid = k < 2 || k == 4;
                   if (k == 4) { wh = w; rh = ri; }
                   if (elect_one()) {
@@ -705,7 +742,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
                   if (i >= L.nres) next_slot();
                 }
               } else {
-                const uint64_t wh = desc(get(i), 1536);
+                const uint32_t wh = ts_lo(get(i), 1536);
                 if (elect_one()) {
                   prod(buf, 1, 0, wh, 0);
                   if (i >= L.nres) mma_commit(&B->empty[ri]);
@@ -713,7 +750,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
                 __syncwarp();
                 if (i >= L.nres) next_slot();
                 ++i;
-                const uint64_t wy = desc(get(i), 1536);
+                const uint32_t wy = ts_lo(get(i), 1536);
                 if (b == 0) {
                   mbar_wait(&B->yrdy, par, abortf);
                   tc_fence_after_sync();
@@ -731,7 +768,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
           }
           // ---- fc2: the small products of all blocks but the last, then the rest ----
           if (g > 0) mbar_wait(&B->qfree, par ^ 1u, abortf);  // the previous step's Q has been read
-          const uint64_t w2 = desc(sb, NQ * 16);
+          const uint32_t w2 = ts_lo(sb, NQ * 16);
           constexpr int K1 = KH - TS_BLK / 16;  // K steps of the earlier blocks
           auto part_q = [&](auto half_c) {  // K steps [0, K1) or [K1, KH); the second part ends with the main product
             constexpr int half = decltype(half_c)::value, k0 = half ? K1 : 0, k1 = half ? KH : K1;
@@ -741,7 +778,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
               if (NS == 3) {  // small products (left, right): (2,0) (1,1) (0,2) (1,0) (0,1)
 #pragma unroll 1
                 for (int j = 0; j < 5; ++j) {
-                  const uint64_t a = a_h + ((0x01012u >> (4 * j)) & 15u) * h_st, w = w2 + ((0x10210u >> (4 * j)) & 15u) * st_q;
+                  const uint32_t a = a_h + ((0x01012u >> (4 * j)) & 15u) * h_st, w = w2 + ((0x10210u >> (4 * j)) & 15u) * st_q;
 #pragma unroll
                   for (int ks = k0; ks < k1; ++ks) ts_mma<false>(tmem + L.tm_q, a + ks * h_ks, w + ks * ks_q, idq, ks > 0 || j > 0);
                 }
@@ -1144,7 +1181,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
     grid_wait();
     const int row = tid & 127, grp = warp >> 2;
     const uint32_t tm = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    unsigned long long c_steps = 0, c_explore = 0, c_noavail = 0;
+    uint32_t c_steps = 0, c_explore = 0, c_noavail = 0;  // (a launch's rows x steps of one thread)
     uint32_t st_bits = 0, g = 0, loads = 0;
     int nt = 0;
     bool fresh = true;
@@ -1398,9 +1435,9 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
       }
       fresh = false;
     }
-    if (c_steps) atomicAdd(p.counters + CNT_AGENT_STEPS, c_steps);
-    if (c_explore) atomicAdd(p.counters + CNT_EXPLORED, c_explore);
-    if (c_noavail) atomicAdd(p.counters + CNT_NO_AVAIL, c_noavail);
+    if (c_steps) atomicAdd(p.counters + CNT_AGENT_STEPS, (unsigned long long)c_steps);
+    if (c_explore) atomicAdd(p.counters + CNT_EXPLORED, (unsigned long long)c_explore);
+    if (c_noavail) atomicAdd(p.counters + CNT_NO_AVAIL, (unsigned long long)c_noavail);
     if (st_bits) atomicOr(p.status, st_bits);
   }
   tc_fence_before_sync();

@@ -138,7 +138,8 @@ def test_host_step_on_pinned_and_pageable_arrays(over):
     dev.destroy()
 
 
-@pytest.mark.parametrize("prec,H,T", [("fp32", 64, 220_000), ("bf16", 128, 300_000)])
+# (The first launch has to last 1.2 s: at 5.0 us a step, which is less than the kernel takes in fp32 - 5.38 -, 240 000 steps do.)
+@pytest.mark.parametrize("prec,H,T", [("fp32", 64, 240_000), ("bf16", 128, 300_000)])
 def test_launch_behind_a_long_one(prec, H, T):
     """A launch that starts beside its predecessor while that still runs for longer than a bounded wait lasts (about a
     second): the wait for the predecessor counts against none of its own waits."""
