@@ -53,6 +53,7 @@ constexpr int TP_QPARTS = 4;
 // availability run up to 9 % faster than with the same test in the product, store or tail warp (5 agents x 55 observations,
 // 16384 environments x 128 steps: 2496 against 2756-2760 us; released at the start: 2757), the aligned ones as before.
 constexpr int TP_RELEASE = 3;
+constexpr uint32_t TP_SCR = 4096;     // scratch of an epilogue warp in launches of a few steps: 32 rows x 128 bytes of hidden state
 constexpr int TP_DST_DEPTH = 16;      // steps of record addresses kept: the loads run at most TP_MAX_STAGES chunks (steps) ahead
 // Register split (setmaxnreg): launched with 128 registers per thread (512 * 128 = 65536); afterwards
 // 256 * 144 + 128 * 112 + 128 * 112 = 65536.
@@ -79,7 +80,7 @@ struct TpBars {
 // M, sms: the launch's batch and the number of blocks it may use (0: the largest tiles, for the shape check).
 // fastx: the launch moves its hidden-state rows through a scratch (modes 1 to 3 of the kernel).
 static TpLayout tp_layout(int n, int D, int A, int rec_bytes, int M = 0, int sms = 0, bool fastx = true,
-                          uint32_t reserve = 0) {
+                          uint32_t reserve = 0, uint32_t scr_warp = TP_SCR) {
   const TcLayout W = tc_layout(n, D, A, rec_bytes);
   TpLayout L;
   memset(&L, 0, sizeof(L));
@@ -114,7 +115,7 @@ static TpLayout tp_layout(int n, int D, int A, int rec_bytes, int M = 0, int sms
   L.chunk_bytes = L.plain ? TP_G * L.obs_bytes + up16(TP_G * L.av_bytes) + 16u : TP_G * L.prefix_bytes;
   uint32_t o = L.wbytes;
   L.off_x = o; o += up16((uint32_t)L.nchunk * TC_LBO_X);
-  L.off_scr = o; o += fastx ? 8 * 2048u : 0;
+  L.off_scr = o; o += fastx ? 8 * scr_warp : 0;
   L.off_oh = o; o += (uint32_t)L.ohc * TC_LBO_A;
   L.off_tail = o; o += 2u * (uint32_t)L.ept * L.tail_bytes;
   L.off_sel = o; o += 4u * TC_ROWS * 8;
@@ -151,8 +152,9 @@ static TpLayout tp_layout(int n, int D, int A, int rec_bytes, int M = 0, int sms
 bool tcp_supported(int n, int D, int A, int H, int prec) {
   if (prec != MARL_PRECISION_BF16 || H != TC_H) return false;
   if (D < 1 || D > 256 || n < 4 || n > 32 || A < 1 || A > 32) return false;
-  // (16 KB are kept back: the domain stated in the header does not move with what a layout happens to leave over)
-  const TpLayout L = tp_layout(n, D, A, rec_bytes_of(n, D, A), 0, 0, true, 8 * TC_LBO_A);
+  // (16 KB are kept back: the domain stated in the header does not move with what a layout happens to leave over; they are
+  // also where the second half of the scratch finds its room, in every shape of the domain)
+  const TpLayout L = tp_layout(n, D, A, rec_bytes_of(n, D, A), 0, 0, true, 8 * TC_LBO_A, TP_SCR / 2);
   // enough staging for loads to run ahead of the network (tp_layout leaves 0 where the ring would be unsafe)
   return L.ept >= TP_G && L.NS >= 3 && L.total <= TC_SMEM_MAX;
 }
@@ -235,9 +237,11 @@ __device__ __forceinline__ void tp_issue_hside(const TpLayout& L, uint32_t sb, u
 // MODE 2 (LAG, one step per launch): reward/done are the outcome of each environment's previous action: they complete
 // the record at pos - 1 and may close the episode BEFORE this step's decision; nothing closes after it.
 // MODE 3: MODE 0 for launches of a few steps, where the tile-to-tile transition is a large part of the time: the
-// hidden-state rows then move coalesced through a scratch and the next tile's rows are prefetched into L2 (modes 1
-// and 2 do the same).  Launches of many steps keep the shorter transition code: its footprint in the step loop's
-// instruction stream and registers costs them more (1.2 %) than the transition saves.
+// hidden-state rows then move coalesced through a scratch.  They leave while fc2 runs, the next tile's come behind them by
+// cp.async while the choice is made, and the cursors and outcomes of the next tile are requested during this one (modes 1
+// and 2 do the same): a list step of 32768 x 8 agents 115.3 -> 89.5 us, 12 to 14 k clocks a tile -> some 9 k.  Launches of many
+// steps keep the shorter transition code: its footprint in the step loop's instruction stream and registers costs them more
+// (1.2 %) than the transition saves.
 template <int NQ, int PM, int MODE>
 __global__ void __launch_bounds__(TP_THREADS, 1)
     actor_tcp_kernel(const __grid_constant__ ActorParams p, const __grid_constant__ TpLayout L) {
@@ -474,23 +478,45 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
       if (my_tiles * T <= TP_RELEASE) grid_release();  // (before the load warp has its first cursors)
       unsigned long long c_episodes = 0, c_trunc = 0;
       uint32_t st_bits = 0, sd = 0, it = 0;
+      // short launches: cursor and outcome of the lane's environment in the next tile, requested during this one
+      int e_n = -1, ne_prev = 0;
+      int32_t slot_n = 0, pos_n = 0;
+      long long epc_n = 0;
+      float reward_n = 0.f;
+      uint32_t done_n = 0;
+      auto next_env = [&](int t) {
+        const int x = t * L.ept + lane;
+        e_n = !(t < p.num_tiles && lane < min(L.ept, p.M - t * L.ept)) ? -1 : LIST ? __ldg(p.env_ids + x) : x;
+      };
+      auto next_cursor = [&](int t) {
+        if (e_n < 0) return;
+        slot_n = p.slot[e_n];
+        pos_n = p.pos[e_n];
+        epc_n = p.ep_count[e_n];
+        reward_n = p.reward[t * L.ept + lane];
+        done_n = p.done[t * L.ept + lane];
+      };
+      if constexpr (FASTX) {
+        next_env(blockIdx.x);
+        next_cursor(blockIdx.x);
+      }
       for (int tile = blockIdx.x; tile < p.num_tiles; tile += gridDim.x) {
         const int ne = min(L.ept, p.M - tile * L.ept);
         const bool mine = lane < ne;
         const int x = tile * L.ept + lane;  // row of the call
-        const int e = (LIST && mine) ? __ldg(p.env_ids + x) : x;
+        const int e = FASTX ? e_n : x;
         int32_t slot = 0, pos = 0, ok = 0;
         long long epc = 0;
         float reward_next = 0.f;
         uint32_t done_next = 0;
         if (mine) {
-          slot = p.slot[e];
-          pos = p.pos[e];
-          epc = p.ep_count[e];
+          slot = FASTX ? slot_n : p.slot[e];
+          pos = FASTX ? pos_n : p.pos[e];
+          epc = FASTX ? epc_n : p.ep_count[e];
           ok = (slot >= 0 && slot < p.E * p.S && pos >= 0 && pos < p.L + (LAG ? 1 : 0)) ? 1 : 0;
           if (!ok) st_bits |= MARL_STATUS_BAD_INDEX;
-          reward_next = p.reward[x];
-          done_next = p.done[x];
+          reward_next = FASTX ? reward_n : p.reward[x];
+          done_next = FASTX ? done_n : p.done[x];
           if (LAG) {
             if (ok && pos > 0) {  // the outcome of the previous action completes its record and may close the episode
               uint8_t* prev = p.ring + (size_t)slot * p.slot_stride + (size_t)(pos - 1) * rec_bytes;
@@ -512,9 +538,9 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
         }
         // Copies the tails of one step (buffer bb, record addresses in tdst_s) to the ring: 16 bytes per lane, the
         // pieces of all environments in one flat loop.
-        auto copy_tails = [&](uint32_t bb) {
+        auto copy_tails = [&](uint32_t bb, int envs) {
           __syncwarp();
-          const uint32_t pieces = L.tail_bytes / 16u, total = (uint32_t)ne * pieces;
+          const uint32_t pieces = L.tail_bytes / 16u, total = (uint32_t)envs * pieces;
           const uint32_t inv = 0xFFFFFFFFu / pieces + 1u;  // idx / pieces == umulhi(idx, inv) for idx < 2^16
           for (uint32_t idx = lane; idx < total; idx += 32) {
             const uint32_t env = __umulhi(idx, inv), pc = idx - env * pieces;
@@ -543,7 +569,13 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
           }
           __syncwarp();
           if (lane == 0) mbar_arrive(&B->flags);  // first: epilogue 3 of this step waits for it
-          if (s > 0) copy_tails(b ^ 1u);           // then the previous step's tails, off the critical path
+          // then the previous step's tails, off the critical path (short launches: the previous tile's too)
+          if constexpr (FASTX) {
+            if (it > 0) copy_tails(b ^ 1u, s > 0 ? ne : ne_prev);
+            if (s == 0) next_env(tile + (int)gridDim.x);
+          } else if (s > 0) {
+            copy_tails(b ^ 1u, ne);
+          }
           if (mine && s + 1 < T) {
             reward_next = p.reward[(size_t)(s + 1) * p.env_step_stride + x];
             done_next = p.done[(size_t)(s + 1) * p.env_step_stride + x];
@@ -564,12 +596,16 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
           }
           ++it;
         }
-        copy_tails((it - 1) & 1);  // the tile's last step
+        if (!FASTX || tile + (int)gridDim.x >= p.num_tiles) copy_tails((it - 1) & 1, ne);  // the tile's last step
         if (mine && ok) {
           p.slot[e] = slot;
           p.pos[e] = pos;
           p.ep_count[e] = epc;
           if (pos > 0) p.slot_len[slot] = pos;
+        }
+        if constexpr (FASTX) {
+          next_cursor(tile + (int)gridDim.x);
+          ne_prev = ne;
         }
       }
       if (c_episodes) atomicAdd(p.counters + CNT_EPISODES, c_episodes);
@@ -791,13 +827,43 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
           tmem_st4(tm_h + (uint32_t)c8 * 4u, pack_bf16x2(hv[0], hv[1]), pack_bf16x2(hv[2], hv[3]), pack_bf16x2(hv[4], hv[5]), pack_bf16x2(hv[6], hv[7]));
         }
     };
-    // this thread's half (32 floats) of tile row r's hidden state in global memory
-    auto h_row = [&](int e0, int r) -> float* {
-      if (!LIST) return p.h + ((size_t)e0 * n + (size_t)r) * TC_H + cb;  // a tile's rows are contiguous
-      const int rel = rowenv_s[r];  // r / n
-      const int env = __ldg(p.env_ids + e0 + rel);
-      return p.h + ((size_t)env * n + (size_t)(r - rel * n)) * TC_H + cb;
+    // ---- short launches: a tile's rows of hidden state, and the scalars beside them, are requested a tile ahead ----
+    const int wrow0 = (warp & 3) * 32;  // first tile row of this warp
+    // A thread owns 128 bytes of its row, so a warp that moves "its own" pieces would touch 32 lines per instruction.  The
+    // rows go through a warp-private scratch instead: eight lanes move one row's 128 bytes, and the scratch's piece index is
+    // xor-ed with the row so that neither side has bank conflicts.
+    uint4* sw = reinterpret_cast<uint4*>(smem + L.off_scr + (uint32_t)warp * TP_SCR);
+    uint32_t grow_n = 0;                // the thread's row in the next tile; its environment and state:
+    int e_n = 0, la_n = -1, pos_n = 0, done_n = 0;
+    auto next_env = [&](int t) {
+      const int e0n = t * L.ept;
+      e_n = !(t < p.num_tiles && row < min(L.ept, p.M - e0n) * n) ? -1 : LIST ? __ldg(p.env_ids + e0n + el) : e0n + el;
     };
+    auto next_scalars = [&](int t) {
+      grow_n = (uint32_t)e_n * (uint32_t)n + (uint32_t)ai;
+      if (e_n < 0) return;
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(p.h + (size_t)grow_n * TC_H + cb));
+      if (half == 0) la_n = p.last_action[grow_n];
+      if (LAG) {
+        pos_n = p.pos[e_n];
+        done_n = p.done[t * L.ept + el];
+      }
+    };
+    auto next_rows = [&]() {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int rl = 4 * j + (lane >> 3);
+        const uint32_t g = __shfl_sync(0xFFFFFFFFu, grow_n, rl);
+        const bool on = __shfl_sync(0xFFFFFFFFu, e_n, rl) >= 0;
+        const float* src = on ? p.h + (size_t)g * TC_H + cb + (lane & 7) * 4 : p.h;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(sw + rl * 8 + ((lane & 7) ^ (rl & 7)))), "l"(src), "r"(on ? 16u : 0u) : "memory");
+      }
+    };
+    if constexpr (FASTX) {
+      next_env(blockIdx.x);
+      next_scalars(blockIdx.x);
+      next_rows();
+    }
 
     for (int tile = blockIdx.x; tile < p.num_tiles; tile += gridDim.x) {
       const int e0 = tile * L.ept;
@@ -805,56 +871,29 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
       const int R = ne * n;
       const bool live = row < R;
       const bool is_row = live && half == 0;  // owner of the row's choice
-      const int e = (LIST && live) ? __ldg(p.env_ids + e0 + el) : e0 + el;
+      const int e = LIST ? e_n : e0 + el;
       const size_t grow = (size_t)e * n + ai;  // global row
       int la = -1;
 
       // ---- tile prologue: hidden state and last actions from global memory ----
       {
         bool carry = live;  // the row continues an episode
-        if (LAG && live) {  // ... unless the late outcome has just ended it
-          const int ps = p.pos[e];
-          if (ps > 0 && (p.done[e0 + el] || ps == p.L)) carry = false;
-        }
-        const int la_mem = (carry && half == 0) ? p.last_action[grow] : -1;  // in flight beside the rows below
-        // A thread owns 128 bytes of its row, so a warp reading "its own" pieces would touch 32 lines per
-        // instruction.  The rows go through a warp-private 2 KB scratch instead: eight lanes fetch one row's 128 bytes, the scratch's piece index is xor-ed with the row so
-        // that neither side has bank conflicts, and each thread then takes its row, 16 rows per pass.
+        if (LAG && live && pos_n > 0 && (done_n || pos_n == p.L)) carry = false;  // ... unless the late outcome has just ended it
+        const int la_mem = !(carry && half == 0) ? -1 : FASTX ? la_n : p.last_action[grow];  // in flight beside the rows below
         if constexpr (FASTX) {
-          uint4* sw = reinterpret_cast<uint4*>(smem + L.off_scr) + warp * 128;  // this warp's scratch
-          const int wrow0 = (warp & 3) * 32;                      // first tile row of this warp
-          uint4 f[2][4];
+          asm volatile("cp.async.wait_all;" ::: "memory");
+          __syncwarp();
 #pragma unroll
-          for (int ps = 0; ps < 2; ++ps)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const int r = wrow0 + ps * 16 + 4 * j + (lane >> 3);
-              f[ps][j] = make_uint4(0u, 0u, 0u, 0u);
-              if (r < R) f[ps][j] = __ldg(reinterpret_cast<const uint4*>(h_row(e0, r)) + (lane & 7));
-            }
-#pragma unroll
-          for (int ps = 0; ps < 2; ++ps) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const int rl = 4 * j + (lane >> 3);
-              sw[rl * 8 + ((lane & 7) ^ (rl & 7))] = f[ps][j];
-            }
-            __syncwarp();
-            if ((lane >> 4) == ps) {
-              const int rl = lane & 15;
-#pragma unroll
-              for (int q = 0; q < 8; ++q) {
-                const uint4 v = sw[rl * 8 + (q ^ (rl & 7))];
-                h[4 * q] = __uint_as_float(v.x); h[4 * q + 1] = __uint_as_float(v.y);
-                h[4 * q + 2] = __uint_as_float(v.z); h[4 * q + 3] = __uint_as_float(v.w);
-              }
-            }
-            __syncwarp();
+          for (int q = 0; q < 8; ++q) {
+            const uint4 v = sw[lane * 8 + (q ^ (lane & 7))];
+            h[4 * q] = __uint_as_float(v.x); h[4 * q + 1] = __uint_as_float(v.y);
+            h[4 * q + 2] = __uint_as_float(v.z); h[4 * q + 3] = __uint_as_float(v.w);
           }
           if (!carry) {
 #pragma unroll
             for (int q = 0; q < 32; ++q) h[q] = 0.f;
           }
+          next_env(tile + (int)gridDim.x);
         } else {
           const float4* src = reinterpret_cast<const float4*>(p.h + grow * TC_H + cb);
 #pragma unroll
@@ -873,17 +912,6 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
         tc_fence_before_sync();
         asm volatile("bar.sync 1, 256;" ::: "memory");  // la_s is read by both threads of a row
         warp_arrive(&B->tiled, lane);
-        // The next tile's hidden state is a first touch of its lines (and often of its page): ask for it now, one
-        // line per thread, so that the next prologue finds it in L2.
-        const int tile_n = tile + (int)gridDim.x;
-        if (FASTX && tile_n < p.num_tiles) {
-          const int e0n = tile_n * L.ept;
-          if (row < min(L.ept, p.M - e0n) * n) {
-            const float* nx = h_row(e0n, row);
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(nx));
-            if (half == 0 && ai == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.last_action + (nx - cb - p.h) / TC_H));
-          }
-        }
       }
 
       if (fresh) mbar_wait(&B->wload, 0, abortf);
@@ -927,6 +955,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
         tmem_st_wait();
         tc_fence_before_sync();
         warp_arrive(&B->yready, lane);
+        if (FASTX && s + 1 == T) next_scalars(tile + (int)gridDim.x);
 
         // ---- epilogue 2: gate math, new hidden state (fp32 registers) and its bf16 operand.
         //      The r and z accumulators hold half the pre-activation: sigmoid(v) = 0.5 * tanh(v / 2) + 0.5 ----
@@ -966,6 +995,27 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
 
         // ---- epilogue 3: the row owners choose and complete the record's tail ----
         mbar_wait(&B->flags, par, abortf);  // close flags of this step written, tail buffer free
+        if constexpr (FASTX) {
+          if (s + 1 == T) {  // the tile's rows leave, the next tile's come
+            const bool zero = live && close_s[b * 32 + el];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              uint4 v = make_uint4(__float_as_uint(h[4 * q]), __float_as_uint(h[4 * q + 1]), __float_as_uint(h[4 * q + 2]), __float_as_uint(h[4 * q + 3]));
+              if (zero) v = make_uint4(0u, 0u, 0u, 0u);
+              sw[lane * 8 + (q ^ (lane & 7))] = v;
+            }
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const int rl = 4 * j + (lane >> 3);
+              const uint32_t g = __shfl_sync(0xFFFFFFFFu, (uint32_t)grow, rl);
+              const uint4 v = sw[rl * 8 + ((lane & 7) ^ (rl & 7))];
+              if (wrow0 + rl < R) reinterpret_cast<uint4*>(p.h + (size_t)g * TC_H + cb)[lane & 7] = v;
+            }
+            __syncwarp();
+            next_rows();
+          }
+        }
         mbar_wait(&B->fc2d, par, abortf);   // (both halves: the hidden operand may be cleared below)
         tc_fence_after_sync();
         if (half == 0) {
@@ -1058,27 +1108,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
 
       // ---- tile epilogue: state back to global memory ----
       if (is_row) p.last_action[grow] = la;
-      if constexpr (FASTX) {
-        uint4* sw = reinterpret_cast<uint4*>(smem + L.off_scr) + warp * 128;
-        const int wrow0 = (warp & 3) * 32;
-#pragma unroll
-      for (int ps = 0; ps < 2; ++ps) {  // the rows leave through the same scratch, coalesced
-        if ((lane >> 4) == ps) {
-          const int rl = lane & 15;
-#pragma unroll
-          for (int q = 0; q < 8; ++q)
-            sw[rl * 8 + (q ^ (rl & 7))] = make_uint4(__float_as_uint(h[4 * q]), __float_as_uint(h[4 * q + 1]),
-                                                     __float_as_uint(h[4 * q + 2]), __float_as_uint(h[4 * q + 3]));
-        }
-        __syncwarp();
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int rl = 4 * j + (lane >> 3), r = wrow0 + ps * 16 + rl;
-          if (r < R) reinterpret_cast<uint4*>(h_row(e0, r))[lane & 7] = sw[rl * 8 + ((lane & 7) ^ (rl & 7))];
-        }
-        __syncwarp();
-      }
-      } else if (live) {
+      if (!FASTX && live) {
         float4* dsth = reinterpret_cast<float4*>(p.h + grow * TC_H + cb);
 #pragma unroll
         for (int q = 0; q < 8; ++q) dsth[q] = make_float4(h[4 * q], h[4 * q + 1], h[4 * q + 2], h[4 * q + 3]);
