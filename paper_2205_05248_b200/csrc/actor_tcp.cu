@@ -34,6 +34,7 @@
 
 #include "actor_tc_layout.cuh"
 #include "common.cuh"
+#include "gates.cuh"
 #include "launch_util.cuh"
 #include "tcgen05.cuh"
 
@@ -64,6 +65,7 @@ struct TpLayout {
   uint32_t prefix_bytes, tail_bytes, chunk_bytes, obs_bytes, av_bytes, rs_env, rs_bytes, off_rstage;
   uint32_t off_W1, off_Wih, off_Whh, off_Bg, off_Bhn, off_W2, off_tab_la, wbytes;
   uint32_t off_x, off_scr, off_oh, off_stage, off_tail, off_sel, off_la, off_close, off_closeany, off_rowenv, off_dstp, off_tdst, off_bar, total;
+  uint32_t av_off, off_bias;  // availability within a staged chunk; fp32 biases and agent columns (ragged variant)
 };
 
 struct TpBars {
@@ -80,7 +82,7 @@ struct TpBars {
 // M, sms: the launch's batch and the number of blocks it may use (0: the largest tiles, for the shape check).
 // fastx: the launch moves its hidden-state rows through a scratch (modes 1 to 3 of the kernel).
 static TpLayout tp_layout(int n, int D, int A, int rec_bytes, int M = 0, int sms = 0, bool fastx = true,
-                          uint32_t reserve = 0, uint32_t scr_warp = TP_SCR) {
+                          uint32_t reserve = 0, uint32_t scr_warp = TP_SCR, bool ragged = false) {
   const TcLayout W = tc_layout(n, D, A, rec_bytes);
   TpLayout L;
   memset(&L, 0, sizeof(L));
@@ -112,7 +114,9 @@ static TpLayout tp_layout(int n, int D, int A, int rec_bytes, int M = 0, int sms
   L.tail_bytes = (uint32_t)rec_bytes - (up16(L.obs_bytes) + up16(L.av_bytes));
   // (plain shapes: a chunk's availability bytes need not start on a 16-byte boundary of the input array; the load
   // then covers the aligned range around them, at most 30 bytes more)
-  L.chunk_bytes = L.plain ? TP_G * L.obs_bytes + up16(TP_G * L.av_bytes) + 16u : TP_G * L.prefix_bytes;
+  // (ragged: the observations' too)
+  L.av_off = TP_G * L.obs_bytes + (ragged ? 16u : 0u);
+  L.chunk_bytes = L.plain ? L.av_off + up16(TP_G * L.av_bytes) + 16u : TP_G * L.prefix_bytes;
   uint32_t o = L.wbytes;
   L.off_x = o; o += up16((uint32_t)L.nchunk * TC_LBO_X);
   L.off_scr = o; o += fastx ? 8 * scr_warp : 0;
@@ -125,6 +129,7 @@ static TpLayout tp_layout(int n, int D, int A, int rec_bytes, int M = 0, int sms
   L.off_rowenv = o; o += TC_ROWS * 4;
   L.off_dstp = o; o += TP_DST_DEPTH * 32 * 8;
   L.off_tdst = o; o += 32 * 8;
+  L.off_bias = o; o += ragged ? 4u * TC_H * 4 + (uint32_t)n * TC_TAB * 4 : 0;  // (a multiple of 16)
   L.off_bar = o; o += (uint32_t)((sizeof(TpBars) + 15) & ~15u);
   L.off_stage = o;
   // plain shapes: the converters also lay observations and availability bytes out as the records want them (each
@@ -182,6 +187,8 @@ constexpr uint64_t TP_K_A = (2 * TC_LBO_A) >> 4, TP_K_X = (2 * TC_LBO_X) >> 4, T
                    TP_K_G = (2 * TP_LBO_G) >> 4;                       // descriptor increments of one K = 16 step
 
 // fc1 of one step: observations x W1, then the one-hot tile x (bias pieces, agent-id columns); commits to fc1d.
+// (RAGGED, here and below: no bias and no agent column among the products; the epilogues add them in fp32.)
+template <bool RAGGED>
 __device__ __forceinline__ void tp_issue_fc1(const TpLayout& L, uint32_t sb, uint32_t tmem, uint64_t* fc1d) {
   using namespace tc;
   tc_fence_after_sync();
@@ -199,7 +206,7 @@ __device__ __forceinline__ void tp_issue_fc1(const TpLayout& L, uint32_t sb, uin
     }
     if (ks < ks_obs) mma_bf16(tmem + TM_FC1, d_x + ks * TP_K_X, d_W1 + ks * TP_K_W1, id64, ks > 0);
 #pragma unroll 1
-    for (ks = 0; ks < ks_oh; ++ks) mma_bf16(tmem + TM_FC1, d_oh + ks * TP_K_A, d_W1oh + ks * TP_K_W1, id64, 1);
+    for (ks = 0; ks < (RAGGED ? 0 : ks_oh); ++ks) mma_bf16(tmem + TM_FC1, d_oh + ks * TP_K_A, d_W1oh + ks * TP_K_W1, id64, 1);
     mma_commit(fc1d);
   }
   __syncwarp();
@@ -207,7 +214,7 @@ __device__ __forceinline__ void tp_issue_fc1(const TpLayout& L, uint32_t sb, uin
 
 // h-side gate products of one step: the first MMA seeds r | z | candidate-input with their biases (contiguous in
 // tensor memory: one N = 192 accumulator), the last one seeds the step's Q accumulator with the output bias.
-template <int NQ>
+template <int NQ, bool RAGGED>
 __device__ __forceinline__ void tp_issue_hside(const TpLayout& L, uint32_t sb, uint32_t tmem, uint32_t qcol) {
   using namespace tc;
   tc_fence_after_sync();
@@ -218,13 +225,13 @@ __device__ __forceinline__ void tp_issue_hside(const TpLayout& L, uint32_t sb, u
     const uint64_t d_Bg = smem_desc(sb + L.off_Bg, TP_LBO_G, 128), d_Bhn = smem_desc(sb + L.off_Bhn, TP_LBO_W1, 128);
     const uint64_t d_W2b = smem_desc(sb + L.off_W2 + 8u * NQ * 16, NQ * 16, 128);            // bias pieces of W2: k-chunks 8, 9
     const uint32_t id64 = idesc_bf16_f32(128, 64), id128 = idesc_bf16_f32(128, 128), id192 = idesc_bf16_f32(128, 192);
-    mma_bf16(tmem + TM_R, d_oh, d_Bg, id192, 0);
+    if (!RAGGED) mma_bf16(tmem + TM_R, d_oh, d_Bg, id192, 0);
 #pragma unroll
     for (int ks = 0; ks < 4; ++ks) {
-      mma_bf16_ts(tmem + TM_R, tmem + TMP_H + ks * 8, d_Whh + ks * TP_K_G, id128, 1);
+      mma_bf16_ts(tmem + TM_R, tmem + TMP_H + ks * 8, d_Whh + ks * TP_K_G, id128, !RAGGED || ks > 0);
       mma_bf16_ts(tmem + TM_HN, tmem + TMP_H + ks * 8, d_Whh_n + ks * TP_K_G, id64, ks > 0);
     }
-    mma_bf16(tmem + TM_HN, d_oh, d_Bhn, id64, 1);
+    if (!RAGGED) mma_bf16(tmem + TM_HN, d_oh, d_Bhn, id64, 1);
     mma_bf16(tmem + qcol, d_oh, d_W2b, idesc_bf16_f32(128, NQ), 0);
   }
   __syncwarp();
@@ -242,7 +249,11 @@ __device__ __forceinline__ void tp_issue_hside(const TpLayout& L, uint32_t sb, u
 // and 2 do the same): a list step of 32768 x 8 agents 115.3 -> 89.5 us, 12 to 14 k clocks a tile -> some 9 k.  Launches of many
 // steps keep the shorter transition code: its footprint in the step loop's instruction stream and registers costs them more
 // (1.2 %) than the transition saves.
-template <int NQ, int PM, int MODE>
+// RAGGED (one step per launch, PM != 0): inputs that start (PM 1: observations on any float; availability on any byte) and end
+// anywhere.  The bulk copies take the aligned range around a chunk as far as it lies inside the call's arrays, the load warp's
+// lanes the bytes that are left at the arrays' ends.  These calls have the accurate gate functions, as on the split-operand
+// kernel, which serves them where a block would have one tile at most.
+template <int NQ, int PM, int MODE, bool RAGGED = false>
 __global__ void __launch_bounds__(TP_THREADS, 1)
     actor_tcp_kernel(const __grid_constant__ ActorParams p, const __grid_constant__ TpLayout L) {
   constexpr bool LIST = MODE == 1 || MODE == 2, LAG = MODE == 2, FASTX = MODE != 0;
@@ -329,7 +340,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
       mbar_wait(&B->wload, 0, abortf);
       if (total > 0) {
         mbar_wait(&B->xready, 0, abortf);
-        tp_issue_fc1(L, sb, tmem, &B->fc1d);
+        tp_issue_fc1<RAGGED>(L, sb, tmem, &B->fc1d);
       }
       for (int g = 0, s = 0; g < total; ++g) {
         const uint32_t par = (uint32_t)g & 1u;
@@ -342,14 +353,21 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
           } else {
             mbar_wait(&B->stepd, par ^ 1u, abortf);
           }
-          tp_issue_hside<NQ>(L, sb, tmem, qcol);
+          tp_issue_hside<NQ, RAGGED>(L, sb, tmem, qcol);
         }
         mbar_wait(&B->yready, par, abortf);
         tc_fence_after_sync();
         if (elect_one()) {
           const uint64_t d_Wih = smem_desc(sb + L.off_Wih, TP_LBO_G, 128);
 #pragma unroll
-          for (int ks = 0; ks < 4; ++ks) mma_bf16_ts(tmem + TM_R, tmem + TMP_Y + ks * 8, d_Wih + ks * TP_K_G, idesc_bf16_f32(128, 192), 1);
+          for (int ks = 0; ks < 4; ++ks) {
+            if (RAGGED && ks == 0) {  // the candidate-input columns start here
+              mma_bf16_ts(tmem + TM_R, tmem + TMP_Y, d_Wih, idesc_bf16_f32(128, 128), 1);
+              mma_bf16_ts(tmem + TM_IN, tmem + TMP_Y, d_Wih + ((2 * TC_H * 16) >> 4), idesc_bf16_f32(128, 64), 0);
+            } else {
+              mma_bf16_ts(tmem + TM_R, tmem + TMP_Y + ks * 8, d_Wih + ks * TP_K_G, idesc_bf16_f32(128, 192), 1);
+            }
+          }
           mma_commit(&B->grud);
         }
         __syncwarp();
@@ -360,7 +378,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
           // one lane looks (lanes looking separately could disagree and split the warp's control flow)
           const uint32_t ready = __shfl_sync(0xFFFFFFFFu, lane == 0 ? (uint32_t)mbar_test_wait(&B->xready, par ^ 1u) | (uint32_t)mbar_test_wait(&B->hready, par) << 1 : 0u, 0);
           if (ready & 1u) {
-            tp_issue_fc1(L, sb, tmem, &B->fc1d);
+            tp_issue_fc1<RAGGED>(L, sb, tmem, &B->fc1d);
             pending = false;
           } else if (ready & 2u) {
             break;
@@ -379,7 +397,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
         __syncwarp();
         if (pending) {
           mbar_wait(&B->xready, par ^ 1u, abortf);
-          tp_issue_fc1(L, sb, tmem, &B->fc1d);
+          tp_issue_fc1<RAGGED>(L, sb, tmem, &B->fc1d);
         }
         // The next step's h-side products need only the new hidden state, which is in place unless an episode
         // of this tile ends with this step (its rows are cleared after fc2): issue them now, off the critical
@@ -390,7 +408,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
         } else {
           // (published by the load warp before this step's inputs were requested: ordered before the fc1 operand)
           if (closeany_s[g & (TP_DST_DEPTH - 1)] == 0) {
-            tp_issue_hside<NQ>(L, sb, tmem, TM_Q + (par ^ 1u) * tp_qstride(NQ));
+            tp_issue_hside<NQ, RAGGED>(L, sb, tmem, TM_Q + (par ^ 1u) * tp_qstride(NQ));
             hside_issued = true;
           }
         }
@@ -453,18 +471,45 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
               mbar_wait(&B->sfree[qslot], qpar, abortf);
             }
             const size_t env0 = (size_t)tile * L.ept + (size_t)(c * TP_G);
-            // availability bytes of the chunk: [a0, a0 + ge n A) of the input array; plain shapes load the 16-byte
-            // aligned range around them (inside the array: the launcher checks that the step's block ends aligned)
-            const size_t a0 = (size_t)s * p.avail_step_stride + env0 * (size_t)(n * A);
-            const size_t b0 = PM != 0 ? a0 & ~(size_t)15 : a0;
-            const uint32_t av_load = PM != 0 ? (uint32_t)(((a0 + (size_t)ge * L.av_bytes + 15) & ~(size_t)15) - b0) : (uint32_t)ge * L.av_bytes;
-            if (lane == 0) mbar_arrive_expect_tx(&B->full[qslot], (uint32_t)ge * L.obs_bytes + av_load);
-            __syncwarp();
-            uint8_t* dst = stage + qslot * L.chunk_bytes;
-            if (lane == 0)
-              bulk_load(dst, p.obs + (size_t)s * p.obs_step_stride + env0 * (size_t)(n * D), (uint32_t)ge * L.obs_bytes,
-                        &B->full[qslot]);
-            if (lane == 1) bulk_load(dst + TP_G * L.obs_bytes, p.avail + b0, av_load, &B->full[qslot]);
+            if constexpr (RAGGED) {
+              uint8_t* dst = stage + qslot * L.chunk_bytes;
+              // bytes [a, a + bytes) of the array [lo, lo + all) to `to` + (a mod 16): the lanes' part, and the bulk copy's
+              auto ends = [&](const uint8_t* lo, size_t all, const uint8_t* a, uint32_t bytes, uint8_t* to, const uint8_t*& from, uint8_t*& at) -> uint32_t {
+                const uintptr_t A0 = reinterpret_cast<uintptr_t>(a), A1 = A0 + bytes, base = A0 & ~(uintptr_t)15;
+                uintptr_t B0 = (reinterpret_cast<uintptr_t>(lo) + 15) & ~(uintptr_t)15, B1 = (reinterpret_cast<uintptr_t>(lo) + all) & ~(uintptr_t)15;
+                if (B0 < base) B0 = base;
+                if (B1 > ((A1 + 15) & ~(uintptr_t)15)) B1 = (A1 + 15) & ~(uintptr_t)15;
+                if (B1 < B0) B1 = B0;
+                const uint32_t head = B0 > A0 ? (uint32_t)((B0 < A1 ? B0 : A1) - A0) : 0u;
+                if ((uint32_t)lane < head) to[A0 - base + lane] = a[lane];
+                if (B1 < A1 && (uint32_t)lane < (uint32_t)(A1 - B1)) to[B1 - base + lane] = reinterpret_cast<const uint8_t*>(B1)[lane];
+                from = reinterpret_cast<const uint8_t*>(B0);
+                at = to + (B0 - base);
+                return (uint32_t)(B1 - B0);
+              };
+              const uint8_t *fo, *fa, *obs = reinterpret_cast<const uint8_t*>(p.obs);
+              uint8_t *to, *ta;
+              const uint32_t lo = ends(obs, (size_t)p.M * L.obs_bytes, obs + env0 * L.obs_bytes, (uint32_t)ge * L.obs_bytes, dst, fo, to);
+              const uint32_t la = ends(p.avail, (size_t)p.M * L.av_bytes, p.avail + env0 * L.av_bytes, (uint32_t)ge * L.av_bytes, dst + L.av_off, fa, ta);
+              __syncwarp();
+              if (lane == 0) mbar_arrive_expect_tx(&B->full[qslot], lo + la);  // (publishes the lanes' bytes)
+              __syncwarp();
+              if (lane == 0 && lo) bulk_load(to, fo, lo, &B->full[qslot]);
+              if (lane == 1 && la) bulk_load(ta, fa, la, &B->full[qslot]);
+            } else {
+              // availability bytes of the chunk: [a0, a0 + ge n A) of the input array; plain shapes load the 16-byte
+              // aligned range around them (inside the array: the launcher checks that the step's block ends aligned)
+              const size_t a0 = (size_t)s * p.avail_step_stride + env0 * (size_t)(n * A);
+              const size_t b0 = PM != 0 ? a0 & ~(size_t)15 : a0;
+              const uint32_t av_load = PM != 0 ? (uint32_t)(((a0 + (size_t)ge * L.av_bytes + 15) & ~(size_t)15) - b0) : (uint32_t)ge * L.av_bytes;
+              if (lane == 0) mbar_arrive_expect_tx(&B->full[qslot], (uint32_t)ge * L.obs_bytes + av_load);
+              __syncwarp();
+              uint8_t* dst = stage + qslot * L.chunk_bytes;
+              if (lane == 0)
+                bulk_load(dst, p.obs + (size_t)s * p.obs_step_stride + env0 * (size_t)(n * D), (uint32_t)ge * L.obs_bytes,
+                          &B->full[qslot]);
+              if (lane == 1) bulk_load(dst + TP_G * L.obs_bytes, p.avail + b0, av_load, &B->full[qslot]);
+            }
             ++q;
             if (++qslot == (uint32_t)NS) {
               qslot = 0;
@@ -676,6 +721,8 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
           const uint32_t q = qbase + (uint32_t)c, qslot = q % (uint32_t)NS, qpar = (q / (uint32_t)NS) & 1u;
           const uint8_t* src = stage + qslot * L.chunk_bytes;
           const unsigned long long* recs = dstp_s + (it & (TP_DST_DEPTH - 1)) * 32 + c * TP_G;  // this chunk's records
+          // ragged: the chunk's observations start at byte `osh` of the staged range
+          const uint32_t osh = RAGGED ? (uint32_t)((reinterpret_cast<uintptr_t>(p.obs) + (size_t)(e0 + c * TP_G) * L.obs_bytes) & 15u) : 0u;
           mbar_wait(&B->full[qslot], qpar, abortf);
           const int items = Rc * L.nchunk;
           if (PM == 1) {
@@ -695,7 +742,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
                 cc[u] = on[u] ? (int)__umulhi((uint32_t)jj, inv_Rc) : 0;
                 rr[u] = on[u] ? jj - cc[u] * Rc : 0;
                 const int envc = rowenv_s[rr[u]];
-                const float* srow = reinterpret_cast<const float*>(src) + rr[u] * D;
+                const float* srow = reinterpret_cast<const float*>(src + osh) + rr[u] * D;
                 drow[u] = reinterpret_cast<float*>(smem + L.off_rstage + qslot * L.rs_bytes + (uint32_t)envc * L.rs_env) + (rr[u] - envc * n) * D;
 #pragma unroll
                 for (int k = 0; k < 8; ++k) v[u][k] = (on[u] && cc[u] * 8 + k < D) ? srow[cc[u] * 8 + k] : 0.f;
@@ -741,8 +788,8 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
             }
           }
           // the chunk's availability bytes, rows contiguous; plain shapes: from byte `shift` of the loaded range
-          const uint8_t* avs = src + TP_G * L.obs_bytes;
-          const uint32_t shift = PM != 0 ? (uint32_t)(((size_t)(e0 + c * TP_G) * (size_t)(n * A)) & 15u) : 0u;
+          const uint8_t* avs = src + (RAGGED ? L.av_off : TP_G * L.obs_bytes);
+          const uint32_t shift = PM != 0 ? (uint32_t)(((RAGGED ? (size_t)reinterpret_cast<uintptr_t>(p.avail) : 0) + (size_t)(e0 + c * TP_G) * (size_t)(n * A)) & 15u) : 0u;
           if (PM != 0) {
             // To the record images (1) or straight to the records (2): word j of an environment's block is put
             // together from the two loaded words that hold its bytes; bytes beyond the block stay zero (padding of
@@ -864,6 +911,21 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
       next_scalars(blockIdx.x);
       next_rows();
     }
+    float* bias_s = reinterpret_cast<float*>(smem + L.off_bias);  // [4][64]: reset and update (halved), candidate input, candidate hidden
+    float* tab_a = bias_s + 4 * TC_H;                             // [n][68]: b1 + W1[:, D + agent]
+    if constexpr (RAGGED) {
+      // from the weight image, where a bias is three bf16 pieces
+      mbar_wait(&B->wload, 0, abortf);
+      auto piece = [&](uint32_t off) { return __uint_as_float((uint32_t)*reinterpret_cast<const uint16_t*>(smem + off) << 16); };
+      auto bias_at = [&](uint32_t off) { return (piece(off) + piece(off + 2)) + piece(off + 4); };
+      if (tid < 4 * TC_H) bias_s[tid] = tid < 3 * TC_H ? bias_at(L.off_Bg + (uint32_t)tid * 16u) : bias_at(L.off_Bhn + (uint32_t)(tid - 3 * TC_H) * 16u);
+      const uint32_t w1x = L.off_W1 + (uint32_t)L.nchunk * TP_LBO_W1;
+      for (int i = tid; i < n * TC_H; i += 256) {
+        const int a = i / TC_H, j = i - a * TC_H, k = 3 + a;
+        tab_a[a * TC_TAB + j] = bias_at(w1x + (uint32_t)j * 16u) + piece(w1x + (uint32_t)(k >> 3) * TP_LBO_W1 + (uint32_t)j * 16u + (uint32_t)(k & 7) * 2u);
+      }
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+    }
 
     for (int tile = blockIdx.x; tile < p.num_tiles; tile += gridDim.x) {
       const int e0 = tile * L.ept;
@@ -941,6 +1003,10 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
             for (int q = 0; q < 4; ++q) {
               float4 l4 = make_float4(0.f, 0.f, 0.f, 0.f);
               if (last >= 0) l4 = *reinterpret_cast<const float4*>(tlr + c16 * 16 + 4 * q);
+              if constexpr (RAGGED) {
+                const float4 a4 = *reinterpret_cast<const float4*>(tab_a + ai * TC_TAB + cb + c16 * 16 + 4 * q);
+                l4 = make_float4(a4.x + l4.x, a4.y + l4.y, a4.z + l4.z, a4.w + l4.w);
+              }
               y[4 * q] = fmaxf(__uint_as_float(v[4 * q]) + l4.x, 0.f);
               y[4 * q + 1] = fmaxf(__uint_as_float(v[4 * q + 1]) + l4.y, 0.f);
               y[4 * q + 2] = fmaxf(__uint_as_float(v[4 * q + 2]) + l4.z, 0.f);
@@ -978,13 +1044,29 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
             tmem_ld_wait();
             if (c8 + 1 < 4) request(c8 + 1, g[(c8 + 1) & 1]);
             uint32_t(&v)[4][8] = g[c8 & 1];
+            if constexpr (RAGGED) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const float rg = fmaf(0.5f, tanh_fast(__uint_as_float(v[0][j])), 0.5f);
-              const float zg = fmaf(0.5f, tanh_fast(__uint_as_float(v[1][j])), 0.5f);
-              const float cand = tanh_fast(fmaf(rg, __uint_as_float(v[3][j]), __uint_as_float(v[2][j])));
-              const float hp = h[c8 * 8 + j];
-              h[c8 * 8 + j] = fmaf(zg, hp - cand, cand);  // (1 - z) * cand + z * h
+              for (int j = 0; j < 8; j += 2) {
+                float a2[4][2];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                  a2[k][0] = __uint_as_float(v[k][j]);
+                  a2[k][1] = __uint_as_float(v[k][j + 1]);
+                }
+                ts_f2 b2[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) b2[k] = *reinterpret_cast<const ts_f2*>(bias_s + k * TC_H + cb + c8 * 8 + j);
+                gates2<true>(a2, b2, h[c8 * 8 + j], h[c8 * 8 + j + 1]);
+              }
+            } else {
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                const float rg = fmaf(0.5f, tanh_fast(__uint_as_float(v[0][j])), 0.5f);
+                const float zg = fmaf(0.5f, tanh_fast(__uint_as_float(v[1][j])), 0.5f);
+                const float cand = tanh_fast(fmaf(rg, __uint_as_float(v[3][j]), __uint_as_float(v[2][j])));
+                const float hp = h[c8 * 8 + j];
+                h[c8 * 8 + j] = fmaf(zg, hp - cand, cand);  // (1 - z) * cand + z * h
+              }
             }
             store_h(c8, c8 + 1);
           }
@@ -1130,7 +1212,8 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
   if (warp == 12) tmem_dealloc(tmem, TM_COLS);
 }
 
-// Whether a dense step of M environments runs on this kernel when its input arrays start on 16-byte boundaries.
+// Whether a dense step of M environments runs on this kernel, kernels asked for by name included, when its input arrays start
+// on 16-byte boundaries.
 bool tcp_takes_batch(int n, int D, int A, int M) {
   return ((size_t)M * n * D * 4) % 16 == 0 && ((size_t)M * n * A) % 16 == 0 && (D % 8 == 0 || M % TP_G == 0);
 }
@@ -1139,31 +1222,45 @@ bool tcp_takes_batch(int n, int D, int A, int M) {
 // needs (the caller then uses the one-tile kernel), or a negative cudaError.
 int launch_actor_tcp(const ActorParams& p_in, int sms, cudaStream_t stream) {
   const int mode = p_in.env_ids == nullptr ? (p_in.T < 8 ? 3 : 0) : (p_in.lagged ? 2 : 1);
-  const TpLayout L = tp_layout(p_in.n, p_in.D, p_in.A, (int)p_in.rl.rec_bytes, p_in.M, sms, mode != 0);
+  // plain shapes: a last chunk of fewer environments need not be a 16-byte multiple, and the aligned range around the last
+  // chunk's availability bytes may end beyond the step's block; nor need the arrays of one call start on 16-byte boundaries.
+  // One-step launches take such inputs if their blocks have more than one tile (split-operand kernel -> this one, us): lists of
+  // 5 x 55 observations 3799 environments 29.2 -> 24.0, 9001 with late outcomes 51.2 -> 34.5, 33333 142 -> 81; dense steps of
+  // 16385 x 5 65 -> 44 (one-tile kernel) and 70 -> 44.  The errors against the oracle are the split-operand kernel's (rms of Q
+  // 3.0e-5 to 4.1e-5, of h 2.1e-6, on both): gates and biases are the same fp32 arithmetic, with biases and agent columns
+  // among the products they were 20 to 45 % larger.
+  const int plain = p_in.D % 8 != 0 ? 1 : (p_in.n * p_in.A) % 16 != 0 ? 2 : 0;
+  const bool aligned = reinterpret_cast<uintptr_t>(p_in.obs) % 16 == 0 && reinterpret_cast<uintptr_t>(p_in.avail) % 16 == 0;
+  const bool whole = aligned && (p_in.obs_step_stride * 4) % 16 == 0 && p_in.avail_step_stride % 16 == 0 &&
+                     (plain != 1 || p_in.M % TP_G == 0) && (plain == 0 || ((size_t)p_in.M * p_in.n * p_in.A) % 16 == 0);
+  const bool ragged = !whole;
+  if (ragged) {
+    if (plain == 0 || p_in.T != 1 || !p_in.ragged_ok || reinterpret_cast<uintptr_t>(p_in.obs) % (plain == 1 ? 4 : 16)) return 0;
+    if ((p_in.M + TC_ROWS / p_in.n - 1) / (TC_ROWS / p_in.n) <= sms) return 0;
+  }
+  const TpLayout L = tp_layout(p_in.n, p_in.D, p_in.A, (int)p_in.rl.rec_bytes, p_in.M, sms, mode != 0, 0, TP_SCR, ragged);
+  if (ragged && L.NS < 3) return 0;
   ActorParams p = p_in;
   p.ept = L.ept;  // (tiles of whole chunks for the plain shapes)
   p.num_tiles = (p.M + L.ept - 1) / L.ept;
-  if (reinterpret_cast<uintptr_t>(p.obs) % 16 || reinterpret_cast<uintptr_t>(p.avail) % 16) return 0;
-  if ((p.obs_step_stride * 4) % 16 || p.avail_step_stride % 16) return 0;
-  // plain shapes: a last chunk of fewer environments would not be a 16-byte multiple, and the aligned range around
-  // the last chunk's availability bytes must end inside the step's block
-  if (L.plain == 1 && p.M % TP_G != 0) return 0;
-  if (L.plain != 0 && ((size_t)p.M * p.n * p.A) % 16 != 0) return 0;
   if (p.lagged && (mode != 2 || p.T != 1)) return 0;  // late outcomes: one step per launch over a list
   auto pick = [&](auto nq) {
     constexpr int Q = decltype(nq)::value;
     auto of_mode = [&](auto md) {
       constexpr int MD = decltype(md)::value;
+      if constexpr (MD != 0) {
+        if (ragged) return L.plain == 1 ? actor_tcp_kernel<Q, 1, MD, true> : actor_tcp_kernel<Q, 2, MD, true>;
+      }
       return L.plain == 1 ? actor_tcp_kernel<Q, 1, MD> : L.plain == 2 ? actor_tcp_kernel<Q, 2, MD> : actor_tcp_kernel<Q, 0, MD>;
     };
     return mode == 3 ? of_mode(std::integral_constant<int, 3>()) : mode == 2 ? of_mode(std::integral_constant<int, 2>())
          : mode == 1 ? of_mode(std::integral_constant<int, 1>()) : of_mode(std::integral_constant<int, 0>());
   };
   auto kernel = L.NQ == 16 ? pick(std::integral_constant<int, 16>()) : pick(std::integral_constant<int, 32>());
-  static uint32_t configured[24][SMEM_OPTIN_DEVICES];
+  static uint32_t configured[48][SMEM_OPTIN_DEVICES];
   {
     const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), L.total,
-                                              configured[(L.NQ == 16 ? 0 : 1) + 2 * L.plain + 6 * mode]);
+                                              configured[(L.NQ == 16 ? 0 : 1) + 2 * L.plain + 6 * mode + (ragged ? 24 : 0)]);
     if (e != cudaSuccess) return -(int)e;
   }
   int grid = p.num_tiles < sms ? p.num_tiles : sms;

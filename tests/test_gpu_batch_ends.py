@@ -1,0 +1,66 @@
+"""One-step launches on inputs that start and end inside a 16-byte unit, on the pipelined kernel: against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2205_05248_b200 import binding, workloads
+from referee import RTOL, check_near_ties, near_tie_rows_allowed, row_rel_err
+
+pytestmark = pytest.mark.gpu
+
+# One tile a block at the most goes to the split-operand kernel: the batches have more rows than 148 tiles of 128.  Rows of 55
+# and 31 observations take the word-by-word path (any float is a start), of 24 only the availability may start and end
+# anywhere; 17 actions take the 32-column kernel; one to four environments in the last chunk; availability blocks of 24
+# bytes.
+SHAPES = [dict(E=3785, n=5, D=55, A=12), dict(E=3787, n=5, D=31, A=17), dict(E=3786, n=5, D=24, A=11), dict(E=4811, n=4, D=9, A=6)]
+
+
+def _at(v, offset):
+    """The same tensor, starting `offset` elements behind a 16-byte boundary, at the very end of its allocation."""
+    buf = torch.empty(offset + v.numel(), dtype=v.dtype, device=v.device)
+    out = buf[offset:].view(v.shape)
+    out.copy_(v)
+    return out
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("kind", ["step", "subset", "lagged"])
+def test_inputs_that_start_and_end_anywhere(kind, shape):
+    cfg = workloads.small_config(**{**dict(H=64, L=3, T=6, precision="bf16", env=dict(done_thresh24=1 << 21)), **shape, "C": 2 * shape["E"]})
+    E, n, A, T = cfg["E"], cfg["n"], cfg["A"], cfg["T"]
+    w = workloads.make_weights(cfg)
+    actor = binding.Actor(cfg)
+    actor.set_weights(w)
+    d_in = actor.env_generate(cfg["env"], 0, T)
+    h_in = [v.cpu().numpy() for v in d_in]
+    g_acts, g_q = actor.set_trace(T, want_q=True)
+    sess = oracle.Session(cfg, w, np.arange(E))
+    rng = np.random.default_rng(5)
+    eps, near, greedy = 0.15, 0, 0
+    for t in range(T):
+        M = E if kind == "step" else E - t  # lists of every length modulo four
+        ids = np.arange(E) if kind == "step" else rng.permutation(E)[:M].astype(np.int32)
+        x = [v[t, :M].contiguous() for v in d_in]
+        x[0], x[1] = _at(x[0], t % 4 if cfg["D"] % 8 else 0), _at(x[1], (0, 1, 7, 15, 16, 3)[t])
+        act = (actor.step(*x, eps) if kind == "step" else actor.step_subset(ids, *x, eps) if kind == "subset" else actor.step_lagged(ids, *x, eps)).cpu().numpy()
+        assert actor.step_kernel == "actor_tcp_kernel"
+        q = g_q[t][torch.as_tensor(ids, device=g_q.device, dtype=torch.long)].cpu().numpy()
+        _, tr = (sess.step_lagged if kind == "lagged" else sess.step_subset)(ids, *[v[t, :M] for v in h_in], eps, adopt=act, trace=("q", "action_free", "explore"))
+        err = row_rel_err(q, tr["q"])
+        assert err.max() <= RTOL["bf16"]
+        diff = np.argwhere(tr["action_free"][None] != act[None])
+        check_near_ties(diff, tr["q"][None], q[None], tr["action_free"][None], act[None], tr["explore"][None])
+        near, greedy = near + len(diff), greedy + int((tr["explore"] == 0).sum())
+    assert near <= near_tie_rows_allowed("bf16", greedy), (near, greedy)
+    st, rv = actor.get_state(), actor.ring_view()
+    for k in ("last_action", "slot", "pos", "ep_count"):
+        assert np.array_equal(st[k].cpu().numpy(), getattr(sess, k)), k
+    assert row_rel_err(st["h"].cpu().numpy(), sess.h).max() <= RTOL["bf16"]
+    for k in ("slot_epid", "slot_len", "slot_complete"):
+        assert np.array_equal(rv[k].cpu().numpy(), sess.ring[k]), k
+    written = np.arange(cfg["L"])[None, :] < sess.ring["slot_len"][:, None]
+    for k in ("obs", "avail", "action", "reward", "done"):
+        assert np.array_equal(rv[k].cpu().numpy()[written], sess.ring[k][written]), k
+    assert actor.status()[0] == 0
+    actor.destroy()
