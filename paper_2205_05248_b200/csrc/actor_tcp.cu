@@ -252,7 +252,7 @@ __device__ __forceinline__ void tp_issue_hside(const TpLayout& L, uint32_t sb, u
 // RAGGED (one step per launch, PM != 0): inputs that start (PM 1: observations on any float; availability on any byte) and end
 // anywhere.  The bulk copies take the aligned range around a chunk as far as it lies inside the call's arrays, the load warp's
 // lanes the bytes that are left at the arrays' ends.  These calls have the accurate gate functions, as on the split-operand
-// kernel, which serves them where a block would have one tile at most.
+// kernel, which serves the small batches.
 template <int NQ, int PM, int MODE, bool RAGGED = false>
 __global__ void __launch_bounds__(TP_THREADS, 1)
     actor_tcp_kernel(const __grid_constant__ ActorParams p, const __grid_constant__ TpLayout L) {
@@ -1224,8 +1224,8 @@ int launch_actor_tcp(const ActorParams& p_in, int sms, cudaStream_t stream) {
   const int mode = p_in.env_ids == nullptr ? (p_in.T < 8 ? 3 : 0) : (p_in.lagged ? 2 : 1);
   // plain shapes: a last chunk of fewer environments need not be a 16-byte multiple, and the aligned range around the last
   // chunk's availability bytes may end beyond the step's block; nor need the arrays of one call start on 16-byte boundaries.
-  // One-step launches take such inputs if their blocks have more than one tile (split-operand kernel -> this one, us): lists of
-  // 5 x 55 observations 3799 environments 29.2 -> 24.0, 9001 with late outcomes 51.2 -> 34.5, 33333 142 -> 81; dense steps of
+  // One-step launches take such inputs from half a tile a block on (split-operand kernel -> this one, us): lists of 5 x 55
+  // observations, 801 environments 19.3 -> 19.0, 1801 22.0 -> 21.7, 3601 29.0 -> 24.7, 9001 with late outcomes 51.2 -> 34.5, 33333 142 -> 81; dense steps of
   // 16385 x 5 65 -> 44 (one-tile kernel) and 70 -> 44.  The errors against the oracle are the split-operand kernel's (rms of Q
   // 3.0e-5 to 4.1e-5, of h 2.1e-6, on both): gates and biases are the same fp32 arithmetic, with biases and agent columns
   // among the products they were 20 to 45 % larger.
@@ -1236,7 +1236,7 @@ int launch_actor_tcp(const ActorParams& p_in, int sms, cudaStream_t stream) {
   const bool ragged = !whole;
   if (ragged) {
     if (plain == 0 || p_in.T != 1 || !p_in.ragged_ok || reinterpret_cast<uintptr_t>(p_in.obs) % (plain == 1 ? 4 : 16)) return 0;
-    if ((p_in.M + TC_ROWS / p_in.n - 1) / (TC_ROWS / p_in.n) <= sms) return 0;
+    if ((p_in.M + TC_ROWS / p_in.n - 1) / (TC_ROWS / p_in.n) <= sms / 2) return 0;
   }
   const TpLayout L = tp_layout(p_in.n, p_in.D, p_in.A, (int)p_in.rl.rec_bytes, p_in.M, sms, mode != 0, 0, TP_SCR, ragged);
   if (ragged && L.NS < 3) return 0;

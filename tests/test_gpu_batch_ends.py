@@ -9,11 +9,12 @@ from referee import RTOL, check_near_ties, near_tie_rows_allowed, row_rel_err
 
 pytestmark = pytest.mark.gpu
 
-# One tile a block at the most goes to the split-operand kernel: the batches have more rows than 148 tiles of 128.  Rows of 55
+# Small batches go to the split-operand kernel: these have more rows than 148 tiles of 128, and one a single tile a block.  Rows of 55
 # and 31 observations take the word-by-word path (any float is a start), of 24 only the availability may start and end
 # anywhere; 17 actions take the 32-column kernel; one to four environments in the last chunk; availability blocks of 24
 # bytes.
-SHAPES = [dict(E=3785, n=5, D=55, A=12), dict(E=3787, n=5, D=31, A=17), dict(E=3786, n=5, D=24, A=11), dict(E=4811, n=4, D=9, A=6)]
+SHAPES = [dict(E=3785, n=5, D=55, A=12), dict(E=3787, n=5, D=31, A=17), dict(E=3786, n=5, D=24, A=11), dict(E=4811, n=4, D=9, A=6),
+          dict(E=1931, n=5, D=55, A=12)]
 
 
 def _at(v, offset):
