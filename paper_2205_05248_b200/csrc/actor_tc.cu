@@ -24,6 +24,7 @@
 //
 // Shared memory: the packed weights (bf16 matrices in operand layout, fp32 bias/one-hot tables), one x/y
 // operand buffer, one hidden-state operand buffer, two sets of ring records (double-buffered over steps).
+#include <cmath>
 #include <cstring>
 #include <vector>
 
@@ -73,12 +74,24 @@ void tc_pack_weights(int n, int D, int A, int H, const float* W1, const float* b
     const uint16_t b = bf16_bits(v);
     memcpy(o + base + operand_offset(N, row, k), &b, 2);
   };
-  // a fp32 value as three bf16 pieces at k0, k0+1, k0+2
+  // a fp32 value as three bf16 pieces at k0, k0+1, k0+2, which add up to it: each the nearest to what is left, beyond the
+  // largest finite bf16 value the next towards zero (the nearest would be infinite, or two of them add up to infinity); an
+  // infinity or a NaN is one piece
   auto put3 = [&](uint32_t base, int N, int row, int k0, float v) {
-    const float p0 = bf16_value(v), p1 = bf16_value(v - p0), p2 = bf16_value(v - p0 - p1);
-    put(base, N, row, k0, p0);
-    put(base, N, row, k0 + 1, p1);
-    put(base, N, row, k0 + 2, p2);
+    float largest;
+    const uint32_t largest_bits = 0x7F7F0000u;
+    memcpy(&largest, &largest_bits, 4);
+    const bool cut = std::fabs(v) > largest;
+    for (int i = 0; i < 3; ++i) {
+      uint32_t u;
+      memcpy(&u, &v, 4);
+      const uint16_t b = cut ? (uint16_t)(u >> 16) : bf16_bits(v);
+      memcpy(o + base + operand_offset(N, row, k0 + i), &b, 2);
+      u = (uint32_t)b << 16;
+      float piece;
+      memcpy(&piece, &u, 4);
+      v = std::isfinite(piece) ? v - piece : 0.f;
+    }
   };
   for (int j = 0; j < H; ++j) {
     for (int k = 0; k < D; ++k) put(L.off_W1, H, j, k, W1[(size_t)j * I + k]);

@@ -129,7 +129,7 @@ static TpLayout tp_layout(int n, int D, int A, int rec_bytes, int M = 0, int sms
   L.off_rowenv = o; o += TC_ROWS * 4;
   L.off_dstp = o; o += TP_DST_DEPTH * 32 * 8;
   L.off_tdst = o; o += 32 * 8;
-  L.off_bias = o; o += ragged ? 4u * TC_H * 4 + (uint32_t)n * TC_TAB * 4 : 0;  // (a multiple of 16)
+  L.off_bias = o; o += ragged ? 4u * TC_H * 4 + (uint32_t)n * TC_TAB * 4 + (uint32_t)L.NQ * 4 : 0;  // (a multiple of 16)
   L.off_bar = o; o += (uint32_t)((sizeof(TpBars) + 15) & ~15u);
   L.off_stage = o;
   // plain shapes: the converters also lay observations and availability bytes out as the records want them (each
@@ -232,7 +232,7 @@ __device__ __forceinline__ void tp_issue_hside(const TpLayout& L, uint32_t sb, u
       mma_bf16_ts(tmem + TM_HN, tmem + TMP_H + ks * 8, d_Whh_n + ks * TP_K_G, id64, ks > 0);
     }
     if (!RAGGED) mma_bf16(tmem + TM_HN, d_oh, d_Bhn, id64, 1);
-    mma_bf16(tmem + qcol, d_oh, d_W2b, idesc_bf16_f32(128, NQ), 0);
+    if (!RAGGED) mma_bf16(tmem + qcol, d_oh, d_W2b, idesc_bf16_f32(128, NQ), 0);
   }
   __syncwarp();
 }
@@ -389,9 +389,9 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
         if (elect_one()) {
           const uint64_t d_W2 = smem_desc(sb + L.off_W2, NQ * 16, 128);
 #pragma unroll
-          for (int ks = 0; ks < 4; ++ks)  // part 0 holds the bias already; parts 1..3 start from zero
+          for (int ks = 0; ks < 4; ++ks)  // part 0 holds the bias already (ragged: starts from zero); parts 1..3 start from zero
             mma_bf16_ts(tmem + qcol + (NQ == 16 ? ks * NQ : 0), tmem + TMP_H + ks * 8, d_W2 + ks * ((2 * NQ * 16) >> 4), idesc_bf16_f32(128, NQ),
-                     (NQ == 16 && ks > 0) ? 0 : 1);
+                     ks == 0 ? !RAGGED : NQ != 16);
           mma_commit(&B->fc2d);
         }
         __syncwarp();
@@ -913,12 +913,14 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
     }
     float* bias_s = reinterpret_cast<float*>(smem + L.off_bias);  // [4][64]: reset and update (halved), candidate input, candidate hidden
     float* tab_a = bias_s + 4 * TC_H;                             // [n][68]: b1 + W1[:, D + agent]
+    float* b2_s = tab_a + n * TC_TAB;                             // [NQ]
     if constexpr (RAGGED) {
       // from the weight image, where a bias is three bf16 pieces
       mbar_wait(&B->wload, 0, abortf);
       auto piece = [&](uint32_t off) { return __uint_as_float((uint32_t)*reinterpret_cast<const uint16_t*>(smem + off) << 16); };
       auto bias_at = [&](uint32_t off) { return (piece(off) + piece(off + 2)) + piece(off + 4); };
       if (tid < 4 * TC_H) bias_s[tid] = tid < 3 * TC_H ? bias_at(L.off_Bg + (uint32_t)tid * 16u) : bias_at(L.off_Bhn + (uint32_t)(tid - 3 * TC_H) * 16u);
+      if (tid < NQ) b2_s[tid] = bias_at(L.off_W2 + (uint32_t)(8 * NQ + tid) * 16u);
       const uint32_t w1x = L.off_W1 + (uint32_t)L.nchunk * TP_LBO_W1;
       for (int i = tid; i < n * TC_H; i += 256) {
         const int a = i / TC_H, j = i - a * TC_H, k = 3 + a;
@@ -1116,6 +1118,10 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
               qv[a] = __float_as_uint((__uint_as_float(qv[a]) + __uint_as_float(q1[a])) + (__uint_as_float(q2[a]) + __uint_as_float(q3[a])));
           }
           tmem_ld_wait();
+          if constexpr (RAGGED) {
+#pragma unroll
+            for (int a = 0; a < NQ; ++a) qv[a] = __float_as_uint(__uint_as_float(qv[a]) + b2_s[a]);
+          }
           tc_fence_before_sync();
           if (is_row) {
             mbar_wait(&B->selready[it & 3], (it >> 2) & 1, abortf);
