@@ -65,7 +65,7 @@ struct TpLayout {
   uint32_t prefix_bytes, tail_bytes, chunk_bytes, obs_bytes, av_bytes, rs_env, rs_bytes, off_rstage;
   uint32_t off_W1, off_Wih, off_Whh, off_Bg, off_Bhn, off_W2, off_tab_la, wbytes;
   uint32_t off_x, off_scr, off_oh, off_stage, off_tail, off_sel, off_la, off_close, off_closeany, off_rowenv, off_dstp, off_tdst, off_bar, total;
-  uint32_t av_off, off_bias;  // availability within a staged chunk; fp32 biases and agent columns (ragged variant)
+  uint32_t av_off, off_bias;  // availability within a staged chunk; fp32 biases and agent columns (accurate gates)
 };
 
 struct TpBars {
@@ -82,7 +82,7 @@ struct TpBars {
 // M, sms: the launch's batch and the number of blocks it may use (0: the largest tiles, for the shape check).
 // fastx: the launch moves its hidden-state rows through a scratch (modes 1 to 3 of the kernel).
 static TpLayout tp_layout(int n, int D, int A, int rec_bytes, int M = 0, int sms = 0, bool fastx = true,
-                          uint32_t reserve = 0, uint32_t scr_warp = TP_SCR, bool ragged = false) {
+                          uint32_t reserve = 0, uint32_t scr_warp = TP_SCR, bool ragged = false, bool acc = false) {
   const TcLayout W = tc_layout(n, D, A, rec_bytes);
   TpLayout L;
   memset(&L, 0, sizeof(L));
@@ -129,7 +129,7 @@ static TpLayout tp_layout(int n, int D, int A, int rec_bytes, int M = 0, int sms
   L.off_rowenv = o; o += TC_ROWS * 4;
   L.off_dstp = o; o += TP_DST_DEPTH * 32 * 8;
   L.off_tdst = o; o += 32 * 8;
-  L.off_bias = o; o += ragged ? 4u * TC_H * 4 + (uint32_t)n * TC_TAB * 4 + (uint32_t)L.NQ * 4 : 0;  // (a multiple of 16)
+  L.off_bias = o; o += acc ? 4u * TC_H * 4 + (uint32_t)n * TC_TAB * 4 + (uint32_t)L.NQ * 4 : 0;  // (a multiple of 16)
   L.off_bar = o; o += (uint32_t)((sizeof(TpBars) + 15) & ~15u);
   L.off_stage = o;
   // plain shapes: the converters also lay observations and availability bytes out as the records want them (each
@@ -187,8 +187,8 @@ constexpr uint64_t TP_K_A = (2 * TC_LBO_A) >> 4, TP_K_X = (2 * TC_LBO_X) >> 4, T
                    TP_K_G = (2 * TP_LBO_G) >> 4;                       // descriptor increments of one K = 16 step
 
 // fc1 of one step: observations x W1, then the one-hot tile x (bias pieces, agent-id columns); commits to fc1d.
-// (RAGGED, here and below: no bias and no agent column among the products; the epilogues add them in fp32.)
-template <bool RAGGED>
+// (ACC, here and below: no bias and no agent column among the products; the epilogues add them in fp32.)
+template <bool ACC>
 __device__ __forceinline__ void tp_issue_fc1(const TpLayout& L, uint32_t sb, uint32_t tmem, uint64_t* fc1d) {
   using namespace tc;
   tc_fence_after_sync();
@@ -206,7 +206,7 @@ __device__ __forceinline__ void tp_issue_fc1(const TpLayout& L, uint32_t sb, uin
     }
     if (ks < ks_obs) mma_bf16(tmem + TM_FC1, d_x + ks * TP_K_X, d_W1 + ks * TP_K_W1, id64, ks > 0);
 #pragma unroll 1
-    for (ks = 0; ks < (RAGGED ? 0 : ks_oh); ++ks) mma_bf16(tmem + TM_FC1, d_oh + ks * TP_K_A, d_W1oh + ks * TP_K_W1, id64, 1);
+    for (ks = 0; ks < (ACC ? 0 : ks_oh); ++ks) mma_bf16(tmem + TM_FC1, d_oh + ks * TP_K_A, d_W1oh + ks * TP_K_W1, id64, 1);
     mma_commit(fc1d);
   }
   __syncwarp();
@@ -214,7 +214,7 @@ __device__ __forceinline__ void tp_issue_fc1(const TpLayout& L, uint32_t sb, uin
 
 // h-side gate products of one step: the first MMA seeds r | z | candidate-input with their biases (contiguous in
 // tensor memory: one N = 192 accumulator), the last one seeds the step's Q accumulator with the output bias.
-template <int NQ, bool RAGGED>
+template <int NQ, bool ACC>
 __device__ __forceinline__ void tp_issue_hside(const TpLayout& L, uint32_t sb, uint32_t tmem, uint32_t qcol) {
   using namespace tc;
   tc_fence_after_sync();
@@ -225,14 +225,14 @@ __device__ __forceinline__ void tp_issue_hside(const TpLayout& L, uint32_t sb, u
     const uint64_t d_Bg = smem_desc(sb + L.off_Bg, TP_LBO_G, 128), d_Bhn = smem_desc(sb + L.off_Bhn, TP_LBO_W1, 128);
     const uint64_t d_W2b = smem_desc(sb + L.off_W2 + 8u * NQ * 16, NQ * 16, 128);            // bias pieces of W2: k-chunks 8, 9
     const uint32_t id64 = idesc_bf16_f32(128, 64), id128 = idesc_bf16_f32(128, 128), id192 = idesc_bf16_f32(128, 192);
-    if (!RAGGED) mma_bf16(tmem + TM_R, d_oh, d_Bg, id192, 0);
+    if (!ACC) mma_bf16(tmem + TM_R, d_oh, d_Bg, id192, 0);
 #pragma unroll
     for (int ks = 0; ks < 4; ++ks) {
-      mma_bf16_ts(tmem + TM_R, tmem + TMP_H + ks * 8, d_Whh + ks * TP_K_G, id128, !RAGGED || ks > 0);
+      mma_bf16_ts(tmem + TM_R, tmem + TMP_H + ks * 8, d_Whh + ks * TP_K_G, id128, !ACC || ks > 0);
       mma_bf16_ts(tmem + TM_HN, tmem + TMP_H + ks * 8, d_Whh_n + ks * TP_K_G, id64, ks > 0);
     }
-    if (!RAGGED) mma_bf16(tmem + TM_HN, d_oh, d_Bhn, id64, 1);
-    if (!RAGGED) mma_bf16(tmem + qcol, d_oh, d_W2b, idesc_bf16_f32(128, NQ), 0);
+    if (!ACC) mma_bf16(tmem + TM_HN, d_oh, d_Bhn, id64, 1);
+    if (!ACC) mma_bf16(tmem + qcol, d_oh, d_W2b, idesc_bf16_f32(128, NQ), 0);
   }
   __syncwarp();
 }
@@ -251,9 +251,10 @@ __device__ __forceinline__ void tp_issue_hside(const TpLayout& L, uint32_t sb, u
 // (1.2 %) than the transition saves.
 // RAGGED (one step per launch, PM != 0): inputs that start (PM 1: observations on any float; availability on any byte) and end
 // anywhere.  The bulk copies take the aligned range around a chunk as far as it lies inside the call's arrays, the load warp's
-// lanes the bytes that are left at the arrays' ends.  These calls have the accurate gate functions, as on the split-operand
-// kernel, which serves the small batches.
-template <int NQ, int PM, int MODE, bool RAGGED = false>
+// lanes the bytes that are left at the arrays' ends.
+// ACC (ragged only): the accurate gate functions, biases and agent columns in fp32, as on the split-operand kernel, which
+// serves these calls' small batches; without it the arithmetic is the one-tile kernel's.
+template <int NQ, int PM, int MODE, bool RAGGED = false, bool ACC = false>
 __global__ void __launch_bounds__(TP_THREADS, 1)
     actor_tcp_kernel(const __grid_constant__ ActorParams p, const __grid_constant__ TpLayout L) {
   constexpr bool LIST = MODE == 1 || MODE == 2, LAG = MODE == 2, FASTX = MODE != 0;
@@ -340,7 +341,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
       mbar_wait(&B->wload, 0, abortf);
       if (total > 0) {
         mbar_wait(&B->xready, 0, abortf);
-        tp_issue_fc1<RAGGED>(L, sb, tmem, &B->fc1d);
+        tp_issue_fc1<ACC>(L, sb, tmem, &B->fc1d);
       }
       for (int g = 0, s = 0; g < total; ++g) {
         const uint32_t par = (uint32_t)g & 1u;
@@ -353,7 +354,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
           } else {
             mbar_wait(&B->stepd, par ^ 1u, abortf);
           }
-          tp_issue_hside<NQ, RAGGED>(L, sb, tmem, qcol);
+          tp_issue_hside<NQ, ACC>(L, sb, tmem, qcol);
         }
         mbar_wait(&B->yready, par, abortf);
         tc_fence_after_sync();
@@ -361,7 +362,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
           const uint64_t d_Wih = smem_desc(sb + L.off_Wih, TP_LBO_G, 128);
 #pragma unroll
           for (int ks = 0; ks < 4; ++ks) {
-            if (RAGGED && ks == 0) {  // the candidate-input columns start here
+            if (ACC && ks == 0) {  // the candidate-input columns start here
               mma_bf16_ts(tmem + TM_R, tmem + TMP_Y, d_Wih, idesc_bf16_f32(128, 128), 1);
               mma_bf16_ts(tmem + TM_IN, tmem + TMP_Y, d_Wih + ((2 * TC_H * 16) >> 4), idesc_bf16_f32(128, 64), 0);
             } else {
@@ -378,7 +379,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
           // one lane looks (lanes looking separately could disagree and split the warp's control flow)
           const uint32_t ready = __shfl_sync(0xFFFFFFFFu, lane == 0 ? (uint32_t)mbar_test_wait(&B->xready, par ^ 1u) | (uint32_t)mbar_test_wait(&B->hready, par) << 1 : 0u, 0);
           if (ready & 1u) {
-            tp_issue_fc1<RAGGED>(L, sb, tmem, &B->fc1d);
+            tp_issue_fc1<ACC>(L, sb, tmem, &B->fc1d);
             pending = false;
           } else if (ready & 2u) {
             break;
@@ -389,15 +390,15 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
         if (elect_one()) {
           const uint64_t d_W2 = smem_desc(sb + L.off_W2, NQ * 16, 128);
 #pragma unroll
-          for (int ks = 0; ks < 4; ++ks)  // part 0 holds the bias already (ragged: starts from zero); parts 1..3 start from zero
+          for (int ks = 0; ks < 4; ++ks)  // part 0 holds the bias already (accurate gates: starts from zero); parts 1..3 start from zero
             mma_bf16_ts(tmem + qcol + (NQ == 16 ? ks * NQ : 0), tmem + TMP_H + ks * 8, d_W2 + ks * ((2 * NQ * 16) >> 4), idesc_bf16_f32(128, NQ),
-                     ks == 0 ? !RAGGED : NQ != 16);
+                     ks == 0 ? !ACC : NQ != 16);
           mma_commit(&B->fc2d);
         }
         __syncwarp();
         if (pending) {
           mbar_wait(&B->xready, par ^ 1u, abortf);
-          tp_issue_fc1<RAGGED>(L, sb, tmem, &B->fc1d);
+          tp_issue_fc1<ACC>(L, sb, tmem, &B->fc1d);
         }
         // The next step's h-side products need only the new hidden state, which is in place unless an episode
         // of this tile ends with this step (its rows are cleared after fc2): issue them now, off the critical
@@ -408,7 +409,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
         } else {
           // (published by the load warp before this step's inputs were requested: ordered before the fc1 operand)
           if (closeany_s[g & (TP_DST_DEPTH - 1)] == 0) {
-            tp_issue_hside<NQ, RAGGED>(L, sb, tmem, TM_Q + (par ^ 1u) * tp_qstride(NQ));
+            tp_issue_hside<NQ, ACC>(L, sb, tmem, TM_Q + (par ^ 1u) * tp_qstride(NQ));
             hside_issued = true;
           }
         }
@@ -914,7 +915,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
     float* bias_s = reinterpret_cast<float*>(smem + L.off_bias);  // [4][64]: reset and update (halved), candidate input, candidate hidden
     float* tab_a = bias_s + 4 * TC_H;                             // [n][68]: b1 + W1[:, D + agent]
     float* b2_s = tab_a + n * TC_TAB;                             // [NQ]
-    if constexpr (RAGGED) {
+    if constexpr (ACC) {
       // from the weight image, where a bias is three bf16 pieces
       mbar_wait(&B->wload, 0, abortf);
       auto piece = [&](uint32_t off) { return __uint_as_float((uint32_t)*reinterpret_cast<const uint16_t*>(smem + off) << 16); };
@@ -1005,7 +1006,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
             for (int q = 0; q < 4; ++q) {
               float4 l4 = make_float4(0.f, 0.f, 0.f, 0.f);
               if (last >= 0) l4 = *reinterpret_cast<const float4*>(tlr + c16 * 16 + 4 * q);
-              if constexpr (RAGGED) {
+              if constexpr (ACC) {
                 const float4 a4 = *reinterpret_cast<const float4*>(tab_a + ai * TC_TAB + cb + c16 * 16 + 4 * q);
                 l4 = make_float4(a4.x + l4.x, a4.y + l4.y, a4.z + l4.z, a4.w + l4.w);
               }
@@ -1046,7 +1047,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
             tmem_ld_wait();
             if (c8 + 1 < 4) request(c8 + 1, g[(c8 + 1) & 1]);
             uint32_t(&v)[4][8] = g[c8 & 1];
-            if constexpr (RAGGED) {
+            if constexpr (ACC) {
 #pragma unroll
               for (int j = 0; j < 8; j += 2) {
                 float a2[4][2];
@@ -1118,7 +1119,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
               qv[a] = __float_as_uint((__uint_as_float(qv[a]) + __uint_as_float(q1[a])) + (__uint_as_float(q2[a]) + __uint_as_float(q3[a])));
           }
           tmem_ld_wait();
-          if constexpr (RAGGED) {
+          if constexpr (ACC) {
 #pragma unroll
             for (int a = 0; a < NQ; ++a) qv[a] = __float_as_uint(__uint_as_float(qv[a]) + b2_s[a]);
           }
@@ -1244,7 +1245,10 @@ int launch_actor_tcp(const ActorParams& p_in, int sms, cudaStream_t stream) {
     if (plain == 0 || p_in.T != 1 || !p_in.ragged_ok || reinterpret_cast<uintptr_t>(p_in.obs) % (plain == 1 ? 4 : 16)) return 0;
     if ((p_in.M + TC_ROWS / p_in.n - 1) / (TC_ROWS / p_in.n) <= sms / 2) return 0;
   }
-  const TpLayout L = tp_layout(p_in.n, p_in.D, p_in.A, (int)p_in.rl.rec_bytes, p_in.M, sms, mode != 0, 0, TP_SCR, ragged);
+  // Dense steps whose launches of several steps and whose small batches go to the one-tile kernel (rows of whole 16-byte units) have
+  // its arithmetic: a rollout is the same however it is divided.  The others have the accurate gates of the split-operand kernel.
+  const bool acc = ragged && !(mode == 3 && p_in.one_tile);
+  const TpLayout L = tp_layout(p_in.n, p_in.D, p_in.A, (int)p_in.rl.rec_bytes, p_in.M, sms, mode != 0, 0, TP_SCR, ragged, acc);
   if (ragged && L.NS < 3) return 0;
   ActorParams p = p_in;
   p.ept = L.ept;  // (tiles of whole chunks for the plain shapes)
@@ -1255,7 +1259,10 @@ int launch_actor_tcp(const ActorParams& p_in, int sms, cudaStream_t stream) {
     auto of_mode = [&](auto md) {
       constexpr int MD = decltype(md)::value;
       if constexpr (MD != 0) {
-        if (ragged) return L.plain == 1 ? actor_tcp_kernel<Q, 1, MD, true> : actor_tcp_kernel<Q, 2, MD, true>;
+        if constexpr (MD == 3) {
+          if (ragged && !acc) return actor_tcp_kernel<Q, 2, MD, true>;  // (the one-tile kernel has no plain 1)
+        }
+        if (ragged) return L.plain == 1 ? actor_tcp_kernel<Q, 1, MD, true, true> : actor_tcp_kernel<Q, 2, MD, true, true>;
       }
       return L.plain == 1 ? actor_tcp_kernel<Q, 1, MD> : L.plain == 2 ? actor_tcp_kernel<Q, 2, MD> : actor_tcp_kernel<Q, 0, MD>;
     };
@@ -1263,10 +1270,10 @@ int launch_actor_tcp(const ActorParams& p_in, int sms, cudaStream_t stream) {
          : mode == 1 ? of_mode(std::integral_constant<int, 1>()) : of_mode(std::integral_constant<int, 0>());
   };
   auto kernel = L.NQ == 16 ? pick(std::integral_constant<int, 16>()) : pick(std::integral_constant<int, 32>());
-  static uint32_t configured[48][SMEM_OPTIN_DEVICES];
+  static uint32_t configured[72][SMEM_OPTIN_DEVICES];
   {
     const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), L.total,
-                                              configured[(L.NQ == 16 ? 0 : 1) + 2 * L.plain + 6 * mode + (ragged ? 24 : 0)]);
+                                              configured[(L.NQ == 16 ? 0 : 1) + 2 * L.plain + 6 * mode + (ragged ? 24 : 0) + (acc ? 24 : 0)]);
     if (e != cudaSuccess) return -(int)e;
   }
   int grid = p.num_tiles < sms ? p.num_tiles : sms;

@@ -79,7 +79,8 @@ struct ActorParams {
   uint64_t agent_type_bits;
   int32_t* type_count;      // [E] types of an environment that are done with the launch (split-operand kernel, zero between launches)
   int32_t early;            // host only: the launch may start beside the kernel before it (see launch_overlapped)
-  int32_t ragged_ok;        // host only: inputs that the pipelined kernel takes with accurate gates (see launch_actor_tcp) may go there
+  int32_t ragged_ok;        // host only: inputs off 16-byte boundaries may go to the pipelined kernel (see launch_actor_tcp)
+  int32_t one_tile;         // host only: the one-tile kernel takes dense launches of the actor
 };
 
 // Everything the episode sampler needs (ring_sample.cu).  Passed by value.

@@ -676,9 +676,10 @@ static void fill_params(marl_actor* a, ActorParams& p) {
   p.trace_q = a->trace_q;
   p.trace_first = a->trace_next;
   p.trace_cap = (a->trace_actions || a->trace_q) ? a->trace_cap : 0;
+  p.ragged_ok = a->use_tcs ? 1 : 0;  // (kernels asked for by name fall back to the CUDA-core kernel)
+  p.one_tile = a->use_tc ? 1 : 0;
   // The first launch on a published image waits for everything before it; the later ones find the image in place and may
   // load it while the kernel before them still runs.
-  p.ragged_ok = a->use_tcs ? 1 : 0;  // (kernels asked for by name fall back to the CUDA-core kernel)
   p.early = a->image_fresh ? 0 : 1;
   a->image_fresh = false;
 }

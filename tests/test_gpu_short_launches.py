@@ -64,3 +64,38 @@ def test_lists_of_several_tiles_a_block_equal_full_steps():
     for a in actors:
         assert a.status()[0] == 0
         a.destroy()
+
+
+# availability of a step that is no 16-byte multiple: one-step launches run here, longer ones on the one-tile kernel
+@pytest.mark.parametrize("shape", [dict(E=3785, n=5, D=24, A=11), dict(E=2999, n=7, D=32, A=17)])
+def test_one_step_launches_of_odd_batches_equal_a_long_one(shape):
+    """A rollout of a batch that is no 16-byte multiple is the same however it is divided: state and choices bit by bit, Q up to the
+    order of its sum."""
+    cfg = workloads.small_config(**{**dict(H=64, L=5, T=14, precision="bf16", env=dict(done_thresh24=1 << 21)), **shape, "C": 2 * shape["E"]})
+    w = workloads.make_weights(cfg)
+    long, short = binding.Actor(cfg), binding.Actor(cfg)
+    staged = long.env_generate(cfg["env"], 0, cfg["T"])
+    for a in (long, short):
+        a.set_weights(w)
+    long.rollout_staged(*staged, cfg["T"], 1.0)
+    t, kernels = 0, set()
+    for part in (1, 1, 4, 1, 3, 1, 2, 1):
+        short.rollout_staged(*[x[t:t + part].clone() for x in staged], part, 1.0)
+        kernels.add((part == 1, short.step_kernel))
+        t += part
+    assert t == cfg["T"] and kernels == {(True, "actor_tcp_kernel"), (False, "actor_tc_kernel")} and long.step_kernel == "actor_tc_kernel"
+    torch.cuda.synchronize()
+    s, u, rs, ru = long.get_state(), short.get_state(), long.ring_view(), short.ring_view()
+    for k in ("h", "last_action", "slot", "pos", "ep_count"):
+        assert torch.equal(s[k], u[k]), k
+    written = torch.arange(cfg["L"], device=s["h"].device)[None, :] < rs["slot_len"][:, None]
+    for k in ("slot_epid", "slot_len", "slot_complete"):
+        assert torch.equal(rs[k], ru[k]), k
+    for k in ("obs", "avail", "action", "reward", "done"):
+        assert torch.equal(rs[k][written], ru[k][written]), k
+    # two orders of 67 terms: each is off by at most 66 roundings (or cuts, 2^-23) of partial sums that the terms' magnitudes bound
+    bound = 2 * 66 * 2.0 ** -23 * float((np.abs(w["W2"]).sum(axis=1) + np.abs(w["b2"])).max())
+    assert float((rs["q"][written] - ru["q"][written]).abs().max()) <= bound
+    assert long.status() == short.status() and long.status()[0] == 0
+    long.destroy()
+    short.destroy()
