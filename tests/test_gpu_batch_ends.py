@@ -65,3 +65,26 @@ def test_inputs_that_start_and_end_anywhere(kind, shape):
         assert np.array_equal(rv[k].cpu().numpy()[written], sess.ring[k][written]), k
     assert actor.status()[0] == 0
     actor.destroy()
+
+
+@pytest.mark.parametrize("kind", ["step", "lagged"])
+def test_staging_slots_that_held_the_ends_of_an_array(kind):
+    """Four tiles a block: the slots that held an array's first and last bytes, which no bulk copy brings, are filled again by bulk
+    copies.  Where the arrays start changes which bytes those are and nothing else."""
+    cfg = workloads.small_config(H=64, L=4, T=4, precision="bf16", env=dict(done_thresh24=1 << 21), E=11999, n=5, D=55, A=12, C=11999)
+    ids = np.random.default_rng(3).permutation(cfg["E"]).astype(np.int32)
+    got = []
+    for offset in (1, 2, 3):
+        a = binding.Actor(cfg)
+        a.set_weights(workloads.make_weights(cfg))
+        x = a.env_generate(cfg["env"], 0, cfg["T"])
+        for t in range(cfg["T"]):
+            inputs = [_at(v[t], o) for v, o in zip(x, (offset, 5 * offset, 0, 0))]
+            a.step(*inputs, 0.1) if kind == "step" else a.step_lagged(ids, *inputs, 0.1)
+            assert a.step_kernel == "actor_tcp_kernel"
+        torch.cuda.synchronize()
+        assert a.status()[0] == 0
+        got.append((a.get_state()["h"].clone(), a.ring_mem.clone()))
+        a.destroy()
+    for h, ring in got[1:]:
+        assert torch.equal(h, got[0][0]) and torch.equal(ring, got[0][1])
