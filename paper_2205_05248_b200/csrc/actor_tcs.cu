@@ -376,7 +376,7 @@ __device__ __forceinline__ uint32_t ts_lo(uint32_t addr, uint32_t lbo) { return 
 
 }  // namespace
 
-template <int NS, int NQ, int H, bool FAST = false>
+template <int NS, int NQ, int H, bool TYPED, bool FAST = false>
 __global__ void __launch_bounds__(TS_THREADS, 1)
     actor_tcs_kernel(const __grid_constant__ ActorParams p, const __grid_constant__ TsLayout L) {
   using namespace tc;
@@ -390,9 +390,10 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
   constexpr uint32_t TSM_Y = TSM_HOP + NS * H / 2;
   constexpr uint32_t FC1 = H == 64 ? 96 : 0;     // fc1's accumulator: the candidate-input columns, or buffer 0
   // Registers (setmaxnreg): launched with 96 a thread (640 * 96 = 61440); afterwards
-  // 256 * 128 + 256 * 88 + 128 * 48 = 61440, at one piece and hidden 128 256 * 136 + 256 * 72 + 128 * 64: there the epilogue
-  // and the issuing warp spill less (16384 environments x 8 agents x 64 steps 3600 -> 3405 us).
-  constexpr bool WIDE = NS == 1 && H == 128;
+  // 256 * 128 + 256 * 88 + 128 * 48 = 61440, at one piece and hidden 128 256 * 136 + 256 * 72 + 128 * 64: there the epilogue and
+  // the issuing warp spill less.  (bf16, accurate gates, narrow -> wide split: 70 environments x 3 agents x 78 steps 595 -> 583 us,
+  // 4001 x 5 x 16 steps 320 -> 323.  Per-type networks keep the narrow one: 1024 x 5 agents x 64 steps 653 us, 664.)
+  constexpr bool WIDE = NS == 1 && H == 128 && !TYPED;
   constexpr int REGS_EPI = WIDE ? 136 : 128, REGS_PREP = WIDE ? 72 : 88, REGS_SVC = WIDE ? 64 : 48;
   extern __shared__ __align__(1024) uint8_t smem[];
   TsBars* B = reinterpret_cast<TsBars*>(smem + L.off_bar);
@@ -412,7 +413,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n = p.n, D = p.D, A = p.A, T = p.T, ept = L.ept;
   const bool lag = p.lagged != 0;
-  const int ntypes = L.ntypes;
+  const int ntypes = TYPED ? L.ntypes : 1;
   const uint32_t rec_bytes = p.rl.rec_bytes;
 
   if (tid == 0) {
@@ -442,20 +443,32 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = B->tmem_base;
+  // With one network a tile has the rows of all n agents.  The input and epilogue warps of most variants take that n from a register
+  // that the compiler does not know to be the parameter: it then keeps fewer of a tile's addresses alive across the steps (bf16,
+  // 40001 environments x 3 agents x 16 steps 635 -> 623 us; 4001 x 3 with 20 actions at hidden 128 200 -> 194; fp32 at hidden 128,
+  // 2001 x 8, 462 -> 456).  Not with the hardware's gates (2001 x 8 agents x 32 steps 246 -> 253) and in fp32 at hidden 64 (one step of
+  // 9001 x 5 agents 52.0 -> 52.4).
+  constexpr bool HIDE_NT = !TYPED && !FAST && !(NS == 3 && H == 64);
   auto rows_per_env = [&](int typ) -> int {  // of a pass: the agents of its unit type
     int nt = ntypes > 1 ? 0 : n;
     if (ntypes > 1)
       for (int i = 0; i < n; ++i) nt += (int)((p.agent_type_bits >> (2 * i)) & 3ull) == typ ? 1 : 0;
     return nt;
   };
-  // Work units: the tiles of type 0, then those of type 1, ...; a block takes every gridDim.x-th.
+  // Work units: the tiles of type 0, then those of type 1, ...; a block takes every gridDim.x-th.  With one network nothing of
+  // this is left in the kernel: walking types at run time cost shared networks up to 4 % (fp32 at hidden 128, 2001 environments x
+  // 8 agents x 16 steps, 481 against 457 us; bf16, 4001 x 5 agents at hidden 128, 339 against 319).
   const int my_tiles = (p.num_tiles * ntypes - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;
   auto unit_at = [&](int& tile, int& typ) -> bool {  // moves a tile number beyond its type's tiles on to the next type
-    while (tile >= p.num_tiles) {
-      tile -= p.num_tiles;
-      if (++typ == ntypes) return false;
+    if constexpr (TYPED) {
+      while (tile >= p.num_tiles) {
+        tile -= p.num_tiles;
+        if (++typ == ntypes) return false;
+      }
+      return true;
+    } else {
+      return tile < p.num_tiles;
     }
-    return true;
   };
 
   if (warp >= 16) {
@@ -478,7 +491,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
       const uint32_t x_st = (uint32_t)nk1 * x_ks;
       constexpr uint32_t y_st = KH * x_ks;
       uint32_t g = 0, ri = 0, rpar = 0;  // steps so far; ring slot and its parity
-      uint32_t loads = 0;  // networks loaded so far
+      uint32_t loads = TYPED ? 0 : 1;  // networks loaded so far
       bool first = true;
 
       // slice i of the step: its address once it is in shared memory
@@ -549,13 +562,17 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
         __syncwarp();
       };
 
-      for (int tile = blockIdx.x, typ = 0, cur = -1; unit_at(tile, typ); tile += gridDim.x) {
-        if (typ != cur) {
-          cur = typ;
-          first = true;
-          if (loads++ > 0) __syncthreads();  // every role has left the previous type
-        }
-        for (int s = 0; s < T; ++s, ++g, first = false) {
+      // The steps of all tiles of a type are one loop: this warp has few registers, and of tile and step only the number of
+      // steps left stays alive (fp32 at hidden 128, 2001 environments x 8 agents x 16 steps: 477 us with a loop over tiles around
+      // one over steps, 460 with this one; hidden 128 in bf16, the same rows x 32 steps, 253 and 244).
+      for (int typ = 0, tile = blockIdx.x; typ < ntypes; ++typ, tile -= p.num_tiles) {
+        if (TYPED && tile >= p.num_tiles) continue;   // no tile of this type is the block's
+        if (TYPED && loads++ > 0) __syncthreads();    // every role has left the previous type
+        const int tiles = (p.num_tiles - 1 - tile) / (int)gridDim.x + 1;
+        if (TYPED) tile += tiles * (int)gridDim.x;
+        first = true;
+#pragma unroll 1
+        for (int left = tiles * T; left > 0; --left, ++g, first = false) {
           const uint32_t par = g & 1;
           // ---- fc1 ----
           if (H == 64) {
@@ -720,8 +737,11 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
       // =========================== weight warp ===========================
       uint32_t ri = 0, rpar = 1, used = 0;
       for (int tile = blockIdx.x, typ = 0, cur = -1; unit_at(tile, typ); tile += gridDim.x) {
-        if (typ == cur) continue;
-        if (cur >= 0) __syncthreads();
+        if (typ == cur) {
+          if (!TYPED) break;
+          continue;
+        }
+        if (TYPED && cur >= 0) __syncthreads();
         cur = typ;
         const uint8_t* img = reinterpret_cast<const uint8_t*>(p.wsplit) + (size_t)typ * p.wsplit_stride;
         const uint8_t* sl = img + L.base_bytes;
@@ -758,7 +778,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
             }
         }
       }
-    } else {
+    } else if (TYPED) {
       for (int tile = blockIdx.x, typ = 0, cur = -1; unit_at(tile, typ); tile += gridDim.x) {
         if (typ != cur && cur >= 0) __syncthreads();
         cur = typ;
@@ -781,11 +801,12 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
     uint8_t* units = smem + L.off_scr + (warp - 8) * L.nu * TS_UNIT;
     const int c4 = lane & 3;  // the unit's columns 4 c4 .. of rows 8 j + lane / 4 are this lane's to copy
     const bool vec = (D & 3) == 0 && (reinterpret_cast<uintptr_t>(p.obs) & 15) == 0;
-    uint32_t c_episodes = 0, c_trunc = 0, st_bits = 0, g = 0, loads = 0;
-    int nt = 0;
+    uint32_t c_episodes = 0, c_trunc = 0, st_bits = 0, g = 0, loads = TYPED ? 0 : 1;
+    int nt = n;
+    if constexpr (HIDE_NT) asm volatile("" : "+r"(nt));
     bool fresh = true;
     for (int tile = blockIdx.x, typ = 0, cur = -1; unit_at(tile, typ); tile += gridDim.x) {
-      if (typ != cur) {
+      if (TYPED && typ != cur) {
         cur = typ;
         nt = rows_per_env(typ);
         fresh = true;
@@ -1104,11 +1125,12 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
     const int row = tid & 127, grp = warp >> 2;
     const uint32_t tm = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     uint32_t c_steps = 0, c_explore = 0, c_noavail = 0;  // (a launch's rows x steps of one thread)
-    uint32_t st_bits = 0, g = 0, loads = 0;
-    int nt = 0;
+    uint32_t st_bits = 0, g = 0, loads = TYPED ? 0 : 1;
+    int nt = n;
+    if constexpr (HIDE_NT) asm volatile("" : "+r"(nt));
     bool fresh = true;
     for (int tile = blockIdx.x, typ = 0, cur = -1; unit_at(tile, typ); tile += gridDim.x) {
-      if (typ != cur) {
+      if (TYPED && typ != cur) {
         cur = typ;
         nt = rows_per_env(typ);
         fresh = true;
@@ -1395,12 +1417,19 @@ int launch_actor_tcs(const ActorParams& p_in, int sms, bool fast_gates, cudaStre
   }
   p.ept = L.ept;
   p.num_tiles = (p.M + L.ept - 1) / L.ept;
-  const int v = fast_gates ? 8 : (ns == 3 ? 0 : 4) + (L.NQ == 16 ? 0 : 2) + (p.H == 64 ? 0 : 1);
-  decltype(&actor_tcs_kernel<3, 16, 64>) kernels[9] = {
-      actor_tcs_kernel<3, 16, 64>, actor_tcs_kernel<3, 16, 128>, actor_tcs_kernel<3, 32, 64>, actor_tcs_kernel<3, 32, 128>,
-      actor_tcs_kernel<1, 16, 64>, actor_tcs_kernel<1, 16, 128>, actor_tcs_kernel<1, 32, 64>, actor_tcs_kernel<1, 32, 128>,
-      actor_tcs_kernel<1, 16, 128, true>};
-  static uint32_t configured[9][SMEM_OPTIN_DEVICES];
+  // One network or one per type, accurate gates: [types][pieces][actions][hidden]; the hardware's gates are the last.  In fp32 at
+  // hidden 64 launches of several steps go to the kernel for several types with one network too: there that one is the faster
+  // (4096 environments x 8 agents x 64 steps 1028 us against 1039, 1482 x 5 x 28 steps 230.7 against 234.1), in one-step launches it
+  // is not (9001 x 5 agents 53.4 against 52.0).
+  const bool typed = ntypes > 1 || (ns == 3 && p.H == 64 && L.NQ == 16 && p.T > 1);
+  const int v = fast_gates ? 16 : (typed ? 8 : 0) + (ns == 3 ? 0 : 4) + (L.NQ == 16 ? 0 : 2) + (p.H == 64 ? 0 : 1);
+  decltype(&actor_tcs_kernel<3, 16, 64, false>) kernels[17] = {
+      actor_tcs_kernel<3, 16, 64, false>, actor_tcs_kernel<3, 16, 128, false>, actor_tcs_kernel<3, 32, 64, false>, actor_tcs_kernel<3, 32, 128, false>,
+      actor_tcs_kernel<1, 16, 64, false>, actor_tcs_kernel<1, 16, 128, false>, actor_tcs_kernel<1, 32, 64, false>, actor_tcs_kernel<1, 32, 128, false>,
+      actor_tcs_kernel<3, 16, 64, true>, actor_tcs_kernel<3, 16, 128, true>, actor_tcs_kernel<3, 32, 64, true>, actor_tcs_kernel<3, 32, 128, true>,
+      actor_tcs_kernel<1, 16, 64, true>, actor_tcs_kernel<1, 16, 128, true>, actor_tcs_kernel<1, 32, 64, true>, actor_tcs_kernel<1, 32, 128, true>,
+      actor_tcs_kernel<1, 16, 128, false, true>};
+  static uint32_t configured[17][SMEM_OPTIN_DEVICES];
   {
     const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernels[v]), L.total, configured[v]);
     if (e != cudaSuccess) return -(int)e;
