@@ -484,7 +484,6 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
                 const uint32_t head = B0 > A0 ? (uint32_t)((B0 < A1 ? B0 : A1) - A0) : 0u;
                 if ((uint32_t)lane < head) to[A0 - base + lane] = a[lane];
                 if (B1 < A1 && (uint32_t)lane < (uint32_t)(A1 - B1)) to[B1 - base + lane] = reinterpret_cast<const uint8_t*>(B1)[lane];
-                if (head != 0 || B1 < A1) fence_proxy_async_smem();  // (a later bulk copy writes these bytes of the slot)
                 from = reinterpret_cast<const uint8_t*>(B0);
                 at = to + (B0 - base);
                 return (uint32_t)(B1 - B0);
@@ -516,6 +515,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
             if (++qslot == (uint32_t)NS) {
               qslot = 0;
               qpar ^= 1u;
+              if constexpr (RAGGED) fence_proxy_async_smem();  // (bulk copies write the slots again, over bytes that lanes wrote)
             }
           }
         }
