@@ -1099,7 +1099,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
               if (wrow0 + rl < R) reinterpret_cast<uint4*>(p.h + (size_t)g * TC_H + cb)[lane & 7] = v;
             }
             __syncwarp();
-            next_rows();
+            if (tile + (int)gridDim.x < p.num_tiles) next_rows();  // (the next tile's prologue waits for them)
           }
         }
         mbar_wait(&B->fc2d, par, abortf);   // (both halves: the hidden operand may be cleared below)
