@@ -138,13 +138,24 @@ def test_host_step_on_pinned_and_pageable_arrays(over):
     dev.destroy()
 
 
-# (The first launch has to last 1.2 s: at 5.0 us a step, which is less than the kernel takes in fp32 - 5.38 -, 240 000 steps do.)
 @pytest.mark.parametrize("prec,H,T", [("fp32", 64, 240_000), ("bf16", 128, 300_000)])
 def test_launch_behind_a_long_one(prec, H, T):
     """A launch that starts beside its predecessor while that still runs for longer than a bounded wait lasts (about a
     second): the wait for the predecessor counts against none of its own waits."""
     cfg = workloads.small_config(H=H, E=1, n=4, D=8, A=4, C=2, L=50, precision=prec, seed=5)
     w = workloads.make_weights(cfg)
+    # steps for a first launch of 1.5 s, whatever a step takes: timed over a twelfth of T, the second of two launches
+    a = binding.Actor(cfg, work_steps=1)
+    a.set_weights(w)
+    probe = a.env_generate(cfg["env"], 0, T // 12)
+    ev = [torch.cuda.Event(enable_timing=True) for _ in range(3)]
+    for e in ev[:2]:
+        e.record()
+        a.rollout_staged(*probe, T // 12, 0.2)
+    ev[2].record()
+    torch.cuda.synchronize()
+    a.destroy()
+    T = max(T, int(1500.0 / ev[1].elapsed_time(ev[2]) * (T // 12)))
     states = []
     for together in (True, False):
         a = binding.Actor(cfg, work_steps=1)
