@@ -63,6 +63,7 @@ def test_inputs_that_start_and_end_anywhere(kind, shape):
     written = np.arange(cfg["L"])[None, :] < sess.ring["slot_len"][:, None]
     for k in ("obs", "avail", "action", "reward", "done"):
         assert np.array_equal(rv[k].cpu().numpy()[written], sess.ring[k][written]), k
+    assert row_rel_err(rv["q"].cpu().numpy()[written], sess.ring["q"][written]).max() <= RTOL["bf16"]
     assert actor.status()[0] == 0
     actor.destroy()
 
@@ -88,3 +89,85 @@ def test_staging_slots_that_held_the_ends_of_an_array(kind):
         a.destroy()
     for h, ring in got[1:]:
         assert torch.equal(h, got[0][0]) and torch.equal(ring, got[0][1])
+
+
+def _pair(shape):
+    cfg = workloads.small_config(**{**dict(H=64, L=4, T=7, precision="bf16", env=dict(done_thresh24=1 << 21)), **shape, "C": 2 * shape["E"]})
+    actors = [binding.Actor(cfg) for _ in range(2)]
+    for a in actors:
+        a.set_weights(workloads.make_weights(cfg))
+    return cfg, actors, actors[0].env_generate(cfg["env"], 0, cfg["T"])
+
+
+def _same(one, two):
+    torch.cuda.synchronize()
+    s, u = one.get_state(), two.get_state()
+    for k in ("h", "last_action", "slot", "pos", "ep_count"):
+        assert torch.equal(s[k], u[k]), k
+    assert torch.equal(one.ring_mem, two.ring_mem)
+    for a in (one, two):
+        assert a.status()[0] == 0
+        a.destroy()
+
+
+@pytest.mark.parametrize("shape", SHAPES[:3])
+def test_pinned_host_arrays_of_a_batch_that_ends_anywhere(shape):
+    """A host step that reads the caller's pinned arrays in place: what the step on device arrays gives."""
+    cfg, (dev, pin), x = _pair(shape)
+    for t in range(cfg["T"]):
+        want = dev.step(*[v[t] if v[t].data_ptr() % 16 == 0 else _at(v[t], 0) for v in x], 0.15)
+        got = pin.step_host(*[v[t].cpu().pin_memory() for v in x], 0.15, torch.empty_like(want, device="cpu").pin_memory())
+        assert torch.equal(got, want.cpu()), t
+        assert dev.step_kernel == pin.step_kernel == "actor_tcp_kernel"
+    _same(dev, pin)
+
+
+@pytest.mark.parametrize("kind", ["step", "subset", "lagged"])
+def test_captured_steps_on_inputs_that_start_anywhere(kind):
+    """Two steps in one graph, replayed: what the same steps give one by one.  (Nothing explores: the draws of a replay are those
+    of its capture.)"""
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        cfg, (cap, ref), x = _pair(SHAPES[0])
+        E, n = cfg["E"], cfg["n"]
+        inputs = [[_at(v[t], o) for v, o in zip(x, (t % 4, t, 0, 0))] for t in range(cfg["T"])]
+        lists = [np.random.default_rng(t).permutation(E).astype(np.int32) for t in range(cfg["T"])]
+        out = [torch.empty((E, n), dtype=torch.int32, device="cuda") for _ in range(cfg["T"])]
+        torch.cuda.synchronize()
+
+        def call(a, t, to=None):
+            if kind == "step":
+                return a.step(*inputs[t], 0.0, to)
+            return a.step_subset(lists[t], *inputs[t], 0.0, lagged=kind == "lagged", actions_out=to)
+        call(cap, 0)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=side):
+            for t in (1, 2):
+                call(cap, t, out[t])
+            assert cap.step_kernel == "actor_tcp_kernel"
+        graph.replay()
+        out[3] = call(cap, 3)
+        want = [call(ref, t) for t in range(4)]
+        torch.cuda.synchronize()
+        assert all(torch.equal(out[t], want[t]) for t in (1, 2, 3))
+        _same(cap, ref)
+    graph.reset()
+
+
+@pytest.mark.parametrize("kind", ["step", "subset", "lagged"])
+def test_a_published_network_on_inputs_that_start_anywhere(kind):
+    """A network published for step 3 is the one that steps 3 and later use, as if it had been loaded there."""
+    cfg, (pub, ref), x = _pair(SHAPES[1])
+    new = workloads.make_weights(cfg, seed=977)
+    ids = np.random.default_rng(1).permutation(cfg["E"]).astype(np.int32)
+    for t in range(cfg["T"]):
+        if t == 1:
+            pub.publish_weights(new, version=2, effective_step=3)
+        if t == 3:
+            ref.set_weights(new, version=2)
+        inputs = [_at(v[t], o) for v, o in zip(x, (1 + t % 3, 2 * t + 1, 0, 0))]
+        a, b = (m.step(*inputs, 0.15) if kind == "step" else m.step_subset(ids, *inputs, 0.15, lagged=kind == "lagged") for m in (pub, ref))
+        assert torch.equal(a, b), t
+        assert pub.step_kernel == ref.step_kernel == "actor_tcp_kernel"
+    assert pub.weights_version == ref.weights_version == 2
+    _same(pub, ref)

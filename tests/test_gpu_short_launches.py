@@ -58,9 +58,29 @@ def test_lists_of_several_tiles_a_block_equal_full_steps():
         c = late.step_lagged(ids, obs[t][sel], avail[t][sel], rew[prev][sel], done[prev][sel], 0.2)
         assert torch.equal(a[sel], b) and torch.equal(a[sel], c), t
     assert all(x.step_kernel == "actor_tcp_kernel" for x in actors)
-    s, u = dense.get_state(), listed.get_state()
+    s, u, v = dense.get_state(), listed.get_state(), late.get_state()
+    rd, rl, rt = dense.ring_view(), listed.ring_view(), late.ring_view()
     for k in ("h", "last_action", "slot", "pos", "ep_count"):
         assert torch.equal(s[k], u[k]), k
+    written = torch.arange(cfg["L"], device=obs.device)[None, :] < rd["slot_len"][:, None]
+    for k in ("slot_epid", "slot_len", "slot_complete"):
+        assert torch.equal(rd[k], rl[k]), k
+    for k in ("obs", "avail", "action", "q", "reward", "done"):
+        assert torch.equal(rd[k][written], rl[k][written]), k
+    # the late actor: everything but the outcome of its last step, which has not arrived
+    going = s["pos"] > 0                                  # (the others' episodes end with that outcome)
+    for k in ("h", "last_action", "slot", "pos", "ep_count"):
+        assert torch.equal(s[k][going], v[k][going]), k
+    assert torch.equal(rd["slot_len"], rt["slot_len"]) and torch.equal(rd["slot_epid"], rt["slot_epid"])
+    ends = torch.zeros_like(rd["slot_complete"])
+    ends[v["slot"][~going].long()] = 1
+    assert torch.equal(rd["slot_complete"], rt["slot_complete"] | ends)
+    for k in ("obs", "avail", "action", "q"):
+        assert torch.equal(rd[k][written], rt[k][written]), k
+    told = written.clone()
+    told[v["slot"].long(), v["pos"].long() - 1] = False
+    for k in ("reward", "done"):
+        assert torch.equal(rd[k][told], rt[k][told]), k
     for a in actors:
         assert a.status()[0] == 0
         a.destroy()
