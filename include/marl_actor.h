@@ -66,7 +66,9 @@ extern "C" {
                                         * so do calls whose availability block (batch * n_agents * n_actions bytes)
                                         * is not a 16-byte multiple when an environment's is not, and calls with an
                                         * environment count that is not a multiple of 4 when obs_dim is not a
-                                        * multiple of 8 */
+                                        * multiple of 8.  (MARL_KERNEL_AUTO: large one-step calls of the latter two
+                                        * kinds stay on the pipelined kernel, with the gate functions of the kernel that
+                                        * takes the actor's launches of several steps) */
 
 #define MARL_MAX_AGENT_TYPES 4
 
@@ -192,7 +194,8 @@ int marl_actor_create(const marl_actor_config_t* cfg, marl_actor_t** out);
 /* Loads the network (Algorithm 2: an iteration starts by fetching the current parameters).  HOST fp32 arrays in
  * [out][in] layout, copied and repacked before the call returns to the caller's stream order:
  *   W1 [H][D+n+A], b1 [H], W_ih [3H][H], b_ih [3H], W_hh [3H][H], b_hh [3H] (row blocks r|z|n),
- *   W2 [A][H], b2 [A].  In bf16 precision the four matrices are rounded to bf16 (RNE); biases stay fp32.
+ *   W2 [A][H], b2 [A].  In bf16 precision the four matrices are rounded to bf16 (RNE); biases stay fp32,
+ *   infinite ones and those beyond bf16's range among them.
  * version is stored and returned by marl_actor_weights_version. */
 int marl_actor_set_weights(marl_actor_t* a, const float* W1, const float* b1, const float* W_ih,
                            const float* b_ih, const float* W_hh, const float* b_hh, const float* W2,
@@ -205,7 +208,7 @@ int marl_actor_set_weights(marl_actor_t* a, const float* W1, const float* b1, co
  * in [0, n_types); the eight weight arrays as for marl_actor_set_weights with a leading [n_types] axis
  * (W1 [K][H][D+n+A], b1 [K][H], ...).  n_types must not exceed the n_agent_types the actor was created with.
  * Blocking, like marl_actor_set_weights, and a pending publication is dropped.  With n_types > 1 the steps run on
- * the general kernel (both precisions; a tile's rows of one type at a time), marl_actor_publish_weights is
+ * the general kernel (both precisions; a tile holds the rows of one type), marl_actor_publish_weights is
  * refused, and marl_actor_kernel_name reports "ffma"; a later marl_actor_set_weights returns to the shared network
  * and the kernel chosen at creation. */
 int marl_actor_set_weights_typed(marl_actor_t* a, int32_t n_types, const int32_t* agent_type, const float* W1,
@@ -242,7 +245,9 @@ int marl_actor_step(marl_actor_t* a, const float* obs, const uint8_t* avail, con
  * done u8[M], actions_out i32[M][n] (may be NULL).  The call consumes one index of the global step counter, which
  * keys the exploration stream as (seed, step, environment, agent) with the environment's own index; a trace row
  * of this step is written at the environment's own index as well.  Runs on the pipelined tensor-core kernel where
- * the actor uses it and the arrays can be bulk-copied (16-byte aligned obs and avail), else on the general kernel.
+ * the actor uses it and obs and avail start and end on 16-byte boundaries.  With the automatic choice it also does where they do not,
+ * obs_dim is not a multiple of 8 or n_agents * n_actions not one of 16, and the list is longer than about half a tile of 128 rows a
+ * multiprocessor, then with the general kernel's accurate gate functions; else on the general kernel.
  * May be captured into a graph, from the actor's first list step on or before: a captured call keeps its list in pinned memory of
  * its own until the actor is destroyed (a replay reads it again). */
 int marl_actor_step_subset(marl_actor_t* a, const int32_t* env_ids, int32_t M, const float* obs,

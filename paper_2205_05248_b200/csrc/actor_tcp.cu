@@ -246,7 +246,7 @@ __device__ __forceinline__ void tp_issue_hside(const TpLayout& L, uint32_t sb, u
 // MODE 3: MODE 0 for launches of a few steps, where the tile-to-tile transition is a large part of the time: the
 // hidden-state rows then move coalesced through a scratch.  They leave while fc2 runs, the next tile's come behind them by
 // cp.async while the choice is made, and the cursors and outcomes of the next tile are requested during this one (modes 1
-// and 2 do the same): a list step of 32768 x 8 agents 115.3 -> 89.5 us, 12 to 14 k clocks a tile -> some 9 k.  Launches of many
+// and 2 do the same): a list step of 32768 x 8 agents 115 -> 90 us, 12 to 14 k clocks a tile -> some 9 k.  Launches of many
 // steps keep the shorter transition code: its footprint in the step loop's instruction stream and registers costs them more
 // (1.2 %) than the transition saves.
 // RAGGED (one step per launch, PM != 0): inputs that start (PM 1: observations on any float; availability on any byte) and end
@@ -987,7 +987,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
         uint8_t* tl = tails + b * tail_set + (uint32_t)el * L.tail_bytes;  // this row's environment tail
 
         // ---- epilogue 1: y = relu(fc1 + W1[:, last action]) -> bf16 operand.  Bias and agent-id column are
-        //      inside the GEMM; fc1 itself finished during the previous step. ----
+        //      inside the GEMM (accurate gates: added here); fc1 itself finished during the previous step. ----
         mbar_wait(&B->fc1d, par, abortf);
         tc_fence_after_sync();
         {
@@ -1227,16 +1227,17 @@ bool tcp_takes_batch(int n, int D, int A, int M) {
 }
 
 // Returns the number of kernels launched, 0 if this launch's pointers do not meet the kernel's alignment
-// needs (the caller then uses the one-tile kernel), or a negative cudaError.
+// needs (the caller then uses another kernel), or a negative cudaError.
 int launch_actor_tcp(const ActorParams& p_in, int sms, cudaStream_t stream) {
   const int mode = p_in.env_ids == nullptr ? (p_in.T < 8 ? 3 : 0) : (p_in.lagged ? 2 : 1);
   // plain shapes: a last chunk of fewer environments need not be a 16-byte multiple, and the aligned range around the last
   // chunk's availability bytes may end beyond the step's block; nor need the arrays of one call start on 16-byte boundaries.
   // One-step launches take such inputs from half a tile a block on (split-operand kernel -> this one, us): lists of 5 x 55
-  // observations, 801 environments 19.3 -> 19.0, 1801 22.0 -> 21.7, 3601 29.0 -> 24.7, 9001 with late outcomes 51.2 -> 34.5, 33333 142 -> 81; dense steps of
-  // 16385 x 5 65 -> 44 (one-tile kernel) and 70 -> 44.  The errors against the oracle are the split-operand kernel's (rms of Q
-  // 3.0e-5 to 4.1e-5, of h 2.1e-6, on both): gates and biases are the same fp32 arithmetic, with biases and agent columns
-  // among the products they were 20 to 45 % larger.
+  // observations, 801 environments 19.3 -> 19.0, 1801 22.0 -> 21.7, 3601 29.0 -> 24.7, 9001 with late outcomes 51 -> 35, 33333 142 -> 81; dense steps of
+  // 16385 x 5, 55 observations 70 -> 44, 80 observations 65 (one-tile kernel) -> 42.
+  // Where the split-operand kernel had these calls the errors against the oracle are its own (rms of Q 3.0e-5 to 4.1e-5, of h 2.1e-6,
+  // on both): gates and biases are the same fp32 arithmetic, with biases and agent columns among the products they were 20 to 45 %
+  // larger.
   const int plain = p_in.D % 8 != 0 ? 1 : (p_in.n * p_in.A) % 16 != 0 ? 2 : 0;
   const bool aligned = reinterpret_cast<uintptr_t>(p_in.obs) % 16 == 0 && reinterpret_cast<uintptr_t>(p_in.avail) % 16 == 0;
   const bool whole = aligned && (p_in.obs_step_stride * 4) % 16 == 0 && p_in.avail_step_stride % 16 == 0 &&

@@ -1,4 +1,4 @@
-// Accurate gate functions of the GRU cell, two columns at a time (split-operand kernel; pipelined kernel's ragged inputs).
+// Accurate gate functions of the GRU cell, two columns at a time (split-operand kernel; accurate variant of the pipelined kernel).
 #pragma once
 
 #include <cuda_runtime.h>

@@ -866,7 +866,7 @@ static int step_list(marl_actor* a, const int32_t* env_ids, int32_t M, const flo
   p.lagged = lagged ? 1 : 0;
   int rc = 0;
   const char* kernel = "actor_tcp_kernel";
-  if (a->use_tcp && c.hidden != 128) {  // 0: these pointers or this list length cannot be bulk-copied
+  if (a->use_tcp && c.hidden != 128) {  // 0: inputs off 16-byte boundaries and too few of them
     tc_tiling(M, c.n_agents, a->sms, &p.ept, &p.num_tiles);
     rc = launch_actor_tcp(p, a->sms, a->stream);
   }
